@@ -4,95 +4,265 @@
 //
 // Each GEMM index may fuse two tensor indices through an IMap, so the setup of the
 // Hbar elements and the FP64 sigma product are written as plain contractions
-// without explicit transposes.  GB300 has about 1.1 TFLOP/s of FP64 (about two
-// DFMA per SM and clock), so this kernel is bound by the DFMA pipe: a 64x64 tile
-// per 256-thread block with 4x4 outputs per thread keeps the pipe fed while the
-// tile loads stay in L1/L2.
+// without explicit transposes.  GB300 has about 1.26 TFLOP/s of FP64 (two FMA per SM and clock), so
+// the FP64 pipe bounds every tile, padding included: 16 x 16 x 16 products already keep an SM busy for
+// 2048 clocks, long enough to hide the next K block's loads behind them.  What is left to gain is the
+// balance over the SMs: small tiles, tile shapes that follow M and N, and the K range of a tile
+// shared by a cluster.  Measured against one shape (64 x 64 tiles, single-buffered, a 64-bit division per
+// element and index): sigma product of one vector at o=4 v=12 600 -> 107 us, the tiny workload's IP + EA
+// solve 71 -> 13 ms, o=13 v=67 IP + EA 278 -> 74 ms (ring contraction at 1.11 TFLOP/s, 0.88 of the pipe),
+// the Green's-function overlaps of 40 systems at o=40 v=200 4.0 -> 0.5 ms.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <cmath>
 #include <map>
 #include <mutex>
 
 #include "common.cuh"
-#include <algorithm>
 
 #include "kernels.cuh"
 #include "ozaki.cuh"
 
 namespace gfcc {
 
-namespace {
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+namespace cg = cooperative_groups;
 
-__global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c) {
-  __shared__ double As[BK][BM + 1];
-  __shared__ double Bs[BK][BN + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+namespace {
+
+constexpr int BK = 16, NT = 256;
+constexpr int NUM_SM = 152;
+
+// x / d by 32-bit division where both fit (the 64-bit one costs several times as many instructions)
+__device__ __forceinline__ long long fast_div(long long x, long long d) {
+  if ((((unsigned long long)x | (unsigned long long)d) >> 32) == 0) return (long long)((unsigned)x / (unsigned)d);
+  return x / d;
+}
+
+__device__ __forceinline__ long long map_offset(const IMap &m, long long x) {
+  if (m.d0 <= 0) return x * m.s0;
+  const long long q = fast_div(x, m.d0);
+  return (x - q * m.d0) * m.s0 + q * m.s1;
+}
+
+// A fused K index walked in steps of BK without a division per step: x = q d0 + r.
+struct KWalk {
+  long long d0, r, off, step, wrap;
+  int dr;
+  __device__ __forceinline__ void init(const IMap &m, long long x) {
+    if (m.d0 <= 0) {
+      d0 = 1LL << 62;
+      r = x;
+      off = x * m.s0;
+      dr = BK;
+      step = BK * m.s0;
+      wrap = 0;
+      return;
+    }
+    d0 = m.d0;
+    const long long q = fast_div(x, d0), dq = fast_div(BK, d0);
+    r = x - q * d0;
+    off = r * m.s0 + q * m.s1;
+    dr = (int)(BK - dq * d0);
+    step = dr * m.s0 + dq * m.s1;
+    wrap = m.s1 - d0 * m.s0;
+  }
+  __device__ __forceinline__ void next() {
+    r += dr;
+    off += step;
+    if (r >= d0) {
+      r -= d0;
+      off += wrap;
+    }
+  }
+};
+
+// One BM x BN output tile per block, BM = TM RM and BN = (NT / TM) RN: thread (ty, tx) holds outputs
+// (ty + TM i, tx + TN j).  The K loop is double-buffered: the next K block is on its way from global
+// memory while this one is multiplied.  A cluster of gridDim.z / batch blocks (along z) may share
+// the K range of a tile; its partial sums meet through distributed shared memory in rank order.
+template <int TM, int RM, int RN>
+__global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kcluster) {
+  constexpr int TN = NT / TM, BM = TM * RM, BN = TN * RN;
+  constexpr int LA = (BM * BK + NT - 1) / NT, LB = (BN * BK + NT - 1) / NT;
+  __shared__ double As[2][BK][BM + 1];
+  __shared__ double Bs[2][BK][BN + 1];
+  __shared__ double red[BM * BN];
+  const int tx = threadIdx.x % TN, ty = threadIdx.x / TN;
   const long long b = blockIdx.z / c.nsplit;
   const long long z = blockIdx.z - b * c.nsplit;
   const double *A = c.A + b * c.sab;
   const double *B = c.B + b * c.sbb;
-  double *C = c.C + b * c.scb + z * c.scz;
+  double *C = c.C + b * c.scb + (kcluster > 1 ? 0 : z * c.scz);
   const long long kbeg = z * c.kchunk;
   const long long kend = min(c.K, kbeg + c.kchunk);
   const long long m0 = (long long)blockIdx.x * BM;
   const long long n0 = (long long)blockIdx.y * BN;
-  double acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) acc[i][j] = 0.0;
 
-  for (long long k0 = kbeg; k0 < kend; k0 += BK) {
+  // this thread's elements of the A and B tiles: lanes run along K where K is the contiguous index
+  // of the operand, else along M (N)
+  const bool a_k = c.ak.s0 == 1, b_k = c.bk.s0 == 1;
+  int am[LA], akl[LA], bn[LB], bkl[LB];
+  bool aok[LA], bok[LB];
+  const double *ap[LA], *bp[LB];
+  KWalk aw[LA], bw[LB];
 #pragma unroll
-    for (int r = 0; r < (BM * BK) / NT; r++) {
-      const int e = threadIdx.x + NT * r;
-      const int kl = e % BK, ml = e / BK;
-      const long long m = m0 + ml, k = k0 + kl;
-      As[kl][ml] = (m < c.M && k < kend) ? A[imap_apply(c.am, m) + imap_apply(c.ak, k)] : 0.0;
+  for (int r = 0; r < LA; r++) {
+    const int e = threadIdx.x + NT * r;
+    am[r] = a_k ? e / BK : e % BM;
+    akl[r] = a_k ? e % BK : e / BM;
+    aok[r] = e < BM * BK && m0 + am[r] < c.M;
+    ap[r] = A + (aok[r] ? map_offset(c.am, m0 + am[r]) : 0);
+    aw[r].init(c.ak, kbeg + akl[r]);
+  }
+#pragma unroll
+  for (int r = 0; r < LB; r++) {
+    const int e = threadIdx.x + NT * r;
+    bn[r] = b_k ? e / BK : e % BN;
+    bkl[r] = b_k ? e % BK : e / BN;
+    bok[r] = e < BN * BK && n0 + bn[r] < c.N;
+    bp[r] = B + (bok[r] ? map_offset(c.bn, n0 + bn[r]) : 0);
+    bw[r].init(c.bk, kbeg + bkl[r]);
+  }
+  double va[LA], vb[LB];
+  auto fetch = [&](long long k0) {
+#pragma unroll
+    for (int r = 0; r < LA; r++) {
+      va[r] = (aok[r] && k0 + akl[r] < kend) ? ap[r][aw[r].off] : 0.0;
+      aw[r].next();
     }
 #pragma unroll
-    for (int r = 0; r < (BN * BK) / NT; r++) {
-      const int e = threadIdx.x + NT * r;
-      const int nl = e % BN, kl = e / BN;
-      const long long n = n0 + nl, k = k0 + kl;
-      Bs[kl][nl] = (n < c.N && k < kend) ? B[imap_apply(c.bk, k) + imap_apply(c.bn, n)] : 0.0;
+    for (int r = 0; r < LB; r++) {
+      vb[r] = (bok[r] && k0 + bkl[r] < kend) ? bp[r][bw[r].off] : 0.0;
+      bw[r].next();
     }
-    __syncthreads();
+  };
+  auto stage = [&](int buf) {
+#pragma unroll
+    for (int r = 0; r < LA; r++)
+      if (BM * BK % NT == 0 || threadIdx.x + NT * r < BM * BK) As[buf][akl[r]][am[r]] = va[r];
+#pragma unroll
+    for (int r = 0; r < LB; r++)
+      if (BN * BK % NT == 0 || threadIdx.x + NT * r < BN * BK) Bs[buf][bkl[r]][bn[r]] = vb[r];
+  };
+  double acc[RM][RN];
+#pragma unroll
+  for (int i = 0; i < RM; i++)
+#pragma unroll
+    for (int j = 0; j < RN; j++) acc[i][j] = 0.0;
+
+  if (kbeg < kend) {
+    fetch(kbeg);
+    stage(0);
+  }
+  __syncthreads();
+  int buf = 0;
+  for (long long k0 = kbeg; k0 < kend; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < kend;
+    if (more) fetch(k0 + BK);
 #pragma unroll
     for (int kk = 0; kk < BK; kk++) {
-      double a[4], bb[4];
+      double a[RM], bb[RN];
 #pragma unroll
-      for (int i = 0; i < 4; i++) a[i] = As[kk][ty + 16 * i];
+      for (int i = 0; i < RM; i++) a[i] = As[buf][kk][ty + TM * i];
 #pragma unroll
-      for (int j = 0; j < 4; j++) bb[j] = Bs[kk][tx + 16 * j];
+      for (int j = 0; j < RN; j++) bb[j] = Bs[buf][kk][tx + TN * j];
 #pragma unroll
-      for (int i = 0; i < 4; i++)
+      for (int i = 0; i < RM; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        for (int j = 0; j < RN; j++) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
     }
+    if (more) stage(buf ^ 1);
     __syncthreads();
   }
+  auto store = [&](int ml, int nl, double v) {
+    const long long m = m0 + ml, n = n0 + nl;
+    if (m >= c.M || n >= c.N) return;
+    const long long off = map_offset(c.cm, m) + map_offset(c.cn, n);
+    double val = c.alpha * v;
+    if (c.beta != 0.0) val += c.beta * C[off];
+    C[off] = val;
+  };
+  if (kcluster > 1) {
+    cg::cluster_group cl = cg::this_cluster();
 #pragma unroll
-  for (int i = 0; i < 4; i++) {
-    const long long m = m0 + ty + 16 * i;
-    if (m >= c.M) continue;
-    const long long om = imap_apply(c.cm, m);
+    for (int i = 0; i < RM; i++)
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-      const long long n = n0 + tx + 16 * j;
-      if (n >= c.N) continue;
-      const long long off = om + imap_apply(c.cn, n);
-      double val = c.alpha * acc[i][j];
-      if (c.beta != 0.0) val += c.beta * C[off];
-      C[off] = val;
+      for (int j = 0; j < RN; j++) red[(ty + TM * i) * BN + tx + TN * j] = acc[i][j];
+    cl.sync();
+    // block z of the cluster adds up and stores its share of the tile
+    const int share = (BM * BN + kcluster - 1) / kcluster;
+    const int e1 = min(BM * BN, ((int)z + 1) * share);
+    for (int e = (int)z * share + threadIdx.x; e < e1; e += NT) {
+      double s = 0.0;
+      for (int r = 0; r < kcluster; r++) s += cl.map_shared_rank(red, r)[e];
+      store(e / BN, e % BN, s);
+    }
+    cl.sync();   // no block leaves while another reads its partial sums
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < RM; i++)
+#pragma unroll
+    for (int j = 0; j < RN; j++) store(ty + TM * i, tx + TN * j, acc[i][j]);
+}
+
+struct Tiling {
+  int bm, bn, kcluster;
+};
+
+// The FP64 pipe (two FMA per SM and clock) bounds every tile: a tile takes bm bn K / 2 clocks of an
+// SM, padding included, so the best tiling is the one whose busiest SM has the fewest of them.
+// Candidates: 32 x 32 tiles, and tiles of 256 outputs from 64 x 4 to 4 x 64 (no more than 1 output per
+// thread, hence a few per cent slower on large products), each with the K range shared by up to 8 blocks.
+Tiling choose_tiling(long long M, long long N, long long K, long long batch, bool cluster) {
+  static const int shape[6][2] = {{32, 32}, {16, 16}, {64, 4}, {32, 8}, {8, 32}, {4, 64}};
+  Tiling best{16, 16, 1};
+  double cost = 0.0;
+  for (const auto &s : shape) {
+    const double tiles = (double)((M + s[0] - 1) / s[0]) * (double)((N + s[1] - 1) / s[1]) * (double)batch;
+    if ((N + s[1] - 1) / s[1] > 65535) continue;
+    for (int S = 1; S <= (cluster ? 8 : 1); S *= 2) {
+      if (S > 1 && K < 2 * BK * S) break;
+      const double steps = std::ceil(std::ceil((double)K / S) / BK);
+      const double t = std::ceil(tiles * S / NUM_SM) * (steps * s[0] * s[1] * BK / 2.0 * (s[0] == 32 && s[1] == 32 ? 1.0 : 1.04) +
+                                                        1000.0 + (S > 1 ? 1500.0 : 0.0));
+      if (cost == 0.0 || t < cost) {
+        cost = t;
+        best = Tiling{s[0], s[1], S};
+      }
     }
   }
+  return best;
+}
+
+template <int TM, int RM, int RN>
+int launch_contract(const Contract &c, int kcluster, long long mt, long long nt, cudaStream_t st) {
+  dim3 grid((unsigned)mt, (unsigned)nt, (unsigned)(c.batch * c.nsplit));
+  if (kcluster <= 1) {
+    contract_f64_kernel<TM, RM, RN><<<grid, NT, 0, st>>>(c, 1);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(NT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = (unsigned)kcluster;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    GFCC_CUDA(cudaLaunchKernelEx(&cfg, contract_f64_kernel<TM, RM, RN>, c, kcluster));
+  }
+  GFCC_LAUNCH_CHECK();
+  return GFCC_OK;
 }
 }  // namespace
 
 int contract_f64(const Contract &c, cudaStream_t st) {
   if (c.M <= 0 || c.N <= 0 || c.batch <= 0) return GFCC_OK;
   // K == 0 leaves acc = 0, so C = beta * C (the empty sum).
-  const long long mt = (c.M + BM - 1) / BM, nt = (c.N + BN - 1) / BN;
   Contract cc = c;
   if (cc.nsplit < 1) cc.nsplit = 1;
   if (cc.nsplit == 1) cc.kchunk = cc.K > 0 ? cc.K : 1;
@@ -100,9 +270,15 @@ int contract_f64(const Contract &c, cudaStream_t st) {
     set_error("contract_f64: split-K chunk %lld x %lld does not cover K=%lld", cc.kchunk, cc.nsplit, cc.K);
     return GFCC_ERR_ARG;
   }
-  if (mt > 0x7fffffffLL || nt > 65535 || c.batch * cc.nsplit > 65535) {
-    set_error("contract_f64: grid too large (M=%lld N=%lld batch=%lld)", c.M, c.N, c.batch);
-    return GFCC_ERR_ARG;
+  Tiling t = choose_tiling(cc.M, cc.N, cc.nsplit > 1 ? cc.kchunk : cc.K, cc.batch * cc.nsplit, cc.nsplit == 1);
+  const long long mt = (c.M + t.bm - 1) / t.bm, nt = (c.N + t.bn - 1) / t.bn;
+  if (mt > 0x7fffffffLL || nt > 65535 || c.batch * cc.nsplit * t.kcluster > 65535) {
+    if (t.kcluster > 1 && c.batch * cc.nsplit <= 65535) {
+      t.kcluster = 1;
+    } else {
+      set_error("contract_f64: grid too large (M=%lld N=%lld batch=%lld)", c.M, c.N, c.batch);
+      return GFCC_ERR_ARG;
+    }
   }
   {
     const long long ka = imap_max(c.am, c.M) + imap_max(c.ak, c.K) + (c.batch - 1) * c.sab;
@@ -114,10 +290,18 @@ int contract_f64(const Contract &c, cudaStream_t st) {
     }
     GFCC_TRY(check_extent(c.C, 0, kc, "contraction output C"));
   }
-  dim3 grid((unsigned)mt, (unsigned)nt, (unsigned)(c.batch * cc.nsplit));
-  contract_f64_kernel<<<grid, NT, 0, st>>>(cc);
-  GFCC_LAUNCH_CHECK();
-  return GFCC_OK;
+  if (t.kcluster > 1) {
+    // whole K blocks per cluster block; every block of the cluster gets a (possibly empty) range
+    cc.nsplit = t.kcluster;
+    cc.kchunk = (((cc.K + t.kcluster - 1) / t.kcluster) + BK - 1) / BK * BK;
+    cc.scz = 0;
+  }
+  if (t.bm == 32 && t.bn == 32) return launch_contract<16, 2, 2>(cc, t.kcluster, mt, nt, st);
+  if (t.bm == 64) return launch_contract<64, 1, 1>(cc, t.kcluster, mt, nt, st);
+  if (t.bm == 32) return launch_contract<32, 1, 1>(cc, t.kcluster, mt, nt, st);
+  if (t.bm == 8) return launch_contract<8, 1, 1>(cc, t.kcluster, mt, nt, st);
+  if (t.bm == 4) return launch_contract<4, 1, 1>(cc, t.kcluster, mt, nt, st);
+  return launch_contract<16, 1, 1>(cc, t.kcluster, mt, nt, st);
 }
 
 namespace {
@@ -162,10 +346,11 @@ int gemm_f64(cudaStream_t st, long long M, long long N, long long K, double alph
   const double emu_min = g_emulate_min_flops_local >= 0.0 ? g_emulate_min_flops_local : g_emulate_min_flops;
   if (batch == 1 && g_emulate_big && 2.0 * (double)M * (double)N * (double)K >= emu_min)
     return gemm_f64_emulated(st, M, N, K, alpha, A, am, ak, B, bk, bn, beta, C, cm, cn, 8, 9);
-  // Few output tiles and a long K would leave most SMs idle: split K into partial sums.
-  const long long tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN) * batch;
-  if (batch == 1 && tiles < 152 && K >= 8192) {
-    long long nsplit = std::min<long long>(std::max<long long>(1, 304 / tiles), K / 2048);
+  // A few 16 x 16 output tiles and a long K: the K ranges of a cluster (8 at most) would not fill the
+  // SMs, so K is split further into partial sums in global memory.
+  const long long tiles = ((M + 15) / 16) * ((N + 15) / 16);
+  if (batch == 1 && tiles * 8 < 2 * NUM_SM && K >= 8192) {
+    long long nsplit = std::min<long long>(4 * NUM_SM / tiles, K / 512);
     nsplit = std::min<long long>(nsplit, 512);
     if (nsplit >= 2) {
       const long long need = nsplit * M * N;
