@@ -78,7 +78,7 @@ extern "C" {
                                      gfcc_solve (for gfcc_mlp_collect); default 0                        */
 #define GFCC_OPT_EMU_FUSED_N 16   /* FP64-accurate products with at most this many columns run all digit
                                      pairs of a tile in one kernel (levels in TMEM); wider ones one GEMM
-                                     per digit pair.  Process-wide; default 512                          */
+                                     per digit pair.  Process-wide; default: every width                  */
 #define GFCC_OPT_GRAPHS     15    /* 1 (default): the Arnoldi steps of the inner solves of the mixed
                                      refinement are captured once per batch size into CUDA graphs and
                                      replayed (not while profiling, not on the legacy default stream)    */

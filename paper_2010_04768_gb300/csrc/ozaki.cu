@@ -25,8 +25,8 @@
 namespace gfcc {
 
 // products with at most this many columns take the fused kernel (all digit pairs of a tile in one
-// CTA, levels in TMEM); wider ones keep one GEMM per digit pair (256-column tiles)
-long long g_fused_max_n = 512;
+// CTA, levels in TMEM); wider ones, and digit counts it does not hold, one GEMM per digit pair
+long long g_fused_max_n = 1LL << 40;
 
 namespace {
 
@@ -183,9 +183,9 @@ int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, d
     set_error("emu_gemm: operands disagree in K (%lld vs %lld)", A.K, B.K);
     return GFCC_ERR_ARG;
   }
-  if (N <= g_fused_max_n && A.S <= 8 && B.S <= 8 && P <= 9 && M <= (1LL << 31) - 1)
+  if (N <= g_fused_max_n && emu_fused_takes(A.S, B.S, P) && M <= (1LL << 31) - 256 && N <= (1LL << 31) - 256)
     return emu_gemm_fused(st, A.dig, A.rows * A.ld, A.S, A.exp2, B.dig, B.rows * B.ld, B.S, B.exp2, A.ld, (int)M,
-                          (int)N, (int)K, P, alpha, beta, C, cm, cn, n0, static_cast<double *>(work));
+                          (int)N, (int)K, P, 6, alpha, beta, C, cm, cn, n0, static_cast<double *>(work));
   const long long nk = (K + 63) / 64;
   const int nz = (int)((nk + KCHUNK_BLOCKS - 1) / KCHUNK_BLOCKS);
   const long long kbs = (nk + nz - 1) / nz;

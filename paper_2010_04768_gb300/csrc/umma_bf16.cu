@@ -20,9 +20,12 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <utility>
 
 #include "common.cuh"
 #include "umma.cuh"
@@ -716,59 +719,176 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 
 // ---------------------------------------------------------------------------------------------
 // FP64-accurate product from digit planes with every digit pair of a tile in one CTA:
-//   C = alpha 2^(eA[m] + eB[n]) sum_L 2^(-6L) sum_{i+j=L, L<=P} A_i B_j^T + beta C.
-// The accumulator of each level L = i + j lives in its own 64-column block of TMEM (8 levels fill
-// the 512 columns).  A stage holds the tile of one A plane i and the tiles of the B planes
-// j = 1 .. min(SB, P - i), so every level of pair (i, j) is fed from the same stage.  A level
-// accumulates at most 8 pairs x 32 K blocks x 64 = 2^14 products of magnitude <= 2^10, so its FP32
-// sums are exact integers; the epilogue adds the levels exactly in two int64 accumulators, forms
-// the FP64 value and writes the FP64 result (or, with a K split, an FP64 partial per split).
-constexpr int EMU_BN = 64, EMU_STAGES = 2, EMU_MAXS = 8;
-constexpr int EMU_A_BYTES = BM * BK * 2, EMU_B_BYTES = EMU_BN * BK * 2;
-constexpr int EMU_STAGE_BYTES = EMU_A_BYTES + EMU_MAXS * EMU_B_BYTES;
-constexpr int EMU_SMEM_BYTES = EMU_STAGES * EMU_STAGE_BYTES + 1024 + 256;
-
-struct EmuMaps {
-  CUtensorMap a[EMU_MAXS];
-  CUtensorMap b[EMU_MAXS];
+//   C = alpha 2^(eA[m] + eB[n]) sum_L 2^(-bL) sum_{i+j=L, L<=P} A_i B_j^T + beta C   (b-bit digits).
+// The accumulator of each level L = i + j lives in its own BN columns of TMEM (8 levels of 64 columns
+// fill it).  The tensor cores read both operands from shared memory, so the work is arranged to
+// read and load each byte as seldom as possible: the B planes of a K block lie one after the other, so one
+// MMA multiplies an A plane with up to 256 / BN of them at once (N = 256) and adds the products to as
+// many consecutive levels; per K block every plane is loaded once (A planes through a ring of slots, B
+// planes double-buffered).  Persistent: one CTA per SM walks the tiles; a producer warp, an MMA warp and
+// epilogue warps of 16 columns each.  A level is an exact integer while it holds at most 2^24 / 2^(2b-2) products:
+// after kc K blocks the epilogue warps add the levels to two int64 accumulators per output (levels
+// 2..5 and 6..9) and the MMA warp starts them anew.  The last step, integer to FP64 with one rounding, is
+// integer arithmetic too (FP64 operations are issued at two per SM and clock).
+// Bound by the tensor cores: 8000 x 3200 x 8000 at level 9 (36 pairs) 7.8 ms, 1.88 PFLOP/s of BF16 products.
+// Before (one GEMM per pair with FP32 partial sums in global memory for wide products, one N = 64 MMA per
+// pair for narrow ones): the residual's ring product of 40 systems at o=40 v=200 9.1 -> 5.4 ms, its other
+// four products 7.3 -> 2.1 ms.
+constexpr int EMU_MAXS = 8, EMU_A_SLOTS = 6, EMU_COLS = 16;   // EMU_COLS: columns of an epilogue thread
+constexpr int EMU_A_BYTES = BM * BK * 2;
+template <int BN>
+struct EmuTile {
+  static constexpr int B_PLANE = BN * BK * 2, B_BYTES = EMU_MAXS * B_PLANE, GROUP = 256 / BN, COLS = EMU_MAXS * BN;
+  static constexpr int EPI_WARPS = 4 * BN / EMU_COLS, THREADS = 64 + 32 * EPI_WARPS;
+  static constexpr int SMEM_BYTES = EMU_A_SLOTS * EMU_A_BYTES + 2 * B_BYTES + 1024 + 512;
 };
 
-__global__ void __launch_bounds__(THREADS, 1)
-    umma_emu_kernel(const __grid_constant__ EmuMaps maps, int SA, int SB, int P, int M, int N, int K,
-                    int kb_per_split, const int *eA, const int *eB, double alpha, double beta, double *C, IMap cm,
-                    IMap cn, long long n0g, double *part, UmmaCtl ctl) {
+struct EmuArgs {
+  int SA, SB, P, bits;          // planes of A and B, highest level, bits of a digit
+  int M, N, nM, nN, nz;         // output, tiles, K splits
+  int nk, kb_per_split, kc;     // K blocks: all, of a split, between two drains
+  const int *eA, *eB;
+  int alpha_exp;                // alpha = alpha_mul 2^alpha_exp
+  double alpha_mul, beta;
+  double *C, *part;
+  IMap rm, cm;                  // row / column maps of C
+  long long r0g, c0g;           // first row / column index
+  UmmaCtl ctl;
+};
+
+__device__ __forceinline__ void tma_load_3d(unsigned dst, const CUtensorMap *map, unsigned mbar, int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(
+          dst),
+      "l"(reinterpret_cast<unsigned long long>(map)), "r"(mbar), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld_8_nowait(unsigned taddr, unsigned (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// (hi 2^sh + lo) 2^e2 rounded once to FP64 (round to nearest, ties to even) with integer operations
+__device__ __forceinline__ double fixed_to_f64(long long hi, long long lo, int sh, int e2) {
+  const __int128 t = ((__int128)hi << sh) + lo;
+  if (t == 0) return 0.0;
+  const bool neg = t < 0;
+  unsigned __int128 u = neg ? -(unsigned __int128)t : (unsigned __int128)t;
+  const unsigned long long uh = (unsigned long long)(u >> 64);
+  const int lz = uh ? __clzll((long long)uh) : 64 + __clzll((long long)(unsigned long long)u);
+  u <<= lz;
+  const unsigned long long top = (unsigned long long)(u >> 64);
+  unsigned long long mant = top >> 11;
+  const unsigned long long rem = top & 0x7ffULL;
+  const bool sticky = (unsigned long long)u != 0;
+  if (rem > 0x400ULL || (rem == 0x400ULL && (sticky || (mant & 1)))) mant++;
+  const int be = 127 - lz + e2 + 1023;   // biased exponent of the leading bit
+  double v;
+  if (be >= 1 && be <= 2045)
+    v = __longlong_as_double((long long)(((unsigned long long)be << 52) + (mant - (1ULL << 52))));
+  else
+    v = scalbn((double)mant, 127 - lz + e2 - 52);
+  return neg ? -v : v;
+}
+
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// The MMAs of one K block at level P, called by a whole warp so that the descriptors stay in uniform
+// registers (built lane by lane, an MMA took about 130 clocks to issue, four times what N = 64 takes to
+// execute); everything but the slot is a compile-time constant.  ita counts the A planes consumed.
+template <int BN, int P>
+__device__ __forceinline__ bool emu_issue_kblock(unsigned tmem, unsigned sa0, unsigned sb, unsigned long long *afull,
+                                                 unsigned long long *aempty, int &ita, bool start,
+                                                 volatile int *consumed_a, volatile int *abort_flag,
+                                                 unsigned long long wait_ns) {
+  using T = EmuTile<BN>;
+  const unsigned long long db = smem_desc(sb);
+#pragma unroll
+  for (int i = 1; i < P; i++, ita++) {
+    const int s = ita % EMU_A_SLOTS;
+    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&afull[s]), (ita / EMU_A_SLOTS) & 1, abort_flag, wait_ns)))
+      return false;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const unsigned long long da = smem_desc(sa0 + s * EMU_A_BYTES);
+    if (elect_one()) {
+      *consumed_a = ita + 1;
+#pragma unroll
+      for (int k = 0; k < BK / 16; k++)
+#pragma unroll
+        for (int j = 1; j <= P - i; j += T::GROUP) {
+          // plane 1 meets every level first (there are P - 1 B planes), so it starts the accumulators
+          const int g = T::GROUP < P - i - j + 1 ? T::GROUP : P - i - j + 1;
+          const unsigned acc = (i > 1 || k > 0) ? 1u : (start ? 0u : 1u);
+          umma_bf16(tmem + (unsigned)((i + j - 2) * BN), da + 2 * k, db + (j - 1) * (T::B_PLANE >> 4) + 2 * k,
+                    idesc_bf16(BM, g * BN), acc);
+        }
+      umma_commit(smem_u32(&aempty[s]));
+    }
+    __syncwarp();
+  }
+  return true;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
+    umma_emu_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                    const __grid_constant__ EmuArgs a) {
+  using T = EmuTile<BN>;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem + EMU_STAGES * EMU_STAGE_BYTES);
-  unsigned long long *full = bars, *empty = bars + EMU_STAGES, *done = bars + 2 * EMU_STAGES;
-  unsigned *tmem_slot = reinterpret_cast<unsigned *>(bars + 2 * EMU_STAGES + 1);
+  unsigned char *smA = smem, *smB = smem + EMU_A_SLOTS * EMU_A_BYTES;
+  unsigned long long *bars = reinterpret_cast<unsigned long long *>(smB + 2 * T::B_BYTES);
+  unsigned long long *afull = bars, *aempty = afull + EMU_A_SLOTS, *bfull = aempty + EMU_A_SLOTS, *bempty = bfull + 2;
+  unsigned long long *accf = bempty + 2, *acce = accf + 1, *drain = acce + 1;
+  unsigned *tmem_slot = reinterpret_cast<unsigned *>(drain + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-  volatile int *issued = reinterpret_cast<volatile int *>(tmem_slot + 2);
-  volatile int *consumed = reinterpret_cast<volatile int *>(tmem_slot + 3);
+  volatile int *issued_a = reinterpret_cast<volatile int *>(tmem_slot + 2), *issued_b = issued_a + 1;
+  volatile int *consumed_a = issued_a + 2, *consumed_b = issued_a + 3;
+  volatile int *go = issued_a + 4;   // the epilogue group's decision per chunk (two in turn)
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * EMU_BN;
-  const int nk_all = (K + BK - 1) / BK;
-  const int kb0 = blockIdx.z * kb_per_split;
-  const int kb1 = min(nk_all, kb0 + kb_per_split);
-  const int nk = kb1 - kb0;
-  const int SAe = min(SA, P - 1);            // A planes with at least one partner
-  const int iters = nk * SAe;                // stages: (K block, A plane)
+  const int tiles = a.nM * a.nN * a.nz;
+  const int SAe = min(a.SA, a.P - 1);   // A planes with at least one partner
+  const int SBe = min(a.SB, a.P - 1);
+  const unsigned long long wait_ns = a.ctl.wait_ns;
+  // tile t: split z, then groups of RASTER_GM row tiles sweep the column tiles
+  auto tile_of = [&](int t, int &m0, int &n0, int &z, int &kb0, int &nk) {
+    z = t / (a.nM * a.nN);
+    const int id = t - z * (a.nM * a.nN);
+    const int first_m = (id / (RASTER_GM * a.nN)) * RASTER_GM;
+    const int gm = min(a.nM - first_m, RASTER_GM);
+    const int r = id - first_m * a.nN;
+    m0 = (first_m + r % gm) * BM;
+    n0 = (r / gm) * BN;
+    kb0 = z * a.kb_per_split;
+    nk = min(a.nk, kb0 + a.kb_per_split) - kb0;
+  };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < EMU_STAGES; s++) {
-      mbar_init(smem_u32(&full[s]), 1);
-      mbar_init(smem_u32(&empty[s]), 1);
+    for (int s = 0; s < EMU_A_SLOTS; s++) {
+      mbar_init(smem_u32(&afull[s]), 1);
+      mbar_init(smem_u32(&aempty[s]), 1);
     }
-    mbar_init(smem_u32(done), 1);
+    for (int s = 0; s < 2; s++) {
+      mbar_init(smem_u32(&bfull[s]), 1);
+      mbar_init(smem_u32(&bempty[s]), 1);
+    }
+    mbar_init(smem_u32(accf), 1);
+    mbar_init(smem_u32(acce), T::EPI_WARPS);
+    mbar_init(smem_u32(drain), 1);
     *abort_flag = 0;
-    *issued = 0;
-    *consumed = 0;
+    *issued_a = *issued_b = *consumed_a = *consumed_b = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {   // TMEM: 8 level accumulators of 64 FP32 columns x 128 lanes
+  if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(512));
+                 "r"(T::COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -776,145 +896,212 @@ __global__ void __launch_bounds__(THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const unsigned tmem = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
-    // ---------------- TMA producer: stage t = (K block t / SAe, A plane t % SAe + 1)
-    for (int t = 0; t < iters && !ctl.skip_loads; t++) {
-      const int s = t % EMU_STAGES;
-      const unsigned ph = (t / EMU_STAGES) & 1;
-      if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns)) break;
-      const int kb = kb0 + t / SAe, i = t % SAe + 1;
-      const int nb = min(SB, P - i);
-      unsigned char *sa = smem + s * EMU_STAGE_BYTES;
-      mbar_expect_tx(smem_u32(&full[s]), EMU_A_BYTES + nb * EMU_B_BYTES);
-      tma_load_2d(smem_u32(sa), &maps.a[i - 1], smem_u32(&full[s]), kb * BK, m0);
-      for (int j = 1; j <= nb; j++)
-        tma_load_2d(smem_u32(sa + EMU_A_BYTES + (j - 1) * EMU_B_BYTES), &maps.b[j - 1], smem_u32(&full[s]), kb * BK,
-                    n0);
-      *issued = t + 1;
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer
-    const unsigned idesc = idesc_bf16(BM, EMU_BN);
-    unsigned started = 0;   // bit L: level L has received its first product
-    bool ok = true;
-    for (int t = 0; t < iters && ok; t++) {
-      const int s = t % EMU_STAGES;
-      const unsigned ph = (t / EMU_STAGES) & 1;
-      if (!mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns)) {
-        ok = false;
-        break;
-      }
-      *consumed = t + 1;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int i = t % SAe + 1;
-      const int nb = min(SB, P - i);
-      const unsigned sa = smem_u32(smem + s * EMU_STAGE_BYTES);
-      for (int j = 1; j <= nb; j++) {
-        const int L = i + j;
-        const unsigned acc_col = tmem + (unsigned)((L - 2) * EMU_BN);
-        const unsigned sb = sa + EMU_A_BYTES + (j - 1) * EMU_B_BYTES;
-#pragma unroll
-        for (int k = 0; k < BK / 16; k++) {
-          const unsigned acc = ((started >> L) & 1u) || k > 0 ? 1u : 0u;
-          umma_bf16(acc_col, smem_desc(sa + 32 * k), smem_desc(sb + 32 * k), idesc, acc);
-        }
-        started |= 1u << L;
-      }
-      umma_commit(smem_u32(&empty[s]));
-    }
-    umma_commit(smem_u32(done));
-  }
-  __syncwarp();
-
-  // ---------------- epilogue: all 4 warps, one row per thread
-  const bool ready = mbar_wait(smem_u32(done), 0, abort_flag, ctl.wait_ns);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (__all_sync(0xffffffffu, ready && !*abort_flag) && nk > 0) {
-    const int row = m0 + warp * 32 + lane;
-    const int ea = row < M ? eA[row] : 0;
-    // The level sums are exact integers below 2^24: they are added in two int64 accumulators,
-    // levels Lhi+1..P with weights 64^(P-L) and 2..Lhi with 64^(Lhi-L) (below 2^45 each), on the
-    // integer pipes; FP64 work is two conversions and one scaled add per output.
-    const int Lhi = min(P, 5);
-#pragma unroll 1
-    for (int c0 = 0; c0 < EMU_BN; c0 += 32) {
-      double acc[32];
-      long long ia[32];
-#pragma unroll
-      for (int q = 0; q < 32; q++) ia[q] = 0;
-#pragma unroll 1
-      for (int L = P; L > Lhi; L--) {
-        const int ilo = max(1, L - SB), ihi = min(SAe, L - 1);   // a level holds products if some i + j = L
-        if (ilo > ihi) continue;
-        float v[32];
-        tmem_ld_32(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)((L - 2) * EMU_BN + c0), v);
-        const int sh = 6 * (P - L);
-#pragma unroll
-        for (int q = 0; q < 32; q++) ia[q] += (long long)__float2int_rn(v[q]) << sh;
-      }
-      const double wlo = ldexp(1.0, -6 * P), whi = ldexp(1.0, -6 * Lhi);
-#pragma unroll
-      for (int q = 0; q < 32; q++) {
-        acc[q] = (double)ia[q] * wlo;
-        ia[q] = 0;
-      }
-#pragma unroll 1
-      for (int L = Lhi; L >= 2; L--) {
-        const int ilo = max(1, L - SB), ihi = min(SAe, L - 1);
-        if (ilo > ihi) continue;
-        float v[32];
-        tmem_ld_32(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)((L - 2) * EMU_BN + c0), v);
-        const int sh = 6 * (Lhi - L);
-#pragma unroll
-        for (int q = 0; q < 32; q++) ia[q] += (long long)__float2int_rn(v[q]) << sh;
-      }
-#pragma unroll
-      for (int q = 0; q < 32; q++) acc[q] = fma((double)ia[q], whi, acc[q]);
-      if (row < M) {
-        const int ncols = min(32, N - (n0 + c0));
-        if (part != nullptr) {
-          double *dst = part + ((long long)blockIdx.z * M + row) * N + n0 + c0;
-#pragma unroll
-          for (int q = 0; q < 32; q++)
-            if (q < ncols) dst[q] = acc[q];
-        } else {
-          const long long ro = imap_apply(cm, row);
-#pragma unroll
-          for (int q = 0; q < 32; q++) {
-            if (q >= ncols) continue;
-            const int col = n0 + c0 + q;
-            const long long off = ro + imap_apply(cn, n0g + col);
-            const double val = alpha * ldexp(acc[q], ea + eB[col]);
-            C[off] = beta != 0.0 ? val + beta * C[off] : val;
+  if (warp == 0) {
+    if (lane == 0 && !a.ctl.skip_loads) {
+      // ---------------- TMA producer: per K block all B planes at once, then the A planes one by one
+      int ita = 0, itb = 0;
+      bool ok = true;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        int m0, n0, z, kb0, nk;
+        tile_of(t, m0, n0, z, kb0, nk);
+        for (int kb = kb0; kb < kb0 + nk && ok; kb++) {
+          const int sb = itb & 1;
+          if (!mbar_wait(smem_u32(&bempty[sb]), ((itb >> 1) & 1) ^ 1, abort_flag, wait_ns)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(smem_u32(&bfull[sb]), SBe * T::B_PLANE);
+          tma_load_3d(smem_u32(smB + sb * T::B_BYTES), &tmB, smem_u32(&bfull[sb]), kb * BK, n0, 0);
+          *issued_b = ++itb;
+          for (int i = 0; i < SAe; i++) {
+            const int s = ita % EMU_A_SLOTS;
+            if (!mbar_wait(smem_u32(&aempty[s]), ((ita / EMU_A_SLOTS) & 1) ^ 1, abort_flag, wait_ns)) {
+              ok = false;
+              break;
+            }
+            mbar_expect_tx(smem_u32(&afull[s]), EMU_A_BYTES);
+            tma_load_3d(smem_u32(smA + s * EMU_A_BYTES), &tmA, smem_u32(&afull[s]), kb * BK, m0, i);
+            *issued_a = ++ita;
           }
         }
       }
     }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer (the whole warp; one elected lane issues)
+    int ita = 0, itb = 0, ch = 0;
+    bool ok = true;
+    const unsigned sa0 = smem_u32(smA);
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      int m0, n0, z, kb0, nk;
+      tile_of(t, m0, n0, z, kb0, nk);
+      for (int c0 = 0; c0 < nk && ok; c0 += a.kc, ch++) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(acce), (ch & 1) ^ 1, abort_flag, wait_ns))) {
+          ok = false;
+          break;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int c1 = min(nk, c0 + a.kc);
+        for (int kb = c0; kb < c1 && ok; kb++, itb++) {
+          const int sbuf = itb & 1;
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bfull[sbuf]), (itb >> 1) & 1, abort_flag, wait_ns))) {
+            ok = false;
+            break;
+          }
+          if (lane == 0) *consumed_b = itb + 1;
+          const unsigned sb = smem_u32(smB + sbuf * T::B_BYTES);
+          const bool start = kb == c0;
+          switch (a.P) {
+#define GFCC_EMU_LEVEL(P)                                                                                       \
+  case P:                                                                                                       \
+    ok = emu_issue_kblock<BN, P>(tmem, sa0, sb, afull, aempty, ita, start, consumed_a, abort_flag, wait_ns); \
+    break;
+            GFCC_EMU_LEVEL(2)
+            GFCC_EMU_LEVEL(3)
+            GFCC_EMU_LEVEL(4)
+            GFCC_EMU_LEVEL(5)
+            GFCC_EMU_LEVEL(6)
+            GFCC_EMU_LEVEL(7)
+            GFCC_EMU_LEVEL(8)
+            GFCC_EMU_LEVEL(9)
+#undef GFCC_EMU_LEVEL
+            default: ok = false; break;
+          }
+          if (ok && elect_one()) umma_commit(smem_u32(&bempty[sbuf]));
+          __syncwarp();
+        }
+        if (ok && elect_one()) umma_commit(smem_u32(accf));
+        __syncwarp();
+      }
+    }
+    if (elect_one()) umma_commit(smem_u32(drain));   // arrives once every MMA issued above has completed
+    __syncwarp();
+  } else {
+    // ---------------- epilogue: warp w reads TMEM lanes 32 (w mod 4) .. + 31, NC of the columns
+    constexpr int NC = EMU_COLS;
+    const int q = warp & 3, part = (warp - 2) >> 2;
+    const int Lhi = min(a.P, 5), b = a.bits;
+    const unsigned trow = tmem + ((unsigned)(q * 32) << 16) + (unsigned)(part * NC);
+    long long hi[NC], lo[NC];
+    int ch = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      int m0, n0, z, kb0, nk;
+      tile_of(t, m0, n0, z, kb0, nk);
+#pragma unroll
+      for (int c = 0; c < NC; c++) hi[c] = lo[c] = 0;
+      for (int c0 = 0; c0 < nk; c0 += a.kc, ch++) {
+        // one lane polls and decides for the group; the other warps block on a named barrier (polling by
+        // all of them takes shared-memory cycles from the loads)
+        if (warp == 2 && lane == 0) {
+          const bool ready = mbar_wait(smem_u32(accf), ch & 1, abort_flag, wait_ns);
+          go[ch & 1] = ready && !*abort_flag ? 1 : 0;
+        }
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * T::EPI_WARPS) : "memory");
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (!go[ch & 1]) {
+          ok = false;
+          break;
+        }
+#pragma unroll
+        for (int g = 0; g < NC; g += 8) {
+          // two levels at a time: hi takes levels 2..Lhi, lo the ones above
+#pragma unroll
+          for (int l = 0; l < EMU_MAXS; l += 2) {
+            unsigned r[2][8];
+            if (2 + l > a.P) break;
+            tmem_ld_8_nowait(trow + (unsigned)(l * BN + g), r[0]);
+            if (3 + l <= a.P) tmem_ld_8_nowait(trow + (unsigned)((l + 1) * BN + g), r[1]);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int d = 0; d < 2; d++) {
+              if (2 + l + d > a.P) break;
+              const int sh = b * ((l < 4 ? Lhi : a.P) - 2 - l - d);
+#pragma unroll
+              for (int c = 0; c < 8; c++) {
+                const long long x = (long long)__float2int_rn(__uint_as_float(r[d][c])) << sh;
+                if (l < 4)
+                  hi[g + c] += x;
+                else
+                  lo[g + c] += x;
+              }
+            }
+          }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(acce)) : "memory");
+      }
+      const int row = m0 + q * 32 + lane;
+      const int c0 = n0 + part * NC;
+      const int sh = b * (a.P - Lhi), e0 = -b * a.P;
+      if (!ok || row >= a.M) {
+        // nothing to store
+      } else if (a.part != nullptr) {
+        double *dst = a.part + ((long long)z * a.M + row) * a.N + c0;
+#pragma unroll
+        for (int c = 0; c < NC; c++)
+          if (c0 + c < a.N) dst[c] = fixed_to_f64(hi[c], lo[c], sh, e0);
+      } else {
+        const int ea = a.eA[row] + a.alpha_exp + e0;
+        double *base = a.C + imap_apply(a.rm, a.r0g + row);
+        // the column offset walks without a division per column
+        const long long x0 = a.c0g + c0;
+        const bool two = a.cm.d0 > 0;
+        long long rr = two ? x0 % a.cm.d0 : 0;
+        long long off = imap_apply(a.cm, x0);
+        const long long wrap = two ? a.cm.s1 - a.cm.d0 * a.cm.s0 : 0;
+#pragma unroll
+        for (int c = 0; c < NC; c++) {
+          if (c0 + c < a.N) {
+            double v = fixed_to_f64(hi[c], lo[c], sh, ea + a.eB[c0 + c]);
+            if (a.alpha_mul != 1.0) v *= a.alpha_mul;
+            if (a.beta != 0.0) v += a.beta * base[off];
+            base[off] = v;
+          }
+          off += a.cm.s0;
+          if (two && ++rr == a.cm.d0) {
+            rr = 0;
+            off += wrap;
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+  __syncwarp();
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // every MMA has completed (the drain barrier); after a time-out also the copies that were issued but
+    // not consumed land before the shared memory goes away (fixed DRAIN_NS limits)
+    volatile int never = 0;
+    mbar_wait(smem_u32(drain), 0, &never, DRAIN_NS);
+    if (*abort_flag) {
+      for (int it = *consumed_a; it < *issued_a; it++)
+        mbar_wait(smem_u32(&afull[it % EMU_A_SLOTS]), (it / EMU_A_SLOTS) & 1, &never, DRAIN_NS);
+      for (int it = *consumed_b; it < *issued_b; it++)
+        mbar_wait(smem_u32(&bfull[it & 1]), (it >> 1) & 1, &never, DRAIN_NS);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (threadIdx.x == 0 && *abort_flag) {
-    // as in umma_bf16_gemm_kernel: the committed products, then the issued copies (fixed limit)
-    volatile int never = 0;
-    mbar_wait(smem_u32(done), 0, &never, DRAIN_NS);
-    for (int t = *consumed; t < *issued; t++)
-      mbar_wait(smem_u32(&full[t % EMU_STAGES]), (t / EMU_STAGES) & 1, &never, DRAIN_NS);
-  }
-  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(T::COLS));
   }
 }
 
 // C = alpha 2^(eA + eB) sum_z part[z] + beta C (the K splits of umma_emu_kernel)
 __global__ void emu_split_reduce_kernel(const double *part, int nz, int M, int N, const int *eA, const int *eB,
-                                        double alpha, double beta, double *C, IMap cm, IMap cn, long long n0g) {
+                                        double alpha, double beta, double *C, IMap cm, IMap cn, long long m0g,
+                                        long long n0g) {
   const long long tot = (long long)M * N;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
     const int m = (int)(t / N), n = (int)(t - (long long)m * N);
     double s = 0.0;
     for (int z = 0; z < nz; z++) s += part[(long long)z * tot + t];
-    const long long off = imap_apply(cm, m) + imap_apply(cn, n0g + n);
+    const long long off = imap_apply(cm, m0g + m) + imap_apply(cn, n0g + n);
     const double val = alpha * ldexp(s, eA[m] + eB[n]);
     C[off] = beta != 0.0 ? val + beta * C[off] : val;
   }
@@ -1187,53 +1374,151 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
   return run(bn);
 }
 
-int emu_fused_splits(long long K) {
-  const int nk = (int)((K + BK - 1) / BK);
-  return (nk + 31) / 32;
+namespace {
+constexpr int EMU_SMS = 152;
+constexpr int EMU_MAX_SPLIT_TILES = 4 * EMU_SMS;   // tiles x K splits of a split product: bounds its partial sums
+
+// Tiling of a fused digit product: tile width, whether A and B change places, K splits.  The model (in
+// clocks of an SM) weighs the MMAs of 36 digit pairs, the loads of 16 planes at about 55 bytes a clock,
+// the drains and the last step of a tile, over the busiest SM.  It does not depend on the digits kept, so that
+// a workspace sized for a shape serves every level.
+struct EmuPlan {
+  int bn = 64, nz = 1;
+  bool swap = false;
+};
+EmuPlan emu_plan(long long M, long long N, long long K) {
+  const long long nk = (K + BK - 1) / BK;
+  EmuPlan best;
+  double cost = 0.0;
+  for (int sw = 0; sw < 2; sw++)
+    for (int bn : {64, 32}) {
+      const long long rows = sw ? N : M, cols = sw ? M : N;
+      const double tiles = (double)((rows + BM - 1) / BM) * (double)((cols + bn - 1) / bn);
+      const double kb = std::max(72.0 * bn, (8.0 * EMU_A_BYTES + 8.0 * bn * BK * 2) / 55.0);
+      for (long long nz = 1; nz == 1 || (nz <= nk / 4 && tiles * nz <= EMU_MAX_SPLIT_TILES); nz = nz < 8 ? nz + 1 : nz * 5 / 4) {
+        const double per = std::ceil((double)nk / nz);
+        const double t = std::ceil(tiles * nz / EMU_SMS) * (per * kb + std::ceil(per / 8) * 64.0 * bn + 45.0 * bn + 2500.0) +
+                         (nz > 1 ? 4000.0 + 8.0 * 2.0 * nz * M * N / 2500.0 : 0.0);
+        if (cost == 0.0 || t < 0.98 * cost) {
+          cost = t;
+          best.bn = bn;
+          best.nz = (int)nz;
+          best.swap = sw != 0;
+        }
+      }
+    }
+  // every split gets at least one K block
+  const long long per = (nk + best.nz - 1) / best.nz;
+  best.nz = (int)((nk + per - 1) / per);
+  return best;
 }
 
-long long emu_fused_work_bytes(long long M, long long N, long long K) {
-  const int nz = emu_fused_splits(K);
-  return nz > 1 ? (long long)nz * M * N * 8 + 256 : 0;
-}
-
-int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, int SA, const int *eA,
-                   const __nv_bfloat16 *Bdig, long long plB, int SB, const int *eB, long long ld, int M, int N, int K,
-                   int P, double alpha, double beta, double *C, IMap cm, IMap cn, long long n0, double *work) {
-  if (M <= 0 || N <= 0) return GFCC_OK;
-  if (SA < 1 || SB < 1 || SA > EMU_MAXS || SB > EMU_MAXS || P < 2 || P > 9 || K <= 0 || (ld % 8) ||
-      (reinterpret_cast<uintptr_t>(Adig) & 15) || (reinterpret_cast<uintptr_t>(Bdig) & 15) || (plA % 8) ||
-      (plB % 8)) {
-    set_error("emu_gemm_fused: unsupported digits (SA=%d SB=%d P=%d) or alignment", SA, SB, P);
+// 3-D K-major BF16 tensor map over digit planes: planes x rows x K, box `planes` x box_rows x 64
+int make_plane_map(CUtensorMap *map, const void *base, long long planes, long long rows, long long K, long long ld,
+                   long long plane, int box_rows, int box_planes) {
+  auto fn = encode_fn();
+  if (fn == nullptr) {
+    set_error("cuTensorMapEncodeTiled is not available from the driver");
+    return GFCC_ERR_CUDA;
+  }
+  const cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)planes};
+  const cuuint64_t strides[2] = {(cuuint64_t)ld * 2, (cuuint64_t)plane * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)BK, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    set_error("cuTensorMapEncodeTiled failed (%d) for planes=%lld rows=%lld K=%lld ld=%lld", (int)r, planes, rows, K, ld);
     return GFCC_ERR_ARG;
   }
-  EmuMaps maps;
-  for (int i = 0; i < SA; i++) GFCC_TRY(make_map(&maps.a[i], Adig + (long long)i * plA, M, K, ld, BM));
-  for (int j = 0; j < SB; j++) GFCC_TRY(make_map(&maps.b[j], Bdig + (long long)j * plB, N, K, ld, EMU_BN));
-  for (int i = SA; i < EMU_MAXS; i++) maps.a[i] = maps.a[0];
-  for (int j = SB; j < EMU_MAXS; j++) maps.b[j] = maps.b[0];
+  return GFCC_OK;
+}
+
+template <int BN>
+int launch_emu(cudaStream_t st, const CUtensorMap &ma, const CUtensorMap &mb, const EmuArgs &a) {
   static bool attr[64] = {false};
   int dev = 0;
   GFCC_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !attr[dev]) {
-    GFCC_CUDA(cudaFuncSetAttribute(umma_emu_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, EMU_SMEM_BYTES));
+    GFCC_CUDA(cudaFuncSetAttribute(umma_emu_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   EmuTile<BN>::SMEM_BYTES));
     if (dev >= 0 && dev < 64) attr[dev] = true;
   }
-  const int nz = emu_fused_splits(K);
-  double *part = nz > 1 ? work : nullptr;
-  if (nz > 1) GFCC_TRY(check_extent_bytes(work, emu_fused_work_bytes(M, N, K), "fused digit GEMM partials"));
-  GFCC_TRY(check_extent(C, 0, imap_max(cm, M) + imap_max(cn, n0 + N), "fused digit GEMM output"));
-  dim3 grid((M + BM - 1) / BM, (N + EMU_BN - 1) / EMU_BN, nz);
-  if (grid.y > 65535 || grid.z > 65535) {
-    set_error("emu_gemm_fused: grid too large");
+  const long long tiles = (long long)a.nM * a.nN * a.nz;
+  umma_emu_kernel<BN><<<(unsigned)std::min<long long>(tiles, EMU_SMS), EmuTile<BN>::THREADS, EmuTile<BN>::SMEM_BYTES, st>>>(
+      ma, mb, a);
+  GFCC_LAUNCH_CHECK();
+  return GFCC_OK;
+}
+}  // namespace
+
+// (grows with N: a workspace sized for a shape serves fewer columns too)
+long long emu_fused_work_bytes(long long M, long long N, long long K) {
+  const long long nk = (K + BK - 1) / BK;
+  return std::min<long long>(std::max<long long>(1, nk / 4) * M * N * 8, 8LL * EMU_MAX_SPLIT_TILES * BM * 64) + 256;
+}
+
+bool emu_fused_takes(int SA, int SB, int P) {
+  return SA >= 1 && SB >= 1 && SA <= EMU_MAXS && SB <= EMU_MAXS && P >= 2 && P <= 9 && P - 1 <= SA && P - 1 <= SB;
+}
+
+int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, int SA, const int *eA,
+                   const __nv_bfloat16 *Bdig, long long plB, int SB, const int *eB, long long ld, int M, int N, int K,
+                   int P, int bits, double alpha, double beta, double *C, IMap cm, IMap cn, long long n0,
+                   double *work, long long m0) {
+  if (M <= 0 || N <= 0) return GFCC_OK;
+  if (!emu_fused_takes(SA, SB, P) || bits < 1 || bits > 7 || K <= 0 || (ld % 8) ||
+      (reinterpret_cast<uintptr_t>(Adig) & 15) || (reinterpret_cast<uintptr_t>(Bdig) & 15) || (plA % 8) ||
+      (plB % 8)) {
+    set_error("emu_gemm_fused: unsupported digits (SA=%d SB=%d P=%d bits=%d) or alignment", SA, SB, P, bits);
     return GFCC_ERR_ARG;
   }
-  umma_emu_kernel<<<grid, THREADS, EMU_SMEM_BYTES, st>>>(maps, SA, SB, P, M, N, K, 32, eA, eB, alpha, beta, C, cm, cn,
-                                                          n0, part, umma_ctl());
-  GFCC_LAUNCH_CHECK();
-  if (nz > 1) {
-    emu_split_reduce_kernel<<<grid1d((long long)M * N), 256, 0, st>>>(part, nz, M, N, eA, eB, alpha, beta, C, cm, cn,
-                                                                       n0);
+  const EmuPlan pl = emu_plan(M, N, K);
+  EmuArgs a;
+  a.SA = SA; a.SB = SB; a.P = P; a.bits = bits;
+  a.M = M; a.N = N;
+  a.eA = eA; a.eB = eB;
+  a.C = C;
+  a.rm = cm; a.cm = cn;
+  a.r0g = m0; a.c0g = n0;
+  if (pl.swap) {
+    std::swap(Adig, Bdig);
+    std::swap(plA, plB);
+    std::swap(a.SA, a.SB);
+    std::swap(a.M, a.N);
+    std::swap(a.eA, a.eB);
+    std::swap(a.rm, a.cm);
+    std::swap(a.r0g, a.c0g);
+  }
+  a.nM = (a.M + BM - 1) / BM;
+  a.nN = (a.N + pl.bn - 1) / pl.bn;
+  a.nz = pl.nz;
+  a.nk = (K + BK - 1) / BK;
+  a.kb_per_split = (a.nk + a.nz - 1) / a.nz;
+  // a level holds up to P - 1 pairs: (P - 1) kc 64 products of at most 2^(2 bits - 2) stay within 2^24
+  a.kc = (1 << (26 - 2 * bits)) / (BK * (P - 1));
+  a.beta = beta;
+  int ex = 0;
+  const double fr = frexp(alpha, &ex);
+  const bool pow2 = fr == 0.5;
+  a.alpha_exp = pow2 ? ex - 1 : 0;
+  a.alpha_mul = pow2 ? 1.0 : alpha;
+  a.ctl = umma_ctl();
+  a.part = a.nz > 1 ? work : nullptr;
+  if ((long long)a.nM * a.nN * a.nz > 0x7fffffffLL || a.kc < 1) {
+    set_error("emu_gemm_fused: too many tiles (M=%d, N=%d)", M, N);
+    return GFCC_ERR_ARG;
+  }
+  if (a.nz > 1) GFCC_TRY(check_extent_bytes(work, emu_fused_work_bytes(M, N, K), "fused digit GEMM partials"));
+  GFCC_TRY(check_extent(C, 0, imap_max(cm, m0 + M) + imap_max(cn, n0 + N), "fused digit GEMM output"));
+  CUtensorMap ma, mb;
+  GFCC_TRY(make_plane_map(&ma, Adig, a.SA, a.M, K, ld, plA, BM, 1));
+  GFCC_TRY(make_plane_map(&mb, Bdig, a.SB, a.N, K, ld, plB, pl.bn, std::min(a.SB, P - 1)));
+  GFCC_TRY(pl.bn == 64 ? launch_emu<64>(st, ma, mb, a) : launch_emu<32>(st, ma, mb, a));
+  if (a.nz > 1) {
+    emu_split_reduce_kernel<<<grid1d((long long)M * N), 256, 0, st>>>(work, a.nz, a.M, a.N, a.eA, a.eB, alpha, beta, C,
+                                                                       a.rm, a.cm, a.r0g, a.c0g);
     GFCC_LAUNCH_CHECK();
   }
   return GFCC_OK;
