@@ -100,7 +100,9 @@ extern "C" {
  * accepted there). */
 #define GFCC_OPT_SETUP_EMULATE_FLOPS 19 /* contexts created GFCC_PREC_MIXED_BF16 evaluate the setup
                                      contractions of at least this many flops from digit planes on
-                                     the tensor cores (FP64-accurate); default 4e12, 0 = all of them   */
+                                     the tensor cores (FP64-accurate); default 4e12, 0 = all of them.
+                                     Smaller ones do so too where the planes are the faster way, unless
+                                     the value is above the default                                    */
 #define GFCC_OPT_WAIT_NS    20    /* limit of the bounded waits of the tensor-core kernels in
                                      nanoseconds (1 .. 1e11); default 1e9.  A wait that runs out makes
                                      the call return GFCC_ERR_TIMEOUT                                   */
@@ -115,9 +117,9 @@ extern "C" {
                                      launches of several waves, 1 always (unless GFCC_OPT_GEMM_PAIR is
                                      1), 2 never                                                        */
 #define GFCC_OPT_CLOSED_SHELL_EMULATE 24 /* closed-shell contexts (gfcc_create_rhf) only: 1 (default) the
-                                     contractions of the operator of at least 1e9 flops (the ring sums,
-                                     oooo) are FP64-accurate products of BF16 digit planes on the tensor
-                                     cores; 0 every contraction on the FP64 units                       */
+                                     contractions of the operator of at least 1e9 flops, and smaller ones
+                                     that are faster so, are FP64-accurate products of BF16 digit planes
+                                     on the tensor cores; 0 every contraction on the FP64 units         */
 
 /* Initial guesses (Algorithm 1, "compute initial guess").  With a guess other than ZERO, gfcc_solve
  * keeps every converged solution X_p(omega) (FP32 complex, n_omega * n_orb * dim * 8 bytes of device
@@ -498,8 +500,8 @@ int gfcc_spectral_adaptive(gfcc_ctx *ctx, int sectors, double omega_min, double 
  *   max_iter    : iterations per equation set (>= 1); Jacobi steps with the Fock-diagonal denominators
  *                 f_ii (+ f_jj) - f_aa (- f_bb), extrapolated by DIIS over the last 8 iterates.
  *   flags       : GFCC_CCSD_EMULATE - contractions of at least 1e10 flops (or the setup threshold
- *                 GFCC_OPT_SETUP_EMULATE_FLOPS when that is lower) through the FP64-accurate digit-plane
- *                 products on the BF16 tensor cores; GFCC_CCSD_GUESS - t1, t2 (and lambda) hold initial iterates on entry
+ *                 GFCC_OPT_SETUP_EMULATE_FLOPS when that is lower), and smaller ones that are faster so,
+ *                 through the FP64-accurate digit-plane products on the BF16 tensor cores; GFCC_CCSD_GUESS - t1, t2 (and lambda) hold initial iterates on entry
  *                 (else both start from zero, Lambda from T).
  *   t1 [o][v], t2 [o][o][v][v] : out (in with GFCC_CCSD_GUESS), host; t2 antisymmetric.
  *   lambda      : NULL (T only) or out [lambda1 (o x v) | lambda2 (o x o x v x v)], the layout

@@ -515,9 +515,14 @@ int create_impl(int o, int v, int L, const double *fock, const double *chol, con
     if (timed) cudaEventRecord(e0, c->stream);
     // mixed-precision contexts build their large FP64 intermediates from digit planes on the
     // tensor cores (FP64-accurate); FP64 contexts keep every contraction on the FP64 units
-    g_emulate_big = precision == GFCC_PREC_MIXED_BF16;
-    s = rhf ? build_hbar_rhf(c, d_fock, d_chol) : build_hbar(c, d_fock, d_chol);
-    g_emulate_big = false;
+    {
+      EmuArena arena;   // the planes' workspace, given back with the set-up
+      g_emulate_big = precision == GFCC_PREC_MIXED_BF16;
+      g_emu_arena = &arena;
+      s = rhf ? build_hbar_rhf(c, d_fock, d_chol) : build_hbar(c, d_fock, d_chol);
+      g_emu_arena = nullptr;
+      g_emulate_big = false;
+    }
     if (timed) {
       cudaEventRecord(e1, c->stream);
       cudaEventSynchronize(e1);

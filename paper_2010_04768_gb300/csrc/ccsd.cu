@@ -38,6 +38,7 @@
 
 #include "ctx.cuh"
 #include "kernels.cuh"
+#include "ozaki.cuh"
 
 namespace gfcc {
 
@@ -608,6 +609,9 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
   }
   const bool prev_emulate = g_emulate_big;
   const double prev_min = g_emulate_min_flops_local;
+  EmuArena arena;   // the digit planes' workspace of the whole call
+  EmuArena *prev_arena = g_emu_arena;
+  g_emu_arena = &arena;
   g_emulate_big = (flags & GFCC_CCSD_EMULATE) != 0;
   // the iteration's large contractions (the vvvv blocks and their ladder products, the ring, the
   // Cholesky sums of the singles) are 1e11-1e12 flops each at medium sizes: below the setup threshold
@@ -671,6 +675,7 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
     s = run(C);
     cudaStreamSynchronize(st);
   }
+  g_emu_arena = prev_arena;
   g_emulate_big = prev_emulate;
   g_emulate_min_flops_local = prev_min;
   cudaGetLastError();

@@ -329,7 +329,8 @@ std::map<cudaStream_t, SplitBuf> g_splitk;
 }  // namespace
 
 thread_local bool g_emulate_big = false;
-double g_emulate_min_flops = 4e12;
+constexpr double EMULATE_MIN_FLOPS_DEFAULT = 4e12;
+double g_emulate_min_flops = EMULATE_MIN_FLOPS_DEFAULT;
 thread_local double g_emulate_min_flops_local = -1.0;
 
 int gemm_f64(cudaStream_t st, long long M, long long N, long long K, double alpha,
@@ -341,11 +342,17 @@ int gemm_f64(cudaStream_t st, long long M, long long N, long long K, double alph
   c.am = am; c.ak = ak; c.bk = bk; c.bn = bn; c.cm = cm; c.cn = cn;
   c.batch = batch; c.sab = sab; c.sbb = sbb; c.scb = scb;
   c.alpha = alpha; c.beta = beta;
-  // Large contractions (setup of big problems) go to the FP64-accurate digit-plane path on the
-  // tensor cores when enabled: at ~1 TFLOP/s of FP64 they would take minutes.
+  // Contractions whose owner allows it (mixed-precision set-up, emulated CCSD, closed-shell operator) run on
+  // the tensor cores from digit planes that hold more bits than FP64 sums keep: all of at least emu_min
+  // flops, and the smaller ones where the planes are faster (unless the threshold was raised above its default).
+  // Without room for the planes the FP64 units do it.
   const double emu_min = g_emulate_min_flops_local >= 0.0 ? g_emulate_min_flops_local : g_emulate_min_flops;
-  if (batch == 1 && g_emulate_big && 2.0 * (double)M * (double)N * (double)K >= emu_min)
-    return gemm_f64_emulated(st, M, N, K, alpha, A, am, ak, B, bk, bn, beta, C, cm, cn, 8, 9);
+  if (batch == 1 && K > 0 && g_emulate_big &&
+      (2.0 * (double)M * (double)N * (double)K >= emu_min ||
+       (g_emulate_min_flops <= EMULATE_MIN_FLOPS_DEFAULT && emulation_pays(M, N, K, false)))) {
+    const int s = gemm_f64_emulated(st, M, N, K, alpha, A, am, ak, B, bk, bn, beta, C, cm, cn);
+    if (s != GFCC_ERR_OOM) return s;
+  }
   // A few 16 x 16 output tiles and a long K: the K ranges of a cluster (8 at most) would not fill the
   // SMs, so K is split further into partial sums in global memory.
   const long long tiles = ((M + 15) / 16) * ((N + 15) / 16);

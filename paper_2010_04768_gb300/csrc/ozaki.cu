@@ -50,16 +50,16 @@ __global__ void rowexp_kernel(const double *A, long long rows, long long K, long
   }
 }
 
-// dig[i][r][k] = i-th base-64 digit of A[r][k] 2^-e[r] (k < K), 0 for K <= k < ld
+// dig[i][r][k] = i-th digit of A[r][k] 2^-e[r] (k < K), 0 for K <= k < ld
 __global__ void slice_kernel(const double *A, long long rows, long long K, long long lda, const int *e, int S,
-                             __nv_bfloat16 *dig, long long ld) {
+                             int bits, __nv_bfloat16 *dig, long long ld) {
   const long long tot = rows * ld;
   const long long plane = rows * ld;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
     const long long r = t / ld, k = t - r * ld;
-    long long Y = k < K ? fixed_point(A[r * lda + k], e[r], 6 * S) : 0;
+    long long Y = k < K ? fixed_point(A[r * lda + k], e[r], bits * S) : 0;
     for (int i = 0; i < S; i++) {
-      const int sh = 6 * (S - 1 - i);
+      const int sh = bits * (S - 1 - i);
       const long long d = sh > 0 ? (Y + (1LL << (sh - 1))) >> sh : Y;
       Y -= d << sh;
       dig[i * plane + t] = __float2bfloat16((float)(int)d);
@@ -110,7 +110,8 @@ long long emu_operand_bytes(long long rows, long long K, int S) {
 }
 
 int emu_slice(cudaStream_t st, const double *A, long long rows, long long K, long long lda, int S, void *mem,
-              EmuOperand &out) {
+              EmuOperand &out, int bits) {
+  out.bits = bits;
   out.rows = rows;
   out.K = K;
   out.ld = (K + 7) / 8 * 8;
@@ -128,7 +129,7 @@ int emu_slice(cudaStream_t st, const double *A, long long rows, long long K, lon
   }
   rowexp_kernel<<<(unsigned)rows, 256, 0, st>>>(A, rows, K, lda, out.exp2);
   GFCC_LAUNCH_CHECK();
-  slice_kernel<<<grid1d(rows * out.ld), 256, 0, st>>>(A, rows, K, lda, out.exp2, S, out.dig, out.ld);
+  slice_kernel<<<grid1d(rows * out.ld), 256, 0, st>>>(A, rows, K, lda, out.exp2, S, bits, out.dig, out.ld);
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -175,17 +176,21 @@ int emu_max_exponent(cudaStream_t st, const EmuOperand &e, int *out) {
 }
 
 int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, double alpha, double beta, double *C,
-             IMap cm, IMap cn, void *work, long long n0) {
+             IMap cm, IMap cn, void *work, long long n0, long long m0) {
   P = std::max(2, P - A.drop);
   const long long M = A.rows, N = B.rows, K = A.K;
   if (M <= 0 || N <= 0) return GFCC_OK;
-  if (B.K != K || A.ld != B.ld) {
-    set_error("emu_gemm: operands disagree in K (%lld vs %lld)", A.K, B.K);
+  if (B.K != K || A.ld != B.ld || A.bits != B.bits) {
+    set_error("emu_gemm: operands disagree in K (%lld vs %lld) or digits (%d vs %d bits)", A.K, B.K, A.bits, B.bits);
     return GFCC_ERR_ARG;
   }
-  if (N <= g_fused_max_n && emu_fused_takes(A.S, B.S, P) && M <= (1LL << 31) - 256 && N <= (1LL << 31) - 256)
+  if ((N <= g_fused_max_n || A.bits != 6) && emu_fused_takes(A.S, B.S, P) && M <= (1LL << 31) - 256 && N <= (1LL << 31) - 256)
     return emu_gemm_fused(st, A.dig, A.rows * A.ld, A.S, A.exp2, B.dig, B.rows * B.ld, B.S, B.exp2, A.ld, (int)M,
-                          (int)N, (int)K, P, 6, alpha, beta, C, cm, cn, n0, static_cast<double *>(work));
+                          (int)N, (int)K, P, A.bits, alpha, beta, C, cm, cn, n0, static_cast<double *>(work), m0);
+  if (A.bits != 6 || m0 != 0) {
+    set_error("emu_gemm: %d-bit digits to level %d are beyond the digit-pair products", A.bits, P);
+    return GFCC_ERR_ARG;
+  }
   const long long nk = (K + 63) / 64;
   const int nz = (int)((nk + KCHUNK_BLOCKS - 1) / KCHUNK_BLOCKS);
   const long long kbs = (nk + nz - 1) / nz;
@@ -236,109 +241,243 @@ int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, d
   return GFCC_OK;
 }
 
+// ---------------------------------------------------------------- strided operands
 namespace {
-// G[r][k] = X[imap(rm, r) + imap(km, k)] for k < K, 0 for K <= k < ld
-__global__ void gather_kernel(const double *X, long long rows, long long K, long long ld, IMap rm, IMap km, long long r0,
-                              double *G) {
-  const long long tot = rows * ld;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const long long r = t / ld, k = t - r * ld;
-    G[t] = k < K ? X[imap_apply(rm, r0 + r) + imap_apply(km, k)] : 0.0;
+
+constexpr int SL_ROWS = 32, SL_K = 64, SL_THREADS = 256;
+
+// Both passes read a SL_ROWS x SL_K tile with the lanes along whichever index of X is contiguous
+// (k_lanes: the K index), so that a transposed operand is read in whole sectors too.
+template <typename F>
+__device__ __forceinline__ void for_tile(bool k_lanes, F f) {
+  for (int e = threadIdx.x; e < SL_ROWS * SL_K; e += SL_THREADS)
+    if (k_lanes)
+      f(e / SL_K, e % SL_K);
+    else
+      f(e % SL_ROWS, e / SL_ROWS);
+}
+
+// be[r] = largest biased exponent among the entries of row r0 + r (be zeroed by the caller); a block
+// covers SL_ROWS rows and `span` K values
+__global__ __launch_bounds__(SL_THREADS) void strided_exp_kernel(const double *X, long long rows, long long K, IMap rm,
+                                                                 IMap km, long long r0, bool k_lanes, int span,
+                                                                 unsigned gx, int *be) {
+  __shared__ int mx[SL_ROWS];
+  __shared__ long long ro[SL_ROWS];
+  const unsigned bx = blockIdx.x % gx, by = blockIdx.x / gx;
+  const long long rb = (long long)bx * SL_ROWS;
+  if (threadIdx.x < SL_ROWS) {
+    mx[threadIdx.x] = 0;
+    ro[threadIdx.x] = rb + threadIdx.x < rows ? imap_apply(rm, r0 + rb + threadIdx.x) : -1;
+  }
+  __syncthreads();
+  const long long kbeg = (long long)by * span, kend = min(K, kbeg + span);
+  if (k_lanes) {
+    // a warp per row: lanes along K
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int r = warp; r < SL_ROWS; r += SL_THREADS / 32) {
+      if (ro[r] < 0) continue;
+      int m = 0;
+      for (long long k = kbeg + lane; k < kend; k += 32)
+        m = max(m, (int)((__double_as_longlong(X[ro[r] + imap_apply(km, k)]) >> 52) & 0x7ff));
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) mx[r] = m;
+    }
+  } else {
+    // lanes along the rows, warps along K
+    const int r = threadIdx.x & 31;
+    int m = 0;
+    if (ro[r] >= 0)
+      for (long long k = kbeg + (threadIdx.x >> 5); k < kend; k += SL_THREADS / 32)
+        m = max(m, (int)((__double_as_longlong(X[ro[r] + imap_apply(km, k)]) >> 52) & 0x7ff));
+    atomicMax(&mx[r], m);
+  }
+  __syncthreads();
+  if (threadIdx.x < SL_ROWS && ro[threadIdx.x] >= 0 && mx[threadIdx.x] > 0) atomicMax(&be[rb + threadIdx.x], mx[threadIdx.x]);
+}
+
+// biased exponent -> e with max_k |X[r][k]| 2^-e in [1/4, 1/2); rows of zeros 0
+__global__ void strided_exp_final_kernel(int *be, long long rows) {
+  const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (r < rows) be[r] = be[r] > 0 ? be[r] - 1021 : 0;
+}
+
+// dig[i][r][k] = i-th digit of X[rm(r0 + r) + km(k)] 2^-e[r] (k < K), 0 for K <= k < ld
+__global__ __launch_bounds__(SL_THREADS) void strided_slice_kernel(const double *X, long long rows, long long K, IMap rm,
+                                                                   IMap km, long long r0, bool k_lanes, const int *e,
+                                                                   int S, int bits, unsigned gx, __nv_bfloat16 *dig,
+                                                                   long long ld) {
+  __shared__ double tile[SL_ROWS][SL_K + 1];
+  __shared__ long long ro[SL_ROWS], ko[SL_K];
+  __shared__ int ex[SL_ROWS];
+  const long long rb = (long long)(blockIdx.x % gx) * SL_ROWS, k0 = (long long)(blockIdx.x / gx) * SL_K;
+  if (threadIdx.x < SL_ROWS) {
+    const bool in = rb + threadIdx.x < rows;
+    ro[threadIdx.x] = in ? imap_apply(rm, r0 + rb + threadIdx.x) : -1;
+    ex[threadIdx.x] = in ? e[rb + threadIdx.x] : 0;
+  } else if (threadIdx.x >= 64 && threadIdx.x < 64 + SL_K) {
+    const int k = threadIdx.x - 64;
+    ko[k] = k0 + k < K ? imap_apply(km, k0 + k) : -1;
+  }
+  __syncthreads();
+  for_tile(k_lanes, [&](int r, int k) { tile[r][k] = (ro[r] >= 0 && ko[k] >= 0) ? X[ro[r] + ko[k]] : 0.0; });
+  __syncthreads();
+  const long long plane = rows * ld;
+  for (int t = threadIdx.x; t < SL_ROWS * SL_K / 2; t += SL_THREADS) {
+    const int r = t / (SL_K / 2), k = 2 * (t % (SL_K / 2));
+    if (ro[r] < 0 || k0 + k >= ld) continue;
+    long long Y0 = fixed_point(tile[r][k], ex[r], bits * S), Y1 = fixed_point(tile[r][k + 1], ex[r], bits * S);
+    __nv_bfloat162 *dst = reinterpret_cast<__nv_bfloat162 *>(dig + (rb + r) * ld + k0 + k);
+    for (int i = 0; i < S; i++) {
+      const int sh = bits * (S - 1 - i);
+      const long long d0 = sh > 0 ? (Y0 + (1LL << (sh - 1))) >> sh : Y0;
+      const long long d1 = sh > 0 ? (Y1 + (1LL << (sh - 1))) >> sh : Y1;
+      Y0 -= d0 << sh;
+      Y1 -= d1 << sh;
+      dst[i * (plane / 2)] = __floats2bfloat162_rn((float)(int)d0, (float)(int)d1);
+    }
   }
 }
+
 }  // namespace
 
+int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long long K, IMap rm, IMap km, long long r0,
+                      int S, int bits, void *mem, EmuOperand &out) {
+  out.rows = rows;
+  out.K = K;
+  out.ld = (K + 7) / 8 * 8;
+  out.S = S;
+  out.bits = bits;
+  unsigned char *p = static_cast<unsigned char *>(mem);
+  out.dig = reinterpret_cast<__nv_bfloat16 *>(p);
+  p += ((long long)S * rows * out.ld * 2 + 255) / 256 * 256;
+  out.exp2 = reinterpret_cast<int *>(p);
+  if (rows <= 0 || K <= 0) return GFCC_OK;
+  GFCC_TRY(check_extent(X, 0, imap_max(rm, r0 + rows) + imap_max(km, K), "digit split input"));
+  GFCC_TRY(check_extent_bytes(mem, emu_operand_bytes(rows, K, S), "digit split output"));
+  const bool k_lanes = km.s0 == 1 || rm.s0 != 1;
+  const long long gx = (rows + SL_ROWS - 1) / SL_ROWS, gy = (out.ld + SL_K - 1) / SL_K;
+  // K values per block of the exponent pass: enough blocks for the chip, at least four tiles each
+  long long span = SL_K * 4;
+  while (gx * ((K + span - 1) / span) > 152 * 16 && span < (1 << 20)) span *= 2;
+  const long long gz = (K + span - 1) / span;
+  if (gx * gy > 0x7fffffffLL || gx * gz > 0x7fffffffLL) {
+    set_error("emu_slice_strided: grid too large (rows %lld, K %lld)", rows, K);
+    return GFCC_ERR_ARG;
+  }
+  GFCC_CUDA(cudaMemsetAsync(out.exp2, 0, sizeof(int) * rows, st));
+  strided_exp_kernel<<<(unsigned)(gx * gz), SL_THREADS, 0, st>>>(X, rows, K, rm, km, r0, k_lanes, (int)span, (unsigned)gx,
+                                                                 out.exp2);
+  GFCC_LAUNCH_CHECK();
+  strided_exp_final_kernel<<<cdiv(rows, 256), 256, 0, st>>>(out.exp2, rows);
+  GFCC_LAUNCH_CHECK();
+  strided_slice_kernel<<<(unsigned)(gx * gy), SL_THREADS, 0, st>>>(X, rows, K, rm, km, r0, k_lanes, out.exp2, S, bits,
+                                                                   (unsigned)gx, out.dig, out.ld);
+  GFCC_LAUNCH_CHECK();
+  return GFCC_OK;
+}
+
+thread_local EmuArena *g_emu_arena = nullptr;
+
+int EmuArena::get(size_t bytes, void **out) {
+  if (cap < bytes) {
+    release();
+    if (dmalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+      return GFCC_ERR_OOM;
+    }
+    cap = bytes;
+  }
+  *out = p;
+  return GFCC_OK;
+}
+
+void EmuArena::release() {
+  if (p) dfree(p);   // cudaFree waits for the work that uses it
+  p = nullptr;
+  cap = 0;
+}
+
+namespace {
+constexpr long long EMU_BLOCK_BYTES = 4LL << 30;
+
+// rows (or columns) of a block whose digit planes stay within EMU_BLOCK_BYTES
+long long block_rows(long long rows, long long K) {
+  const long long per = (K + 7) / 8 * 8 * 2 * F64_DIGITS + 8;
+  return std::min(rows, std::max<long long>(256, EMU_BLOCK_BYTES / per / 128 * 128));
+}
+
+long long up256(long long x) { return (x + 255) / 256 * 256; }
+}  // namespace
+
+// FP64 units: 1.1 TFLOP/s on 16 x 16 tiles.  Digit planes: 36 pairs of BF16 products at about 1.1e15
+// flop/s on padded tiles, the split of both operands (two reads of 8 bytes, eight planes of 2 bytes, at
+// about 3 TB/s), and some 8 launches.  Error against quad sums (relative, Gaussian entries): FP64 units 1.9e-16,
+// 3.0e-16, 6.0e-16, 1.4e-15 at K = 64, 300, 1280, 6400; planes 2.1e-16, 2.3e-16, 2.4e-16, 4.0e-16; entries that
+// decay along K as the Cholesky vectors do: 2.6, 4.6, 7.6, 6.8 against 2.8, 3.0, 3.5, 3.5 (1e-16).  Sums too short
+// for the planes to be the more accurate stay on the FP64 units.
+// What it gives: set-up of a mixed IP context at o=40 v=200 L=800 3489 -> 143 ms, IP + EA set-up and solve at
+// o=20 v=100 365 -> 48 ms, CCSD and Lambda at o=16 v=80 404 -> 112 ms, closed-shell solve at o=30 v=150 96 -> 55 ms.
+bool emulation_pays(long long M, long long N, long long K, bool a_ready) {
+  if (K < 160) return false;
+  const double m16 = (double)((M + 15) / 16 * 16), n16 = (double)((N + 15) / 16 * 16);
+  const double f64 = 2.0 * m16 * n16 * (double)K / 1.1e12;
+  const double m128 = (double)((M + 127) / 128 * 128), n32 = (double)((N + 31) / 32 * 32);
+  const double n128 = (double)((N + 127) / 128 * 128), m32 = (double)((M + 31) / 32 * 32);
+  const double tile = std::min(m128 * n32, n128 * m32);
+  const double emu = 36.0 * 2.0 * tile * (double)((K + 63) / 64 * 64) / 1.1e15 + 32.0 * ((a_ready ? 0.0 : (double)M) + (double)N) * (double)K / 3e12 + (a_ready ? 3e-5 : 4e-5);
+  return emu < f64;
+}
+
+int gemm_f64_emulated_pre(cudaStream_t st, const EmuOperand &A, long long N, const double *B, IMap bk, IMap bn,
+                          double alpha, double beta, double *C, IMap cm, IMap cn) {
+  const long long M = A.rows, K = A.K;
+  if (M <= 0 || N <= 0) return GFCC_OK;
+  GFCC_TRY(check_extent(B, 0, imap_max(bk, K) + imap_max(bn, N), "emulated contraction operand B"));
+  GFCC_TRY(check_extent(C, 0, imap_max(cm, M) + imap_max(cn, N), "emulated contraction output C"));
+  const long long nb = block_rows(N, K);
+  const long long bbytes = up256(emu_operand_bytes(nb, K, F64_DIGITS)), wbytes = emu_fused_work_bytes(M, nb, K);
+  EmuArena local;
+  EmuArena *ar = g_emu_arena ? g_emu_arena : &local;
+  void *mem = nullptr;
+  if (ar->get((size_t)(bbytes + wbytes), &mem) < 0) {
+    set_error("emulated contraction: cannot allocate its temporaries (M=%lld N-block=%lld K=%lld)", M, nb, K);
+    return GFCC_ERR_OOM;
+  }
+  void *gw = static_cast<unsigned char *>(mem) + bbytes;
+  EmuOperand eb;
+  for (long long n0 = 0; n0 < N; n0 += nb) {
+    GFCC_TRY(emu_slice_strided(st, B, std::min(nb, N - n0), K, bn, bk, n0, F64_DIGITS, F64_BITS, mem, eb));
+    GFCC_TRY(emu_gemm(st, A, eb, F64_LEVEL, alpha, beta, C, cm, cn, gw, n0));
+  }
+  return GFCC_OK;
+}
+
 int gemm_f64_emulated(cudaStream_t st, long long M, long long N, long long K, double alpha, const double *A, IMap am,
-                      IMap ak, const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn, int S,
-                      int P) {
+                      IMap ak, const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn) {
   if (M <= 0 || N <= 0) return GFCC_OK;
   GFCC_TRY(check_extent(A, 0, imap_max(am, M) + imap_max(ak, K), "emulated contraction operand A"));
   GFCC_TRY(check_extent(B, 0, imap_max(bk, K) + imap_max(bn, N), "emulated contraction operand B"));
   GFCC_TRY(check_extent(C, 0, imap_max(cm, M) + imap_max(cn, N), "emulated contraction output C"));
-  const long long ld = (K + 7) / 8 * 8;
-  // column blocks of B / C sized so that one pass stays within about 12 GB of temporaries
-  const long long budget = 12LL << 30;
-  const long long nk = (K + 63) / 64, nz = (nk + KCHUNK_BLOCKS - 1) / KCHUNK_BLOCKS;
-  const long long per_col = ld * 8 + (long long)S * ld * 2 + nz * M * 4 + M * 8;
-  long long nb = std::max<long long>(256, budget / std::max<long long>(per_col, 1));
-  nb = std::min(nb, N);
-  void *ag = nullptr, *adig = nullptr, *bg = nullptr, *bdig = nullptr, *w = nullptr;
-  int s = GFCC_OK;
-  if (dmalloc(&ag, sizeof(double) * M * ld) != cudaSuccess || dmalloc(&adig, emu_operand_bytes(M, K, S)) != cudaSuccess ||
-      dmalloc(&bg, sizeof(double) * nb * ld) != cudaSuccess || dmalloc(&bdig, emu_operand_bytes(nb, K, S)) != cudaSuccess ||
-      dmalloc(&w, emu_gemm_work_bytes(M, nb, K)) != cudaSuccess) {
-    cudaGetLastError();
-    set_error("emulated contraction: cannot allocate its temporaries (M=%lld N-block=%lld K=%lld)", M, nb, K);
-    s = GFCC_ERR_OOM;
-  }
+  const long long mb = block_rows(M, K), nb = block_rows(N, K);
+  const long long abytes = up256(emu_operand_bytes(mb, K, F64_DIGITS)), bbytes = up256(emu_operand_bytes(nb, K, F64_DIGITS));
+  EmuArena local;
+  EmuArena *ar = g_emu_arena ? g_emu_arena : &local;
+  void *mem = nullptr;
+  GFCC_TRY(ar->get((size_t)(abytes + bbytes + emu_fused_work_bytes(mb, nb, K)), &mem));
+  void *bm = static_cast<unsigned char *>(mem) + abytes, *gw = static_cast<unsigned char *>(bm) + bbytes;
   EmuOperand ea, eb;
-  if (s == GFCC_OK) {
-    gather_kernel<<<grid1d(M * ld), 256, 0, st>>>(A, M, K, ld, am, ak, 0, static_cast<double *>(ag));
-    if (cudaGetLastError() != cudaSuccess) s = GFCC_ERR_CUDA;
-    count_launch();
-  }
-  if (s == GFCC_OK) s = emu_slice(st, static_cast<double *>(ag), M, K, ld, S, adig, ea);
-  for (long long n0 = 0; n0 < N && s == GFCC_OK; n0 += nb) {
-    const long long cols = std::min(nb, N - n0);
-    gather_kernel<<<grid1d(cols * ld), 256, 0, st>>>(B, cols, K, ld, bn, bk, n0, static_cast<double *>(bg));
-    count_launch();
-    if (cudaGetLastError() != cudaSuccess) {
-      s = GFCC_ERR_CUDA;
-      break;
+  for (long long m0 = 0; m0 < M; m0 += mb) {
+    const long long rows = std::min(mb, M - m0);
+    GFCC_TRY(emu_slice_strided(st, A, rows, K, am, ak, m0, F64_DIGITS, F64_BITS, mem, ea));
+    for (long long n0 = 0; n0 < N; n0 += nb) {
+      const long long cols = std::min(nb, N - n0);
+      if (m0 == 0 || nb < N) GFCC_TRY(emu_slice_strided(st, B, cols, K, bn, bk, n0, F64_DIGITS, F64_BITS, bm, eb));
+      GFCC_TRY(emu_gemm(st, ea, eb, F64_LEVEL, alpha, beta, C, cm, cn, gw, n0, m0));
     }
-    s = emu_slice(st, static_cast<double *>(bg), cols, K, ld, S, bdig, eb);
-    if (s == GFCC_OK) s = emu_gemm(st, ea, eb, P, alpha, beta, C, cm, cn, w, n0);
   }
-  if (s == GFCC_OK && cudaStreamSynchronize(st) != cudaSuccess) {
-    set_error("emulated contraction failed: %s", cudaGetErrorString(cudaGetLastError()));
-    s = GFCC_ERR_CUDA;
-  }
-  for (void *p : {ag, adig, bg, bdig, w}) dfree(p);
-  return s;
-}
-
-int gemm_f64_emulated_pre(cudaStream_t st, const EmuOperand &A, long long N, const double *B, IMap bk, IMap bn,
-                          double alpha, double beta, double *C, IMap cm, IMap cn, int P) {
-  const long long M = A.rows, K = A.K, S = A.S;
-  if (M <= 0 || N <= 0) return GFCC_OK;
-  GFCC_TRY(check_extent(B, 0, imap_max(bk, K) + imap_max(bn, N), "emulated contraction operand B"));
-  GFCC_TRY(check_extent(C, 0, imap_max(cm, M) + imap_max(cn, N), "emulated contraction output C"));
-  const long long ld = (K + 7) / 8 * 8;
-  if (A.ld != ld) {
-    set_error("emulated contraction: the sliced operand's row stride %lld is not %lld", A.ld, ld);
-    return GFCC_ERR_ARG;
-  }
-  const long long budget = 12LL << 30;
-  const long long nk = (K + 63) / 64, nz = (nk + KCHUNK_BLOCKS - 1) / KCHUNK_BLOCKS;
-  const long long per_col = ld * 8 + S * ld * 2 + nz * M * 4 + M * 8;
-  long long nb = std::max<long long>(256, budget / std::max<long long>(per_col, 1));
-  nb = std::min(nb, N);
-  void *bg = nullptr, *bdig = nullptr, *w = nullptr;
-  int s = GFCC_OK;
-  if (dmalloc(&bg, sizeof(double) * nb * ld) != cudaSuccess || dmalloc(&bdig, emu_operand_bytes(nb, K, (int)S)) != cudaSuccess ||
-      dmalloc(&w, emu_gemm_work_bytes(M, nb, K)) != cudaSuccess) {
-    cudaGetLastError();
-    set_error("emulated contraction: cannot allocate its temporaries (M=%lld N-block=%lld K=%lld)", M, nb, K);
-    s = GFCC_ERR_OOM;
-  }
-  EmuOperand eb;
-  for (long long n0 = 0; n0 < N && s == GFCC_OK; n0 += nb) {
-    const long long cols = std::min(nb, N - n0);
-    gather_kernel<<<grid1d(cols * ld), 256, 0, st>>>(B, cols, K, ld, bn, bk, n0, static_cast<double *>(bg));
-    count_launch();
-    if (cudaGetLastError() != cudaSuccess) {
-      s = GFCC_ERR_CUDA;
-      break;
-    }
-    s = emu_slice(st, static_cast<double *>(bg), cols, K, ld, (int)S, bdig, eb);
-    if (s == GFCC_OK) s = emu_gemm(st, A, eb, P, alpha, beta, C, cm, cn, w, n0);
-  }
-  if (s == GFCC_OK && cudaStreamSynchronize(st) != cudaSuccess) {
-    set_error("emulated contraction failed: %s", cudaGetErrorString(cudaGetLastError()));
-    s = GFCC_ERR_CUDA;
-  }
-  for (void *q : {bg, bdig, w}) dfree(q);
-  return s;
+  return GFCC_OK;
 }
 
 }  // namespace gfcc

@@ -8,13 +8,14 @@
 
 namespace gfcc {
 
-// An FP64 matrix (rows x K, K-major) split into S base-64 digit planes with a power-of-two
-// scale per row: A[r][k] ~= 2^exp2[r] sum_i dig[i][r][k] 64^-(i+1).
+// An FP64 matrix (rows x K, K-major) split into S planes of balanced `bits`-bit digits (6: base 64) with
+// a power-of-two scale per row: A[r][k] ~= 2^exp2[r] sum_i dig[i][r][k] 2^(-bits (i+1)).
 struct EmuOperand {
   __nv_bfloat16 *dig = nullptr;   // [S][rows][ld]
   int *exp2 = nullptr;            // [rows]
   long long rows = 0, K = 0, ld = 0;
   int S = 0;
+  int bits = 6;
   // levels this operand's products may drop (as the A operand of emu_gemm) while keeping the error
   // bound of the level-P product of the operator with its Fock-like diagonal (set at setup: see
   // emu_level_drop)
@@ -32,22 +33,44 @@ static inline int emu_level_drop(int e_max, double min_diag) {
 
 long long emu_operand_bytes(long long rows, long long K, int S);
 int emu_slice(cudaStream_t st, const double *A, long long rows, long long K, long long lda, int S, void *mem,
-              EmuOperand &out);
+              EmuOperand &out, int bits = 6);
 long long emu_gemm_work_bytes(long long M, long long N, long long K);
 void emu_set_fused_max_n(long long n);   // widest product (columns) for the fused digit kernel
 // C(m, n) = alpha * sum_k A[m][k] B[n][k] + beta * C(m, n) with digit pairs i + j <= P
-// (the output column index of B's row n is n0 + n)
+// (the output row index of A's row m is m0 + m, the column index of B's row n is n0 + n)
 int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, double alpha, double beta, double *C,
-             IMap cm, IMap cn, void *work, long long n0 = 0);
-// A strided FP64 contraction (the index maps of gemm_f64) evaluated from digit planes: operands are
-// gathered K-major, split into S digits, multiplied pairwise (i + j <= P) and combined in FP64.
-int gemm_f64_emulated(cudaStream_t st, long long M, long long N, long long K, double alpha, const double *A, IMap am,
-                      IMap ak, const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn, int S,
-                      int P);
+             IMap cm, IMap cn, void *work, long long n0 = 0, long long m0 = 0);
+// Digits of the contractions that take the place of FP64 ones: 8 digits of 7 bits hold 56 bits below the
+// row scale (an FP64 sum keeps 53 below each of its partial sums), pairs to level 9.
+constexpr int F64_DIGITS = 8, F64_BITS = 7, F64_LEVEL = 9;
 
-// The same with A already split into digit planes (rows x K, K-major; emu_slice with S digits): only B
+// Split rows r0 .. r0 + rows - 1 of a strided matrix, X[rm(r) + km(k)], into digit planes.  `mem` holds
+// emu_operand_bytes(rows, K, S).
+int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long long K, IMap rm, IMap km, long long r0,
+                      int S, int bits, void *mem, EmuOperand &out);
+
+// Workspace of the emulated contractions below: kept by its owner between calls, grown on demand.
+struct EmuArena {
+  void *p = nullptr;
+  size_t cap = 0;
+  int get(size_t bytes, void **out);   // GFCC_ERR_OOM (with no message kept) when it cannot grow
+  void release();
+  ~EmuArena() { release(); }
+};
+// the calling thread's arena (nullptr: a call allocates and frees its own)
+extern thread_local EmuArena *g_emu_arena;
+
+// A strided FP64 contraction (the index maps of gemm_f64) evaluated from digit planes (F64_DIGITS of
+// F64_BITS): operands are gathered K-major and split, multiplied pairwise and combined with one rounding.
+// Blocks of rows and columns keep the planes within EMU_BLOCK_BYTES each.  GFCC_ERR_OOM: nothing written.
+int gemm_f64_emulated(cudaStream_t st, long long M, long long N, long long K, double alpha, const double *A, IMap am,
+                      IMap ak, const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn);
+// whether the digit planes are faster than the FP64 units (time models of both; a_ready: A is split already)
+bool emulation_pays(long long M, long long N, long long K, bool a_ready);
+
+// The same with A already split into digit planes (rows x K, K-major, F64_DIGITS of F64_BITS): only B
 // (given through its index maps, N columns) is gathered and split per call.
 int gemm_f64_emulated_pre(cudaStream_t st, const EmuOperand &A, long long N, const double *B, IMap bk, IMap bn,
-                          double alpha, double beta, double *C, IMap cm, IMap cn, int P);
+                          double alpha, double beta, double *C, IMap cm, IMap cn);
 
 }  // namespace gfcc

@@ -29,12 +29,10 @@
 
 namespace gfcc {
 
-// Contractions of at least this many flops run on the FP64-accurate digit-plane path when the
-// context's emulation option is on (the ring sums and the oooo term at useful sizes; the narrow ones
-// stay on the FP64 units); the digit planes of the ring matrices are cut once at setup with the
-// digit count and pair level of the setup's emulated contractions
+// With the context's emulation option on, the operator's contractions run from digit planes (F64_DIGITS of
+// F64_BITS, more bits than FP64 sums keep): those of at least this many flops, and the smaller ones where the
+// planes are faster.  The planes of the constant operands are cut once at setup.
 constexpr double RHF_EMULATE_MIN_FLOPS = 1e9;
-constexpr int RHF_EMU_DIGITS = 8, RHF_EMU_LEVEL = 9;
 
 namespace {
 
@@ -351,26 +349,6 @@ int build_hbar_rhf(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
   GFCC_LAUNCH_CHECK();
   rhf_fold_kernel<<<cdiv(ov, 128), 128, 0, st>>>(c->rM2, o, v, c->Foo, c->Fvv, -1.0, 1.0);
   GFCC_LAUNCH_CHECK();
-  // digit planes of the three ring matrices, sliced once here for the digit-plane operator (when the
-  // three together take at most a quarter of the free device memory)
-  {
-    const long long eb = emu_operand_bytes(ov, ov, RHF_EMU_DIGITS);
-    size_t fr = 0, tot = 0;
-    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-      cudaGetLastError();
-      fr = 0;
-    }
-    if (3.0 * (double)eb <= 0.25 * (double)fr) {
-      gfcc::EmuOperand *ops[3] = {&c->rM1e, &c->rM2e, &c->rM3e};
-      double *mats[3] = {c->rM1, c->rM2, c->rM3};
-      for (int k = 0; k < 3; k++) {
-        double *mem;
-        GFCC_TRY(dev_alloc(c, &mem, eb / 8 + 1));
-        GFCC_TRY(emu_slice(st, mats[k], ov, ov, ov, RHF_EMU_DIGITS, mem, *ops[k]));
-      }
-    }
-  }
-
   // ---- [(i,j,a)][e | m] = [-t_ij^ea | -W_maij]
   {
     double *T3;
@@ -404,6 +382,31 @@ int build_hbar_rhf(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     GFCC_TRY(permute4(st, df, c->Fov, isf, c->rU1 + o, osm, 2.0, 1.0));                   // m = i
     GFCC_TRY(permute4(st, df, c->Fov, isf, c->rU1 + o, osn, -1.0, 1.0));                  // n = i
   }
+  // digit planes of the operator's matrices, in the order of what they save, as long as they take at most a
+  // quarter of the device memory that is free
+  {
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+      cudaGetLastError();
+      fr = 0;
+    }
+    double left = 0.25 * (double)fr;
+    auto planes = [&](const double *X, long long rows, long long K, IMap rm, IMap km, EmuOperand &e) -> int {
+      const long long bytes = emu_operand_bytes(rows, K, F64_DIGITS);
+      if ((double)bytes > left) return GFCC_OK;
+      left -= (double)bytes;
+      double *mem;
+      GFCC_TRY(dev_alloc(c, &mem, bytes / 8 + 1));
+      return emu_slice_strided(st, X, rows, K, rm, km, 0, F64_DIGITS, F64_BITS, mem, e);
+    };
+    GFCC_TRY(planes(c->rM1, ov, ov, imap1(ov), imap1(1), c->rM1e));
+    GFCC_TRY(planes(c->rM2, ov, ov, imap1(ov), imap1(1), c->rM2e));
+    GFCC_TRY(planes(c->rM3, ov, ov, imap1(ov), imap1(1), c->rM3e));
+    GFCC_TRY(planes(c->Woooo, oo, oo, imap1(1), imap1(oo), c->rWqe));
+    GFCC_TRY(planes(c->rWT, o2v, v + o, imap1(v + o), imap1(1), c->rWTe));
+    GFCC_TRY(planes(c->rVz, v, o2v, imap1(o2v), imap1(1), c->rVze));
+    GFCC_TRY(planes(c->rU1, o, o + o2v, imap1(o + o2v), imap1(1), c->rU1e));
+  }
   GFCC_TRY(dev_alloc(c, &c->diag_ip, c->dim_ip));
   rhf_diag_kernel<<<grid1d(c->dim_ip), 256, 0, st>>>(c->Foo, c->Fvv, o, v, c->diag_ip);
   GFCC_LAUNCH_CHECK();
@@ -415,20 +418,24 @@ namespace {
 struct EmulateScope {
   bool prev_big;
   double prev_min;
-  explicit EmulateScope(bool on) : prev_big(g_emulate_big), prev_min(g_emulate_min_flops_local) {
+  EmuArena *prev_arena;
+  EmulateScope(bool on, EmuArena *arena)
+      : prev_big(g_emulate_big), prev_min(g_emulate_min_flops_local), prev_arena(g_emu_arena) {
     g_emulate_big = on;
+    g_emu_arena = arena;
     g_emulate_min_flops_local = on ? RHF_EMULATE_MIN_FLOPS : prev_min;
   }
   ~EmulateScope() {
     g_emulate_big = prev_big;
     g_emulate_min_flops_local = prev_min;
+    g_emu_arena = prev_arena;
   }
 };
 }  // namespace
 
 int apply_ip_rhf(gfcc_ctx *c, const SysBatch &b, double *work) {
   cudaStream_t st = c->stream;
-  EmulateScope emu(c->rhf_emulate != 0);
+  EmulateScope emu(c->rhf_emulate != 0, &c->emu_arena);
   const long long o = c->o, v = c->v, ov = o * v, oo = o * o, o2v = oo * v, C2 = 2LL * b.nsys, dim = c->dim_ip;
   double *P = work;                    // [z (v rows) | r1u (o) | r2u (o^2 v)] x C2
   double *r1u = P + v * C2;
@@ -438,23 +445,28 @@ int apply_ip_rhf(gfcc_ctx *c, const SysBatch &b, double *work) {
   PhaseTimer tsig(c, PH_SIGMA, b.nsys * rhf_sigma_flops(c));
   rhf_unpack_kernel<<<grid1d(dim * b.nsys), 256, 0, st>>>(b, dim, C2, r1u);
   GFCC_LAUNCH_CHECK();
+  // C (+)= X B with X's digit planes where the operator runs on them, else through gemm_f64
+  auto product = [&](const double *X, IMap xm, IMap xk, const EmuOperand &Xe, long long M, long long N, long long K,
+                     const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn) -> int {
+    if (c->rhf_emulate && Xe.dig != nullptr &&
+        (2.0 * (double)M * (double)N * (double)K >= RHF_EMULATE_MIN_FLOPS || emulation_pays(M, N, K, true))) {
+      const int s = gemm_f64_emulated_pre(st, Xe, N, B, bk, bn, 1.0, beta, C, cm, cn);
+      if (s != GFCC_ERR_OOM) return s;
+    }
+    return gemm_f64(st, M, N, K, 1.0, X, xm, xk, B, bk, bn, beta, C, cm, cn);
+  };
   // z[e][c] = Vz[e][(m,n,f)] r2u[(m,n,f)][c];  S2 = [-t | -W_maij] [z; r1u]
-  GFCC_TRY(gemm_f64(st, v, C2, o2v, 1.0, c->rVz, imap1(o2v), imap1(1), r2u, imap1(C2), imap1(1), 0.0, P, imap1(C2),
-                    imap1(1)));
-  GFCC_TRY(gemm_f64(st, o2v, C2, v + o, 1.0, c->rWT, imap1(v + o), imap1(1), P, imap1(C2), imap1(1), 0.0, S2, imap1(C2),
-                    imap1(1)));
+  GFCC_TRY(product(c->rVz, imap1(o2v), imap1(1), c->rVze, v, C2, o2v, r2u, imap1(C2), imap1(1), 0.0, P, imap1(C2),
+                   imap1(1)));
+  GFCC_TRY(product(c->rWT, imap1(v + o), imap1(1), c->rWTe, o2v, C2, v + o, P, imap1(C2), imap1(1), 0.0, S2, imap1(C2),
+                   imap1(1)));
   // + W_mnij r_mn^a
-  GFCC_TRY(gemm_f64(st, oo, v * C2, oo, 1.0, c->Woooo, imap1(1), imap1(oo), r2u, imap1(v * C2), imap1(1), 1.0, S2,
-                    imap1(v * C2), imap1(1)));
+  GFCC_TRY(product(c->Woooo, imap1(1), imap1(oo), c->rWqe, oo, v * C2, oo, r2u, imap1(v * C2), imap1(1), 1.0, S2,
+                   imap1(v * C2), imap1(1)));
   {
-    const double rflops = 2.0 * (double)ov * (double)ov * (double)(o * C2);
-    PhaseTimer tr(c, PH_RING, 3.0 * rflops);
-    // the ring matrix k times the B operand (maps bk, bn) into S2 (maps cm, cn): from its digit
-    // planes cut at setup when the operator runs on digit planes, else through gemm_f64
+    PhaseTimer tr(c, PH_RING, 6.0 * (double)ov * (double)ov * (double)(o * C2));
     auto ring = [&](const double *Mk, const EmuOperand &Ek, IMap bk, IMap bn, IMap cm, IMap cn) -> int {
-      if (c->rhf_emulate && Ek.dig != nullptr && rflops >= RHF_EMULATE_MIN_FLOPS)
-        return gemm_f64_emulated_pre(st, Ek, o * C2, r2u, bk, bn, 1.0, 1.0, S2, cm, cn, RHF_EMU_LEVEL);
-      return gemm_f64(st, ov, o * C2, ov, 1.0, Mk, imap1(ov), imap1(1), r2u, bk, bn, 1.0, S2, cm, cn);
+      return product(Mk, imap1(ov), imap1(1), Ek, ov, o * C2, ov, r2u, bk, bn, 1.0, S2, cm, cn);
     };
     // + M1[(i,a)][(m,e)] r[m][j][e]
     GFCC_TRY(ring(c->rM1, c->rM1e, imap2(v, C2, ov * C2), imap2(C2, 1, v * C2), imap2(v, C2, ov * C2),
@@ -464,8 +476,8 @@ int apply_ip_rhf(gfcc_ctx *c, const SysBatch &b, double *work) {
     GFCC_TRY(ring(c->rM3, c->rM3e, imap2(v, C2, ov * C2), imap2(C2, 1, v * C2), imap1(C2), imap2(C2, 1, ov * C2)));
   }
   // S1 = U1 [r1u; r2u]
-  GFCC_TRY(gemm_f64(st, o, C2, o + o2v, 1.0, c->rU1, imap1(o + o2v), imap1(1), r1u, imap1(C2), imap1(1), 0.0, S1,
-                    imap1(C2), imap1(1)));
+  GFCC_TRY(product(c->rU1, imap1(o + o2v), imap1(1), c->rU1e, o, C2, o + o2v, r1u, imap1(C2), imap1(1), 0.0, S1,
+                   imap1(C2), imap1(1)));
   rhf_epilogue_kernel<<<grid1d(dim * b.nsys), 256, 0, st>>>(b, dim, C2, r1u, S1);
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;

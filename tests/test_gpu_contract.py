@@ -34,3 +34,22 @@ def test_sigma_over_tile_shapes(o, v, L, nvec):
         ref = np.stack([ref_of(x) for x in X])
         assert np.abs(g.sigma(sector, X) - ref).max() <= 1e-12 * np.abs(ref).max()
     g.close()
+
+
+@pytest.mark.parametrize("flops", [0.0, 4e12, 1e18])
+@pytest.mark.parametrize("o,v,L", [(1, 2, 3), (3, 7, 9), (7, 33, 41), (12, 61, 243)])
+def test_setup_on_digit_planes(o, v, L, flops):
+    """FP64 sigma of mixed-precision contexts whose set-up contractions (every order of strides the Hbar
+    elements need) all run on digit planes, where they pay, or never: each within the FP64 bound."""
+    pr = make_problem(o, v, L, seed=o + 5 * v, t1_std=0.05, t2_std=0.05, chol_sigma=0.3 if o < 10 else 0.05)
+    gfcc.set_process_option(gfcc.OPT_SETUP_EMULATE_FLOPS, flops)
+    try:
+        g = gfcc.GFCC(pr, precision="mixed")
+    finally:
+        gfcc.set_process_option(gfcc.OPT_SETUP_EMULATE_FLOPS, 4e12)
+    orc = GFCCOracle(pr.fock, pr.chol, pr.t1, pr.t2, o=o)
+    for sector, n, ref_of in (("IP", g.dims()[0], orc.ip_sigma), ("EA", g.dims()[1], orc.ea_sigma)):
+        x = random_vector(1, n) + 1j * random_vector(2, n)
+        ref = ref_of(x)
+        assert np.abs(g.sigma(sector, x)[0] - ref).max() <= 1e-12 * np.abs(ref).max()
+    g.close()
