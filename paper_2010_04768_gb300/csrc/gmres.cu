@@ -9,7 +9,7 @@
 // (CGS2): both passes are batched dot products / vector updates that stream the
 // Krylov basis once each, which suits HBM better than the sequential modified
 // Gram-Schmidt of the oracle and is as stable.  The (m+1) x m Hessenberg matrix
-// of each system is reduced by complex Givens rotations on the device, one thread
+// of each system is reduced by complex Givens rotations on the device, one block
 // per system; a system leaves its cycle when the rotated residual estimate
 // reaches tol ||b|| (or on breakdown), and every cycle ends with the true
 // residual b - A x recomputed by the operator.
@@ -242,116 +242,158 @@ __global__ void cycle_start_kernel(int nsys, const double *nrm2, int NV, const d
   state[s] = ST_IN_CYCLE;
 }
 
-// Givens update of column k for systems in cycle.
+// The least-squares state of the systems (one entry per system, column k of m).
+struct Lsq {
+  int m;
+  double *H, *cs, *sn, *g;
+  const double *bnorm;
+  double tol;
+  int *state, *kcyc, *iters;
+  double *est;
+};
+constexpr int LSQ_MAX = 66;   // m + 2 <= 66
+
+// Givens update of column k of system s, by one block.
 //   h[s*NV + i], i <= k: Gram-Schmidt coefficients (pass 1 + pass 2); h[s*NV + k+1]: ||w||^2 (real part)
-__global__ void givens_kernel(int nsys, int k, int m, const double *h, int NV, double *H, double *cs, double *sn,
-                              double *g, const double *bnorm, double tol, int *state, int *kcyc, int *iters,
-                              double *est) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsys || state[s] != ST_IN_CYCLE) return;
+// The rotations before k act on the column one after the other, a_{i+1} = conj(c_i) h_{i+1} - s_i a_i (s_i
+// is real: the subdiagonal is), the only serial chain; loads, products and the rotated column
+// t_i = c_i a_i + s_i h_{i+1} are spread over the threads.
+__device__ void givens_update(const Lsq &q, int s, int k, const double *h, int NV) {
+  __shared__ double2 hh[LSQ_MAX], cc[LSQ_MAX], aa[LSQ_MAX], pq[LSQ_MAX];
+  __shared__ double ss[LSQ_MAX];
+  const int t = threadIdx.x, m = q.m;
   const double2 *hs = reinterpret_cast<const double2 *>(h) + (long long)s * NV;
-  double2 *Hs = reinterpret_cast<double2 *>(H) + (long long)s * (m + 1) * m;   // column-major [col][row], ld m+1
-  double2 *css = reinterpret_cast<double2 *>(cs) + (long long)s * m;
-  double2 *sns = reinterpret_cast<double2 *>(sn) + (long long)s * m;
-  double2 *gs = reinterpret_cast<double2 *>(g) + (long long)s * (m + 1);
-  double2 col[65];
-  for (int i = 0; i <= k; i++) col[i] = hs[i];
-  const double hk1 = sqrt(fmax(hs[k + 1].x, 0.0));
-  col[k + 1] = make_double2(hk1, 0.0);
-  for (int i = 0; i < k; i++) {   // previous rotations: [c, s; -conj(s), conj(c)]
-    const double2 c = css[i], sv = sns[i], a = col[i], b = col[i + 1];
-    const double2 t = make_double2(c.x * a.x - c.y * a.y + sv.x * b.x - sv.y * b.y,
-                                   c.x * a.y + c.y * a.x + sv.x * b.y + sv.y * b.x);
-    const double2 u = make_double2(-(sv.x * a.x + sv.y * a.y) + (c.x * b.x + c.y * b.y),
-                                   -(sv.x * a.y - sv.y * a.x) + (c.x * b.y - c.y * b.x));
-    col[i] = t;
-    col[i + 1] = u;
+  double2 *css = reinterpret_cast<double2 *>(q.cs) + (long long)s * m;
+  double2 *sns = reinterpret_cast<double2 *>(q.sn) + (long long)s * m;
+  double2 *gs = reinterpret_cast<double2 *>(q.g) + (long long)s * (m + 1);
+  double2 *Hk = reinterpret_cast<double2 *>(q.H) + (long long)s * (m + 1) * m + (long long)k * (m + 1);
+  if (t <= k + 1) hh[t] = hs[t];
+  if (t < k) {
+    const double2 c = css[t], b = hs[t + 1];
+    cc[t] = c;
+    ss[t] = sns[t].x;
+    pq[t] = make_double2(c.x * b.x + c.y * b.y, c.x * b.y - c.y * b.x);   // conj(c) h_{t+1}
   }
-  const double2 a = col[k], b = col[k + 1];
-  const double den = sqrt(a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y);
-  double2 c, sv;
-  if (den > 0.0) {
-    c = make_double2(a.x / den, -a.y / den);    // conj(a) / den
-    sv = make_double2(b.x / den, -b.y / den);   // conj(b) / den
-  } else {
-    c = make_double2(1.0, 0.0);
-    sv = make_double2(0.0, 0.0);
+  __syncthreads();
+  if (t == 0) {
+    double2 a = hh[0];
+    aa[0] = a;
+    for (int i = 0; i < k; i++) {
+      a = make_double2(pq[i].x - ss[i] * a.x, pq[i].y - ss[i] * a.y);
+      aa[i + 1] = a;
+    }
+    const double hk1 = sqrt(fmax(hh[k + 1].x, 0.0));
+    const double den = sqrt(a.x * a.x + a.y * a.y + hk1 * hk1);
+    double2 c, sv;
+    if (den > 0.0) {
+      c = make_double2(a.x / den, -a.y / den);    // conj(a) / den
+      sv = make_double2(hk1 / den, 0.0);
+    } else {
+      c = make_double2(1.0, 0.0);
+      sv = make_double2(0.0, 0.0);
+    }
+    css[k] = c;
+    sns[k] = sv;
+    const double2 gk = gs[k];
+    const double2 g1 = make_double2(-sv.x * gk.x, -sv.x * gk.y);                              // -s g_k
+    gs[k + 1] = g1;
+    gs[k] = make_double2(c.x * gk.x - c.y * gk.y, c.x * gk.y + c.y * gk.x);                   // c g_k
+    Hk[k] = make_double2(den, 0.0);
+    q.iters[s] += 1;
+    const double bn = q.bnorm[s], res = sqrt(g1.x * g1.x + g1.y * g1.y);
+    q.est[s] = bn > 0.0 ? res / bn : 0.0;
+    const bool breakdown = !(hk1 > 1e-14 * den);
+    if (res <= q.tol * bn || breakdown || k + 1 == m || den == 0.0) {
+      q.state[s] = ST_CYCLE_DONE;
+      q.kcyc[s] = k + 1;
+    }
   }
-  css[k] = c;
-  sns[k] = sv;
-  col[k] = make_double2(den, 0.0);
-  col[k + 1] = make_double2(0.0, 0.0);
-  const double2 gk = gs[k];
-  gs[k + 1] = make_double2(-(sv.x * gk.x + sv.y * gk.y), -(sv.x * gk.y - sv.y * gk.x));   // -conj(s) g_k
-  gs[k] = make_double2(c.x * gk.x - c.y * gk.y, c.x * gk.y + c.y * gk.x);                  // c g_k
-  for (int i = 0; i <= k; i++) Hs[(long long)k * (m + 1) + i] = col[i];
-  iters[s] += 1;
-  const double res = sqrt(gs[k + 1].x * gs[k + 1].x + gs[k + 1].y * gs[k + 1].y);
-  est[s] = bnorm[s] > 0.0 ? res / bnorm[s] : 0.0;
-  const bool breakdown = !(hk1 > 1e-14 * den);
-  if (res <= tol * bnorm[s] || breakdown || k + 1 == m || den == 0.0) {
-    state[s] = ST_CYCLE_DONE;
-    kcyc[s] = k + 1;
+  __syncthreads();
+  if (t < k) {
+    const double2 c = cc[t], a = aa[t], b = hh[t + 1];
+    Hk[t] = make_double2(c.x * a.x - c.y * a.y + ss[t] * b.x, c.x * a.y + c.y * a.x + ss[t] * b.y);
   }
 }
 
-// y = R^-1 g (back substitution on the rotated Hessenberg), stored in y[s*NV + i]
-__global__ void backsolve_kernel(int nsys, int m, const double *H, const double *g, const int *state, const int *kcyc,
-                                 double *y, int NV) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsys || state[s] != ST_CYCLE_DONE) return;
+// y = R^-1 g (back substitution on the rotated Hessenberg), stored in y[s*NV + i]; one block of 64 threads
+// per system (thread i holds the remainder of row i; m <= 64), column by column
+__global__ __launch_bounds__(64) void backsolve_kernel(int m, const double *H, const double *g, const int *state,
+                                                       const int *kcyc, double *y, int NV) {
+  __shared__ double2 xj;
+  const int s = blockIdx.x, i = threadIdx.x;
+  if (state[s] != ST_CYCLE_DONE) return;
   const double2 *Hs = reinterpret_cast<const double2 *>(H) + (long long)s * (m + 1) * m;
   const double2 *gs = reinterpret_cast<const double2 *>(g) + (long long)s * (m + 1);
   double2 *ys = reinterpret_cast<double2 *>(y) + (long long)s * NV;
   const int k = kcyc[s];
-  for (int i = k - 1; i >= 0; i--) {
-    double2 acc = gs[i];
-    for (int j = i + 1; j < k; j++) {
-      const double2 r = Hs[(long long)j * (m + 1) + i], yj = ys[j];
-      acc.x -= r.x * yj.x - r.y * yj.y;
-      acc.y -= r.x * yj.y + r.y * yj.x;
+  double2 acc = i < k ? gs[i] : make_double2(0.0, 0.0);
+  double2 r = k > 0 && i < k ? Hs[(long long)(k - 1) * (m + 1) + i] : make_double2(0.0, 0.0);
+  for (int j = k - 1; j >= 0; j--) {
+    // r = R[i][j] (rows i <= j); the next column is loaded while this one is used
+    const double2 nx = j > 0 && i < j ? Hs[(long long)(j - 1) * (m + 1) + i] : make_double2(0.0, 0.0);
+    if (i == j) {
+      const double dd = r.x * r.x + r.y * r.y;
+      xj = dd > 0.0 ? make_double2((acc.x * r.x + acc.y * r.y) / dd, (acc.y * r.x - acc.x * r.y) / dd)
+                    : make_double2(0.0, 0.0);
     }
-    const double2 d = Hs[(long long)i * (m + 1) + i];
-    const double dd = d.x * d.x + d.y * d.y;
-    ys[i] = dd > 0.0 ? make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd)
-                     : make_double2(0.0, 0.0);
+    __syncthreads();
+    const double2 x = xj;
+    if (i < j) {
+      acc.x -= r.x * x.x - r.y * x.y;
+      acc.y -= r.x * x.y + r.y * x.x;
+    }
+    if (i == j) ys[i] = x;
+    r = nx;
+    __syncthreads();
   }
-  for (int i = k; i < NV; i++) ys[i] = make_double2(0.0, 0.0);
+  for (int t = k + i; t < NV; t += 64) ys[t] = make_double2(0.0, 0.0);
 }
-
-__global__ void coef_add_kernel(int nsys, int nv, double *h, const double *h2, int NV, const int *state, int want) {
-  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (t >= (long long)nsys * nv) return;
-  const int s = (int)(t / nv), i = (int)(t % nv);
-  if (state[s] != want) return;
-  const long long q = 2 * ((long long)s * NV + i);
-  h[q] += h2[q];
-  h[q + 1] += h2[q + 1];
-}
-
 
 // ---------------------------------------------------------------- fused Gram-Schmidt passes
-// Both passes stream the Krylov basis of a system once per chunk of CGS_CHUNK elements.  They are
-// HBM-bound, so what matters is the number of independent loads each thread has in flight:
+// Both passes stream the Krylov basis of a system once per chunk of elements.  They are
+// HBM-bound, so what matters is the number of independent loads in flight:
 // * dots: each warp of a block owns whole basis vectors (i = warp, warp + 8, ...; i = nv is w
 //   itself, for ||w||^2) and sweeps the chunk with CGS_UNROLL independent loads per lane; w is
 //   re-read by every warp from L1.  No block-level reduction: one warp shuffle per vector.
 // * update: every thread owns two elements and accumulates sum_i c_i V_i over batches of
 //   CGS_BATCH vectors whose loads are predicated (not branched), so they issue together.
-constexpr int CGS_THREADS = 256, CGS_CHUNK = 4096, CGS_UNROLL = 8, CGS_BATCH = 8;
+// The chunk length follows the number of systems in cycle, so that a few systems fill the chip too
+// (256 elements at least).  The last block of a system adds up its chunks' partial sums in chunk order and takes
+// what follows from them: coefficients, the test for a second pass, the Givens update.  With a kernel
+// for each of these (twelve launches a step) a step of the 30 systems of o=27 v=133 took 208 us beside
+// 30 us of least squares; now 5 launches.
+constexpr int CGS_THREADS = 256, CGS_MIN_CHUNK = 256, CGS_MAX_CHUNK = 4096, CGS_BLOCKS = 1200, CGS_UNROLL = 8, CGS_BATCH = 8;
 constexpr double REORTH_THETA_F32 = 0.01;   // FP32 Krylov vectors: second pass where ||w'|| < 0.1 ||w||
 
+// true in the block of system s that finishes last (counter left at zero for the next kernel)
+__device__ __forceinline__ bool last_block(unsigned *cnt, int s) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(&cnt[s], 1u) == gridDim.x - 1;
+    if (last) cnt[s] = 0;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last != 0;
+}
+
+// out[s*NV + i] = <V_i, w> for i < nv, ||w||^2 for i = nv, for the systems in cycle (second pass: of those, the
+// flagged ones).  grid (chunks of `clen` elements, systems)
 template <typename T>
 __global__ __launch_bounds__(CGS_THREADS) void cgs_dots_kernel(const T *V, long long vs, long long vi, int nv,
-                                                               const T *w, long long n, int nch, const int *state,
-                                                               int want, double *partial, int NV) {
-  const int s = blockIdx.y, chunk = blockIdx.x;
-  if (state[s] != want) return;
+                                                               const T *w, long long n, int clen, const int *state,
+                                                               const int *flag, double *partial, int NV, double *out,
+                                                               unsigned *cnt) {
+  const int s = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
+  if (state[s] != ST_IN_CYCLE || (flag != nullptr && !flag[s])) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long e0 = (long long)chunk * CGS_CHUNK;
-  const long long e1 = e0 + CGS_CHUNK < n ? e0 + CGS_CHUNK : n;
+  const long long e0 = (long long)chunk * clen;
+  const long long e1 = e0 + clen < n ? e0 + clen : n;
   const T *ws = w + 2 * s * vs;
   const T *Vs = V + 2 * s * vs;
+  double2 *ps = reinterpret_cast<double2 *>(partial) + (long long)s * NV * nch;
   for (int i = warp; i <= nv; i += CGS_THREADS / 32) {
     const T *vp = i < nv ? Vs + 2 * i * vi : ws;   // slot nv: ||w||^2
     T ar = T(0), ai = T(0);
@@ -380,30 +422,83 @@ __global__ __launch_bounds__(CGS_THREADS) void cgs_dots_kernel(const T *V, long 
       acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
       acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
     }
-    if (lane == 0) reinterpret_cast<double2 *>(partial)[((long long)s * NV + i) * nch + chunk] = acc;
+    if (lane == 0) ps[(long long)i * nch + chunk] = acc;
+  }
+  if (!last_block(cnt, s)) return;
+  for (int i = warp; i <= nv; i += CGS_THREADS / 32) {
+    double2 acc = make_double2(0.0, 0.0);
+    for (int c = lane; c < nch; c += 32) {
+      const double2 x = __ldcg(&ps[(long long)i * nch + c]);
+      acc.x += x.x;
+      acc.y += x.y;
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
+      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
+    }
+    if (lane == 0) reinterpret_cast<double2 *>(out)[(long long)s * NV + i] = acc;
   }
 }
 
-// w -= V h2 (in place), then the partial squared norm of w (slot 0)
-template <typename T>
-__global__ __launch_bounds__(CGS_THREADS) void cgs_update_norm_kernel(const T *V, long long vs, long long vi, int nv,
-                                                                      T *w, long long n, int nch, const int *state,
-                                                                      int want, const double *h2, double *partial,
-                                                                      int NV) {
+// w -= V coef (in place) and the squared norm of w.
+// First pass (SECOND false): sets flag[s] where the pass cancelled so much of w that it needs the second one
+// (Daniel, Gragg, Kaufman & Stewart 1976: ||w'||^2 < theta ||w||^2), else h[nv] = ||w'||^2.
+// Second pass: over the flagged systems, h += h2 and h[nv] = ||w''||^2.  Its last block (of a system that is
+// not flagged, its first) makes the Givens update of column nv - 1.
+template <typename T, bool SECOND>
+__global__ __launch_bounds__(CGS_THREADS) void cgs_update_kernel(const T *V, long long vs, long long vi, int nv, T *w,
+                                                                 long long n, int clen, int *flag, double *h,
+                                                                 const double *h2, double theta, double *partial,
+                                                                 int NV, unsigned *cnt, Lsq q) {
   __shared__ CT<T> hh[72];
   __shared__ double sh[CGS_THREADS / 32];
-  const int s = blockIdx.y, chunk = blockIdx.x;
-  if (state[s] != want) return;
+  const int s = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
+  if (q.state[s] != ST_IN_CYCLE) return;
+  double2 *hs = reinterpret_cast<double2 *>(h) + (long long)s * NV;
+  if (SECOND && !flag[s]) {
+    // the other blocks of the system may still read state[s]; both outcomes are a return
+    if (chunk == 0) givens_update(q, s, nv - 1, h, NV);
+    return;
+  }
+  const double2 *cf = SECOND ? reinterpret_cast<const double2 *>(h2) + (long long)s * NV : hs;
   for (int i = threadIdx.x; i < nv; i += CGS_THREADS) {
-    const double2 c = reinterpret_cast<const double2 *>(h2)[(long long)s * NV + i];
+    const double2 c = cf[i];
     hh[i] = mkc<T>(c.x, c.y);
   }
   __syncthreads();
-  const long long e0 = (long long)chunk * CGS_CHUNK;
-  const long long e1 = e0 + CGS_CHUNK < n ? e0 + CGS_CHUNK : n;
+  const long long e0 = (long long)chunk * clen;
+  const long long e1 = e0 + clen < n ? e0 + clen : n;
   T *ws = w + 2 * s * vs;
   const T *Vs = V + 2 * s * vs;
   T nn = T(0);
+  if (clen <= CGS_THREADS) {   // one element per thread
+    const long long e = e0 + threadIdx.x;
+    if (e < e1) {
+      CT<T> acc = mkc<T>(0.0, 0.0);
+      int i0 = 0;
+      for (; i0 + 2 * CGS_BATCH <= nv; i0 += 2 * CGS_BATCH) {
+        CT<T> a[2 * CGS_BATCH];
+#pragma unroll
+        for (int j = 0; j < 2 * CGS_BATCH; j++) a[j] = ldc(Vs + 2 * (long long)(i0 + j) * vi, e);
+#pragma unroll
+        for (int j = 0; j < 2 * CGS_BATCH; j++) {
+          const CT<T> c = hh[i0 + j];
+          acc.x += c.x * a[j].x - c.y * a[j].y;
+          acc.y += c.x * a[j].y + c.y * a[j].x;
+        }
+      }
+      for (; i0 < nv; i0++) {
+        const CT<T> a = ldc(Vs + 2 * (long long)i0 * vi, e), c = hh[i0];
+        acc.x += c.x * a.x - c.y * a.y;
+        acc.y += c.x * a.y + c.y * a.x;
+      }
+      CT<T> x = ldc(ws, e);
+      x.x -= acc.x;
+      x.y -= acc.y;
+      stc(ws, e, x);
+      nn = x.x * x.x + x.y * x.y;
+    }
+  } else
   for (long long e = e0 + threadIdx.x; e < e1; e += 2 * CGS_THREADS) {
     const long long f = e + CGS_THREADS;
     const bool inf = f < e1;
@@ -454,40 +549,35 @@ __global__ __launch_bounds__(CGS_THREADS) void cgs_update_norm_kernel(const T *V
   for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
   __syncthreads();
+  double2 *ps = reinterpret_cast<double2 *>(partial) + (long long)s * NV * nch;
   if (threadIdx.x == 0) {
     double tot = 0.0;
     for (int k = 0; k < CGS_THREADS / 32; k++) tot += sh[k];
-    reinterpret_cast<double2 *>(partial)[((long long)s * NV) * nch + chunk] = make_double2(tot, 0.0);
+    ps[chunk] = make_double2(tot, 0.0);
   }
-}
-
-// Selective reorthogonalisation (Daniel, Gragg, Kaufman & Stewart 1976): a second Gram-Schmidt
-// pass only where the first one cancelled more than half of w (||w'||^2 < ||w||^2 / 2).
-__global__ void reorth_flag_kernel(int nsys, const int *state, int want, const double *h, const double *w2, int NV,
-                                   int nv, double theta, int *flag) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsys) return;
-  const double before = h[2 * ((long long)s * NV + nv)];    // ||w||^2 from the first pass
-  const double after = w2[2 * ((long long)s * NV)];          // ||w'||^2
-  flag[s] = (state[s] == want && after < theta * before) ? 1 : 0;
-}
-
-// h[s][i] += h2[s][i] (i < nv) and h[s][nv] = ||w||^2 for the flagged systems; copy the final norm
-__global__ void reorth_merge_kernel(int nsys, int nv, double *h, const double *h2, const double *n1, const double *n2,
-                                    int NV, const int *state, int want, const int *flag) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsys || state[s] != want) return;
-  double2 *hs = reinterpret_cast<double2 *>(h) + (long long)s * NV;
-  const double2 *h2s = reinterpret_cast<const double2 *>(h2) + (long long)s * NV;
-  if (flag[s]) {
-    for (int i = 0; i < nv; i++) {
-      hs[i].x += h2s[i].x;
-      hs[i].y += h2s[i].y;
+  if (!last_block(cnt, s)) return;
+  if (threadIdx.x < 32) {
+    double tot = 0.0;
+    for (int c = threadIdx.x; c < nch; c += 32) tot += __ldcg(&ps[c]).x;
+    for (int off = 16; off > 0; off >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, off);
+    if (threadIdx.x == 0) {
+      if (SECOND) {
+        hs[nv] = make_double2(tot, 0.0);
+      } else {
+        const bool again = tot < theta * hs[nv].x;
+        flag[s] = again ? 1 : 0;
+        if (!again) hs[nv] = make_double2(tot, 0.0);
+      }
     }
-    hs[nv] = make_double2(n2[2 * (long long)s * NV], 0.0);
-  } else {
-    hs[nv] = make_double2(n1[2 * (long long)s * NV], 0.0);
   }
+  if (!SECOND) return;
+  const double2 *h2s = reinterpret_cast<const double2 *>(h2) + (long long)s * NV;
+  for (int i = threadIdx.x; i < nv; i += CGS_THREADS) {
+    hs[i].x += h2s[i].x;
+    hs[i].y += h2s[i].y;
+  }
+  __syncthreads();
+  givens_update(q, s, nv - 1, h, NV);
 }
 
 __global__ void set_state_kernel(int nsys, int *state, int from, int to) {
@@ -545,9 +635,15 @@ long long dbl_of(long long count) {
 }
 }  // namespace
 
+// chunks of partial sums per system: the norms' chunks, or enough for CGS_BLOCKS blocks from few systems
+static long long partial_chunks_per_system(long long n, int nsys) {
+  const long long fine = (n + CGS_MIN_CHUNK - 1) / CGS_MIN_CHUNK;
+  return std::max((n + DOT_CHUNK - 1) / DOT_CHUNK, std::min<long long>(fine, CGS_BLOCKS / std::max(1, nsys) + 1));
+}
+
 long long gmres_work_doubles(const gfcc_ctx *c, int sector, long long n, int nsys, int m, bool mixed) {
   const long long NV = m + 2;
-  const long long nch = (n + DOT_CHUNK - 1) / DOT_CHUNK;   // the finer of the two chunkings
+  const long long nch = partial_chunks_per_system(n, nsys);
   const bool f32 = mixed && c->inner_fp64 == 0;
   long long w = 0;
   const long long vb = 2LL * nsys * (m + 1) * n, vv = 2LL * nsys * n;
@@ -579,7 +675,8 @@ int Gmres::init(gfcc_ctx *ctx, int sec, long long dim, int ns, int mm, double *w
   m = mm;
   NV = m + 2;
   nch = (int)((n + DOT_CHUNK - 1) / DOT_CHUNK);
-  const long long nch_alloc = (n + DOT_CHUNK - 1) / DOT_CHUNK;
+  const long long nch_alloc = partial_chunks_per_system(n, nsys);
+  partial_chunks = nch_alloc * nsys;
   double *p = work;
   auto take = [&](double *&dst, long long cnt) {
     dst = p;
@@ -611,6 +708,7 @@ int Gmres::init(gfcc_ctx *ctx, int sec, long long dim, int ns, int mm, double *w
   iters = kcyc + nsys;
   rflag = iters + nsys;
   act = rflag + nsys;
+  blk_cnt = reinterpret_cast<unsigned *>(act + nsys);
   if (mixed) {
     take(X, 2LL * nsys * n);
     take(R, 2LL * nsys * n);
@@ -712,48 +810,30 @@ int Gmres::mdot(const double *Vb, long long vs, long long vi, int nv, const doub
 }
 
 template <typename T>
-int Gmres::cgs2_t(const T *Vb, long long vs, int nv, T *w, cudaStream_t st) {
-  const int nchc = (int)((n + CGS_CHUNK - 1) / CGS_CHUNK);   // partial holds nch_alloc >= nchc chunks
-  dim3 grid(nchc, nsys);
-  const int TH = 256;
-  // pass p (0: dots and norm, 2: update and norm) over the systems whose filter array equals `want`
-  auto pass = [&](int p, const double *coef, const int *filt, int want) -> int {
-    if (p == 0)
-      cgs_dots_kernel<T><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, nchc, filt, want, partial, NV);
-    else
-      cgs_update_norm_kernel<T><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, nchc, filt, want, coef, partial,
-                                                             NV);
-    GFCC_LAUNCH_CHECK();
-    return GFCC_OK;
-  };
-  auto final = [&](int nvv, double *out, const int *filt, int want) -> int {
-    mdot_final_kernel<<<cdiv(nsys * (long long)nvv * 32, 256), 256, 0, st>>>(partial, nsys, nvv, NV, nchc, filt, want,
-                                                                             out, 0);
-    GFCC_LAUNCH_CHECK();
-    return GFCC_OK;
-  };
-  int *flag = rflag;
-  // pass 1: h = V^H w and ||w||^2 (slot nv)
-  GFCC_TRY(pass(0, nullptr, state, ST_IN_CYCLE));
-  GFCC_TRY(final(nv + 1, h, state, ST_IN_CYCLE));
-  // pass 2: w -= V h, ||w'||^2
-  GFCC_TRY(pass(2, h, state, ST_IN_CYCLE));
-  GFCC_TRY(final(1, nrm, state, ST_IN_CYCLE));
-  // passes 3-4 only where the first pass cancelled most of w
-  // Second pass where ||w'||^2 < theta ||w||^2.  The orthogonality lost by the new vector is about
-  // the relative rounding error of the pass times ||w|| / ||w'||: FP64 solves reorthogonalise below
-  // 1/sqrt(2) (the usual twice-is-enough test); the FP32 inner solves of the refinement, which stop
-  // at a relative residual of 3e-4 and are corrected by the FP64-accurate outer residual, only where
-  // the first pass cancelled more than 90% of w (orthogonality loss <= 10 x about 1e-6 per vector).
+int Gmres::arnoldi_t(const T *Vb, long long vs, int k, T *w, int active, double tol, cudaStream_t st) {
+  const int nv = k + 1;
+  // chunks: enough blocks for the systems in cycle, within the partial sums' room
+  const long long cap = std::max<long long>(1, partial_chunks / nsys);
+  long long nchc = std::min<long long>(cap, std::max(1, CGS_BLOCKS / std::max(1, active)));
+  nchc = std::max(nchc, (n + CGS_MAX_CHUNK - 1) / CGS_MAX_CHUNK);
+  int clen = (int)(((n + nchc - 1) / nchc + CGS_MIN_CHUNK - 1) / CGS_MIN_CHUNK * CGS_MIN_CHUNK);
+  dim3 grid((unsigned)((n + clen - 1) / clen), (unsigned)nsys);
+  // The orthogonality lost by the new vector is about the relative rounding error of the pass times
+  // ||w|| / ||w'||: FP64 solves take the second pass below 1/sqrt(2) (the usual twice-is-enough test);
+  // the FP32 inner solves of the refinement, which stop at a relative residual of 3e-4 and are
+  // corrected by the FP64-accurate outer residual, only where the first pass cancelled more than 90% of w
+  // (orthogonality loss <= 10 x about 1e-6 per vector).
   const double theta = sizeof(T) == sizeof(float) ? REORTH_THETA_F32 : 0.5;
-  reorth_flag_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, state, ST_IN_CYCLE, h, nrm, NV, nv, theta, flag);
+  const Lsq q{m, H, cs, sn, g, bnorm, tol, state, kcyc, iters, est};
+  cgs_dots_kernel<T><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, state, nullptr, partial, NV, h, blk_cnt);
   GFCC_LAUNCH_CHECK();
-  GFCC_TRY(pass(0, nullptr, flag, 1));
-  GFCC_TRY(final(nv, h2, flag, 1));
-  GFCC_TRY(pass(2, h2, flag, 1));
-  GFCC_TRY(final(1, nrm + 2 * NV * (long long)nsys, flag, 1));
-  reorth_merge_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, nv, h, h2, nrm, nrm + 2 * NV * (long long)nsys, NV, state,
-                                                     ST_IN_CYCLE, flag);
+  cgs_update_kernel<T, false><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, rflag, h, nullptr, theta, partial,
+                                                            NV, blk_cnt, q);
+  GFCC_LAUNCH_CHECK();
+  cgs_dots_kernel<T><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, state, rflag, partial, NV, h2, blk_cnt);
+  GFCC_LAUNCH_CHECK();
+  cgs_update_kernel<T, true><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, rflag, h, h2, theta, partial, NV,
+                                                           blk_cnt, q);
   GFCC_LAUNCH_CHECK();
   vscale_kernel<T><<<vscale_grid(n, nsys), 256, 0, st>>>(w, vs, n, h, NV, nv, state, ST_IN_CYCLE);
   GFCC_LAUNCH_CHECK();
@@ -808,6 +888,7 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
   GFCC_CUDA(cudaMemsetAsync(Vt, 0, sizeof(T) * 2 * nsys * (m + 1) * n, st));
   GFCC_CUDA(cudaMemsetAsync(iters, 0, sizeof(int) * nsys, st));
   GFCC_CUDA(cudaMemsetAsync(state, 0, sizeof(int) * nsys, st));   // ST_PENDING
+  GFCC_CUDA(cudaMemsetAsync(blk_cnt, 0, sizeof(unsigned) * nsys, st));
   // ||b||
   GFCC_TRY(mdot_t<T>(Bt, n, 0, 1, Bt, n, nrm, ST_PENDING, 0));
   norm_from_partial_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, nrm, NV, bnorm);
@@ -869,19 +950,13 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
       auto step = [&]() -> int {
         GFCC_TRY(op_t<T>(vk, vs, w, vs, nact, act));
         // Gram-Schmidt against the basis: one classical pass (dots with ||w||^2, then update with
-        // ||w'||^2), a second pass only where needed, then w /= ||w||.  Algorithmic bytes of one
+        // ||w'||^2), a second pass only where needed, the Givens update, then w /= ||w||.  Algorithmic bytes of one
         // classical pass per system: dots read k+1 basis vectors and w, the update reads k+1 basis
         // vectors and reads / writes w, the scaling reads / writes w.
         {
           const double bytes = (double)active * (2.0 * (k + 1) + 5.0) * (double)n * 2.0 * sizeof(T);
           PhaseTimer ta(c, PH_ARNOLDI, bytes);
-          GFCC_TRY(cgs2_t<T>(Vt, vs, k + 1, w, st));
-        }
-        {
-          PhaseTimer tl(c, PH_LSQ);
-          givens_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, k, m, h, NV, H, cs, sn, g, bnorm, tol, state, kcyc,
-                                                       iters, est);
-          GFCC_LAUNCH_CHECK();
+          GFCC_TRY(arnoldi_t<T>(Vt, vs, k, w, active, tol, st));
         }
         return GFCC_OK;
       };
@@ -926,8 +1001,11 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
       GFCC_TRY(plan_active());
     }
     // x += V y
-    backsolve_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, m, H, g, state, kcyc, y, NV);
-    GFCC_LAUNCH_CHECK();
+    {
+      PhaseTimer tl(c, PH_LSQ);
+      backsolve_kernel<<<nsys, 64, 0, st>>>(m, H, g, state, kcyc, y, NV);
+      GFCC_LAUNCH_CHECK();
+    }
     vupdate_kernel<T><<<grid1d(n * nsys), TH, 0, st>>>(Vt, vs, n, m, kcyc, y, NV, 1.0, Ut, n, n, nsys, state,
                                                        ST_CYCLE_DONE);
     GFCC_LAUNCH_CHECK();

@@ -36,6 +36,8 @@ struct Gmres {
   double *H = nullptr, *cs = nullptr, *sn = nullptr, *g = nullptr;
   double *bnorm = nullptr, *relres = nullptr, *est = nullptr, *omega = nullptr;
   int *state = nullptr, *kcyc = nullptr, *iters = nullptr, *rflag = nullptr;
+  unsigned *blk_cnt = nullptr;      // per system: blocks of the running kernel that have finished
+  long long partial_chunks = 0;     // chunks of partial sums over all systems that `partial` holds
   int *act = nullptr;   // the systems the operator runs on in an Arnoldi step (see solve_t)
   double *relres0 = nullptr;   // relative residual of the initial iterate (first true residual)
   double *sigma_work = nullptr;
@@ -93,8 +95,9 @@ struct Gmres {
   template <typename T>
   int mdot_t(const T *Vb, long long vs, long long vi, int nv, const T *w, long long ws, double *out, int want,
              int accumulate);
+  // orthogonalise and normalise w against V_0..V_k and update the least squares (`active` systems in cycle)
   template <typename T>
-  int cgs2_t(const T *Vb, long long vs, int nv, T *w, cudaStream_t st);
+  int arnoldi_t(const T *Vb, long long vs, int k, T *w, int active, double tol, cudaStream_t st);
   template <typename T>
   int solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool use_x0);
 };
