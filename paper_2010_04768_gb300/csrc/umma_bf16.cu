@@ -147,6 +147,14 @@ __device__ __forceinline__ void umma_bf16(unsigned d_tmem, unsigned long long a,
       : "memory");
 }
 
+// One lane of a converged warp.  The MMA loops run in a whole warp and issue from the elected lane, so that
+// descriptors and barrier addresses stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  unsigned p;
+  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void umma_commit(unsigned mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
 }
@@ -237,29 +245,28 @@ __global__ void __launch_bounds__(THREADS, 1)
       tma_load_2d(smem_u32(sb), &tmB, smem_u32(&full[s]), (kb0 + kb) * BK, n0);
       *issued = kb + 1;
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
     // ---------------- MMA issuer
     const unsigned idesc = idesc_bf16(BM, BN);
-    bool ok = true;
-    for (int kb = 0; kb < nk && ok; kb++) {
+    const unsigned long long d0 = smem_desc(smem_u32(smem));
+    for (int kb = 0; kb < nk; kb++) {
       const int s = kb % STAGES;
       const unsigned ph = (kb / STAGES) & 1;
-      if (!mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns)) {
-        ok = false;
-        break;
-      }
-      *consumed = kb + 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned sa = smem_u32(smem + s * STAGE_BYTES);
-      const unsigned sb = sa + A_BYTES;
+      const unsigned long long da = d0 + s * (STAGE_BYTES >> 4), db = da + (A_BYTES >> 4);
+      if (elect_one()) {
+        *consumed = kb + 1;
 #pragma unroll
-      for (int k = 0; k < BK / 16; k++) {
-        // advance 16 BF16 (32 bytes) along K inside the 128-byte swizzle atom
-        umma_bf16(tmem, smem_desc(sa + 32 * k), smem_desc(sb + 32 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+        for (int k = 0; k < BK / 16; k++) {
+          // advance 16 BF16 (32 bytes) along K inside the 128-byte swizzle atom
+          umma_bf16(tmem, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+        }
+        umma_commit(smem_u32(&empty[s]));
       }
-      umma_commit(smem_u32(&empty[s]));
+      __syncwarp();
     }
-    umma_commit(smem_u32(done));   // arrives when every MMA issued above has completed
+    if (elect_one()) umma_commit(smem_u32(done));   // arrives when every MMA issued above has completed
   }
   __syncwarp();
 
@@ -411,39 +418,40 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- MMA issuer: accumulator lt & 1 of the CTA's lt-th tile
-      const unsigned idesc = idesc_bf16(BM, BN);
-      int it = 0, lt = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, lt++) {
-        int m0, n0, kb0, nk;
-        long long zoff;
-        tile_of(t, m0, n0, kb0, nk, zoff);
-        const int buf = lt & 1;
-        if (!mbar_wait(smem_u32(&acce[buf]), ((lt >> 1) & 1) ^ 1, abort_flag, ctl.wait_ns)) break;
+    // ---------------- MMA issuer: accumulator lt & 1 of the CTA's lt-th tile
+    const unsigned idesc = idesc_bf16(BM, BN);
+    const unsigned long long d0 = smem_desc(smem_u32(smem));
+    int it = 0, lt = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, lt++) {
+      int m0, n0, kb0, nk;
+      long long zoff;
+      tile_of(t, m0, n0, kb0, nk, zoff);
+      const int buf = lt & 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acce[buf]), ((lt >> 1) & 1) ^ 1, abort_flag, ctl.wait_ns))) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const unsigned acc = tmem + (unsigned)(buf * BN);
+      for (int kb = 0; kb < nk; kb++, it++) {
+        const int s = it % STAGES;
+        const unsigned ph = (it / STAGES) & 1;
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) {
+          ok = false;
+          break;
+        }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const unsigned acc = tmem + (unsigned)(buf * BN);
-        for (int kb = 0; kb < nk; kb++, it++) {
-          const int s = it % STAGES;
-          const unsigned ph = (it / STAGES) & 1;
-          if (!mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns)) {
-            ok = false;
-            break;
-          }
+        const unsigned long long da = d0 + s * (STAGE_BYTES >> 4), db = da + (A_BYTES >> 4);
+        if (elect_one()) {
           *consumed = it + 1;
-          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const unsigned sa = smem_u32(smem + s * STAGE_BYTES);
-          const unsigned sb = sa + A_BYTES;
 #pragma unroll
-          for (int k = 0; k < BK / 16; k++)
-            umma_bf16(acc, smem_desc(sa + 32 * k), smem_desc(sb + 32 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
+          for (int k = 0; k < BK / 16; k++) umma_bf16(acc, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
           umma_commit(smem_u32(&empty[s]));
         }
-        if (ok) umma_commit(smem_u32(&accf[buf]));
+        __syncwarp();
       }
-      umma_commit(smem_u32(drain));   // arrives once every MMA issued above has completed
+      if (ok && elect_one()) umma_commit(smem_u32(&accf[buf]));
+      __syncwarp();
     }
+    if (elect_one()) umma_commit(smem_u32(drain));   // arrives once every MMA issued above has completed
   } else {
     // ---------------- epilogue warps 2..5: rows 32 (warp mod 4) + lane of each tile
     const int q = warp & 3;
@@ -642,27 +650,26 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       tma_load_2d_pair(smem_u32(sb), &tmB, fb, (kb0 + kb) * BK, nb0);
       *issued = kb + 1;
     }
-  } else if (warp == 1 && lane == 0 && leader) {
+  } else if (warp == 1 && leader) {
     // ---------------- MMA issuer (leader only): M = 256 over the pair, N = 256
     const unsigned idesc = idesc_bf16(2 * BM, PAIR_BN);
-    bool ok = true;
-    for (int kb = 0; kb < nk && ok; kb++) {
+    const unsigned long long d0 = smem_desc(smem_u32(smem));
+    for (int kb = 0; kb < nk; kb++) {
       const int s = kb % PAIR_STAGES;
       const unsigned ph = (kb / PAIR_STAGES) & 1;
-      if (!mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns)) {
-        ok = false;
-        break;
-      }
-      *consumed = kb + 1;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned sa = smem_u32(smem + s * PAIR_STAGE_BYTES);
-      const unsigned sb = sa + PAIR_A_BYTES;
+      const unsigned long long da = d0 + s * (PAIR_STAGE_BYTES >> 4), db = da + (PAIR_A_BYTES >> 4);
+      if (elect_one()) {
+        *consumed = kb + 1;
 #pragma unroll
-      for (int k = 0; k < BK / 16; k++)
-        umma_bf16_pair(tmem, smem_desc(sa + 32 * k), smem_desc(sb + 32 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
-      umma_commit_pair(smem_u32(&empty[s]));
+        for (int k = 0; k < BK / 16; k++)
+          umma_bf16_pair(tmem, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+        umma_commit_pair(smem_u32(&empty[s]));
+      }
+      __syncwarp();
     }
-    umma_commit_pair(smem_u32(done));   // both CTAs: every MMA issued above has completed
+    if (elect_one()) umma_commit_pair(smem_u32(done));   // both CTAs: every MMA issued above has completed
   }
   __syncwarp();
 
@@ -791,12 +798,6 @@ __device__ __forceinline__ double fixed_to_f64(long long hi, long long lo, int s
   else
     v = scalbn((double)mant, 127 - lz + e2 - 52);
   return neg ? -v : v;
-}
-
-__device__ __forceinline__ bool elect_one() {
-  unsigned p;
-  asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
-  return p != 0;
 }
 
 // The MMAs of one K block at level P, called by a whole warp so that the descriptors stay in uniform
