@@ -15,6 +15,8 @@
 //   is applied here in FP64: IP y = x + sigma_off(u) (preconditioned), (z + d) x + sigma_off(x);
 //   EA y = x - sigma_off(u), (z - d) x - sigma_off(x); without omega y = d x + sigma_off(x).
 #pragma once
+#include <algorithm>
+
 #include "sigma.cuh"
 
 namespace gfcc {
@@ -27,7 +29,7 @@ template <typename TIn>
 constexpr int run_len() {
   return sizeof(TIn) == 4 ? 16 : 8;   // packed elements per block
 }
-// systems per launch: the shared tile run_len x (2 ns + 1) stays below 33 KB
+// systems per launch: the shared tile run_len x (ns + 1) pairs stays below 33 KB
 template <typename TIn>
 constexpr int max_systems() {
   return 256;
@@ -56,9 +58,22 @@ __device__ __forceinline__ void store_y(const SysBatch &b, int s, long long mu, 
 }
 
 // sgn = +1 IP, -1 EA; diag = the operator's Fock-like diagonal (MODE_OFFDIAG)
-template <int MODE>
-__device__ __forceinline__ void combine(const SysBatch &b, int s, long long mu, double sr, double si,
-                                        const double *diag, double sgn) {
+template <int MODE, typename TIn>
+__device__ __forceinline__ void combine(const SysBatch &b, int s, long long mu, TIn tr, TIn ti, const double *diag,
+                                        double sgn) {
+  if constexpr (MODE == MODE_OFFDIAG && sizeof(TIn) == 4) {
+    // the preconditioned inner operator on FP32 vectors, y = x +/- sigma_off: one FP32 addition (eight
+    // conversions and additions on the FP64 pipe instead held the epilogue to a third of the memory rate)
+    if (b.xf != nullptr && b.diag != nullptr && b.omega != nullptr) {
+      if (!sys_stores(b, s)) return;
+      const long long v = sysv(b, s);
+      const float2 x = reinterpret_cast<const float2 *>(b.xf)[v * b.ldx + mu];
+      const float f = (float)sgn;
+      reinterpret_cast<float2 *>(b.yf)[v * b.ldy + mu] = make_float2(fmaf(f, tr, x.x), fmaf(f, ti, x.y));
+      return;
+    }
+  }
+  const double sr = tr, si = ti;
   double xr, xi;
   load_x(b, s, mu, xr, xi);
   double yr, yi;
@@ -95,52 +110,87 @@ __device__ __forceinline__ void combine(const SysBatch &b, int s, long long mu, 
   store_y(b, s, mu, yr, yi);
 }
 
-// IP 2h1p block: one block per (pair p = (i<j), run of a); grid (Po, cdiv(v, run)), dynamic shared
-// memory run * (C2 + 1) * sizeof(TIn)
+template <typename TIn>
+struct Pair;
+template <>
+struct Pair<float> {
+  using type = float2;
+};
+template <>
+struct Pair<double> {
+  using type = double2;
+};
+
+// the one-index block (IP 1h: n1 = o, sgn +1; EA 1p: n1 = v, sgn -1): S1[m][c], by the blocks past the first
+// `first` of the grid's x dimension
 template <typename TIn, int MODE>
-__global__ __launch_bounds__(THREADS) void ip2_kernel(SysBatch b, int o, int v, long long C2, int s0, int ns,
-                                                       const TIn *T, const TIn *Q, const TIn *U, const double *diag) {
+__device__ __forceinline__ void one_index(const SysBatch &b, int n1, long long C2, const TIn *S1, const double *diag,
+                                          double sgn, int s0, int ns, int first) {
+  if (blockIdx.y != 0) return;
+  const int tot = n1 * ns;
+  for (int t = (blockIdx.x - first) * THREADS + threadIdx.x; t < tot; t += (gridDim.x - first) * THREADS) {
+    const int s = t / n1, m = t - s * n1;
+    const typename Pair<TIn>::type v = reinterpret_cast<const typename Pair<TIn>::type *>(S1 + m * C2)[s0 + s];
+    combine<MODE, TIn>(b, s0 + s, m, v.x, v.y, diag, sgn);
+  }
+}
+
+// IP 2h1p block: one block per (pair p = (i<j), run of a); grid (Po + blocks of the 1h part, cdiv(v, run)),
+// dynamic shared memory run * (ns + 1) * 2 sizeof(TIn).  A thread handles both planes of a system.
+template <typename TIn, int MODE>
+__global__ __launch_bounds__(THREADS) void ip2_kernel(SysBatch b, int o, int v, long long C2, int s0, int ns, int Po,
+                                                       const TIn *T, const TIn *Q, const TIn *U, const TIn *S1,
+                                                       const double *diag) {
+  using P2 = typename Pair<TIn>::type;
   extern __shared__ __align__(16) unsigned char smem[];
-  TIn *tile = reinterpret_cast<TIn *>(smem);
+  P2 *tile = reinterpret_cast<P2 *>(smem);
   constexpr int A = run_len<TIn>();
+  if ((int)blockIdx.x >= Po) {
+    one_index<TIn, MODE>(b, o, C2, S1, diag, 1.0, s0, ns, Po);
+    return;
+  }
   const long long p = blockIdx.x;
   const int a0 = blockIdx.y * A;
   long long i, j;
   pair_decode(p, o, i, j);
-  const long long Cl = 2LL * ns, ld = Cl + 1, c0 = 2LL * s0;
-  const int cl = (int)Cl;   // at most 2 max_systems()
-  for (int t = threadIdx.x; t < A * cl; t += THREADS) {
-    const int al = t / cl;
-    const long long c = t - al * cl;
-    const long long a = a0 + al;
-    if (a >= v) continue;
-    const long long tij = ((i * v + a) * o + j) * C2 + c0 + c;
-    const long long tji = ((j * v + a) * o + i) * C2 + c0 + c;
-    const long long qij = ((i * o + j) * v + a) * C2 + c0 + c;
-    tile[al * ld + c] = T[tij] - T[tji] + Q[qij] + U[tij];
+  const int ld = ns + 1, na = min(A, v - a0);
+  for (int t = threadIdx.x; t < na * ns; t += THREADS) {
+    const int al = t / ns, s = t - al * ns;
+    const long long a = a0 + al, c = s0 + s;
+    const P2 tij = reinterpret_cast<const P2 *>(T + ((i * v + a) * o + j) * C2)[c];
+    const P2 tji = reinterpret_cast<const P2 *>(T + ((j * v + a) * o + i) * C2)[c];
+    const P2 q = reinterpret_cast<const P2 *>(Q + ((i * o + j) * v + a) * C2)[c];
+    const P2 u = reinterpret_cast<const P2 *>(U + ((i * v + a) * o + j) * C2)[c];
+    P2 r;
+    r.x = tij.x - tji.x + q.x + u.x;
+    r.y = tij.y - tji.y + q.y + u.y;
+    tile[al * ld + s] = r;
   }
   __syncthreads();
   for (int t = threadIdx.x; t < A * ns; t += THREADS) {
     const int s = t / A, al = t - s * A;
-    const long long a = a0 + al;
-    if (a >= v) continue;
-    const long long mu = o + p * v + a;
-    combine<MODE>(b, s0 + s, mu, (double)tile[al * ld + 2 * s], (double)tile[al * ld + 2 * s + 1], diag, 1.0);
+    if (al >= na) continue;
+    const P2 r = tile[al * ld + s];
+    combine<MODE, TIn>(b, s0 + s, o + p * v + a0 + al, r.x, r.y, diag, 1.0);
   }
 }
 
-// EA 2p1h block: one block per (i, run of pairs a<b); grid (o, cdiv(Pv, run))
+// EA 2p1h block: one block per (i, run of pairs a<b); grid (o + blocks of the 1p part, cdiv(Pv, run))
 template <typename TIn, int MODE>
 __global__ __launch_bounds__(THREADS) void ea2_kernel(SysBatch b, int o, int v, long long Pv, long long C2, int s0,
-                                                       int ns, const TIn *T, const TIn *Qp, const TIn *U,
+                                                       int ns, const TIn *T, const TIn *Qp, const TIn *U, const TIn *S1,
                                                        const double *diag) {
+  using P2 = typename Pair<TIn>::type;
   extern __shared__ __align__(16) unsigned char smem[];
-  TIn *tile = reinterpret_cast<TIn *>(smem);
+  P2 *tile = reinterpret_cast<P2 *>(smem);
   constexpr int A = run_len<TIn>();
   __shared__ int pa[A], pb[A];   // the block's pairs (a < b), decoded once
+  if ((int)blockIdx.x >= o) {
+    one_index<TIn, MODE>(b, v, C2, S1, diag, -1.0, s0, ns, o);
+    return;
+  }
   const long long i = blockIdx.x;
   const long long ab0 = (long long)blockIdx.y * A;
-  const long long Cl = 2LL * ns, ld = Cl + 1, c0 = 2LL * s0;
   if (threadIdx.x < A && ab0 + threadIdx.x < Pv) {
     long long a, bb;
     pair_decode(ab0 + threadIdx.x, v, a, bb);
@@ -148,50 +198,41 @@ __global__ __launch_bounds__(THREADS) void ea2_kernel(SysBatch b, int o, int v, 
     pb[threadIdx.x] = (int)bb;
   }
   __syncthreads();
-  const int cl = (int)Cl;   // at most 2 max_systems()
-  for (int t = threadIdx.x; t < A * cl; t += THREADS) {
-    const int al = t / cl;
-    const long long c = t - al * cl;
-    const long long ab = ab0 + al;
-    if (ab >= Pv) continue;
-    const long long a = pa[al], bb = pb[al];
-    const long long tiba = ((i * v + bb) * v + a) * C2 + c0 + c;
-    const long long tiab = ((i * v + a) * v + bb) * C2 + c0 + c;
-    const long long qq = (ab * o + i) * C2 + c0 + c;
-    tile[al * ld + c] = T[tiba] - T[tiab] + Qp[qq] + U[tiba];
+  const int ld = ns + 1, na = (int)min((long long)A, Pv - ab0);
+  for (int t = threadIdx.x; t < na * ns; t += THREADS) {
+    const int al = t / ns, s = t - al * ns;
+    const long long ab = ab0 + al, a = pa[al], bb = pb[al], c = s0 + s;
+    const P2 tiba = reinterpret_cast<const P2 *>(T + ((i * v + bb) * v + a) * C2)[c];
+    const P2 tiab = reinterpret_cast<const P2 *>(T + ((i * v + a) * v + bb) * C2)[c];
+    const P2 q = reinterpret_cast<const P2 *>(Qp + (ab * o + i) * C2)[c];
+    const P2 u = reinterpret_cast<const P2 *>(U + ((i * v + bb) * v + a) * C2)[c];
+    P2 r;
+    r.x = tiba.x - tiab.x + q.x + u.x;
+    r.y = tiba.y - tiab.y + q.y + u.y;
+    tile[al * ld + s] = r;
   }
   __syncthreads();
   for (int t = threadIdx.x; t < A * ns; t += THREADS) {
     const int s = t / A, al = t - s * A;
-    const long long ab = ab0 + al;
-    if (ab >= Pv) continue;
-    const long long mu = v + i * Pv + ab;
-    combine<MODE>(b, s0 + s, mu, (double)tile[al * ld + 2 * s], (double)tile[al * ld + 2 * s + 1], diag, -1.0);
+    if (al >= na) continue;
+    const P2 r = tile[al * ld + s];
+    combine<MODE, TIn>(b, s0 + s, v + i * Pv + ab0 + al, r.x, r.y, diag, -1.0);
   }
 }
 
-// the one-index block (IP 1h: n1 = o, sgn +1; EA 1p: n1 = v, sgn -1): S1[m][c]
-template <typename TIn, int MODE>
-__global__ void one_kernel(SysBatch b, int n1, long long C2, const TIn *S1, const double *diag, double sgn) {
-  const long long tot = (long long)n1 * b.nsys;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const int s = (int)(t / n1);
-    const long long m = t - (long long)s * n1;
-    combine<MODE>(b, s, m, (double)S1[m * C2 + 2 * s], (double)S1[m * C2 + 2 * s + 1], diag, sgn);
-  }
-}
+// blocks for the one-index block of n1 entries of ns systems
+static inline int one_index_blocks(int n1, int ns) { return (int)cdiv((long long)n1 * ns, THREADS); }
 
 template <typename TIn, int MODE>
 int launch_ip(cudaStream_t st, const SysBatch &b, int o, int v, const TIn *S1, const TIn *T, const TIn *Q,
               const TIn *U, const double *diag) {
-  const long long C2 = 2LL * b.nsys, Po = (long long)o * (o - 1) / 2;
+  const long long C2 = 2LL * b.nsys, Po = v > 0 ? (long long)o * (o - 1) / 2 : 0;
   constexpr int A = run_len<TIn>();
-  one_kernel<TIn, MODE><<<grid1d((long long)o * b.nsys), THREADS, 0, st>>>(b, o, C2, S1, diag, 1.0);
-  GFCC_LAUNCH_CHECK();
-  for (int s0 = 0; Po > 0 && v > 0 && s0 < b.nsys; s0 += max_systems<TIn>()) {
+  for (int s0 = 0; s0 < b.nsys; s0 += max_systems<TIn>()) {
     const int ns = b.nsys - s0 < max_systems<TIn>() ? b.nsys - s0 : max_systems<TIn>();
-    const size_t sm = (size_t)A * (2 * ns + 1) * sizeof(TIn);
-    ip2_kernel<TIn, MODE><<<dim3((unsigned)Po, cdiv(v, A)), THREADS, sm, st>>>(b, o, v, C2, s0, ns, T, Q, U, diag);
+    const size_t sm = (size_t)A * (ns + 1) * 2 * sizeof(TIn);
+    ip2_kernel<TIn, MODE><<<dim3((unsigned)Po + one_index_blocks(o, ns), std::max(1u, cdiv(v, A))), THREADS, sm, st>>>(
+        b, o, v, C2, s0, ns, (int)Po, T, Q, U, S1, diag);
     GFCC_LAUNCH_CHECK();
   }
   return GFCC_OK;
@@ -202,13 +243,11 @@ int launch_ea(cudaStream_t st, const SysBatch &b, int o, int v, long long Pv, co
               const TIn *Qp, const TIn *U, const double *diag) {
   const long long C2 = 2LL * b.nsys;
   constexpr int A = run_len<TIn>();
-  one_kernel<TIn, MODE><<<grid1d((long long)v * b.nsys), THREADS, 0, st>>>(b, v, C2, S1, diag, -1.0);
-  GFCC_LAUNCH_CHECK();
-  for (int s0 = 0; Pv > 0 && o > 0 && s0 < b.nsys; s0 += max_systems<TIn>()) {
+  for (int s0 = 0; s0 < b.nsys; s0 += max_systems<TIn>()) {
     const int ns = b.nsys - s0 < max_systems<TIn>() ? b.nsys - s0 : max_systems<TIn>();
-    const size_t sm = (size_t)A * (2 * ns + 1) * sizeof(TIn);
-    ea2_kernel<TIn, MODE><<<dim3((unsigned)o, cdiv(Pv, A)), THREADS, sm, st>>>(b, o, v, Pv, C2, s0, ns, T, Qp, U,
-                                                                                diag);
+    const size_t sm = (size_t)A * (ns + 1) * 2 * sizeof(TIn);
+    ea2_kernel<TIn, MODE><<<dim3((unsigned)o + one_index_blocks(v, ns), std::max(1u, cdiv(Pv, A))), THREADS, sm, st>>>(
+        b, o, v, Pv, C2, s0, ns, T, Qp, U, S1, diag);
     GFCC_LAUNCH_CHECK();
   }
   return GFCC_OK;

@@ -176,33 +176,39 @@ __global__ void vupdate_kernel(const T *V, long long vs_stride, long long vi_str
 }
 
 // w_s *= 1 / scale[s] (real scale stored as the real part of a complex entry scale[s*NV + idx]).
-// Grid (cdiv(2n, VSCALE_PER_BLOCK), nsys): the factor is formed once per thread; each thread scales
-// VSCALE_UNROLL reals with independent loads.
-constexpr int VSCALE_UNROLL = 4, VSCALE_PER_BLOCK = 256 * VSCALE_UNROLL;
+// Grid (cdiv(n, VSCALE_PER_BLOCK), nsys): the factor is formed once per block (a root and a division in
+// FP64 per thread held this kernel to a quarter of the memory rate: 54 us for 100 MB); each thread scales
+// VSCALE_UNROLL elements with independent loads.
+constexpr int VSCALE_UNROLL = 8, VSCALE_PER_BLOCK = 256 * VSCALE_UNROLL;
 template <typename T>
-__global__ void vscale_kernel(T *w, long long ws_stride, long long n, const double *nrm2, int NV, int idx,
-                              const int *state, int want) {
+__global__ __launch_bounds__(256) void vscale_kernel(T *w, long long ws_stride, long long n, const double *nrm2, int NV,
+                                                     int idx, const int *state, int want) {
+  __shared__ T factor;
   const int s = blockIdx.y;
   if (state != nullptr && state[s] != want) return;
   const double nn = nrm2[2 * ((long long)s * NV + idx)];
   if (!(nn > 0.0)) return;
-  const T inv = (T)(1.0 / sqrt(nn));
   T *ws = w + 2 * s * ws_stride;
-  const long long n2 = 2 * n, t0 = (long long)blockIdx.x * VSCALE_PER_BLOCK + threadIdx.x;
-  T x[VSCALE_UNROLL];
+  const long long t0 = (long long)blockIdx.x * VSCALE_PER_BLOCK + threadIdx.x;
+  CT<T> x[VSCALE_UNROLL];
 #pragma unroll
   for (int u = 0; u < VSCALE_UNROLL; u++) {
-    const long long t = t0 + (long long)u * blockDim.x;
-    x[u] = t < n2 ? ws[t] : (T)0;
+    const long long t = t0 + (long long)u * 256;
+    x[u] = t < n ? ldc(ws, t) : mkc<T>(0.0, 0.0);
   }
+  if (threadIdx.x == 0) factor = (T)(1.0 / sqrt(nn));
+  __syncthreads();
+  const T inv = factor;
 #pragma unroll
   for (int u = 0; u < VSCALE_UNROLL; u++) {
-    const long long t = t0 + (long long)u * blockDim.x;
-    if (t < n2) ws[t] = x[u] * inv;
+    const long long t = t0 + (long long)u * 256;
+    x[u].x *= inv;
+    x[u].y *= inv;
+    if (t < n) stc(ws, t, x[u]);
   }
 }
 static inline dim3 vscale_grid(long long n, int nsys) {
-  return dim3((unsigned)std::max<long long>(1, (2 * n + VSCALE_PER_BLOCK - 1) / VSCALE_PER_BLOCK), (unsigned)nsys);
+  return dim3((unsigned)std::max<long long>(1, (n + VSCALE_PER_BLOCK - 1) / VSCALE_PER_BLOCK), (unsigned)nsys);
 }
 
 // r_s = b_s - w_s for systems that are not finished
@@ -315,38 +321,52 @@ __device__ void givens_update(const Lsq &q, int s, int k, const double *h, int N
   }
 }
 
-// y = R^-1 g (back substitution on the rotated Hessenberg), stored in y[s*NV + i]; one block of 64 threads
-// per system (thread i holds the remainder of row i; m <= 64), column by column
-__global__ __launch_bounds__(64) void backsolve_kernel(int m, const double *H, const double *g, const int *state,
+// y = R^-1 g (back substitution on the rotated Hessenberg), stored in y[s*NV + i]; one warp per system: lane l
+// owns y_l and y_{l+32} (m <= 64), a row's products are added pairwise over the warp while the next row is on
+// its way (one thread walking the rows through global memory took 0.7 ms at k = 60)
+__global__ __launch_bounds__(32) void backsolve_kernel(int m, const double *H, const double *g, const int *state,
                                                        const int *kcyc, double *y, int NV) {
-  __shared__ double2 xj;
-  const int s = blockIdx.x, i = threadIdx.x;
+  const int s = blockIdx.x, lane = threadIdx.x;
   if (state[s] != ST_CYCLE_DONE) return;
-  const double2 *Hs = reinterpret_cast<const double2 *>(H) + (long long)s * (m + 1) * m;
+  const double2 *Hs = reinterpret_cast<const double2 *>(H) + (long long)s * (m + 1) * m;   // [column][row], ld m + 1
   const double2 *gs = reinterpret_cast<const double2 *>(g) + (long long)s * (m + 1);
   double2 *ys = reinterpret_cast<double2 *>(y) + (long long)s * NV;
   const int k = kcyc[s];
-  double2 acc = i < k ? gs[i] : make_double2(0.0, 0.0);
-  double2 r = k > 0 && i < k ? Hs[(long long)(k - 1) * (m + 1) + i] : make_double2(0.0, 0.0);
-  for (int j = k - 1; j >= 0; j--) {
-    // r = R[i][j] (rows i <= j); the next column is loaded while this one is used
-    const double2 nx = j > 0 && i < j ? Hs[(long long)(j - 1) * (m + 1) + i] : make_double2(0.0, 0.0);
-    if (i == j) {
-      const double dd = r.x * r.x + r.y * r.y;
-      xj = dd > 0.0 ? make_double2((acc.x * r.x + acc.y * r.y) / dd, (acc.y * r.x - acc.x * r.y) / dd)
-                    : make_double2(0.0, 0.0);
+  const double2 zero = make_double2(0.0, 0.0);
+  // entries (row i, columns l and l + 32) right of or on the diagonal
+  auto entry = [&](int i, int j) { return i >= 0 && j >= i && j < k ? Hs[(long long)j * (m + 1) + i] : zero; };
+  double2 y0 = zero, y1 = zero;
+  double2 r0 = entry(k - 1, lane), r1 = entry(k - 1, lane + 32);
+  for (int i = k - 1; i >= 0; i--) {
+    const double2 n0 = entry(i - 1, lane), n1 = entry(i - 1, lane + 32);
+    const double2 gi = gs[i];
+    double2 p = zero;
+    if (lane > i) {
+      p.x += r0.x * y0.x - r0.y * y0.y;
+      p.y += r0.x * y0.y + r0.y * y0.x;
     }
-    __syncthreads();
-    const double2 x = xj;
-    if (i < j) {
-      acc.x -= r.x * x.x - r.y * x.y;
-      acc.y -= r.x * x.y + r.y * x.x;
+    if (lane + 32 > i) {
+      p.x += r1.x * y1.x - r1.y * y1.y;
+      p.y += r1.x * y1.y + r1.y * y1.x;
     }
-    if (i == j) ys[i] = x;
-    r = nx;
-    __syncthreads();
+    for (int off = 16; off > 0; off >>= 1) {
+      p.x += __shfl_xor_sync(0xffffffffu, p.x, off);
+      p.y += __shfl_xor_sync(0xffffffffu, p.y, off);
+    }
+    if (lane == (i & 31)) {
+      const double2 d = i < 32 ? r0 : r1;
+      const double ax = gi.x - p.x, ay = gi.y - p.y, dd = d.x * d.x + d.y * d.y;
+      const double2 v = dd > 0.0 ? make_double2((ax * d.x + ay * d.y) / dd, (ay * d.x - ax * d.y) / dd) : zero;
+      if (i < 32)
+        y0 = v;
+      else
+        y1 = v;
+      ys[i] = v;
+    }
+    r0 = n0;
+    r1 = n1;
   }
-  for (int t = k + i; t < NV; t += 64) ys[t] = make_double2(0.0, 0.0);
+  for (int t = k + lane; t < NV; t += 32) ys[t] = zero;
 }
 
 // ---------------------------------------------------------------- fused Gram-Schmidt passes
@@ -597,7 +617,12 @@ __global__ void unprecondition_kernel(T *U, long long n, int nsys, const double 
     const double d2 = dr * dr + di * di;
     const CT<T> u = ldc(U, t);
     const double ux = u.x, uy = u.y;
-    stc(U, t, mkc<T>((ux * dr + uy * di) / d2, (uy * dr - ux * di) / d2));
+    if (sizeof(T) == sizeof(float)) {   // one FP64 division: the quotients are rounded to FP32 anyway
+      const double inv = 1.0 / d2;
+      stc(U, t, mkc<T>((ux * dr + uy * di) * inv, (uy * dr - ux * di) * inv));
+    } else {
+      stc(U, t, mkc<T>((ux * dr + uy * di) / d2, (uy * dr - ux * di) / d2));
+    }
   }
 }
 
@@ -1003,7 +1028,7 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
     // x += V y
     {
       PhaseTimer tl(c, PH_LSQ);
-      backsolve_kernel<<<nsys, 64, 0, st>>>(m, H, g, state, kcyc, y, NV);
+      backsolve_kernel<<<nsys, 32, 0, st>>>(m, H, g, state, kcyc, y, NV);
       GFCC_LAUNCH_CHECK();
     }
     vupdate_kernel<T><<<grid1d(n * nsys), TH, 0, st>>>(Vt, vs, n, m, kcyc, y, NV, 1.0, Ut, n, n, nsys, state,

@@ -605,7 +605,6 @@ int build_hbar(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     c->ld_ov = round8(ov);
     c->ld_o2 = round8(oo);
     c->ld_o = round8(o);
-    c->ld_o2v = round8(o2v);
     c->ld_v = round8(v);
     c->ld_k1 = round8(o2v + o);
     double *t;
@@ -641,8 +640,8 @@ int build_hbar(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     GFCC_TRY(alloc_bf16(c, &c->WT_bf, o2v * c->ld_ot));
     concat_bf16_kernel<<<grid1d(o2v * c->ld_ot), 256, 0, st>>>(c->W1, o, c->T3, v, o2v, c->WT_bf, c->ld_ot);
     GFCC_LAUNCH_CHECK();
-    GFCC_TRY(alloc_bf16(c, &c->V3_bf, v * c->ld_o2v));
-    GFCC_TRY(to_bf16(st, c->V3, v, o2v, o2v, 1.0, c->V3_bf, c->ld_o2v));
+    GFCC_TRY(alloc_bf16(c, &c->VU_bf, (v + o) * c->ld_k1));
+    GFCC_TRY(to_bf16(st, c->V3, v, o2v, o2v, 1.0, c->VU_bf, c->ld_k1));
     // U1x[i] = [U1[i][(m,e,n)] | -Foo_offdiag[m][i]]
     {
       const long long d[4] = {1, 1, o, o2v};
@@ -652,8 +651,7 @@ int build_hbar(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     }
     u1_foo_kernel<<<cdiv(oo, 128), 128, 0, st>>>(t, o, o2v, o2v + o, c->Foo);
     GFCC_LAUNCH_CHECK();
-    GFCC_TRY(alloc_bf16(c, &c->U1_bf, o * c->ld_k1));
-    GFCC_TRY(to_bf16(st, t, o, o2v + o, o2v + o, 1.0, c->U1_bf, c->ld_k1));
+    GFCC_TRY(to_bf16(st, t, o, o2v + o, o2v + o, 1.0, c->VU_bf + v * c->ld_k1, c->ld_k1));
 
     // the other digit-plane operands (oooo, [ovoo | three-body], three-body Z, 1h row)
     {
@@ -701,7 +699,6 @@ int build_hbar(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     c->ld_o = round8(o);
     c->ld_v = round8(v);
     c->ld_pv = round8(std::max<long long>(Pv, 1));
-    c->ld_ov2 = round8(ov2);
     c->ld_k1e = round8(ov2 + v);
     const int S = c->emu_S;
     auto slice = [&](const double *A, long long rows, long long K, long long lda, EmuOperand &e) -> int {
@@ -737,8 +734,8 @@ int build_hbar(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
       GFCC_LAUNCH_CHECK();
       GFCC_TRY(slice(wt, ov2, v + o, v + o, c->eWTe));
     }
-    GFCC_TRY(alloc_bf16(c, &c->V3e_bf, o * c->ld_ov2));
-    GFCC_TRY(to_bf16(st, c->V3e, o, ov2, ov2, 1.0, c->V3e_bf, c->ld_ov2));
+    GFCC_TRY(alloc_bf16(c, &c->VUe_bf, (o + v) * c->ld_k1e));
+    GFCC_TRY(to_bf16(st, c->V3e, o, ov2, ov2, 1.0, c->VUe_bf, c->ld_k1e));
     // [V3e | 0]: padded to the K of the 1p row
     {
       const long long d[4] = {1, 1, o, ov2};
@@ -764,8 +761,7 @@ int build_hbar(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     GFCC_LAUNCH_CHECK();
     GFCC_TRY(slice(t, v, ov2 + v, ov2 + v, c->eU1e));
     GFCC_TRY(set_level_drops(c, 1.0, -0.5, {&c->eWre, &c->eWp, &c->eWTe, &c->eV3e, &c->eU1e}));
-    GFCC_TRY(alloc_bf16(c, &c->U1e_bf, v * c->ld_k1e));
-    GFCC_TRY(to_bf16(st, t, v, ov2 + v, ov2 + v, 1.0, c->U1e_bf, c->ld_k1e));
+    GFCC_TRY(to_bf16(st, t, v, ov2 + v, ov2 + v, 1.0, c->VUe_bf + o * c->ld_k1e, c->ld_k1e));
   }
   GFCC_CUDA(cudaStreamSynchronize(st));
   return GFCC_OK;

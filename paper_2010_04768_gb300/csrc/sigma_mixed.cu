@@ -13,10 +13,10 @@
 // Contractions (all D[m][n] = A[m][k] B[n][k], BF16 K-major, FP32 out):
 //   ring  T[(i,a)][(j,c)]  = Wr[(i,a)][(m,e)]   r2b[(j,c)][(m,e)],  r2b = r2[m,j,e]
 //   oooo  Q[(i,j)][(a,c)]  = Wq[(i,j)][(m,n)]   r2o[(a,c)][(m,n)],  r2o = r2[m,n,a]
-//   3-body Z[e][c]         = V3[e][(m,f,n)]     rk[c][(m,f,n)]       (split K)
+//   3-body, 1h
+//         [Z[e]; S1[i]][c] = [V3 | 0; U1x][(m,e,n)|m]  rk[c][(m,e,n)|m]     (split K)
 //   ovoo + 3-body
 //         U[(i,a,j)][c]    = [W1 | T3][(i,a,j)][m | e]  rz[c][m | e],  rz = [r1 | Z]
-//   1h    S1[i][c]         = U1x[i][(m,e,n)|m]  rk[c][(m,e,n)|m]     (split K)
 #include <cuda_bf16.h>
 
 #include "ctx.cuh"
@@ -64,6 +64,17 @@ __device__ __forceinline__ Cz r2_at(const SysBatch &b, int o, int v, int s, int 
     u.i = -u.i;
   }
   return u;
+}
+
+// element m of the one-index block of system s into row c = 2 s + re/im of rk (after o2v columns) and r1
+__device__ __forceinline__ void put_r1(const SysBatch &b, int s, int m, long long off, long long ldk,
+                                       __nv_bfloat16 *rk, long long ld1, __nv_bfloat16 *r1) {
+  const Cz u = load_u(b, s, m);
+  const __nv_bfloat16 hr = __float2bfloat16(u.r), hi = __float2bfloat16(u.i);
+  rk[(long long)(2 * s) * ldk + off + m] = hr;
+  rk[(long long)(2 * s + 1) * ldk + off + m] = hi;
+  r1[(long long)(2 * s) * ld1 + m] = hr;
+  r1[(long long)(2 * s + 1) * ld1 + m] = hi;
 }
 
 // r2b[(j, c)][(m, e)] = r2[m, j, e]
@@ -147,7 +158,8 @@ __device__ __forceinline__ int quo(unsigned q, unsigned long long rcp) {
 
 __global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v, unsigned long long rcp_o,
                                                         long long ld_ov, long long ld_o2, long long ld_k1,
-                                                        __nv_bfloat16 *r2b, __nv_bfloat16 *r2o, __nv_bfloat16 *rk) {
+                                                        __nv_bfloat16 *r2b, __nv_bfloat16 *r2o, __nv_bfloat16 *rk,
+                                                        long long ld_ot, __nv_bfloat16 *rz) {
   extern __shared__ float2 tl[];   // [o][UNPACK_ET + 1]
   constexpr int LD = UNPACK_ET + 1;
   const int e0 = blockIdx.x * UNPACK_ET, m = blockIdx.y, s = blockIdx.z;
@@ -162,6 +174,7 @@ __global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v
     }
     tl[j * LD + el] = val;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) put_r1(b, s, m, (long long)o * o * v, ld_k1, rk, ld_ot, rz);
   __syncthreads();
   // ring: rows (j, 2 s + p), columns m v + e0 .. m v + e0 + et
   for (int t = threadIdx.x; t < 2 * o * UNPACK_ET; t += blockDim.x) {
@@ -187,33 +200,37 @@ __global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v
   }
 }
 
-// rk[c][o2v + m] = r1[m] and r1b[c][m] = r1[m]
+// rk[c][o2v + m] = r1[m] and r1b[c][m] = r1[m] (the general unpacking; unpack_ip_kernel writes them itself)
 __global__ void unpack_r1_kernel(SysBatch b, int o, int v, long long ldk, __nv_bfloat16 *rk, long long ld1,
                                  __nv_bfloat16 *r1b) {
-  const long long o2v = (long long)o * o * v;
-  const int C2 = 2 * b.nsys;
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= C2 * o) return;
-  const int c = t / o, m = t % o;
-  const Cz u = load_u(b, c >> 1, m);
-  const __nv_bfloat16 h = __float2bfloat16((c & 1) ? u.i : u.r);
-  rk[(long long)c * ldk + o2v + m] = h;
-  r1b[(long long)c * ld1 + m] = h;
+  if (t < b.nsys * o) put_r1(b, t / o, t % o, (long long)o * o * v, ldk, rk, ld1, r1b);
 }
 
-// out[r][c] = sum_z part[z][r][c] (in place into part[0]); optional BF16 transposed copy outT[c][r]
-__global__ void reduce_splits_kernel(float *part, int nsplit, long long rows, long long cols, long long zstride,
-                                     __nv_bfloat16 *outT, long long ldT) {
-  const long long tot = rows * cols;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    float s = part[t];
-    for (int z = 1; z < nsplit; z++) s += part[z * zstride + t];
-    part[t] = s;
-    if (outT != nullptr) {
-      const long long r = t / cols, c = t % cols;
-      outT[c * ldT + r] = __float2bfloat16(s);
-    }
+// Partial sums part[z][r][c] over the K splits: rows r < nz_rows (the three-body Z) go to zT[c][r] in BF16,
+// rows r >= nz_rows (the one-index block) to S1[r - nz_rows][c].  A block adds 32 outputs, eight threads to
+// each: with one thread for an output, which walks all splits, it took 14.7 us whatever the size.
+__global__ __launch_bounds__(256) void reduce_splits_kernel(const float *part, int nsplit, int rows, int cols,
+                                                            int nz_rows, __nv_bfloat16 *zT, long long ldT, float *S1) {
+  __shared__ float sh[8][33];
+  const long long tot = (long long)rows * cols;
+  const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const long long t = (long long)blockIdx.x * 32 + x;
+  float s = 0.f;
+  if (t < tot) {
+#pragma unroll 4
+    for (int z = y; z < nsplit; z += 8) s += part[z * tot + t];
   }
+  sh[y][x] = s;
+  __syncthreads();
+  if (y != 0 || t >= tot) return;
+#pragma unroll
+  for (int k = 1; k < 8; k++) s += sh[k][x];
+  const int r = (int)(t / cols), c = (int)(t - (long long)r * cols);
+  if (r < nz_rows)
+    zT[c * ldT + r] = __float2bfloat16(s);
+  else
+    S1[(long long)(r - nz_rows) * cols + c] = s;
 }
 
 // ---------------------------------------------------------------------------------------- EA
@@ -238,11 +255,14 @@ __device__ __forceinline__ Cz y2_at(const SysBatch &b, int v, long long Pv, int 
 //   long K rk[c][(m, a, e)]     = -Y[a][e]  (= y2[m, e, a])
 // both along e.  grid (cdiv(v, 32), cdiv(v, 32), o * nsys), block (32, 8).
 __global__ void unpack_ea_tile_kernel(SysBatch b, int o, int v, long long Pv, long long ld_ov, long long ldk,
-                                      __nv_bfloat16 *r2e, __nv_bfloat16 *rk) {
+                                      __nv_bfloat16 *r2e, __nv_bfloat16 *rk, long long ld_ot, __nv_bfloat16 *rz) {
   __shared__ float2 tile[32][33];
   const int e0 = blockIdx.x * 32, a0 = blockIdx.y * 32;
   const int m = (int)(blockIdx.z % (unsigned)o), s = (int)(blockIdx.z / (unsigned)o);
   const int C2 = 2 * b.nsys;
+  // the 1p block, by the blocks of one (a tile, m)
+  if (a0 == 0 && m == 0 && threadIdx.y == 0 && e0 + (int)threadIdx.x < v)
+    put_r1(b, s, e0 + threadIdx.x, (long long)o * v * v, ldk, rk, ld_ot, rz);
   const bool below = e0 + 31 < a0;   // every a > e: packed pairs (e, a) run along a
   for (int r = threadIdx.y; r < 32; r += 8) {
     const int a = below ? a0 + threadIdx.x : a0 + r, e = below ? e0 + r : e0 + threadIdx.x;
@@ -284,25 +304,11 @@ __global__ void unpack_ea_pairs_kernel(SysBatch b, int o, int v, long long Pv, l
   out[(row + 1) * ld + ef] = __float2bfloat16(u.i);
 }
 
-// rk[c][o v v + e] = y1[e] and r1[c][e] = y1[e], both planes; grid (cdiv(v, 256), nsys)
-__global__ void unpack_ea_y1_kernel(SysBatch b, int o, int v, long long ldk, __nv_bfloat16 *rk, long long ld1,
-                                    __nv_bfloat16 *r1) {
-  const int s = blockIdx.y, e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= v) return;
-  const long long ov2 = (long long)o * v * v;
-  const Cz u = load_u(b, s, e);
-  const __nv_bfloat16 hr = __float2bfloat16(u.r), hi = __float2bfloat16(u.i);
-  rk[(long long)(2 * s) * ldk + ov2 + e] = hr;
-  rk[(long long)(2 * s + 1) * ldk + ov2 + e] = hi;
-  r1[(long long)(2 * s) * ld1 + e] = hr;
-  r1[(long long)(2 * s + 1) * ld1 + e] = hi;
-}
-
-constexpr int KSPLIT = 64;   // split of the long-K contractions (Z, 1h row) into partial sums
+constexpr int KSPLIT = 76;   // split of the long-K contraction (Z and the one-index row): two row tiles fill 152 SMs
 
 struct MixedWork {
   __nv_bfloat16 *r2b, *r2o, *rk, *rz;
-  float *T, *Q, *U, *Zp, *S1p;
+  float *T, *Q, *U, *Zp, *S1;
   long long bytes;
 };
 
@@ -322,8 +328,8 @@ MixedWork layout(const gfcc_ctx *c, int nsys, void *base) {
   w.T = reinterpret_cast<float *>(take(o * v * o * C2 * 4));
   w.Q = reinterpret_cast<float *>(take(o * o * v * C2 * 4));
   w.U = reinterpret_cast<float *>(take(o * v * o * C2 * 4));
-  w.Zp = reinterpret_cast<float *>(take(KSPLIT * v * C2 * 4));
-  w.S1p = reinterpret_cast<float *>(take(KSPLIT * o * C2 * 4));
+  w.Zp = reinterpret_cast<float *>(take(KSPLIT * (v + o) * C2 * 4));
+  w.S1 = reinterpret_cast<float *>(take(o * C2 * 4));
   w.bytes = p - static_cast<unsigned char *>(base);
   return w;
 }
@@ -332,7 +338,7 @@ MixedWork layout(const gfcc_ctx *c, int nsys, void *base) {
 
 struct MixedWorkEA {
   __nv_bfloat16 *r2e, *r2p, *rk, *rz;
-  float *T, *Qp, *U, *Zp, *S1p;
+  float *T, *Qp, *U, *Zp, *S1;
   long long bytes;
 };
 
@@ -352,8 +358,8 @@ MixedWorkEA layout_ea(const gfcc_ctx *c, int nsys, void *base) {
   w.T = reinterpret_cast<float *>(take(o * v * v * C2 * 4));
   w.Qp = reinterpret_cast<float *>(take(std::max<long long>(Pv, 1) * o * C2 * 4));
   w.U = reinterpret_cast<float *>(take(ov2 * C2 * 4));
-  w.Zp = reinterpret_cast<float *>(take(KSPLIT * o * C2 * 4));
-  w.S1p = reinterpret_cast<float *>(take(KSPLIT * v * C2 * 4));
+  w.Zp = reinterpret_cast<float *>(take(KSPLIT * (o + v) * C2 * 4));
+  w.S1 = reinterpret_cast<float *>(take(v * C2 * 4));
   w.bytes = p - static_cast<unsigned char *>(base);
   return w;
 }
@@ -380,7 +386,7 @@ int apply_ip_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
     const unsigned long long rcp_o = ((1ULL << 32) + (unsigned long long)o - 1) / (unsigned long long)o;
     const size_t sm = (size_t)o * (UNPACK_ET + 1) * sizeof(float2);
     unpack_ip_kernel<<<dim3(cdiv(v, UNPACK_ET), (unsigned)o, (unsigned)b.nsys), 256, sm, st>>>(
-        b, (int)o, (int)v, rcp_o, c->ld_ov, c->ld_o2, c->ld_k1, w.r2b, w.r2o, w.rk);
+        b, (int)o, (int)v, rcp_o, c->ld_ov, c->ld_o2, c->ld_k1, w.r2b, w.r2o, w.rk, c->ld_ot, w.rz);
     GFCC_LAUNCH_CHECK();
   } else {
     unpack_ring_kernel<<<grid1d(o * C2 * ov), 256, 0, st>>>(b, (int)o, (int)v, c->ld_ov, w.r2b);
@@ -391,9 +397,9 @@ int apply_ip_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
     unpack_k_tiled_kernel<<<dim3(cdiv(o, 32), cdiv(v, 32), o * C2), dim3(32, 8), 0, st>>>(b, (int)o, (int)v,
                                                                                           c->ld_k1, w.rk);
     GFCC_LAUNCH_CHECK();
+    unpack_r1_kernel<<<cdiv(b.nsys * o, 128), 128, 0, st>>>(b, (int)o, (int)v, c->ld_k1, w.rk, c->ld_ot, w.rz);
+    GFCC_LAUNCH_CHECK();
   }
-  unpack_r1_kernel<<<cdiv(C2 * o, 128), 128, 0, st>>>(b, (int)o, (int)v, c->ld_k1, w.rk, c->ld_ot, w.rz);
-  GFCC_LAUNCH_CHECK();
   }
   {
     PhaseTimer tr(c, PH_RING_BF16, 2.0 * (double)ov * (double)ov * (double)(o * C2));
@@ -405,24 +411,20 @@ int apply_ip_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
                                                  (double)o * (o2v + o)));
     GFCC_TRY(gemm_bf16_tn(st, c->Wq_bf, c->ld_o2, w.r2o, c->ld_o2, w.Q, v * C2, (int)oo, (int)(v * C2), (int)oo, 1.0f,
                           0.0f));
-    // three-body: Z (split K) -> BF16 transposed into rz[c][o + e]; then U = [W1 | T3] [r1 | Z]
-    const int zs = umma_splits((int)o2v, KSPLIT);
-    GFCC_TRY(gemm_bf16_tn(st, c->V3_bf, c->ld_o2v, w.rk, c->ld_k1, w.Zp, C2, (int)v, (int)C2, (int)o2v, 1.0f, 0.0f, zs,
-                          v * C2));
-    reduce_splits_kernel<<<grid1d(v * C2), 256, 0, st>>>(w.Zp, zs, v, C2, v * C2, w.rz + o, c->ld_ot);
+    // three-body Z and the 1h row in one product (split K); Z -> BF16 transposed into rz[c][o + e]; then
+    // U = [W1 | T3] [r1 | Z]
+    const int zs = umma_splits((int)(o2v + o), KSPLIT);
+    GFCC_TRY(gemm_bf16_tn(st, c->VU_bf, c->ld_k1, w.rk, c->ld_k1, w.Zp, C2, (int)(v + o), (int)C2, (int)(o2v + o), 1.0f,
+                          0.0f, zs, (v + o) * C2));
+    reduce_splits_kernel<<<cdiv((v + o) * C2, 32), 256, 0, st>>>(w.Zp, zs, (int)(v + o), (int)C2, (int)v, w.rz + o,
+                                                                 c->ld_ot, w.S1);
     GFCC_LAUNCH_CHECK();
     GFCC_TRY(gemm_bf16_tn(st, c->WT_bf, c->ld_ot, w.rz, c->ld_ot, w.U, C2, (int)o2v, (int)C2, (int)(o + v), 1.0f,
                           0.0f));
-    // 1h row (split K)
-    const int ss = umma_splits((int)(o2v + o), KSPLIT);
-    GFCC_TRY(gemm_bf16_tn(st, c->U1_bf, c->ld_k1, w.rk, c->ld_k1, w.S1p, C2, (int)o, (int)C2, (int)(o2v + o), 1.0f, 0.0f,
-                          ss, o * C2));
-    reduce_splits_kernel<<<grid1d(o * C2), 256, 0, st>>>(w.S1p, ss, o, C2, o * C2, nullptr, 0);
-    GFCC_LAUNCH_CHECK();
   }
   {
     PhaseTimer tp(c, PH_EPILOGUE, 4.0 * C2 * (3.0 * o2v + o) + (b.xf ? 16.0 : 32.0) * b.nsys * c->dim_ip);
-    GFCC_TRY((epi::launch_ip<float, epi::MODE_OFFDIAG>(st, b, (int)o, (int)v, w.S1p, w.T, w.Q, w.U, c->diag_ip)));
+    GFCC_TRY((epi::launch_ip<float, epi::MODE_OFFDIAG>(st, b, (int)o, (int)v, w.S1, w.T, w.Q, w.U, c->diag_ip)));
   }
   return GFCC_OK;
 }
@@ -440,16 +442,13 @@ int apply_ea_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
   {
     PhaseTimer tu(c, PH_UNPACK);
     unpack_ea_tile_kernel<<<dim3(cdiv(v, 32), cdiv(v, 32), (unsigned)(o * b.nsys)), dim3(32, 8), 0, st>>>(
-        b, (int)o, (int)v, Pv, c->ld_ov, c->ld_k1e, w.r2e, w.rk);
+        b, (int)o, (int)v, Pv, c->ld_ov, c->ld_k1e, w.r2e, w.rk, c->ld_ot, w.rz);
     GFCC_LAUNCH_CHECK();
     if (Pv > 0) {
       unpack_ea_pairs_kernel<<<dim3(cdiv(Pv, 256), (unsigned)(o * b.nsys)), 256, 0, st>>>(b, (int)o, (int)v, Pv,
                                                                                         c->ld_pv, w.r2p);
       GFCC_LAUNCH_CHECK();
     }
-    unpack_ea_y1_kernel<<<dim3(cdiv(v, 256), (unsigned)b.nsys), 256, 0, st>>>(b, (int)o, (int)v, c->ld_k1e, w.rk,
-                                                                              c->ld_ot, w.rz);
-    GFCC_LAUNCH_CHECK();
   }
   // T[(i,b)][(a,c)] = Wr_ea[(i,b)][(m,e)] y2[m,a,e]
   {
@@ -465,24 +464,20 @@ int apply_ea_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
   }
   {
     PhaseTimer tob(c, PH_BF16_OTHER, 2.0 * C2 * ((double)o * ov2 + (double)ov2 * (v + o) + (double)v * (ov2 + v)));
-    // U[(i,b,a)][c] = [W3 | T3e] [y1 | Z],  Z[m][c] = V3e[m][(n,f,e)] y2[n,e,f] (split K, into rz[c][v + m])
-    const int zs = umma_splits((int)ov2, KSPLIT);
-    GFCC_TRY(gemm_bf16_tn(st, c->V3e_bf, c->ld_ov2, w.rk, c->ld_k1e, w.Zp, C2, (int)o, (int)C2, (int)ov2, 1.0f, 0.0f,
-                          zs, o * C2));
-    reduce_splits_kernel<<<grid1d(o * C2), 256, 0, st>>>(w.Zp, zs, o, C2, o * C2, w.rz + v, c->ld_ot);
+    // Z[m][c] = V3e[m][(n,f,e)] y2[n,e,f] (into rz[c][v + m]) and the 1p row [U1e | Fvv off-diagonal][a] . [y2 | y1](c)
+    // in one product (split K); then U[(i,b,a)][c] = [W3 | T3e] [y1 | Z]
+    const int zs = umma_splits((int)(ov2 + v), KSPLIT);
+    GFCC_TRY(gemm_bf16_tn(st, c->VUe_bf, c->ld_k1e, w.rk, c->ld_k1e, w.Zp, C2, (int)(o + v), (int)C2, (int)(ov2 + v),
+                          1.0f, 0.0f, zs, (o + v) * C2));
+    reduce_splits_kernel<<<cdiv((o + v) * C2, 32), 256, 0, st>>>(w.Zp, zs, (int)(o + v), (int)C2, (int)o, w.rz + v,
+                                                                 c->ld_ot, w.S1);
     GFCC_LAUNCH_CHECK();
     GFCC_TRY(gemm_bf16_tn(st, c->WTe_bf, c->ld_ot, w.rz, c->ld_ot, w.U, C2, (int)ov2, (int)C2, (int)(v + o), 1.0f,
                           0.0f));
-    // 1p row: S1[a][c] = [U1e | Fvv off-diagonal][a] . [y2 | y1](c) (split K)
-    const int ss = umma_splits((int)(ov2 + v), KSPLIT);
-    GFCC_TRY(gemm_bf16_tn(st, c->U1e_bf, c->ld_k1e, w.rk, c->ld_k1e, w.S1p, C2, (int)v, (int)C2, (int)(ov2 + v), 1.0f,
-                          0.0f, ss, v * C2));
-    reduce_splits_kernel<<<grid1d(v * C2), 256, 0, st>>>(w.S1p, ss, v, C2, v * C2, nullptr, 0);
-    GFCC_LAUNCH_CHECK();
   }
   {
     PhaseTimer tp(c, PH_EPILOGUE, 4.0 * C2 * (2.0 * ov2 + (double)Pv * o + v) + (b.xf ? 16.0 : 32.0) * b.nsys * c->dim_ea);
-    GFCC_TRY((epi::launch_ea<float, epi::MODE_OFFDIAG>(st, b, (int)o, (int)v, Pv, w.S1p, w.T, w.Qp, w.U,
+    GFCC_TRY((epi::launch_ea<float, epi::MODE_OFFDIAG>(st, b, (int)o, (int)v, Pv, w.S1, w.T, w.Qp, w.U,
                                                        c->diag_ea)));
   }
   return GFCC_OK;
