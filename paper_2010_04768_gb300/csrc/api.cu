@@ -634,6 +634,15 @@ int prepare_kept(gfcc_ctx *c, int sector, long long n, int n_omega, int n_orb, c
   return GFCC_OK;
 }
 
+// K splits of the overlap contraction: chunks of at most 8192 elements, and shorter ones (512 at least) while the
+// 16 x 16 output tiles would leave SMs idle (one tile of 8192 elements takes 0.5 ms of its SM: the overlaps of a
+// small molecule took 0.6 ms on a handful of them)
+long long overlap_splits(long long n, long long rows, long long cols) {
+  const long long tiles = std::max<long long>(1, ((rows + 15) / 16) * ((cols + 15) / 16));
+  const long long fill = std::min<long long>((n + 511) / 512, (4 * 152 + tiles - 1) / tiles);
+  return std::max<long long>((n + 8191) / 8192, fill);
+}
+
 int solve_impl_inner(gfcc_ctx *c, int n_omega, const double *d_om, double eta, const OrbLists &ol, double tol,
                      double *d_G) {
   cudaStream_t st = c->stream;
@@ -676,7 +685,8 @@ int solve_impl_inner(gfcc_ctx *c, int n_omega, const double *d_om, double eta, c
     if (keep) GFCC_TRY(prepare_kept(c, sector, n, n_omega, n_orb, d_om, d_orb, eta));
     const int nsys = choose_batch(c, sector, n, ntasks);
     const int m = mixed ? c->inner_restart : c->restart;
-    const long long nsplit = (n + 8191) / 8192;
+    const long long nsplit = overlap_splits(n, 2LL * nsys, n_left);
+    const long long kchunk = (n + nsplit - 1) / nsplit;
     const long long gw = gmres_work_doubles(c, sector, n, nsys, m, mixed);
     // guess workspace: Gram, features, model outputs, coefficients, predictions, deltas, p/n,
     // Gram partials; then the ints (neighbour slots, counts, kinds, store slots)
@@ -829,7 +839,7 @@ int solve_impl_inner(gfcc_ctx *c, int n_omega, const double *d_om, double eta, c
             k.B = Cl; k.bk = imap1(1); k.bn = imap1(n);
             k.C = part; k.cm = imap1(n_left); k.cn = imap1(1);
             k.M = 2LL * ns; k.N = n_left; k.K = n;
-            k.nsplit = nsplit; k.kchunk = 8192; k.scz = 2LL * ns * n_left;
+            k.nsplit = nsplit; k.kchunk = kchunk; k.scz = 2LL * ns * n_left;
             GFCC_TRY(contract_f64(k, st));
             overlap_scatter_kernel<<<grid1d((long long)ns * n_left), 256, 0, st>>>(
                 part, (int)nsplit, ns, ns, n_left, d_twf, d_ta, ip ? 1 : 0, ol.nP, ol.nQ, d_G);
@@ -970,7 +980,7 @@ int solve_impl_inner(gfcc_ctx *c, int n_omega, const double *d_om, double eta, c
       k.B = Cl; k.bk = imap1(1); k.bn = imap1(n);
       k.C = part; k.cm = imap1(n_left); k.cn = imap1(1);
       k.M = 2LL * nsys; k.N = n_left; k.K = n;
-      k.nsplit = nsplit; k.kchunk = 8192; k.scz = 2LL * nsys * n_left;
+      k.nsplit = nsplit; k.kchunk = kchunk; k.scz = 2LL * nsys * n_left;
       GFCC_TRY(contract_f64(k, st));
       overlap_scatter_kernel<<<grid1d((long long)nb * n_left), 256, 0, st>>>(part, (int)nsplit, nsys, nb, n_left,
                                                                               d_tw, d_ta, ip ? 1 : 0, ol.nP, ol.nQ,
