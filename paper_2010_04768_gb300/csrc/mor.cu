@@ -16,8 +16,8 @@
 // exceeds drop_tol times its norm before.  Projection: the new basis vectors are paired as the real and
 // imaginary planes of complex vectors and sent through the context's sigma product (FP64, or the
 // FP64-accurate digit-plane product in mixed-precision contexts), Hhat = S W^T by an FP64 contraction.
-// Model solves: one CTA per frequency builds z I +/- Hhat in global memory and runs Gaussian
-// elimination with partial pivoting on it for all right-hand sides at once (O(N_omega m^3), the cost
+// Model solves: one CTA per frequency builds z I +/- Hhat in shared memory (global when it is too large)
+// and runs Gaussian elimination with partial pivoting on it for all right-hand sides at once (O(N_omega m^3), the cost
 // the paper states for this step).  The model residual b - A(omega) S Xhat = b - z S Xhat -/+ W Xhat
 // of a model solution needs no sigma product (the driver's error indicator).
 #include <algorithm>
@@ -27,7 +27,9 @@
 
 #include "ctx.cuh"
 #include "kernels.cuh"
+#include "ozaki.cuh"
 #include "sigma.cuh"
+#include "umma.cuh"
 
 struct gfcc_mor {
   gfcc_ctx *c = nullptr;
@@ -138,122 +140,175 @@ __global__ void mor_real_kernel(const double *z, long long n, int rows, double *
     out[t] = z[2 * t];
 }
 
-// Model solves: one CTA per frequency w.  A = z_w I + s Hhat (complex, m x m, row-major in work
-// [w][m][m]), right-hand sides bh [m][nb] (real), solution X [w][m][nb] complex; then
+// Model solves: one CTA per frequency w.  [A | X] = [z_w I + s Hhat | bh] (complex, m x (m + nb), row-major, in
+// shared memory when it fits, else in work [w][m][m + nb]); solution X [w][m][nb] complex; then
 // G[w][a][b] (IP: a over rhs, b over left; EA: a over left, b over rhs) = sum_k ch[k][left] X[k][rhs].
-// Gaussian elimination with partial pivoting by rows; threads split the trailing updates.
+// Gaussian elimination with partial pivoting by rows; threads split the trailing updates, the back
+// substitution runs by columns.  Bound by the FP64 pipe (m^3 / 3 complex FMAs) once the pivot search is a warp's and
+// the matrix is in shared memory: 256 frequencies at m = 72, nb = 12 took 4 ms with a serial search over the block
+// and one thread per right-hand side in the back substitution.
 __global__ __launch_bounds__(MT) void mor_model_solve_kernel(const double *Hh, int m, const double *omegas, double eta,
                                                              double zsign, double hsign, const double *bh, int nb,
                                                              const double *ch, int nl, int is_ip, double2 *Aw,
                                                              double2 *Xw, double *G) {
+  extern __shared__ __align__(16) double2 sm[];
   __shared__ int piv;
-  __shared__ double pval[MT];
-  __shared__ int pidx[MT];
-  const int w = blockIdx.x;
-  double2 *A = Aw + (long long)w * m * m;
-  double2 *X = Xw + (long long)w * m * nb;
+  __shared__ double2 inv_s;
+  const int w = blockIdx.x, ld = m + nb, t0 = threadIdx.x, lane = t0 & 31, warp = t0 >> 5;
+  double2 *lm = sm;                                                       // multipliers of a step [m]
+  double2 *A = Aw != nullptr ? Aw + (long long)w * m * ld : sm + m;       // [m][ld]
   const double om = omegas[w];
-  for (long long t = threadIdx.x; t < (long long)m * m; t += MT) {
-    const int i = (int)(t / m), j = (int)(t % m);
-    A[t] = make_double2(hsign * Hh[t] + (i == j ? om : 0.0), i == j ? zsign * eta : 0.0);
+  for (int t = t0; t < m * ld; t += MT) {
+    const int i = t / ld, j = t - i * ld;
+    A[t] = j < m ? make_double2(hsign * Hh[(long long)i * m + j] + (i == j ? om : 0.0), i == j ? zsign * eta : 0.0)
+                 : make_double2(bh[(long long)i * nb + (j - m)], 0.0);
   }
-  for (long long t = threadIdx.x; t < (long long)m * nb; t += MT) X[t] = make_double2(bh[t], 0.0);
   __syncthreads();
   for (int k = 0; k < m; k++) {
-    // pivot: largest |A[i][k]| over i >= k
-    double best = -1.0;
-    int bi = k;
-    for (int i = k + threadIdx.x; i < m; i += MT) {
-      const double2 a = A[(long long)i * m + k];
-      const double mag = a.x * a.x + a.y * a.y;
-      if (mag > best) {
-        best = mag;
-        bi = i;
-      }
-    }
-    pval[threadIdx.x] = best;
-    pidx[threadIdx.x] = bi;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double b = -1.0;
-      int idx = k;
-      for (int t = 0; t < MT; t++)
-        if (pval[t] > b) {
-          b = pval[t];
-          idx = pidx[t];
+    // pivot: largest |A[i][k]| over i >= k (the lowest i of equal ones)
+    if (warp == 0) {
+      double best = -1.0;
+      int bi = k;
+      for (int i = k + lane; i < m; i += 32) {
+        const double2 a = A[(long long)i * ld + k];
+        const double mag = a.x * a.x + a.y * a.y;
+        if (mag > best) {
+          best = mag;
+          bi = i;
         }
-      piv = idx;
+      }
+      for (int off = 16; off > 0; off >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+        if (ob > best || (ob == best && oi < bi)) {
+          best = ob;
+          bi = oi;
+        }
+      }
+      if (lane == 0) {
+        const double2 d = A[(long long)bi * ld + k];
+        const double dd = d.x * d.x + d.y * d.y;
+        piv = bi;
+        inv_s = dd > 0.0 ? make_double2(d.x / dd, -d.y / dd) : make_double2(0.0, 0.0);
+      }
     }
     __syncthreads();
     const int p = piv;
-    if (p != k) {
-      for (int j = threadIdx.x; j < m; j += MT) {
-        const double2 t = A[(long long)k * m + j];
-        A[(long long)k * m + j] = A[(long long)p * m + j];
-        A[(long long)p * m + j] = t;
+    const double2 inv = inv_s;
+    if (p != k)
+      for (int j = k + t0; j < ld; j += MT) {
+        const double2 t = A[(long long)k * ld + j];
+        A[(long long)k * ld + j] = A[(long long)p * ld + j];
+        A[(long long)p * ld + j] = t;
       }
-      for (int j = threadIdx.x; j < nb; j += MT) {
-        const double2 t = X[(long long)k * nb + j];
-        X[(long long)k * nb + j] = X[(long long)p * nb + j];
-        X[(long long)p * nb + j] = t;
-      }
-    }
     __syncthreads();
-    const double2 d = A[(long long)k * m + k];
-    const double dd = d.x * d.x + d.y * d.y;
-    const double2 inv = dd > 0.0 ? make_double2(d.x / dd, -d.y / dd) : make_double2(0.0, 0.0);
     // eliminate below: row i -= l_i row k, l_i = A[i][k] / A[k][k] (columns > k and the right-hand sides)
-    const int rows = m - k - 1, cols = m - k - 1 + nb;
-    for (long long t = threadIdx.x; t < (long long)rows * cols; t += MT) {
-      const int i = k + 1 + (int)(t / cols), jj = (int)(t % cols);
-      const double2 a = A[(long long)i * m + k];
-      const double2 l = make_double2(a.x * inv.x - a.y * inv.y, a.x * inv.y + a.y * inv.x);
-      double2 *dst;
-      double2 src;
-      if (jj < m - k - 1) {
-        dst = &A[(long long)i * m + k + 1 + jj];
-        src = A[(long long)k * m + k + 1 + jj];
-      } else {
-        dst = &X[(long long)i * nb + (jj - (m - k - 1))];
-        src = X[(long long)k * nb + (jj - (m - k - 1))];
+    for (int i = k + 1 + t0; i < m; i += MT) {
+      const double2 a = A[(long long)i * ld + k];
+      lm[i] = make_double2(a.x * inv.x - a.y * inv.y, a.x * inv.y + a.y * inv.x);
+    }
+    __syncthreads();
+    const double2 *rk = A + (long long)k * ld;
+    for (int i = k + 1 + warp; i < m; i += MT / 32) {
+      const double2 l = lm[i];
+      double2 *ri = A + (long long)i * ld;
+      for (int j = k + 1 + lane; j < ld; j += 32) {
+        double2 v = ri[j];
+        const double2 src = rk[j];
+        v.x -= l.x * src.x - l.y * src.y;
+        v.y -= l.x * src.y + l.y * src.x;
+        ri[j] = v;
       }
-      double2 v = *dst;
-      v.x -= l.x * src.x - l.y * src.y;
-      v.y -= l.x * src.y + l.y * src.x;
-      *dst = v;
     }
     __syncthreads();
   }
-  // back substitution, one right-hand side per thread
-  for (int r = threadIdx.x; r < nb; r += MT) {
-    for (int i = m - 1; i >= 0; i--) {
-      double2 acc = X[(long long)i * nb + r];
-      for (int j = i + 1; j < m; j++) {
-        const double2 a = A[(long long)i * m + j], x = X[(long long)j * nb + r];
-        acc.x -= a.x * x.x - a.y * x.y;
-        acc.y -= a.x * x.y + a.y * x.x;
-      }
-      const double2 d = A[(long long)i * m + i];
-      const double dd = d.x * d.x + d.y * d.y;
-      X[(long long)i * nb + r] =
-          dd > 0.0 ? make_double2((acc.x * d.x + acc.y * d.y) / dd, (acc.y * d.x - acc.x * d.y) / dd)
-                   : make_double2(0.0, 0.0);
+  // back substitution, column by column: x_i = X_i / A[i][i], then rows above lose A[r][i] x_i
+  for (int i = m - 1; i >= 0; i--) {
+    double2 *xi = A + (long long)i * ld + m;
+    const double2 d = A[(long long)i * ld + i];
+    const double dd = d.x * d.x + d.y * d.y;
+    for (int r = t0; r < nb; r += MT) {
+      const double2 a = xi[r];
+      xi[r] = dd > 0.0 ? make_double2((a.x * d.x + a.y * d.y) / dd, (a.y * d.x - a.x * d.y) / dd)
+                       : make_double2(0.0, 0.0);
     }
+    __syncthreads();
+    for (int t = t0; t < i * nb; t += MT) {
+      const int row = t / nb, r = t - row * nb;
+      const double2 a = A[(long long)row * ld + i], x = xi[r];
+      double2 *v = A + (long long)row * ld + m + r;
+      v->x -= a.x * x.x - a.y * x.y;
+      v->y -= a.x * x.y + a.y * x.x;
+    }
+    __syncthreads();
   }
-  __syncthreads();
+  for (int t = t0; t < m * nb; t += MT) {
+    const int k = t / nb, r = t - k * nb;
+    Xw[(long long)w * m * nb + t] = A[(long long)k * ld + m + r];
+  }
   if (G == nullptr) return;
-  for (int t = threadIdx.x; t < nb * nl; t += MT) {
+  for (int t = t0; t < nb * nl; t += MT) {
     const int r = t / nl, q = t % nl;   // rhs r, left q
     double gr = 0.0, gi = 0.0;
     for (int k = 0; k < m; k++) {
       const double cq = ch[(long long)k * nl + q];
-      const double2 x = X[(long long)k * nb + r];
+      const double2 x = A[(long long)k * ld + m + r];
       gr += cq * x.x;
       gi += cq * x.y;
     }
     const long long idx = is_ip ? ((long long)w * nb + r) * nl + q : ((long long)w * nl + q) * nb + r;
     G[2 * idx] = gr;
     G[2 * idx + 1] = gi;
+  }
+}
+
+// Coefficient rows of the model residuals as products with [S | W]: for row c = 2 (w nb + r) + re/im,
+// C[c][k] = re/im of z_w X[w][k][r], C[c][m + k] = wsign re/im of X[w][k][r]
+__global__ void mor_coef_kernel(const double2 *Xw, int m, int nb, long long pairs, const double *omegas, double eta,
+                                double zsign, double wsign, double *C) {
+  const long long tot = pairs * m;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
+    const long long pr = t / m;
+    const int k = (int)(t - pr * m), w = (int)(pr / nb), r = (int)(pr - (long long)w * nb);
+    const double2 x = Xw[((long long)w * m + k) * nb + r];
+    const double zr = omegas[w], zi = zsign * eta;
+    double *re = C + 4 * pr * m + k, *im = re + 2 * m;
+    re[0] = zr * x.x - zi * x.y;
+    im[0] = zr * x.y + zi * x.x;
+    re[m] = wsign * x.x;
+    im[m] = wsign * x.y;
+  }
+}
+
+// out[2 pr] = ||b_r - (A x)_pr||^2 and out[2 pr + 1] = ||b_r||^2 from Ax [2 pr + re/im][n], one block per pair
+__global__ __launch_bounds__(MT) void mor_resnorm_kernel(const double *Ax, const double *B, long long n, int nb,
+                                                         double *out) {
+  __shared__ double sh[2][MT / 32];
+  const long long pr = blockIdx.x;
+  const double *ar = Ax + 2 * pr * n, *ai = ar + n, *b = B + (pr % nb) * n;
+  double rr = 0.0, bb = 0.0;
+  for (long long e = threadIdx.x; e < n; e += MT) {
+    const double x = b[e], d = x - ar[e], i = ai[e];
+    rr += d * d + i * i;
+    bb += x * x;
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    rr += __shfl_xor_sync(0xffffffffu, rr, off);
+    bb += __shfl_xor_sync(0xffffffffu, bb, off);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sh[0][threadIdx.x >> 5] = rr;
+    sh[1][threadIdx.x >> 5] = bb;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0, c = 0.0;
+    for (int t = 0; t < MT / 32; t++) {
+      a += sh[0][t];
+      c += sh[1][t];
+    }
+    out[2 * pr] = a;
+    out[2 * pr + 1] = c;
   }
 }
 
@@ -322,18 +377,17 @@ int grow(gfcc_mor *M, size_t bytes) {
 int ensure_cap(gfcc_mor *M, int need) {
   if (need <= M->cap) return GFCC_OK;
   const int cap = std::max(need, std::max(64, 2 * M->cap));
-  double *S = nullptr, *W = nullptr, *H = nullptr;
+  double *S = nullptr, *W = nullptr, *H = nullptr;   // W follows S: the residual products read [S | W] as one operand
   const size_t vb = sizeof(double) * (size_t)cap * (size_t)M->n;
-  if (dmalloc(reinterpret_cast<void **>(&S), vb) != cudaSuccess ||
-      dmalloc(reinterpret_cast<void **>(&W), vb) != cudaSuccess ||
+  if (dmalloc(reinterpret_cast<void **>(&S), 2 * vb) != cudaSuccess ||
       dmalloc(reinterpret_cast<void **>(&H), sizeof(double) * (size_t)cap * cap) != cudaSuccess) {
     cudaGetLastError();
     dfree(S);
-    dfree(W);
     dfree(H);
     set_error("model-order reduction: cannot allocate a subspace of %d vectors (%.3f GB)", cap, 2.0 * vb / 1e9);
     return GFCC_ERR_OOM;
   }
+  W = S + (size_t)cap * (size_t)M->n;
   cudaStream_t st = M->c->stream;
   if (M->m > 0) {
     GFCC_CUDA(cudaMemcpyAsync(S, M->S, sizeof(double) * (size_t)M->m * M->n, cudaMemcpyDeviceToDevice, st));
@@ -343,7 +397,6 @@ int ensure_cap(gfcc_mor *M, int need) {
     GFCC_CUDA(cudaStreamSynchronize(st));
   }
   dfree(M->S);
-  dfree(M->W);
   dfree(M->H);
   M->S = S;
   M->W = W;
@@ -456,13 +509,33 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   // host lists -> device, right-hand sides (complex, real part only) and left vectors
   int *d_lists = nullptr;
   double *buf = nullptr;
-  // frequencies per model launch: their dense model matrices and solutions within about 4 GB
-  const long long per_w = 16LL * m * (m + nb);
-  const long long wb = std::max<long long>(1, std::min<long long>({(long long)n_omega, 256LL, (4LL << 30) / per_w}));
-  const size_t need = sizeof(double) * (size_t)(2LL * nb * n + (long long)nb * n + (long long)nl * n +
-                                                (long long)m * (nb + nl) + 2LL * wb * m * m + 2LL * wb * m * nb +
-                                                2LL * n_omega * nb * nl + n_omega + 2LL * wb * nb + 64);
-  GFCC_TRY(grow(M, need));
+  // The residuals of mixed-precision contexts are products [S | W] x on digit planes (the FP64 units take
+  // 8 n m operations per frequency and right-hand side: 26 ms for 500 x 12 at n = 9616, m = 72, against 4 ms); other
+  // contexts and models too small to gain keep the FP64 kernel.  Short sums are as accurate as that kernel here: the
+  // residuals of models of 36 vectors over 9616 and 6280 elements were within 6e-14 (rms, of ||b||) of quad sums
+  // either way.
+  const bool mixed = h_relres != nullptr && c->precision == GFCC_PREC_MIXED_BF16;
+  bool planes = mixed && emulation_pays(2LL * std::min(n_omega, 304) * nb, n, std::max(2 * m, 160), false);
+  long long per_pair, wb;
+  size_t need;
+  auto layout = [&]() {
+    per_pair = planes ? 16LL * n + 32LL * m : 0;   // A x and the coefficient rows
+    // frequencies per model launch: their dense model matrices, solutions and residuals within about 4 GB
+    const long long per_w = 16LL * m * (m + nb) + per_pair * nb;
+    wb = std::max<long long>(1, std::min<long long>({(long long)n_omega, 304LL, (4LL << 30) / per_w}));
+    need = sizeof(double) * (size_t)(2LL * nb * n + (long long)nb * n + (long long)nl * n + (long long)m * (nb + nl) +
+                                     2LL * wb * m * (m + nb) + 2LL * wb * m * nb + 2LL * n_omega * nb * nl + n_omega +
+                                     2LL * wb * nb + 64) +
+           (size_t)(per_pair * wb * nb);
+  };
+  layout();
+  int g = grow(M, need);
+  if (g == GFCC_ERR_OOM && planes) {
+    planes = false;
+    layout();
+    g = grow(M, need);
+  }
+  GFCC_TRY(g);
   if (dmalloc(reinterpret_cast<void **>(&d_lists), sizeof(int) * (nb + nl) + 16) != cudaSuccess) {
     cudaGetLastError();
     set_error("gfcc_mor_green: allocation failed");
@@ -475,10 +548,12 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   double *bh = Cl + (long long)nl * n;       // [m][nb]
   double *ch = bh + (long long)m * nb;       // [m][nl]
   double2 *Aw = reinterpret_cast<double2 *>(ch + (long long)m * nl);
-  double2 *Xw = Aw + wb * m * m;
+  double2 *Xw = Aw + wb * m * (m + nb);
   double *Gd = reinterpret_cast<double *>(Xw + wb * m * nb);
   double *om = Gd + 2LL * n_omega * nb * nl;
   double *res = om + n_omega;
+  double *Ax = res + 2LL * wb * nb;                    // [2 wb nb][n]
+  double *Cx = Ax + (planes ? 2LL * wb * nb * n : 0);  // [2 wb nb][2 m]
   int s = GFCC_OK;
   auto done = [&](int code) {
     dfree(d_lists);
@@ -516,20 +591,60 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   }
   const double zsign = ip ? -1.0 : 1.0, hsign = ip ? 1.0 : -1.0;
   std::vector<double> hres(2 * wb * nb);
+  // the model matrix in shared memory where it fits (multipliers + m x (m + nb))
+  const size_t smem_lm = sizeof(double2) * (size_t)m, smem_all = smem_lm + sizeof(double2) * (size_t)m * (m + nb);
+  const bool in_smem = smem_all <= 220 * 1024;
+  const size_t smem = in_smem ? smem_all : smem_lm;
+  if (smem > 48 * 1024)
+    GFCC_CUDA(cudaFuncSetAttribute(mor_model_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  EmuArena arena;   // digit planes of the residual products
+  EmuArena *prev_arena = g_emu_arena;
   for (int w0 = 0; w0 < n_omega; w0 += (int)wb) {
     const int nw = std::min<int>((int)wb, n_omega - w0);
-    mor_model_solve_kernel<<<nw, MT, 0, st>>>(Hm, m, om + w0, eta, zsign, hsign, bh, nb, ch, nl, ip ? 1 : 0, Aw, Xw,
-                                              Gd + 2LL * w0 * nb * nl);
+    mor_model_solve_kernel<<<nw, MT, smem, st>>>(Hm, m, om + w0, eta, zsign, hsign, bh, nb, ch, nl, ip ? 1 : 0,
+                                                 in_smem ? nullptr : Aw, Xw, Gd + 2LL * w0 * nb * nl);
     GFCC_LAUNCH_CHECK();
     if (h_relres) {
-      GFCC_CUDA(cudaMemsetAsync(res, 0, sizeof(double) * 2 * nw * nb, st));
-      mor_residual_kernel<<<dim3(cdiv(n, MT), (unsigned)(nw * nb)), MT, 0, st>>>(
-          M->S, M->W, n, m, Xw, nb, om + w0, eta, zsign, ip ? 1.0 : -1.0, Br, res);
-      GFCC_LAUNCH_CHECK();
+      const double wsign = ip ? 1.0 : -1.0;
+      bool done_planes = false;
+      if (planes) {
+        // Ax[c][e] = sum_k Cx[c][k] [S | W][k][e], then ||b - A x||^2 per pair
+        const long long pairs = (long long)nw * nb;
+        mor_coef_kernel<<<grid1d(pairs * m), MT, 0, st>>>(Xw, m, nb, pairs, om + w0, eta, zsign, wsign, Cx);
+        GFCC_LAUNCH_CHECK();
+        g_emu_arena = &arena;
+        if (w0 == 0) s = umma_error_reset(st);
+        if (s == GFCC_OK)
+          s = gemm_f64_emulated(st, 2 * pairs, n, 2LL * m, 1.0, Cx, imap1(2LL * m), imap1(1), M->S,
+                                imap2(m, n, (long long)M->cap * n), imap1(1), 0.0, Ax, imap1(n), imap1(1));
+        g_emu_arena = prev_arena;
+        if (s == GFCC_OK) {
+          mor_resnorm_kernel<<<(unsigned)pairs, MT, 0, st>>>(Ax, Br, n, nb, res);
+          GFCC_LAUNCH_CHECK();
+          done_planes = true;
+        } else if (s != GFCC_ERR_OOM) {
+          dfree(Hm);
+          return done(s);
+        }
+        s = GFCC_OK;   // no room for the planes: the FP64 units
+      }
+      if (!done_planes) {
+        GFCC_CUDA(cudaMemsetAsync(res, 0, sizeof(double) * 2 * nw * nb, st));
+        mor_residual_kernel<<<dim3(cdiv(n, MT), (unsigned)(nw * nb)), MT, 0, st>>>(
+            M->S, M->W, n, m, Xw, nb, om + w0, eta, zsign, wsign, Br, res);
+        GFCC_LAUNCH_CHECK();
+      }
       GFCC_CUDA(cudaMemcpyAsync(hres.data(), res, sizeof(double) * 2 * nw * nb, cudaMemcpyDeviceToHost, st));
       GFCC_CUDA(cudaStreamSynchronize(st));
       for (int t = 0; t < nw * nb; t++)
         h_relres[(long long)w0 * nb + t] = hres[2 * t + 1] > 0.0 ? std::sqrt(hres[2 * t] / hres[2 * t + 1]) : 0.0;
+    }
+  }
+  if (planes) {
+    const int e = umma_error_check(st);
+    if (e < 0) {
+      dfree(Hm);
+      return done(e);
     }
   }
   dfree(Hm);
@@ -623,7 +738,6 @@ void gfcc_mor_destroy(gfcc_mor *M) {
   if (M == nullptr) return;
   if (M->c && M->c->stream) cudaStreamSynchronize(M->c->stream);
   dfree(M->S);
-  dfree(M->W);
   dfree(M->H);
   dfree(M->work);
   delete M;
