@@ -2,8 +2,9 @@
 // collection from kept solutions, and the gfcc_mlp_* entry points.
 //
 // All layers are small (27 -> 256 -> 256 -> 16): the model is latency-bound, so the kernels are
-// plain SIMT code: one 256-thread block per system for inference, a 32 x 32 tiled GEMM with fused
-// bias / ReLU / ReLU-mask epilogues for training.
+// plain SIMT code: one 256-thread block per system for inference; for training five launches a
+// minibatch, of 16 x 32 tiled products with fused normalisation / bias / ReLU / ReLU mask / row sums and a
+// kernel for the output layer and the loss of each sample.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -112,108 +113,213 @@ __global__ void mlp_refresh_kernel(const T *P, int nin, int nh, int nout, W *w1t
   }
 }
 
-// C[m][n] = sum_k A(m,k) B(k,n) (+ bias[n]); A(m,k) = A[m*as0 + k*as1], B(k,n) = B[k*bs0 + n*bs1].
-// mask: C = 0 where mask[m][n] <= 0 (ReLU derivative); C2: relu(C) as well.
+// One product of a training launch: C[m][n] = sum_k A(m,k) B(k,n) (+ bias[n]), A(m,k) = A[m*as0 + k*as1],
+// B(k,n) = B[k*bs0 + n*bs1]; mask: C = 0 where mask[m][n] <= 0 (ReLU derivative); relu: C = max(C, 0);
+// rowsum[m] = sum_k A(m,k) (bias gradients).
 template <typename T>
-__global__ __launch_bounds__(256) void mlp_gemm_kernel(int M, int N, int K, const T *A, long long as0, long long as1,
-                                                       const T *B, long long bs0, long long bs1, const T *bias,
-                                                       const T *mask, T *C, T *C2, long long ldc) {
-  __shared__ T As[32][33];
-  __shared__ T Bs[32][33];
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const int m0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-  T acc[4] = {T(0), T(0), T(0), T(0)};
-  for (int k0 = 0; k0 < K; k0 += 32) {
-    for (int r = ty; r < 32; r += 8) {
-      const int m = m0 + r, k = k0 + tx;
-      As[r][tx] = (m < M && k < K) ? A[(long long)m * as0 + (long long)k * as1] : T(0);
-      const int kk = k0 + r, n = n0 + tx;
-      Bs[r][tx] = (kk < K && n < N) ? B[(long long)kk * bs0 + (long long)n * bs1] : T(0);
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < 32; k++) {
-      const T b = Bs[k][tx];
-#pragma unroll
-      for (int r = 0; r < 4; r++) acc[r] += As[ty + 8 * r][k] * b;
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int r = 0; r < 4; r++) {
-    const int m = m0 + ty + 8 * r, n = n0 + tx;
-    if (m >= M || n >= N) continue;
-    T v = acc[r] + (bias ? bias[n] : T(0));
-    const long long idx = (long long)m * ldc + n;
-    if (mask && !(mask[idx] > T(0))) v = T(0);
-    C[idx] = v;
-    if (C2) C2[idx] = v > T(0) ? v : T(0);
-  }
-}
+struct MlpGemm {
+  int M = 0, N = 0, K = 0;
+  const T *A = nullptr;
+  long long as0 = 0, as1 = 0;
+  const T *B = nullptr;
+  long long bs0 = 0, bs1 = 0;
+  const T *bias = nullptr, *mask = nullptr;
+  T *C = nullptr;
+  long long ldc = 0;
+  T *rowsum = nullptr;
+  bool relu = false;
+};
 
-// db[n] = sum_m D[m][n]
+// Products of one launch, each on its range of blocks.  feat != nullptr: A of the first product is the
+// normalised features (feat[ids[m]][k] - mu[k]) / sd[k] (ids == nullptr: m), also written to Xn.
+// loss_out != nullptr: one more block adds up lossv.
 template <typename T>
-__global__ void mlp_colsum_kernel(int M, int N, const T *D, T *db) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  T s = T(0);
-  for (int m = 0; m < M; m++) s += D[(long long)m * N + n];
-  db[n] = s;
-}
+struct MlpGroup {
+  MlpGemm<T> g[3];
+  int n = 0;
+  const double *feat = nullptr;
+  const int *ids = nullptr;
+  const T *mu = nullptr, *sd = nullptr;
+  T *Xn = nullptr;
+  int nloss = 0;
+  const double *lossv = nullptr;
+  double *loss_out = nullptr;
+};
 
-// Per sample: loss = a^H Gm a / Gm_00 (a = (sum c - 1, c), c_k = y_2k + i y_2k+1) and its gradient
-// d loss / d y = 2 Re / Im ((Gm a)_0 + (Gm a)_k) / Gm_00, scaled by 1 / batch.
+constexpr int GM = 16, GN = 32;   // output tile of a block
+
+// Bound by the latency of its loads: 16 x 32 tiles give 256 x 256 outputs 128 blocks, and 128 values (64 in FP64)
+// of K a step keep 24 loads of every thread in flight while the step before is summed.  A product of 256 x 256 x 256
+// in FP32 takes 10 us from a cold cache (21 us on 32 x 32 tiles with 32 of K a step; 17 us without the loads ahead),
+// loss and gradient of 256 samples 0.13 ms (0.29 ms in fourteen launches).
 template <typename T>
-__global__ void mlp_loss_kernel(int Bn, const T *Y, const double *Gm, double inv_b, T *dY, double *lossv) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= Bn) return;
-  const double2 *G = reinterpret_cast<const double2 *>(Gm) + (long long)s * GUESS_G;
-  const T *y = Y + (long long)s * GUESS_NO;
-  T *dy = dY + (long long)s * GUESS_NO;
-  const double g00 = G[0].x;
-  if (!(g00 > 0.0)) {
-    for (int k = 0; k < GUESS_NO; k++) dy[k] = T(0);
-    lossv[s] = 0.0;
+__global__ __launch_bounds__(256) void mlp_gemm_kernel(MlpGroup<T> p) {
+  constexpr int KC = sizeof(T) == 8 ? 64 : 128;
+  __shared__ __align__(16) T As[KC][GM + 2];
+  __shared__ T Bs[KC][GN + 1];
+  const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+  int tile = blockIdx.x, gi = 0;
+  for (; gi < p.n; gi++) {
+    const int nt = ((p.g[gi].M + GM - 1) / GM) * ((p.g[gi].N + GN - 1) / GN);
+    if (tile < nt) break;
+    tile -= nt;
+  }
+  if (gi == p.n) {   // the loss block
+    __shared__ double sh[256];
+    double s = 0.0;
+    for (int i = tid; i < p.nloss; i += 256) s += p.lossv[i];
+    sh[tid] = s;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (tid < w) sh[tid] += sh[tid + w];
+      __syncthreads();
+    }
+    if (tid == 0) *p.loss_out = sh[0];
     return;
   }
-  double2 a[GUESS_K + 1];
-  a[0] = make_double2(-1.0, 0.0);
-  for (int k = 0; k < GUESS_K; k++) {
-    a[k + 1] = make_double2((double)y[2 * k], (double)y[2 * k + 1]);
-    a[0].x += a[k + 1].x;
-    a[0].y += a[k + 1].y;
-  }
-  double2 ga[GUESS_K + 1];
-  double num = 0.0;
-  for (int j = 0; j <= GUESS_K; j++) {
-    double2 t = make_double2(0.0, 0.0);
-    for (int l = 0; l <= GUESS_K; l++) {
-      const double2 g = G[j * (GUESS_K + 1) + l];
-      t.x += g.x * a[l].x - g.y * a[l].y;
-      t.y += g.x * a[l].y + g.y * a[l].x;
+  const MlpGemm<T> &g = p.g[gi];
+  const int tn = (g.N + GN - 1) / GN;
+  const int m0 = (tile / tn) * GM, n0 = (tile % tn) * GN;
+  const bool norm = gi == 0 && p.feat != nullptr, ak = norm || g.as1 == 1, bn = g.bs1 == 1;
+  T acc[2] = {T(0), T(0)}, rs = T(0);
+  constexpr int NA = GM * KC / 256, NB = KC * GN / 256;
+  T ra[NA], rb[NB];
+  auto fetch = [&](int k0) {   // one step of both operands, all loads before the first use
+#pragma unroll
+    for (int u = 0; u < NA; u++) {
+      const int t = tid + 256 * u, m = m0 + (ak ? t / KC : t % GM), k = k0 + (ak ? t % KC : t / GM);
+      ra[u] = T(0);
+      if (m < g.M && k < g.K) {
+        if (norm) {
+          const long long id = p.ids ? p.ids[m] : m;
+          ra[u] = (T)((p.feat[id * g.K + k] - (double)p.mu[k]) / (double)p.sd[k]);
+        } else {
+          ra[u] = g.A[(long long)m * g.as0 + (long long)k * g.as1];
+        }
+      }
     }
-    ga[j] = t;
-    num += a[j].x * t.x + a[j].y * t.y;
+#pragma unroll
+    for (int u = 0; u < NB; u++) {
+      const int t = tid + 256 * u, n = n0 + (bn ? t % GN : t / KC), k = k0 + (bn ? t / GN : t % KC);
+      rb[u] = (k < g.K && n < g.N) ? g.B[(long long)k * g.bs0 + (long long)n * g.bs1] : T(0);
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < g.K; k0 += KC) {
+#pragma unroll
+    for (int u = 0; u < NA; u++) {
+      const int t = tid + 256 * u, mi = ak ? t / KC : t % GM, ki = ak ? t % KC : t / GM;
+      As[ki][mi] = ra[u];
+      if (norm && n0 == 0 && m0 + mi < g.M && k0 + ki < g.K) p.Xn[(long long)(m0 + mi) * g.K + k0 + ki] = ra[u];
+    }
+#pragma unroll
+    for (int u = 0; u < NB; u++) {
+      const int t = tid + 256 * u;
+      Bs[bn ? t / GN : t % KC][bn ? t % GN : t / KC] = rb[u];
+    }
+    __syncthreads();
+    if (k0 + KC < g.K) fetch(k0 + KC);
+    const int kn = min(KC, (g.K - k0 + 15) / 16 * 16);
+#pragma unroll 16
+    for (int k = 0; k < kn; k++) {
+      const T b = Bs[k][tx];
+      acc[0] += As[k][2 * ty] * b;
+      acc[1] += As[k][2 * ty + 1] * b;
+    }
+    if (g.rowsum != nullptr && n0 == 0)   // 16 lanes a row
+      for (int k = tx & 15; k < kn; k += 16) rs += As[k][2 * ty + (tx >> 4)];
+    __syncthreads();
   }
-  lossv[s] = num / g00;
-  const double sc = 2.0 * inv_b / g00;
-  for (int k = 0; k < GUESS_K; k++) {
-    dy[2 * k] = (T)(sc * (ga[0].x + ga[k + 1].x));
-    dy[2 * k + 1] = (T)(sc * (ga[0].y + ga[k + 1].y));
+  if (g.rowsum != nullptr && n0 == 0) {
+    for (int off = 8; off > 0; off >>= 1) rs += __shfl_xor_sync(0xffffffffu, rs, off);
+    const int m = m0 + 2 * ty + (tx >> 4);
+    if ((tx & 15) == 0 && m < g.M) g.rowsum[m] = rs;
+  }
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    const int m = m0 + 2 * ty + r, n = n0 + tx;
+    if (m >= g.M || n >= g.N) continue;
+    T v = acc[r] + (g.bias ? g.bias[n] : T(0));
+    const long long idx = (long long)m * g.ldc + n;
+    if (g.mask && !(g.mask[idx] > T(0))) v = T(0);
+    if (g.relu) v = v > T(0) ? v : T(0);
+    g.C[idx] = v;
   }
 }
 
-__global__ void sum_kernel(int n, const double *x, double *out) {
-  __shared__ double sh[256];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) s += x[i];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
+// Output layer, loss and their gradients, one warp per sample:
+// y = H2 W3^T + b3; loss = a^H Gm a / Gm_00 (a = (sum c - 1, c), c_k = y_2k + i y_2k+1);
+// d loss / d y = 2 Re / Im ((Gm a)_0 + (Gm a)_k) / Gm_00, scaled by 1 / batch; dZ2 = (dY W3) * [H2 > 0].
+// Lane j < 9 forms (Gm a)_j.  One thread a sample took 29 us for 256 samples, and the two products 17 us each.
+constexpr int HEAD_WARPS = 4;
+template <typename T>
+__global__ __launch_bounds__(32 * HEAD_WARPS) void mlp_head_kernel(int Bn, int nh, const T *H2, const T *W3, const T *b3,
+                                                                   const double *Gm, const int *ids, double inv_b, T *dY,
+                                                                   T *dZ2, double *lossv) {
+  static_assert(GUESS_NO == 2 * GUESS_K && GUESS_K < 32 && GUESS_G == (GUESS_K + 1) * (GUESS_K + 1), "head layout");
+  const int lane = threadIdx.x & 31, s = blockIdx.x * HEAD_WARPS + (threadIdx.x >> 5);
+  if (s >= Bn) return;
+  const double2 *G = reinterpret_cast<const double2 *>(Gm) + (long long)(ids ? ids[s] : s) * GUESS_G;
+  constexpr int NG = GUESS_K + 1;
+  double2 g[NG];   // row `lane` of the Gram matrix
+#pragma unroll
+  for (int l = 0; l < NG; l++) g[l] = lane < NG ? G[lane * NG + l] : make_double2(0.0, 0.0);
+  const double g00 = __shfl_sync(0xffffffffu, g[0].x, 0);
+  T y[GUESS_NO];
+#pragma unroll
+  for (int o = 0; o < GUESS_NO; o++) y[o] = T(0);
+  for (int i = lane; i < nh; i += 32) {
+    const T h = H2[(long long)s * nh + i];
+#pragma unroll
+    for (int o = 0; o < GUESS_NO; o++) y[o] += W3[(long long)o * nh + i] * h;
   }
-  if (threadIdx.x == 0) *out = sh[0];
+#pragma unroll
+  for (int o = 0; o < GUESS_NO; o++) {
+    for (int off = 16; off > 0; off >>= 1) y[o] += __shfl_xor_sync(0xffffffffu, y[o], off);
+    y[o] += b3[o];
+  }
+  T dy[GUESS_NO];
+  if (!(g00 > 0.0)) {
+#pragma unroll
+    for (int o = 0; o < GUESS_NO; o++) dy[o] = T(0);
+    if (lane == 0) lossv[s] = 0.0;
+  } else {
+    double2 a[NG];
+    a[0] = make_double2(-1.0, 0.0);
+#pragma unroll
+    for (int k = 0; k < GUESS_K; k++) {
+      a[k + 1] = make_double2((double)y[2 * k], (double)y[2 * k + 1]);
+      a[0].x += a[k + 1].x;
+      a[0].y += a[k + 1].y;
+    }
+    double2 t = make_double2(0.0, 0.0), al = make_double2(0.0, 0.0);
+#pragma unroll
+    for (int l = 0; l < NG; l++) {
+      t.x += g[l].x * a[l].x - g[l].y * a[l].y;
+      t.y += g[l].x * a[l].y + g[l].y * a[l].x;
+      if (l == lane) al = a[l];
+    }
+    double num = lane < NG ? al.x * t.x + al.y * t.y : 0.0;
+    for (int off = 16; off > 0; off >>= 1) num += __shfl_xor_sync(0xffffffffu, num, off);
+    if (lane == 0) lossv[s] = num / g00;
+    const double sc = 2.0 * inv_b / g00;
+    const double t0x = __shfl_sync(0xffffffffu, t.x, 0), t0y = __shfl_sync(0xffffffffu, t.y, 0);
+#pragma unroll
+    for (int k = 0; k < GUESS_K; k++) {
+      dy[2 * k] = (T)(sc * (t0x + __shfl_sync(0xffffffffu, t.x, k + 1)));
+      dy[2 * k + 1] = (T)(sc * (t0y + __shfl_sync(0xffffffffu, t.y, k + 1)));
+    }
+  }
+#pragma unroll
+  for (int o = 0; o < GUESS_NO; o++)
+    if (lane == o) dY[(long long)s * GUESS_NO + o] = dy[o];
+  for (int i = lane; i < nh; i += 32) {
+    T v = T(0);
+#pragma unroll
+    for (int o = 0; o < GUESS_NO; o++) v += dy[o] * W3[(long long)o * nh + i];
+    const long long idx = (long long)s * nh + i;
+    dZ2[idx] = H2[idx] > T(0) ? v : T(0);
+  }
 }
 
 // Adam (Kingma & Ba 2015) on the trained prefix of the parameters.
@@ -227,25 +333,6 @@ __global__ void mlp_adam_kernel(long long n, T *P, const T *G, T *Mo, T *Vo, dou
     Mo[i] = (T)m;
     Vo[i] = (T)v;
     P[i] = (T)((double)P[i] - lr * (m / bc1) / (sqrt(v / bc2) + eps));
-  }
-}
-
-// Xn[r] = (feat[ids[r]] - mu) / sd in the training precision, Gb[r] = gram[ids[r]].
-template <typename T>
-__global__ void mlp_gather_kernel(int Bn, const int *ids, const double *feat, const double *gram, const T *P,
-                                  long long omu, long long osd, T *Xn, double *Gb) {
-  const long long per = GUESS_NF + 2 * GUESS_G;
-  const long long tot = per * Bn;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const int r = (int)(t / per);
-    const int u = (int)(t - (long long)r * per);
-    const long long id = ids[r];
-    if (u < GUESS_NF) {
-      Xn[(long long)r * GUESS_NF + u] = (T)((feat[id * GUESS_NF + u] - (double)P[omu + u]) / (double)P[osd + u]);
-    } else {
-      const int g = u - GUESS_NF;
-      Gb[(long long)r * 2 * GUESS_G + g] = gram[id * 2 * GUESS_G + g];
-    }
   }
 }
 
@@ -302,11 +389,26 @@ int ensure_ws(gfcc_mlp *m, size_t bytes) {
   return GFCC_OK;
 }
 
+// Pinned staging buffer of at least `bytes` (kept by the model, 16 MB at most); false: there is none
+bool ensure_stage(gfcc_mlp *m, size_t bytes) {
+  if (bytes > (size_t(16) << 20)) return false;
+  if (m->stage_bytes >= bytes) return true;
+  if (m->stage) cudaFreeHost(m->stage);
+  m->stage = nullptr;
+  m->stage_bytes = 0;
+  if (cudaMallocHost(reinterpret_cast<void **>(&m->stage), bytes) != cudaSuccess) {
+    cudaGetLastError();
+    m->stage = nullptr;
+    return false;
+  }
+  m->stage_bytes = bytes;
+  return true;
+}
+
 // Training workspace for a batch of Bn samples (T = training precision).
 struct TrainWs {
-  void *Xn, *Z1, *H1, *Z2, *H2, *Y, *dY, *dZ2, *dZ1;   // T arrays
-  double *Gb, *lossv, *feat, *gram, *acc;
-  int *ids;
+  void *Xn, *H1, *H2, *dY, *dZ2, *dZ1;   // T arrays
+  double *lossv, *feat, *gram, *acc;     // feat | gram: one block, as in the host staging buffer
   size_t bytes;
 };
 // base == nullptr: only the size (w.bytes) is meaningful
@@ -320,67 +422,95 @@ TrainWs train_layout(const gfcc_mlp *m, int Bn, void *base, long long nacc) {
     return r;
   };
   w.Xn = take(ts * Bn * m->nin);
-  w.Z1 = take(ts * Bn * m->nh);
   w.H1 = take(ts * Bn * m->nh);
-  w.Z2 = take(ts * Bn * m->nh);
   w.H2 = take(ts * Bn * m->nh);
-  w.Y = take(ts * Bn * m->nout);
   w.dY = take(ts * Bn * m->nout);
   w.dZ2 = take(ts * Bn * m->nh);
   w.dZ1 = take(ts * Bn * m->nh);
-  w.Gb = static_cast<double *>(take(sizeof(double) * Bn * 2 * GUESS_G));
   w.lossv = static_cast<double *>(take(sizeof(double) * Bn));
-  w.feat = static_cast<double *>(take(sizeof(double) * Bn * GUESS_NF));
-  w.gram = static_cast<double *>(take(sizeof(double) * Bn * 2 * GUESS_G));
+  w.gram = static_cast<double *>(take(sizeof(double) * Bn * (2 * GUESS_G + GUESS_NF)));
+  w.feat = base ? w.gram + (size_t)Bn * 2 * GUESS_G : nullptr;
   w.acc = static_cast<double *>(take(sizeof(double) * std::max<long long>(nacc, 1)));
-  w.ids = static_cast<int *>(take(sizeof(int) * Bn));
   w.bytes = off;
   return w;
 }
 
 template <typename T>
-int gemm(cudaStream_t st, int M, int N, int K, const T *A, long long as0, long long as1, const T *B, long long bs0,
-         long long bs1, const T *bias, const T *mask, T *C, T *C2, long long ldc) {
-  if (M <= 0 || N <= 0) return GFCC_OK;
-  mlp_gemm_kernel<T><<<dim3(cdiv(N, 32), cdiv(M, 32)), 256, 0, st>>>(M, N, K, A, as0, as1, B, bs0, bs1, bias, mask, C,
-                                                                    C2, ldc);
+int launch(cudaStream_t st, const MlpGroup<T> &p) {
+  long long blocks = p.loss_out ? 1 : 0;
+  for (int i = 0; i < p.n; i++) blocks += (long long)cdiv(p.g[i].M, GM) * cdiv(p.g[i].N, GN);
+  mlp_gemm_kernel<T><<<(unsigned)blocks, 256, 0, st>>>(p);
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
 
-// Forward (training precision) of Bn gathered samples, loss per sample, and (want_grad) the
-// gradient of the mean loss into m->Gr.
 template <typename T>
-int fwd_bwd(gfcc_mlp *m, const TrainWs &w, int Bn, bool want_grad) {
+MlpGemm<T> product(int M, int N, int K, const T *A, long long as0, long long as1, const T *B, long long bs0,
+                   long long bs1, T *C) {
+  MlpGemm<T> g;
+  g.M = M;
+  g.N = N;
+  g.K = K;
+  g.A = A;
+  g.as0 = as0;
+  g.as1 = as1;
+  g.B = B;
+  g.bs0 = bs0;
+  g.bs1 = bs1;
+  g.C = C;
+  g.ldc = N;
+  return g;
+}
+
+// Forward (training precision) of Bn samples (features and Gram matrices ids[s] of feat and gram; ids ==
+// nullptr: s), the sum of their losses into *loss_out and the gradient of the mean loss into m->Gr.
+template <typename T>
+int fwd_bwd(gfcc_mlp *m, const TrainWs &w, int Bn, const int *ids, const double *feat, const double *gram,
+            double *loss_out) {
   cudaStream_t st = m->stream;
   const Offsets o = offsets(m->nin, m->nh, m->nout);
   const int nin = m->nin, nh = m->nh, nout = m->nout;
   T *P = static_cast<T *>(m->P), *G = static_cast<T *>(m->Gr);
-  T *Xn = static_cast<T *>(w.Xn), *Z1 = static_cast<T *>(w.Z1), *H1 = static_cast<T *>(w.H1);
-  T *Z2 = static_cast<T *>(w.Z2), *H2 = static_cast<T *>(w.H2), *Y = static_cast<T *>(w.Y);
+  T *Xn = static_cast<T *>(w.Xn), *H1 = static_cast<T *>(w.H1), *H2 = static_cast<T *>(w.H2);
   T *dY = static_cast<T *>(w.dY), *dZ2 = static_cast<T *>(w.dZ2), *dZ1 = static_cast<T *>(w.dZ1);
-  // Z1 = Xn W1^T + b1, H1 = relu(Z1); Z2 = H1 W2^T + b2, H2 = relu(Z2); Y = H2 W3^T + b3
-  GFCC_TRY(gemm<T>(st, Bn, nh, nin, Xn, nin, 1, P + o.W1, 1, nin, P + o.b1, nullptr, Z1, H1, nh));
-  GFCC_TRY(gemm<T>(st, Bn, nh, nh, H1, nh, 1, P + o.W2, 1, nh, P + o.b2, nullptr, Z2, H2, nh));
-  GFCC_TRY(gemm<T>(st, Bn, nout, nh, H2, nh, 1, P + o.W3, 1, nh, P + o.b3, nullptr, Y, nullptr, nout));
-  mlp_loss_kernel<T><<<cdiv(Bn, 128), 128, 0, st>>>(Bn, Y, w.Gb, 1.0 / Bn, dY, w.lossv);
+  // H1 = relu(Xn W1^T + b1); H2 = relu(H1 W2^T + b2)
+  MlpGroup<T> l1, l2, b2, b1;
+  l1.n = 1;
+  l1.g[0] = product<T>(Bn, nh, nin, nullptr, 0, 0, P + o.W1, 1, nin, H1);
+  l1.g[0].bias = P + o.b1;
+  l1.g[0].relu = true;
+  l1.feat = feat;
+  l1.ids = ids;
+  l1.mu = P + o.mu;
+  l1.sd = P + o.sd;
+  l1.Xn = Xn;
+  GFCC_TRY(launch(st, l1));
+  l2.n = 1;
+  l2.g[0] = product<T>(Bn, nh, nh, H1, nh, 1, P + o.W2, 1, nh, H2);
+  l2.g[0].bias = P + o.b2;
+  l2.g[0].relu = true;
+  GFCC_TRY(launch(st, l2));
+  // Y = H2 W3^T + b3, losses, dY, dZ2 = (dY W3) * [Z2 > 0]
+  mlp_head_kernel<T><<<cdiv(Bn, HEAD_WARPS), 32 * HEAD_WARPS, 0, st>>>(Bn, nh, H2, P + o.W3, P + o.b3, gram, ids,
+                                                                      1.0 / Bn, dY, dZ2, w.lossv);
   GFCC_LAUNCH_CHECK();
-  if (!want_grad) return GFCC_OK;
-  // dW3 = dY^T H2, db3 = colsum dY; dZ2 = (dY W3) * [Z2 > 0]
-  GFCC_TRY(gemm<T>(st, nout, nh, Bn, dY, 1, nout, H2, nh, 1, nullptr, nullptr, G + o.W3, nullptr, nh));
-  mlp_colsum_kernel<T><<<cdiv(nout, 128), 128, 0, st>>>(Bn, nout, dY, G + o.b3);
-  GFCC_LAUNCH_CHECK();
-  GFCC_TRY(gemm<T>(st, Bn, nh, nout, dY, nout, 1, P + o.W3, nh, 1, nullptr, Z2, dZ2, nullptr, nh));
-  // dW2 = dZ2^T H1, db2 = colsum dZ2; dZ1 = (dZ2 W2) * [Z1 > 0]
-  GFCC_TRY(gemm<T>(st, nh, nh, Bn, dZ2, 1, nh, H1, nh, 1, nullptr, nullptr, G + o.W2, nullptr, nh));
-  mlp_colsum_kernel<T><<<cdiv(nh, 128), 128, 0, st>>>(Bn, nh, dZ2, G + o.b2);
-  GFCC_LAUNCH_CHECK();
-  GFCC_TRY(gemm<T>(st, Bn, nh, nh, dZ2, nh, 1, P + o.W2, nh, 1, nullptr, Z1, dZ1, nullptr, nh));
-  // dW1 = dZ1^T Xn, db1 = colsum dZ1
-  GFCC_TRY(gemm<T>(st, nh, nin, Bn, dZ1, 1, nh, Xn, nin, 1, nullptr, nullptr, G + o.W1, nullptr, nin));
-  mlp_colsum_kernel<T><<<cdiv(nh, 128), 128, 0, st>>>(Bn, nh, dZ1, G + o.b1);
-  GFCC_LAUNCH_CHECK();
-  return GFCC_OK;
+  // dZ1 = (dZ2 W2) * [Z1 > 0]; dW2 = dZ2^T H1, db2 = colsum dZ2; dW3 = dY^T H2, db3 = colsum dY
+  b2.n = 3;
+  b2.g[0] = product<T>(nh, nh, Bn, dZ2, 1, nh, H1, nh, 1, G + o.W2);
+  b2.g[0].rowsum = G + o.b2;
+  b2.g[1] = product<T>(Bn, nh, nh, dZ2, nh, 1, P + o.W2, nh, 1, dZ1);
+  b2.g[1].mask = H1;
+  b2.g[2] = product<T>(nout, nh, Bn, dY, 1, nout, H2, nh, 1, G + o.W3);
+  b2.g[2].rowsum = G + o.b3;
+  GFCC_TRY(launch(st, b2));
+  // dW1 = dZ1^T Xn, db1 = colsum dZ1; the sum of the losses
+  b1.n = 1;
+  b1.g[0] = product<T>(nh, nin, Bn, dZ1, 1, nh, Xn, nin, 1, G + o.W1);
+  b1.g[0].rowsum = G + o.b1;
+  b1.nloss = Bn;
+  b1.lossv = w.lossv;
+  b1.loss_out = loss_out;
+  return launch(st, b1);
 }
 
 int refresh(gfcc_mlp *m) {
@@ -429,15 +559,6 @@ int array_to_host(const gfcc_mlp *m, const void *d, long long count, double *h) 
     GFCC_CUDA(cudaStreamSynchronize(m->stream));
     for (long long i = 0; i < count; i++) h[i] = f[i];
   }
-  return GFCC_OK;
-}
-
-template <typename T>
-int gather(gfcc_mlp *m, const TrainWs &w, int Bn, const int *ids, const double *feat, const double *gram) {
-  const Offsets o = offsets(m->nin, m->nh, m->nout);
-  mlp_gather_kernel<T><<<grid1d((long long)Bn * (GUESS_NF + 2 * GUESS_G)), 256, 0, m->stream>>>(
-      Bn, ids, feat, gram, static_cast<const T *>(m->P), o.mu, o.sd, static_cast<T *>(w.Xn), w.Gb);
-  GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
 
@@ -588,6 +709,7 @@ void gfcc_mlp_destroy(gfcc_mlp *m) {
   if (m->stream) cudaStreamSynchronize(m->stream);
   for (void *p : {m->P, m->Mo, m->Vo, m->Gr, m->Pinf, m->ws, static_cast<void *>(m->feat), static_cast<void *>(m->gram)})
     if (p) dfree(p);
+  if (m->stage) cudaFreeHost(m->stage);
   if (m->stream) cudaStreamDestroy(m->stream);
   delete m;
 }
@@ -653,22 +775,41 @@ static int host_batch_step(gfcc_mlp *m, int nb, const double *features, const do
   const size_t need = train_layout(m, nb, nullptr, 1).bytes + 256;
   GFCC_TRY(ensure_ws(m, need));
   const TrainWs w = train_layout(m, nb, m->ws, 1);
-  std::vector<int> ids(nb);
-  for (int i = 0; i < nb; i++) ids[i] = i;
-  GFCC_CUDA(cudaMemcpyAsync(w.feat, features, sizeof(double) * nb * GUESS_NF, cudaMemcpyHostToDevice, m->stream));
-  GFCC_CUDA(cudaMemcpyAsync(w.gram, gram, sizeof(double) * nb * 2 * GUESS_G, cudaMemcpyHostToDevice, m->stream));
-  GFCC_CUDA(cudaMemcpyAsync(w.ids, ids.data(), sizeof(int) * nb, cudaMemcpyHostToDevice, m->stream));
   const bool f64 = m->precision == GFCC_MLP_FP64;
-  GFCC_TRY(f64 ? gather<double>(m, w, nb, w.ids, w.feat, w.gram) : gather<float>(m, w, nb, w.ids, w.feat, w.gram));
-  GFCC_TRY(f64 ? fwd_bwd<double>(m, w, nb, true) : fwd_bwd<float>(m, w, nb, true));
-  sum_kernel<<<1, 256, 0, m->stream>>>(nb, w.lossv, w.acc);
-  GFCC_LAUNCH_CHECK();
-  double tot = 0.0;
-  GFCC_CUDA(cudaMemcpyAsync(&tot, w.acc, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
-  if (grad) {
-    GFCC_TRY(array_to_host(m, m->Gr, m->ntrain, grad));
-    for (long long i = m->ntrain; i < m->nparam; i++) grad[i] = 0.0;
+  // One copy each way through pinned memory (bounded; larger batches copy from the caller's arrays): pageable copies
+  // of 0.4 MB in and 0.3 MB out took a third of the call.
+  const size_t fb = sizeof(double) * nb * GUESS_NF, gb = sizeof(double) * nb * 2 * GUESS_G;
+  const size_t rb = (tsize(m) * m->ntrain + 15) & ~size_t(15);   // gradient, then the loss in its untrained tail
+  const bool staged = ensure_stage(m, std::max(fb + gb, rb + sizeof(double)));
+  if (staged) {
+    std::memcpy(m->stage, gram, gb);
+    std::memcpy(m->stage + gb, features, fb);
+    GFCC_CUDA(cudaMemcpyAsync(w.gram, m->stage, gb + fb, cudaMemcpyHostToDevice, m->stream));
+  } else {
+    GFCC_CUDA(cudaMemcpyAsync(w.gram, gram, gb, cudaMemcpyHostToDevice, m->stream));
+    GFCC_CUDA(cudaMemcpyAsync(w.feat, features, fb, cudaMemcpyHostToDevice, m->stream));
   }
+  double *loss_out = reinterpret_cast<double *>(static_cast<char *>(m->Gr) + rb);
+  static_assert(2 * GUESS_NF * sizeof(float) >= 16 + sizeof(double), "the loss fits the gradient's tail");
+  GFCC_TRY(f64 ? fwd_bwd<double>(m, w, nb, nullptr, w.feat, w.gram, loss_out)
+               : fwd_bwd<float>(m, w, nb, nullptr, w.feat, w.gram, loss_out));
+  double tot = 0.0;
+  if (grad && staged) {
+    GFCC_CUDA(cudaMemcpyAsync(m->stage, m->Gr, rb + sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+    GFCC_CUDA(cudaStreamSynchronize(m->stream));
+    std::memcpy(&tot, m->stage + rb, sizeof(double));
+    if (f64) {
+      std::memcpy(grad, m->stage, sizeof(double) * m->ntrain);
+    } else {
+      const float *f = reinterpret_cast<const float *>(m->stage);
+      for (long long i = 0; i < m->ntrain; i++) grad[i] = f[i];
+    }
+  } else {
+    GFCC_CUDA(cudaMemcpyAsync(&tot, loss_out, sizeof(double), cudaMemcpyDeviceToHost, m->stream));
+    if (grad) GFCC_TRY(array_to_host(m, m->Gr, m->ntrain, grad));
+  }
+  if (grad)
+    for (long long i = m->ntrain; i < m->nparam; i++) grad[i] = 0.0;
   if (lr > 0.0) {
     GFCC_TRY(f64 ? adam<double>(m, lr) : adam<float>(m, lr));
     GFCC_TRY(refresh(m));
@@ -722,11 +863,8 @@ int gfcc_mlp_train(gfcc_mlp *m, int steps, int minibatch, double lr, unsigned lo
   GFCC_CUDA(cudaMemcpyAsync(d_ids, ids.data(), sizeof(int) * ids.size(), cudaMemcpyHostToDevice, m->stream));
   for (int s = 0; s < steps; s++) {
     const int *sid = d_ids + (size_t)s * minibatch;
-    GFCC_TRY(f64 ? gather<double>(m, w, minibatch, sid, m->feat, m->gram)
-                 : gather<float>(m, w, minibatch, sid, m->feat, m->gram));
-    GFCC_TRY(f64 ? fwd_bwd<double>(m, w, minibatch, true) : fwd_bwd<float>(m, w, minibatch, true));
-    sum_kernel<<<1, 256, 0, m->stream>>>(minibatch, w.lossv, w.acc + s);
-    GFCC_LAUNCH_CHECK();
+    GFCC_TRY(f64 ? fwd_bwd<double>(m, w, minibatch, sid, m->feat, m->gram, w.acc + s)
+                 : fwd_bwd<float>(m, w, minibatch, sid, m->feat, m->gram, w.acc + s));
     GFCC_TRY(f64 ? adam<double>(m, lr) : adam<float>(m, lr));
   }
   GFCC_TRY(refresh(m));

@@ -20,6 +20,8 @@ struct gfcc_mlp {
   long long ns = 0, cap = 0;
   void *ws = nullptr;     // training / inference workspace
   size_t ws_bytes = 0;
+  char *stage = nullptr;  // pinned staging of a host minibatch and its gradient
+  size_t stage_bytes = 0;
   cudaStream_t stream = nullptr;
 };
 
