@@ -175,42 +175,6 @@ __global__ void vupdate_kernel(const T *V, long long vs_stride, long long vi_str
   }
 }
 
-// w_s *= 1 / scale[s] (real scale stored as the real part of a complex entry scale[s*NV + idx]).
-// Grid (cdiv(n, VSCALE_PER_BLOCK), nsys): the factor is formed once per block (a root and a division in
-// FP64 per thread held this kernel to a quarter of the memory rate: 54 us for 100 MB); each thread scales
-// VSCALE_UNROLL elements with independent loads.
-constexpr int VSCALE_UNROLL = 8, VSCALE_PER_BLOCK = 256 * VSCALE_UNROLL;
-template <typename T>
-__global__ __launch_bounds__(256) void vscale_kernel(T *w, long long ws_stride, long long n, const double *nrm2, int NV,
-                                                     int idx, const int *state, int want) {
-  __shared__ T factor;
-  const int s = blockIdx.y;
-  if (state != nullptr && state[s] != want) return;
-  const double nn = nrm2[2 * ((long long)s * NV + idx)];
-  if (!(nn > 0.0)) return;
-  T *ws = w + 2 * s * ws_stride;
-  const long long t0 = (long long)blockIdx.x * VSCALE_PER_BLOCK + threadIdx.x;
-  CT<T> x[VSCALE_UNROLL];
-#pragma unroll
-  for (int u = 0; u < VSCALE_UNROLL; u++) {
-    const long long t = t0 + (long long)u * 256;
-    x[u] = t < n ? ldc(ws, t) : mkc<T>(0.0, 0.0);
-  }
-  if (threadIdx.x == 0) factor = (T)(1.0 / sqrt(nn));
-  __syncthreads();
-  const T inv = factor;
-#pragma unroll
-  for (int u = 0; u < VSCALE_UNROLL; u++) {
-    const long long t = t0 + (long long)u * 256;
-    x[u].x *= inv;
-    x[u].y *= inv;
-    if (t < n) stc(ws, t, x[u]);
-  }
-}
-static inline dim3 vscale_grid(long long n, int nsys) {
-  return dim3((unsigned)std::max<long long>(1, (n + VSCALE_PER_BLOCK - 1) / VSCALE_PER_BLOCK), (unsigned)nsys);
-}
-
 // r_s = b_s - w_s for systems that are not finished
 template <typename T>
 __global__ void resid_form_kernel(const T *B, const T *W, T *R, long long r_stride, long long n, int nsys,
@@ -282,9 +246,27 @@ __device__ void givens_update(const Lsq &q, int s, int k, const double *h, int N
   }
   __syncthreads();
   if (t == 0) {
+    const double2 gk = gs[k];
+    const double bn = q.bnorm[s];
+    const int it = q.iters[s];
     double2 a = hh[0];
     aa[0] = a;
-    for (int i = 0; i < k; i++) {
+    int i = 0;
+    for (; i + 8 <= k; i += 8) {   // the operands of eight steps ahead of their chain
+      double2 pv[8];
+      double sv[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        pv[u] = pq[i + u];
+        sv[u] = ss[i + u];
+      }
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        a = make_double2(pv[u].x - sv[u] * a.x, pv[u].y - sv[u] * a.y);
+        aa[i + u + 1] = a;
+      }
+    }
+    for (; i < k; i++) {
       a = make_double2(pq[i].x - ss[i] * a.x, pq[i].y - ss[i] * a.y);
       aa[i + 1] = a;
     }
@@ -300,13 +282,12 @@ __device__ void givens_update(const Lsq &q, int s, int k, const double *h, int N
     }
     css[k] = c;
     sns[k] = sv;
-    const double2 gk = gs[k];
     const double2 g1 = make_double2(-sv.x * gk.x, -sv.x * gk.y);                              // -s g_k
     gs[k + 1] = g1;
     gs[k] = make_double2(c.x * gk.x - c.y * gk.y, c.x * gk.y + c.y * gk.x);                   // c g_k
     Hk[k] = make_double2(den, 0.0);
-    q.iters[s] += 1;
-    const double bn = q.bnorm[s], res = sqrt(g1.x * g1.x + g1.y * g1.y);
+    q.iters[s] = it + 1;
+    const double res = sqrt(g1.x * g1.x + g1.y * g1.y);
     q.est[s] = bn > 0.0 ? res / bn : 0.0;
     const bool breakdown = !(hk1 > 1e-14 * den);
     if (res <= q.tol * bn || breakdown || k + 1 == m || den == 0.0) {
@@ -319,6 +300,48 @@ __device__ void givens_update(const Lsq &q, int s, int k, const double *h, int N
     const double2 c = cc[t], a = aa[t], b = hh[t + 1];
     Hk[t] = make_double2(c.x * a.x - c.y * a.y + ss[t] * b.x, c.x * a.y + c.y * a.x + ss[t] * b.y);
   }
+}
+
+// w_s *= 1 / scale[s] (real scale stored as the real part of a complex entry scale[s*NV + idx]).
+// Grid (cdiv(n, VSCALE_PER_BLOCK), nsys): the factor is formed once per block (a root and a division in
+// FP64 per thread held this kernel to a quarter of the memory rate: 54 us for 100 MB); each thread scales
+// VSCALE_UNROLL elements with independent loads.
+constexpr int VSCALE_UNROLL = 8, VSCALE_PER_BLOCK = 256 * VSCALE_UNROLL;
+// GIVENS: one more block per system makes the Givens update of column idx - 1 meanwhile (a system that it takes
+// out of its cycle may or may not be scaled; the vector is not used again).
+template <typename T, bool GIVENS>
+__global__ __launch_bounds__(256) void vscale_kernel(T *w, long long ws_stride, long long n, const double *nrm2, int NV,
+                                                     int idx, const int *state, int want, Lsq q) {
+  __shared__ T factor;
+  const int s = blockIdx.y;
+  if (state != nullptr && state[s] != want) return;
+  if (GIVENS && blockIdx.x == gridDim.x - 1) {
+    givens_update(q, s, idx - 1, nrm2, NV);
+    return;
+  }
+  const double nn = nrm2[2 * ((long long)s * NV + idx)];
+  if (!(nn > 0.0)) return;
+  T *ws = w + 2 * s * ws_stride;
+  const long long t0 = (long long)blockIdx.x * VSCALE_PER_BLOCK + threadIdx.x;
+  CT<T> x[VSCALE_UNROLL];
+#pragma unroll
+  for (int u = 0; u < VSCALE_UNROLL; u++) {
+    const long long t = t0 + (long long)u * 256;
+    x[u] = t < n ? ldc(ws, t) : mkc<T>(0.0, 0.0);
+  }
+  if (threadIdx.x == 0) factor = (T)(1.0 / sqrt(nn));
+  __syncthreads();
+  const T inv = factor;
+#pragma unroll
+  for (int u = 0; u < VSCALE_UNROLL; u++) {
+    const long long t = t0 + (long long)u * 256;
+    x[u].x *= inv;
+    x[u].y *= inv;
+    if (t < n) stc(ws, t, x[u]);
+  }
+}
+static inline dim3 vscale_grid(long long n, int nsys) {
+  return dim3((unsigned)std::max<long long>(1, (n + VSCALE_PER_BLOCK - 1) / VSCALE_PER_BLOCK), (unsigned)nsys);
 }
 
 // y = R^-1 g (back substitution on the rotated Hessenberg), stored in y[s*NV + i]; one warp per system: lane l
@@ -371,18 +394,27 @@ __global__ __launch_bounds__(32) void backsolve_kernel(int m, const double *H, c
 
 // ---------------------------------------------------------------- fused Gram-Schmidt passes
 // Both passes stream the Krylov basis of a system once per chunk of elements.  They are
-// HBM-bound, so what matters is the number of independent loads in flight:
-// * dots: each warp of a block owns whole basis vectors (i = warp, warp + 8, ...; i = nv is w
-//   itself, for ||w||^2) and sweeps the chunk with CGS_UNROLL independent loads per lane; w is
-//   re-read by every warp from L1.  No block-level reduction: one warp shuffle per vector.
+// HBM-bound, so what matters is the number of independent loads in flight, and that the blocks make one wave:
+// * dots: each warp of a block owns whole basis vectors (i = warp, warp + 4, ...; i = nv is w
+//   itself, for ||w||^2; of fewer vectors than warps, parts of the chunk) and sweeps the chunk with 8 or 16
+//   independent loads per lane that pass L1 by; w is re-read by every warp from L1.  No block-level reduction: one
+//   warp shuffle per vector.
 // * update: every thread owns two elements and accumulates sum_i c_i V_i over batches of
 //   CGS_BATCH vectors whose loads are predicated (not branched), so they issue together.
-// The chunk length follows the number of systems in cycle, so that a few systems fill the chip too
-// (256 elements at least).  The last block of a system adds up its chunks' partial sums in chunk order and takes
-// what follows from them: coefficients, the test for a second pass, the Givens update.  With a kernel
-// for each of these (twelve launches a step) a step of the 30 systems of o=27 v=133 took 208 us beside
-// 30 us of least squares; now 5 launches.
-constexpr int CGS_THREADS = 256, CGS_MIN_CHUNK = 256, CGS_MAX_CHUNK = 4096, CGS_BLOCKS = 1200, CGS_UNROLL = 8, CGS_BATCH = 8;
+// The chunk length follows the number of systems in cycle, so that their blocks are as many as the chip holds at
+// once.  The last block of a system adds up its chunks' partial sums in chunk order and takes
+// what follows from them: coefficients, the test for a second pass.  The Givens update runs beside the scaling of the
+// new vector.
+// At 30 systems of o=27 v=133 (n = 46710, FP32) and 51 vectors the dots take 77 us and the update 57 us (3.9 and
+// 5.3 TB/s of basis read from HBM, the rest from L2); blocks of eight warps, 1.13 and 1.46 waves of them, and w read
+// from L1 between the basis loads took 107 and 78 us.
+constexpr int CGS_THREADS = 256, CGS_MIN_CHUNK = 256, CGS_BATCH = 8;
+constexpr int DOT_WARPS = 4, DOT_RUN = 4096;   // FP32 sums of at most DOT_RUN / 32 terms, then FP64
+template <typename T>
+struct CgsShape {   // blocks per SM (by registers), elements a round of the dots
+  static constexpr bool F32 = sizeof(T) == sizeof(float);
+  static constexpr int DOT_UNROLL = 8, DOT_PER_SM = 8, UPD_PER_SM = 4;
+};
 constexpr double REORTH_THETA_F32 = 0.01;   // FP32 Krylov vectors: second pass where ||w'|| < 0.1 ||w||
 
 // true in the block of system s that finishes last (counter left at zero for the next kernel)
@@ -399,87 +431,120 @@ __device__ __forceinline__ bool last_block(unsigned *cnt, int s) {
   return last != 0;
 }
 
+__device__ __forceinline__ float2 ldc_stream(const float *p, long long i) {
+  return __ldcg(reinterpret_cast<const float2 *>(p) + i);
+}
+__device__ __forceinline__ double2 ldc_stream(const double *p, long long i) {
+  return __ldcg(reinterpret_cast<const double2 *>(p) + i);
+}
+
+// sum over U rounds of 32 elements from e (this lane's) below e1
+template <typename T, int U, bool TAIL>
+__device__ __forceinline__ void dot_round(const T *vp, const T *ws, long long e, long long e1, T &ar, T &ai) {
+  CT<T> a[U];
+#pragma unroll
+  for (int u = 0; u < U; u++) a[u] = !TAIL || e + 32 * u < e1 ? ldc_stream(vp, e + 32 * u) : mkc<T>(0.0, 0.0);
+#pragma unroll
+  for (int u = 0; u < U; u++) {
+    const CT<T> x = !TAIL || e + 32 * u < e1 ? ldc(ws, e + 32 * u) : mkc<T>(0.0, 0.0);
+    ar += a[u].x * x.x + a[u].y * x.y;
+    ai += a[u].x * x.y - a[u].y * x.x;
+  }
+}
+
 // out[s*NV + i] = <V_i, w> for i < nv, ||w||^2 for i = nv, for the systems in cycle (second pass: of those, the
 // flagged ones).  grid (chunks of `clen` elements, systems)
 template <typename T>
-__global__ __launch_bounds__(CGS_THREADS) void cgs_dots_kernel(const T *V, long long vs, long long vi, int nv,
-                                                               const T *w, long long n, int clen, const int *state,
-                                                               const int *flag, double *partial, int NV, double *out,
-                                                               unsigned *cnt) {
+__global__ __launch_bounds__(32 * DOT_WARPS, CgsShape<T>::DOT_PER_SM) void cgs_dots_kernel(
+    const T *V, long long vs, long long vi, int nv, const T *w, long long n, int clen, const int *state, const int *flag,
+    double *partial, int NV, double *out, unsigned *cnt) {
+  constexpr int U = CgsShape<T>::DOT_UNROLL;
+  __shared__ double2 parts[DOT_WARPS];
   const int s = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
   if (state[s] != ST_IN_CYCLE || (flag != nullptr && !flag[s])) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long e0 = (long long)chunk * clen;
-  const long long e1 = e0 + clen < n ? e0 + clen : n;
   const T *ws = w + 2 * s * vs;
   const T *Vs = V + 2 * s * vs;
   double2 *ps = reinterpret_cast<double2 *>(partial) + (long long)s * NV * nch;
-  for (int i = warp; i <= nv; i += CGS_THREADS / 32) {
+  // fewer FP32 vectors than warps: `split` warps a vector, each on its part of the chunk (FP64 Krylov vectors are
+  // those of small systems, where a chunk is one round)
+  const int split = CgsShape<T>::F32 && nv + 1 < DOT_WARPS ? DOT_WARPS / (nv + 1) : 1;
+  const int plen = split == 1 ? clen : (clen / split + 31) / 32 * 32;
+  const long long c1 = min((long long)(chunk + 1) * clen, n);
+  const long long e0 = (long long)chunk * clen + (warp % split) * plen;
+  const long long e1 = min(e0 + plen, c1);
+  for (int i = warp / split; i <= nv; i += DOT_WARPS / split) {
     const T *vp = i < nv ? Vs + 2 * i * vi : ws;   // slot nv: ||w||^2
-    T ar = T(0), ai = T(0);
-    long long e = e0 + lane;
-    // full rounds: CGS_UNROLL unconditional loads of the basis vector and of w in flight per lane
-    for (; e + 32 * (CGS_UNROLL - 1) < e1; e += 32 * CGS_UNROLL) {
-      CT<T> a[CGS_UNROLL], x[CGS_UNROLL];
-#pragma unroll
-      for (int u = 0; u < CGS_UNROLL; u++) {
-        a[u] = ldc(vp, e + 32 * u);
-        x[u] = ldc(ws, e + 32 * u);
-      }
-#pragma unroll
-      for (int u = 0; u < CGS_UNROLL; u++) {
-        ar += a[u].x * x[u].x + a[u].y * x[u].y;
-        ai += a[u].x * x[u].y - a[u].y * x[u].x;
-      }
+    double2 acc = make_double2(0.0, 0.0);
+    for (long long r0 = e0; r0 < e1; r0 += DOT_RUN) {
+      const long long r1 = min(r0 + DOT_RUN, e1);
+      T ar = T(0), ai = T(0);
+      long long e = r0 + lane;
+      if (CgsShape<T>::F32)
+        for (; e + 32 * (2 * U - 1) < r1; e += 32 * 2 * U) dot_round<T, 2 * U, false>(vp, ws, e, r1, ar, ai);
+      for (; e + 32 * (U - 1) < r1; e += 32 * U) dot_round<T, U, false>(vp, ws, e, r1, ar, ai);
+      if (e < r1) dot_round<T, U, true>(vp, ws, e, r1, ar, ai);
+      acc.x += (double)ar;
+      acc.y += (double)ai;
     }
-    for (; e < e1; e += 32) {
-      const CT<T> a = ldc(vp, e), x = ldc(ws, e);
-      ar += a.x * x.x + a.y * x.y;
-      ai += a.x * x.y - a.y * x.x;
-    }
-    double2 acc = make_double2((double)ar, (double)ai);
     for (int off = 16; off > 0; off >>= 1) {
       acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
       acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
     }
-    if (lane == 0) ps[(long long)i * nch + chunk] = acc;
+    if (lane == 0) {
+      if (split == 1)
+        ps[(long long)i * nch + chunk] = acc;
+      else
+        parts[warp] = acc;
+    }
+    if (split > 1) break;   // one vector a warp
+  }
+  if (split > 1) {
+    __syncthreads();
+    if (threadIdx.x <= nv) {
+      double2 acc = parts[threadIdx.x * split];
+      for (int p = 1; p < split; p++) {
+        acc.x += parts[threadIdx.x * split + p].x;
+        acc.y += parts[threadIdx.x * split + p].y;
+      }
+      ps[(long long)threadIdx.x * nch + chunk] = acc;
+    }
   }
   if (!last_block(cnt, s)) return;
-  for (int i = warp; i <= nv; i += CGS_THREADS / 32) {
+  // four lanes a vector, eight loads of each in flight
+  for (int i0 = 0; i0 <= nv; i0 += 8 * DOT_WARPS) {
+    const int i = i0 + threadIdx.x / 4;
     double2 acc = make_double2(0.0, 0.0);
-    for (int c = lane; c < nch; c += 32) {
-      const double2 x = __ldcg(&ps[(long long)i * nch + c]);
-      acc.x += x.x;
-      acc.y += x.y;
+    if (i <= nv) {
+#pragma unroll 8
+      for (int c = threadIdx.x & 3; c < nch; c += 4) {
+        const double2 x = __ldcg(&ps[(long long)i * nch + c]);
+        acc.x += x.x;
+        acc.y += x.y;
+      }
     }
-    for (int off = 16; off > 0; off >>= 1) {
+    for (int off = 2; off > 0; off >>= 1) {
       acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
       acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
     }
-    if (lane == 0) reinterpret_cast<double2 *>(out)[(long long)s * NV + i] = acc;
+    if (i <= nv && (threadIdx.x & 3) == 0) reinterpret_cast<double2 *>(out)[(long long)s * NV + i] = acc;
   }
 }
 
 // w -= V coef (in place) and the squared norm of w.
 // First pass (SECOND false): sets flag[s] where the pass cancelled so much of w that it needs the second one
 // (Daniel, Gragg, Kaufman & Stewart 1976: ||w'||^2 < theta ||w||^2), else h[nv] = ||w'||^2.
-// Second pass: over the flagged systems, h += h2 and h[nv] = ||w''||^2.  Its last block (of a system that is
-// not flagged, its first) makes the Givens update of column nv - 1.
+// Second pass: over the flagged systems, h += h2 and h[nv] = ||w''||^2.
 template <typename T, bool SECOND>
-__global__ __launch_bounds__(CGS_THREADS) void cgs_update_kernel(const T *V, long long vs, long long vi, int nv, T *w,
+__global__ __launch_bounds__(CGS_THREADS, CgsShape<T>::UPD_PER_SM) void cgs_update_kernel(const T *V, long long vs, long long vi, int nv, T *w,
                                                                  long long n, int clen, int *flag, double *h,
                                                                  const double *h2, double theta, double *partial,
-                                                                 int NV, unsigned *cnt, Lsq q) {
+                                                                 int NV, unsigned *cnt, const int *state) {
   __shared__ CT<T> hh[72];
   __shared__ double sh[CGS_THREADS / 32];
   const int s = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
-  if (q.state[s] != ST_IN_CYCLE) return;
+  if (state[s] != ST_IN_CYCLE || (SECOND && !flag[s])) return;
   double2 *hs = reinterpret_cast<double2 *>(h) + (long long)s * NV;
-  if (SECOND && !flag[s]) {
-    // the other blocks of the system may still read state[s]; both outcomes are a return
-    if (chunk == 0) givens_update(q, s, nv - 1, h, NV);
-    return;
-  }
   const double2 *cf = SECOND ? reinterpret_cast<const double2 *>(h2) + (long long)s * NV : hs;
   for (int i = threadIdx.x; i < nv; i += CGS_THREADS) {
     const double2 c = cf[i];
@@ -596,8 +661,6 @@ __global__ __launch_bounds__(CGS_THREADS) void cgs_update_kernel(const T *V, lon
     hs[i].x += h2s[i].x;
     hs[i].y += h2s[i].y;
   }
-  __syncthreads();
-  givens_update(q, s, nv - 1, h, NV);
 }
 
 __global__ void set_state_kernel(int nsys, int *state, int from, int to) {
@@ -660,10 +723,11 @@ long long dbl_of(long long count) {
 }
 }  // namespace
 
-// chunks of partial sums per system: the norms' chunks, or enough for CGS_BLOCKS blocks from few systems
+// chunks of partial sums per system: the norms' chunks, or enough to fill the chip from few systems (all of them,
+// or the last few in cycle)
 static long long partial_chunks_per_system(long long n, int nsys) {
   const long long fine = (n + CGS_MIN_CHUNK - 1) / CGS_MIN_CHUNK;
-  return std::max((n + DOT_CHUNK - 1) / DOT_CHUNK, std::min<long long>(fine, CGS_BLOCKS / std::max(1, nsys) + 1));
+  return std::max((n + DOT_CHUNK - 1) / DOT_CHUNK, std::min<long long>(fine, std::max(256, 152 * 8 / std::max(1, nsys) + 1)));
 }
 
 long long gmres_work_doubles(const gfcc_ctx *c, int sector, long long n, int nsys, int m, bool mixed) {
@@ -837,12 +901,17 @@ int Gmres::mdot(const double *Vb, long long vs, long long vi, int nv, const doub
 template <typename T>
 int Gmres::arnoldi_t(const T *Vb, long long vs, int k, T *w, int active, double tol, cudaStream_t st) {
   const int nv = k + 1;
-  // chunks: enough blocks for the systems in cycle, within the partial sums' room
+  // chunks: the blocks of the systems in cycle fill the chip once, within the partial sums' room
   const long long cap = std::max<long long>(1, partial_chunks / nsys);
-  long long nchc = std::min<long long>(cap, std::max(1, CGS_BLOCKS / std::max(1, active)));
-  nchc = std::max(nchc, (n + CGS_MAX_CHUNK - 1) / CGS_MAX_CHUNK);
-  int clen = (int)(((n + nchc - 1) / nchc + CGS_MIN_CHUNK - 1) / CGS_MIN_CHUNK * CGS_MIN_CHUNK);
-  dim3 grid((unsigned)((n + clen - 1) / clen), (unsigned)nsys);
+  auto chunk = [&](int per_sm, int step) {
+    const long long c = std::min<long long>(cap, std::max(1, 152 * per_sm / std::max(1, active)));
+    return (int)(((n + c - 1) / c + step - 1) / step * step);
+  };
+  using Shape = CgsShape<T>;
+  const int dlen = chunk(Shape::DOT_PER_SM, 32 * Shape::DOT_UNROLL);
+  int ulen = chunk(Shape::UPD_PER_SM, CGS_THREADS);
+  if (ulen > CGS_THREADS) ulen = (ulen + 2 * CGS_THREADS - 1) / (2 * CGS_THREADS) * (2 * CGS_THREADS);
+  const dim3 dgrid((unsigned)((n + dlen - 1) / dlen), (unsigned)nsys), ugrid((unsigned)((n + ulen - 1) / ulen), (unsigned)nsys);
   // The orthogonality lost by the new vector is about the relative rounding error of the pass times
   // ||w|| / ||w'||: FP64 solves take the second pass below 1/sqrt(2) (the usual twice-is-enough test);
   // the FP32 inner solves of the refinement, which stop at a relative residual of 3e-4 and are
@@ -850,17 +919,19 @@ int Gmres::arnoldi_t(const T *Vb, long long vs, int k, T *w, int active, double 
   // (orthogonality loss <= 10 x about 1e-6 per vector).
   const double theta = sizeof(T) == sizeof(float) ? REORTH_THETA_F32 : 0.5;
   const Lsq q{m, H, cs, sn, g, bnorm, tol, state, kcyc, iters, est};
-  cgs_dots_kernel<T><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, state, nullptr, partial, NV, h, blk_cnt);
+  cgs_dots_kernel<T><<<dgrid, 32 * DOT_WARPS, 0, st>>>(Vb, vs, n, nv, w, n, dlen, state, nullptr, partial, NV, h, blk_cnt);
   GFCC_LAUNCH_CHECK();
-  cgs_update_kernel<T, false><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, rflag, h, nullptr, theta, partial,
-                                                            NV, blk_cnt, q);
+  cgs_update_kernel<T, false><<<ugrid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, ulen, rflag, h, nullptr, theta, partial,
+                                                             NV, blk_cnt, state);
   GFCC_LAUNCH_CHECK();
-  cgs_dots_kernel<T><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, state, rflag, partial, NV, h2, blk_cnt);
+  cgs_dots_kernel<T><<<dgrid, 32 * DOT_WARPS, 0, st>>>(Vb, vs, n, nv, w, n, dlen, state, rflag, partial, NV, h2, blk_cnt);
   GFCC_LAUNCH_CHECK();
-  cgs_update_kernel<T, true><<<grid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, clen, rflag, h, h2, theta, partial, NV,
-                                                           blk_cnt, q);
+  cgs_update_kernel<T, true><<<ugrid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, ulen, rflag, h, h2, theta, partial, NV,
+                                                            blk_cnt, state);
   GFCC_LAUNCH_CHECK();
-  vscale_kernel<T><<<vscale_grid(n, nsys), 256, 0, st>>>(w, vs, n, h, NV, nv, state, ST_IN_CYCLE);
+  dim3 vgrid = vscale_grid(n, nsys);
+  vgrid.x += 1;
+  vscale_kernel<T, true><<<vgrid, 256, 0, st>>>(w, vs, n, h, NV, nv, state, ST_IN_CYCLE, q);
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -938,7 +1009,7 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
     cycle_start_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, nrm, NV, bnorm, tol, max_iters, m + 1, state, iters,
                                                       relres, g, H);
     GFCC_LAUNCH_CHECK();
-    vscale_kernel<T><<<vscale_grid(n, nsys), 256, 0, st>>>(Vt, vs, n, nrm, NV, 0, state, ST_IN_CYCLE);
+    vscale_kernel<T, false><<<vscale_grid(n, nsys), 256, 0, st>>>(Vt, vs, n, nrm, NV, 0, state, ST_IN_CYCLE, Lsq{});
     GFCC_LAUNCH_CHECK();
     if (cycle == 0) GFCC_CUDA(cudaMemcpyAsync(relres0, relres, sizeof(double) * nsys, cudaMemcpyDeviceToDevice, st));
     first = false;
