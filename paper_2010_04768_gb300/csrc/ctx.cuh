@@ -103,7 +103,7 @@ struct gfcc_ctx {
   // the rows of both long-K products, [V3 | 0] over [U1 | off-diagonal -Fbar_oo of the 1h row]: [e, i][(m,f,n) | m],
   // ld_k1
   __nv_bfloat16 *VU_bf = nullptr;
-  long long ld_ov = 0, ld_o2 = 0, ld_o = 0, ld_v = 0, ld_k1 = 0, ld_ot = 0;
+  long long ld_ov = 0, ld_o2 = 0, ld_k1 = 0, ld_ot = 0;
 
   // digit planes of the FP64 IP operands for the FP64-accurate residual on the tensor cores
   // (full Fock folding, same GEMM roles as the BF16 operands; V3 padded to the K of U1x)

@@ -105,7 +105,7 @@ __global__ void finalize_kernel(const long long *acc, long long M, long long N, 
 }  // namespace
 
 long long emu_operand_bytes(long long rows, long long K, int S) {
-  const long long ld = (K + 7) / 8 * 8;
+  const long long ld = emu_ld(K);
   return (long long)S * rows * ld * 2 + ((rows * 4 + 255) / 256) * 256 + 256;
 }
 
@@ -114,7 +114,7 @@ int emu_slice(cudaStream_t st, const double *A, long long rows, long long K, lon
   out.bits = bits;
   out.rows = rows;
   out.K = K;
-  out.ld = (K + 7) / 8 * 8;
+  out.ld = emu_ld(K);
   out.S = S;
   unsigned char *p = static_cast<unsigned char *>(mem);
   out.dig = reinterpret_cast<__nv_bfloat16 *>(p);
@@ -345,7 +345,7 @@ int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long lon
                       int S, int bits, void *mem, EmuOperand &out) {
   out.rows = rows;
   out.K = K;
-  out.ld = (K + 7) / 8 * 8;
+  out.ld = emu_ld(K);
   out.S = S;
   out.bits = bits;
   unsigned char *p = static_cast<unsigned char *>(mem);
@@ -404,7 +404,7 @@ constexpr long long EMU_BLOCK_BYTES = 4LL << 30;
 
 // rows (or columns) of a block whose digit planes stay within EMU_BLOCK_BYTES
 long long block_rows(long long rows, long long K) {
-  const long long per = (K + 7) / 8 * 8 * 2 * F64_DIGITS + 8;
+  const long long per = emu_ld(K) * 2 * F64_DIGITS + 8;
   return std::min(rows, std::max<long long>(256, EMU_BLOCK_BYTES / per / 128 * 128));
 }
 

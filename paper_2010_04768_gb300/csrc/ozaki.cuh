@@ -8,6 +8,11 @@
 
 namespace gfcc {
 
+// Row stride of digit planes: whole 128-byte lines where a row has one (a K block of 64 digits that straddles two
+// lines is fetched as both)
+static inline long long emu_ld(long long K) { return K >= 64 ? (K + 63) / 64 * 64 : (K + 7) / 8 * 8; }
+
+
 // An FP64 matrix (rows x K, K-major) split into S planes of balanced `bits`-bit digits (6: base 64) with
 // a power-of-two scale per row: A[r][k] ~= 2^exp2[r] sum_i dig[i][r][k] 2^(-bits (i+1)).
 struct EmuOperand {

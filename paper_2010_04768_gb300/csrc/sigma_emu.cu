@@ -245,7 +245,7 @@ EmuWorkEA emu_layout_ea(const gfcc_ctx *c, int nsub, void *base) {
   auto op = [&](EmuOperand &e, long long rows, long long K) {
     e.rows = rows;
     e.K = K;
-    e.ld = (K + 7) / 8 * 8;
+    e.ld = emu_ld(K);
     e.S = (int)S;
     e.dig = reinterpret_cast<__nv_bfloat16 *>(take(S * rows * e.ld * 2));
     e.exp2 = reinterpret_cast<int *>(take(rows * 4));
@@ -293,7 +293,7 @@ EmuWork emu_layout(const gfcc_ctx *c, int nsub, void *base) {
   auto op = [&](EmuOperand &e, long long rows, long long K) {
     e.rows = rows;
     e.K = K;
-    e.ld = (K + 7) / 8 * 8;
+    e.ld = emu_ld(K);
     e.S = (int)S;
     e.dig = reinterpret_cast<__nv_bfloat16 *>(take(S * rows * e.ld * 2));
     e.exp2 = reinterpret_cast<int *>(take(rows * 4));

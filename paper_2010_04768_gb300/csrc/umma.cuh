@@ -28,7 +28,7 @@ bool emu_fused_takes(int SA, int SB, int P);   // digit counts and level that em
 // Tile autotuning (on by default): the first call of each GEMM shape with beta == 0 times the
 // 64 / 128 / 256-column tiles and every later call of the shape uses the fastest.
 void umma_set_autotune(bool on);
-// CTA-pair tile (cta_group::2, 256 x 256 per pair): 0 timed by the autotuner beside the one-CTA tiles
+// CTA-pair tile (cta_group::2, 256 rows x 128, 192 or 256 columns per pair): 0 timed by the autotuner beside the one-CTA tiles
 // (default), 1 used whenever it applies, 2 never
 void umma_set_pair_mode(int mode);
 // persistent tile loop (one CTA per SM, two TMEM accumulators): 0 timed by the autotuner (default),

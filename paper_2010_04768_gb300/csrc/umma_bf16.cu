@@ -174,6 +174,48 @@ __device__ __forceinline__ void tmem_ld_32(unsigned taddr, float (&v)[32]) {
   for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
 }
 
+// A warp's 32 x 32 block of an accumulator (v: its row `lane`) to D[row0 ..][col0 ..] through shared memory (buf: 32
+// rows of STORE_LD floats of this warp), so that stores run along rows: eight lanes a row of four columns each, or a
+// lane a column where D does not align.  Rows straight from the registers are 32 separate 16-byte pieces a store:
+// 96957 x 60 outputs took 24 us whatever K.
+constexpr int STORE_LD = 36, STORE_BYTES = 32 * STORE_LD * 4;
+__device__ __forceinline__ void store_block(float *buf, const float (&v)[32], float alpha, float beta, float *D,
+                                            long long ldd, int row0, int M, int col0, int N) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < 32; i += 4)
+    *reinterpret_cast<float4 *>(buf + lane * STORE_LD + i) =
+        make_float4(alpha * v[i], alpha * v[i + 1], alpha * v[i + 2], alpha * v[i + 3]);
+  __syncwarp();
+  const int ncols = min(32, N - col0), rows = min(32, M - row0);
+  float *base = D + (long long)row0 * ldd + col0;
+  if (((ldd | ncols) & 3) == 0 && (reinterpret_cast<uintptr_t>(base) & 15) == 0) {
+    const int r0 = lane >> 3, c = (lane & 7) * 4;
+    if (c < ncols) {
+#pragma unroll
+      for (int i = 0; i < 8; i++) {
+        const int r = r0 + 4 * i;
+        if (r >= rows) break;
+        float4 x = *reinterpret_cast<const float4 *>(buf + r * STORE_LD + c);
+        float4 *dst = reinterpret_cast<float4 *>(base + r * ldd + c);
+        if (beta != 0.0f) {
+          const float4 d = *dst;
+          x = make_float4(x.x + beta * d.x, x.y + beta * d.y, x.z + beta * d.z, x.w + beta * d.w);
+        }
+        *dst = x;
+      }
+    }
+  } else if (lane < ncols) {
+#pragma unroll 8
+    for (int r = 0; r < rows; r++) {
+      const float x = buf[r * STORE_LD + lane];
+      float *dst = base + r * ldd + lane;
+      *dst = beta != 0.0f ? x + beta * *dst : x;
+    }
+  }
+  __syncwarp();
+}
+
 template <int BN, int ST>
 __global__ void __launch_bounds__(THREADS, 1)
     umma_bf16_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float *D,
@@ -275,31 +317,14 @@ __global__ void __launch_bounds__(THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   // tcgen05.ld is warp-collective: take the decision per warp
   if (__all_sync(0xffffffffu, ready && !*abort_flag)) {
-    const int row = m0 + warp * 32 + lane;
+    // every load has landed and every MMA has completed: the stages hold the blocks on their way out
+    float *buf = reinterpret_cast<float *>(smem + warp * STORE_BYTES);
+    const int row0 = m0 + warp * 32;
 #pragma unroll 1
-    for (int c0 = 0; c0 < BN; c0 += 32) {
+    for (int c0 = 0; c0 < BN && n0 + c0 < N && row0 < M; c0 += 32) {
       float v[32];
       tmem_ld_32(tmem + ((unsigned)(warp * 32) << 16) + c0, v);
-      if (row < M) {
-        float *dst = D + (long long)row * ldd + n0 + c0;
-        const int ncols = min(32, N - (n0 + c0));
-        if (ncols == 32 && beta == 0.0f && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4)
-            *reinterpret_cast<float4 *>(dst + i) = make_float4(alpha * v[i], alpha * v[i + 1], alpha * v[i + 2],
-                                                               alpha * v[i + 3]);
-        } else if (ncols == 32 && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float4 d = *reinterpret_cast<const float4 *>(dst + i);
-            *reinterpret_cast<float4 *>(dst + i) =
-                make_float4(alpha * v[i] + beta * d.x, alpha * v[i + 1] + beta * d.y, alpha * v[i + 2] + beta * d.z,
-                            alpha * v[i + 3] + beta * d.w);
-          }
-        } else {
-          for (int i = 0; i < ncols; i++) dst[i] = alpha * v[i] + (beta != 0.0f ? beta * dst[i] : 0.0f);
-        }
-      }
+      store_block(buf, v, alpha, beta, D, ldd, row0, M, n0 + c0, N);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -333,7 +358,7 @@ template <int BN>
 struct PTile {
   static constexpr int STAGES = BN == 256 ? 4 : 6;
   static constexpr int A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 512;
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 512 + 4 * STORE_BYTES;
 };
 
 template <int BN>
@@ -455,6 +480,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
   } else {
     // ---------------- epilogue warps 2..5: rows 32 (warp mod 4) + lane of each tile
     const int q = warp & 3;
+    float *out = reinterpret_cast<float *>(smem + STAGES * STAGE_BYTES + 512 + q * STORE_BYTES);
     int lt = 0;
     for (int t = blockIdx.x; t < tiles; t += gridDim.x, lt++) {
       int m0, n0, kb0, nk;
@@ -464,32 +490,12 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
       const bool ready = mbar_wait(smem_u32(&accf[buf]), (lt >> 1) & 1, abort_flag, ctl.wait_ns);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (!__all_sync(0xffffffffu, ready && !*abort_flag)) break;
-      const int row = m0 + q * 32 + lane;
-      float *Dz = D + zoff;
+      const int row0 = m0 + q * 32;
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
+      for (int c0 = 0; c0 < BN && n0 + c0 < N && row0 < M; c0 += 32) {
         float v[32];
         tmem_ld_32(tmem + ((unsigned)(q * 32) << 16) + (unsigned)(buf * BN + c0), v);
-        if (row < M && n0 + c0 < N) {
-          float *dst = Dz + (long long)row * ldd + n0 + c0;
-          const int ncols = min(32, N - (n0 + c0));
-          if (ncols == 32 && beta == 0.0f && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4 *>(dst + i) = make_float4(alpha * v[i], alpha * v[i + 1], alpha * v[i + 2],
-                                                                 alpha * v[i + 3]);
-          } else if (ncols == 32 && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              const float4 d = *reinterpret_cast<const float4 *>(dst + i);
-              *reinterpret_cast<float4 *>(dst + i) =
-                  make_float4(alpha * v[i] + beta * d.x, alpha * v[i + 1] + beta * d.y, alpha * v[i + 2] + beta * d.z,
-                              alpha * v[i + 3] + beta * d.w);
-            }
-          } else {
-            for (int i = 0; i < ncols; i++) dst[i] = alpha * v[i] + (beta != 0.0f ? beta * dst[i] : 0.0f);
-          }
-        }
+        store_block(out, v, alpha, beta, D + zoff, ldd, row0, M, n0 + c0, N);
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
@@ -527,10 +533,14 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
 // barriers of both CTAs (multicast); each CTA's TMEM holds its own 128 rows of the accumulator and
 // each CTA writes them.  Same bounded waits and abort path as the one-CTA kernel; the pair meets at a
 // cluster barrier before either frees its TMEM and exits.
-constexpr int PAIR_BN = 256, PAIR_HALF = 128, PAIR_STAGES = 6;
-constexpr int PAIR_A_BYTES = BM * BK * 2, PAIR_B_BYTES = PAIR_HALF * BK * 2;
-constexpr int PAIR_STAGE_BYTES = PAIR_A_BYTES + PAIR_B_BYTES;
-constexpr int PAIR_SMEM_BYTES = PAIR_STAGES * PAIR_STAGE_BYTES + 1024 + 256;
+// Tiles of 192 and 128 columns fill the chip where 256 would leave the last wave of its 76 pairs nearly empty.
+template <int PBN>
+struct PairTile {
+  static constexpr int HALF = PBN / 2, STAGES = PBN == 256 ? 6 : (PBN == 192 ? 7 : 8);
+  static constexpr int A_BYTES = BM * BK * 2, B_BYTES = HALF * BK * 2, STAGE_BYTES = A_BYTES + B_BYTES;
+  static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+  static constexpr int TMEM_COLS = PBN > 128 ? 256 : 128;   // a power of two
+};
 
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
@@ -579,15 +589,18 @@ __device__ __forceinline__ void umma_commit_pair(unsigned mbar) {
       : "memory");
 }
 
+template <int PBN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     umma_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float *D,
                           long long ldd, int M, int N, int K, float alpha, float beta, int kb_per_split,
                           long long split_stride, UmmaCtl ctl) {
+  constexpr int STAGES = PairTile<PBN>::STAGES, A_BYTES = PairTile<PBN>::A_BYTES,
+                STAGE_BYTES = PairTile<PBN>::STAGE_BYTES, TMEM_COLS = PairTile<PBN>::TMEM_COLS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem + PAIR_STAGES * PAIR_STAGE_BYTES);
-  unsigned long long *full = bars, *empty = bars + PAIR_STAGES, *done = bars + 2 * PAIR_STAGES;
-  unsigned *tmem_slot = reinterpret_cast<unsigned *>(bars + 2 * PAIR_STAGES + 1);
+  unsigned long long *bars = reinterpret_cast<unsigned long long *>(smem + STAGES * STAGE_BYTES);
+  unsigned long long *full = bars, *empty = bars + STAGES, *done = bars + 2 * STAGES;
+  unsigned *tmem_slot = reinterpret_cast<unsigned *>(bars + 2 * STAGES + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
   volatile int *issued = reinterpret_cast<volatile int *>(tmem_slot + 2);
   volatile int *consumed = reinterpret_cast<volatile int *>(tmem_slot + 3);
@@ -607,8 +620,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     n_tile = r / gm;
   }
   const int m0 = mp_tile * (2 * BM) + (int)rank * BM;        // this CTA's rows
-  const int n0 = n_tile * PAIR_BN;                            // the pair's columns
-  const int nb0 = n0 + (int)rank * PAIR_HALF;                 // this CTA's half of the B tile
+  const int n0 = n_tile * PBN;                            // the pair's columns
+  const int nb0 = n0 + (int)rank * PairTile<PBN>::HALF;                 // this CTA's half of the B tile
   const int nk_all = (K + BK - 1) / BK;
   const int kb0 = blockIdx.z * kb_per_split;
   const int kb1 = min(nk_all, kb0 + kb_per_split);
@@ -616,7 +629,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   D += (long long)blockIdx.z * split_stride;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < PAIR_STAGES; s++) {
+    for (int s = 0; s < STAGES; s++) {
       mbar_init(smem_u32(&full[s]), 1);
       mbar_init(smem_u32(&empty[s]), 1);
     }
@@ -628,7 +641,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   }
   if (warp == 0) {   // TMEM of both CTAs: 256 FP32 columns x 128 lanes each (one warp per CTA)
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(PAIR_BN));
+                 "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -639,12 +652,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer (both CTAs): loads complete on the leader's full barriers
     for (int kb = 0; kb < nk && !ctl.skip_loads; kb++) {
-      const int s = kb % PAIR_STAGES;
-      const unsigned ph = (kb / PAIR_STAGES) & 1;
+      const int s = kb % STAGES;
+      const unsigned ph = (kb / STAGES) & 1;
       if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns)) break;
-      unsigned char *sa = smem + s * PAIR_STAGE_BYTES;
-      unsigned char *sb = sa + PAIR_A_BYTES;
-      if (leader) mbar_expect_tx(smem_u32(&full[s]), 2 * PAIR_STAGE_BYTES);
+      unsigned char *sa = smem + s * STAGE_BYTES;
+      unsigned char *sb = sa + A_BYTES;
+      if (leader) mbar_expect_tx(smem_u32(&full[s]), 2 * STAGE_BYTES);
       const unsigned fb = map_to_rank(smem_u32(&full[s]), 0);
       tma_load_2d_pair(smem_u32(sa), &tmA, fb, (kb0 + kb) * BK, m0);
       tma_load_2d_pair(smem_u32(sb), &tmB, fb, (kb0 + kb) * BK, nb0);
@@ -652,14 +665,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1 && leader) {
     // ---------------- MMA issuer (leader only): M = 256 over the pair, N = 256
-    const unsigned idesc = idesc_bf16(2 * BM, PAIR_BN);
+    const unsigned idesc = idesc_bf16(2 * BM, PBN);
     const unsigned long long d0 = smem_desc(smem_u32(smem));
     for (int kb = 0; kb < nk; kb++) {
-      const int s = kb % PAIR_STAGES;
-      const unsigned ph = (kb / PAIR_STAGES) & 1;
+      const int s = kb % STAGES;
+      const unsigned ph = (kb / STAGES) & 1;
       if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned long long da = d0 + s * (PAIR_STAGE_BYTES >> 4), db = da + (PAIR_A_BYTES >> 4);
+      const unsigned long long da = d0 + s * (STAGE_BYTES >> 4), db = da + (A_BYTES >> 4);
       if (elect_one()) {
         *consumed = kb + 1;
 #pragma unroll
@@ -679,31 +692,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const bool failed = *reinterpret_cast<volatile unsigned *>(&g_umma_error) != 0;
   if (__all_sync(0xffffffffu, ready && !*abort_flag && !failed) && nk > 0) {
-    const int row = m0 + warp * 32 + lane;
+    // the pair's MMAs have completed and all loads landed: the stages hold the blocks on their way out
+    float *buf = reinterpret_cast<float *>(smem + warp * STORE_BYTES);
+    const int row0 = m0 + warp * 32;
 #pragma unroll 1
-    for (int c0 = 0; c0 < PAIR_BN; c0 += 32) {
+    for (int c0 = 0; c0 < PBN && n0 + c0 < N && row0 < M; c0 += 32) {
       float v[32];
       tmem_ld_32(tmem + ((unsigned)(warp * 32) << 16) + c0, v);
-      if (row < M && n0 + c0 < N) {
-        float *dst = D + (long long)row * ldd + n0 + c0;
-        const int ncols = min(32, N - (n0 + c0));
-        if (ncols == 32 && beta == 0.0f && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4)
-            *reinterpret_cast<float4 *>(dst + i) = make_float4(alpha * v[i], alpha * v[i + 1], alpha * v[i + 2],
-                                                               alpha * v[i + 3]);
-        } else if (ncols == 32 && ((reinterpret_cast<uintptr_t>(dst) & 15) == 0)) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float4 d = *reinterpret_cast<const float4 *>(dst + i);
-            *reinterpret_cast<float4 *>(dst + i) =
-                make_float4(alpha * v[i] + beta * d.x, alpha * v[i + 1] + beta * d.y, alpha * v[i + 2] + beta * d.z,
-                            alpha * v[i + 3] + beta * d.w);
-          }
-        } else {
-          for (int i = 0; i < ncols; i++) dst[i] = alpha * v[i] + (beta != 0.0f ? beta * dst[i] : 0.0f);
-        }
-      }
+      store_block(buf, v, alpha, beta, D, ldd, row0, M, n0 + c0, N);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -714,13 +710,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     volatile int never = 0;
     mbar_wait(smem_u32(done), 0, &never, DRAIN_NS);
     for (int kb = *consumed; kb < *issued; kb++)
-      mbar_wait(smem_u32(&full[kb % PAIR_STAGES]), (kb / PAIR_STAGES) & 1, &never, DRAIN_NS);
+      mbar_wait(smem_u32(&full[kb % STAGES]), (kb / STAGES) & 1, &never, DRAIN_NS);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync_all();   // neither CTA frees its TMEM or shared memory while the pair's work is in flight
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(PAIR_BN));
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
   }
 }
 
@@ -1175,7 +1171,7 @@ namespace {
 bool g_autotune = true;
 // 0: the autotuner also times the CTA-pair tile; 1: the pair tile whenever it applies; 2: never
 int g_pair_mode = 0;
-constexpr int TILE_PAIR = 512;   // autotuner key of the 256 x 256 CTA-pair tile
+constexpr int TILE_PAIR = 512;   // autotuner key offset of the CTA-pair tiles (+ their width)
 constexpr int TILE_PERSIST = 1024;   // autotuner key offset of the persistent kernel (+ its tile width)
 // 0: the autotuner also times the persistent kernel; 1: always the persistent kernel; 2: never
 int g_persist_mode = 0;
@@ -1242,28 +1238,29 @@ int launch_umma_persist(cudaStream_t st, const __nv_bfloat16 *A, long long lda, 
   return GFCC_OK;
 }
 
+template <int PBN>
 int launch_umma_pair(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const __nv_bfloat16 *B, long long ldb,
                      float *D, long long ldd, int M, int N, int K, float alpha, float beta, int nsplit, int kbs,
                      long long split_stride) {
   CUtensorMap ma, mb;
   GFCC_TRY(make_map(&ma, A, M, K, lda, BM));
-  GFCC_TRY(make_map(&mb, B, N, K, ldb, PAIR_HALF));
+  GFCC_TRY(make_map(&mb, B, N, K, ldb, PairTile<PBN>::HALF));
   static bool attr[64] = {false};
   int dev = 0;
   GFCC_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !attr[dev]) {
-    GFCC_CUDA(cudaFuncSetAttribute(umma_pair_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   PAIR_SMEM_BYTES));
+    GFCC_CUDA(cudaFuncSetAttribute(umma_pair_gemm_kernel<PBN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   PairTile<PBN>::SMEM_BYTES));
     if (dev >= 0 && dev < 64) attr[dev] = true;
   }
   const long long mp = (M + 2 * BM - 1) / (2 * BM);
-  if ((N + PAIR_BN - 1) / PAIR_BN > 65535 || nsplit > 65535 || 2 * mp > 0x7fffffffLL) {
+  if ((N + PBN - 1) / PBN > 65535 || nsplit > 65535 || 2 * mp > 0x7fffffffLL) {
     set_error("gemm_bf16_tn: grid too large (M=%d, N=%d, nsplit=%d)", M, N, nsplit);
     return GFCC_ERR_ARG;
   }
-  dim3 grid((unsigned)(2 * mp), (N + PAIR_BN - 1) / PAIR_BN, nsplit);
-  umma_pair_gemm_kernel<<<grid, THREADS, PAIR_SMEM_BYTES, st>>>(ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
-                                                                 split_stride, umma_ctl());
+  dim3 grid((unsigned)(2 * mp), (N + PBN - 1) / PBN, nsplit);
+  umma_pair_gemm_kernel<PBN><<<grid, THREADS, PairTile<PBN>::SMEM_BYTES, st>>>(ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
+                                                                              split_stride, umma_ctl());
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1302,13 +1299,17 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
   GFCC_TRY(check_extent_bytes(B, (long long)(N - 1) * ldb * 2 + (long long)K * 2, "bf16 GEMM operand B"));
   GFCC_TRY(check_extent_bytes(D, ((long long)(M - 1) * ldd + N + (long long)(nsplit - 1) * split_stride) * 4,
                               "bf16 GEMM output D"));
-  // tile widths: 64 / 128 / 256 columns per CTA, TILE_PAIR (256 x 256 over a CTA pair), or
+  // tile widths: 64 / 128 / 256 columns per CTA, TILE_PAIR + 128 / 192 / 256 (256 rows over a CTA pair), or
   // TILE_PERSIST + 64 / 128 / 256 (the persistent kernel with that width)
   auto run = [&](int bn) -> int {
     if (bn == 64) return launch_umma<64>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
     if (bn == 128) return launch_umma<128>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
-    if (bn == TILE_PAIR)
-      return launch_umma_pair(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
+    if (bn == TILE_PAIR + 128)
+      return launch_umma_pair<128>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
+    if (bn == TILE_PAIR + 192)
+      return launch_umma_pair<192>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
+    if (bn == TILE_PAIR + 256)
+      return launch_umma_pair<256>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
     if (bn == TILE_PERSIST + 64)
       return launch_umma_persist<64>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
     if (bn == TILE_PERSIST + 128)
@@ -1317,9 +1318,18 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
       return launch_umma_persist<256>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
     return launch_umma<256>(st, A, lda, B, ldb, D, ldd, M, N, K, alpha, beta, nsplit, kbs, split_stride);
   };
-  // the pair kernel needs two row tiles and pays off on wide products with a long K loop
+  // the pair kernel needs two row tiles and pays off on wide products with a long K loop; its widths by the waves of
+  // 76 pairs (clocks of a tile: a K block's loads at 55 bytes a clock, some 16 a column and 6000 for its ends).
+  // 3591 x 1620 x 3591: 192 columns 38 us, 256 columns 50 us; 8000 x 3200 x 8000: 256 columns 257 us, 128 348 us.
   const bool pair_ok = g_pair_mode != 2 && M > BM && N > 128 && kbs >= 8;
-  if (g_pair_mode == 1) return pair_ok ? run(TILE_PAIR) : run(N <= 64 ? 64 : (N <= 128 ? 128 : 256));
+  auto pair_cost = [&](int w) {
+    const long long tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + w - 1LL) / w) * nsplit;
+    return (double)((tiles + 75) / 76) * (kbs * (298.0 + 1.16 * w) + 16.0 * w + 6000.0);
+  };
+  const int pair_best = pair_cost(256) <= std::min(pair_cost(192), pair_cost(128)) ? 256
+                        : pair_cost(192) <= pair_cost(128)                       ? 192
+                                                                                 : 128;
+  if (g_pair_mode == 1) return pair_ok ? run(TILE_PAIR + pair_best) : run(N <= 64 ? 64 : (N <= 128 ? 128 : 256));
   const int narrow = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
   if (g_persist_mode == 1) return run(TILE_PERSIST + narrow);
   // the persistent kernel pays off once a launch has several waves of tiles
@@ -1342,19 +1352,22 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
       if (it != g_tune.end()) best = it->second;
     }
     if (best == 0) {
-      // first call of this shape: time every tile width (second of two launches each, CUDA events on
+      // first call of this shape: time every tile width (the last two of three launches each, CUDA events on
       // the stream; beta == 0, so the repeated launches leave the same D) and keep the fastest
       cudaEvent_t e0, e1;
       GFCC_CUDA(cudaEventCreate(&e0));
       GFCC_CUDA(cudaEventCreate(&e1));
       float best_ms = 0.0f;
-      for (int cand : {64, 128, 256, TILE_PAIR, TILE_PERSIST + 64, TILE_PERSIST + 128, TILE_PERSIST + 256}) {
-        const int w = cand > TILE_PERSIST ? cand - TILE_PERSIST : cand;
-        if (cand == TILE_PAIR ? !pair_ok
-                              : ((cand > TILE_PERSIST && !persist_ok) || (w > 64 && w / 2 >= N)))
+      for (int cand : {64, 128, 256, TILE_PAIR + 128, TILE_PAIR + 192, TILE_PAIR + 256, TILE_PERSIST + 64,
+                       TILE_PERSIST + 128, TILE_PERSIST + 256}) {
+        const int w = cand > TILE_PERSIST ? cand - TILE_PERSIST : cand > TILE_PAIR ? cand - TILE_PAIR : cand;
+        if (cand > TILE_PAIR && cand < TILE_PERSIST
+                ? !pair_ok || pair_cost(w) > 1.15 * pair_cost(pair_best)
+                : ((cand > TILE_PERSIST && !persist_ok) || (w > 64 && w / 2 >= N)))
           continue;   // never better
         GFCC_TRY(run(cand));
         GFCC_CUDA(cudaEventRecord(e0, st));
+        GFCC_TRY(run(cand));
         GFCC_TRY(run(cand));
         GFCC_CUDA(cudaEventRecord(e1, st));
         GFCC_CUDA(cudaEventSynchronize(e1));
