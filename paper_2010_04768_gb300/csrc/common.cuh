@@ -79,10 +79,11 @@ __host__ __device__ __forceinline__ long long pair_start(long long i, long long 
 __host__ __device__ __forceinline__ long long pair_index(long long i, long long j, long long m) {
   return pair_start(i, m) + (j - i - 1);
 }
-// Inverse of pair_index (closed form from the quadratic, then an exact integer correction).
+// Inverse of pair_index (closed form from the quadratic in FP32, a step or two off, then an exact integer
+// correction; the FP64 square root of every thread held the epilogues to a third of the memory rate).
 __device__ __forceinline__ void pair_decode(long long idx, long long m, long long &i, long long &j) {
-  const double b = 2.0 * (double)m - 1.0;
-  long long ii = (long long)((b - sqrt(fmax(b * b - 8.0 * (double)idx, 0.0))) * 0.5);
+  const float b = 2.0f * (float)m - 1.0f;
+  long long ii = (long long)((b - sqrtf(fmaxf(b * b - 8.0f * (float)idx, 0.0f))) * 0.5f);
   if (ii < 0) ii = 0;
   if (ii > m - 2) ii = m - 2;
   while (ii > 0 && pair_start(ii, m) > idx) ii--;

@@ -413,7 +413,7 @@ constexpr int DOT_WARPS = 4, DOT_RUN = 4096;   // FP32 sums of at most DOT_RUN /
 template <typename T>
 struct CgsShape {   // blocks per SM (by registers), elements a round of the dots
   static constexpr bool F32 = sizeof(T) == sizeof(float);
-  static constexpr int DOT_UNROLL = 8, DOT_PER_SM = 8, UPD_PER_SM = 4;
+  static constexpr int DOT_UNROLL = 8, DOT_PER_SM = F32 ? 8 : 5, UPD_PER_SM = 4;
 };
 constexpr double REORTH_THETA_F32 = 0.01;   // FP32 Krylov vectors: second pass where ||w'|| < 0.1 ||w||
 
@@ -473,7 +473,7 @@ __global__ __launch_bounds__(32 * DOT_WARPS, CgsShape<T>::DOT_PER_SM) void cgs_d
   const long long c1 = min((long long)(chunk + 1) * clen, n);
   const long long e0 = (long long)chunk * clen + (warp % split) * plen;
   const long long e1 = min(e0 + plen, c1);
-  for (int i = warp / split; i <= nv; i += DOT_WARPS / split) {
+  auto dot = [&](int i) -> double2 {   // this lane's part of <V_i, w> over the warp's part of the chunk
     const T *vp = i < nv ? Vs + 2 * i * vi : ws;   // slot nv: ||w||^2
     double2 acc = make_double2(0.0, 0.0);
     for (long long r0 = e0; r0 < e1; r0 += DOT_RUN) {
@@ -487,17 +487,41 @@ __global__ __launch_bounds__(32 * DOT_WARPS, CgsShape<T>::DOT_PER_SM) void cgs_d
       acc.x += (double)ar;
       acc.y += (double)ai;
     }
+    return acc;
+  };
+  if (split == 1) {
+    // four vectors at a time: their eight sums over the lanes scatter as they are added (9 FP64 additions instead of
+    // 40; at 51 vectors those of the plain butterfly took as long on the FP64 pipe as half of the loads)
+    for (int i0 = warp; i0 <= nv; i0 += 4 * DOT_WARPS) {
+      double v[8];
+#pragma unroll
+      for (int g = 0; g < 4; g++) {
+        const int i = i0 + g * DOT_WARPS;
+        const double2 d = i <= nv ? dot(i) : make_double2(0.0, 0.0);
+        v[2 * g] = d.x;
+        v[2 * g + 1] = d.y;
+      }
+#pragma unroll
+      for (int h = 4; h > 0; h >>= 1) {
+        const bool up = lane & (4 * h);
+#pragma unroll
+        for (int k = 0; k < h; k++) {
+          const double give = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+          v[k] = keep + __shfl_xor_sync(0xffffffffu, give, 4 * h);
+        }
+      }
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+      const int k = (lane >> 4) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1), i = i0 + (k >> 1) * DOT_WARPS;
+      if ((lane & 3) == 0 && i <= nv) reinterpret_cast<double *>(ps)[2 * ((long long)i * nch + chunk) + (k & 1)] = v[0];
+    }
+  } else if (warp / split <= nv) {
+    double2 acc = dot(warp / split);
     for (int off = 16; off > 0; off >>= 1) {
       acc.x += __shfl_xor_sync(0xffffffffu, acc.x, off);
       acc.y += __shfl_xor_sync(0xffffffffu, acc.y, off);
     }
-    if (lane == 0) {
-      if (split == 1)
-        ps[(long long)i * nch + chunk] = acc;
-      else
-        parts[warp] = acc;
-    }
-    if (split > 1) break;   // one vector a warp
+    if (lane == 0) parts[warp] = acc;
   }
   if (split > 1) {
     __syncthreads();

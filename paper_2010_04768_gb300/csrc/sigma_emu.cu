@@ -22,21 +22,39 @@ namespace gfcc {
 
 namespace {
 
-// e[c] (c = 2 s + re/im) with max_mu |x_s| * 2^-e in [1/4, 1/2)
-__global__ void plane_exp_kernel(const double *x, long long ldx, long long n, int *e) {
-  __shared__ double sh[32];
-  const int c = blockIdx.x, s = c >> 1, t = c & 1;
-  double mx = 0.0;
-  for (long long mu = threadIdx.x; mu < n; mu += blockDim.x) mx = fmax(mx, fabs(x[2 * (s * ldx + mu) + t]));
-  for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) mx = fmax(mx, sh[w]);
-    int E = 0;
-    if (mx > 0.0) frexp(mx, &E);
-    e[c] = mx > 0.0 ? E + 1 : 0;
+// e[c] (c = 2 s + re/im) with max_mu |x_s| * 2^-e in [1/4, 1/2).  First the largest exponent field of the plane
+// (e zeroed before; grid (chunks, systems)), on the integer units, then the shift.  With one block a plane and FP64
+// maxima it took 120 us for the 80 planes of 40 systems at o=40 v=200.
+__global__ __launch_bounds__(256) void plane_exp_kernel(const double *x, long long ldx, long long n, int *e) {
+  const int s = blockIdx.y, lane = threadIdx.x & 31;
+  const double2 *xs = reinterpret_cast<const double2 *>(x) + s * ldx;
+  int mr = 0, mi = 0;
+#pragma unroll 4
+  for (long long mu = (long long)blockIdx.x * 256 + threadIdx.x; mu < n; mu += (long long)gridDim.x * 256) {
+    const double2 u = xs[mu];
+    const int er = (__double2hiint(u.x) >> 20) & 0x7ff, ei = (__double2hiint(u.y) >> 20) & 0x7ff;
+    if (er < 0x7ff) mr = max(mr, er);
+    if (ei < 0x7ff) mi = max(mi, ei);
   }
+  mr = __reduce_max_sync(0xffffffffu, mr);
+  mi = __reduce_max_sync(0xffffffffu, mi);
+  if (lane == 0) {
+    if (mr > 0) atomicMax(&e[2 * s], mr);
+    if (mi > 0) atomicMax(&e[2 * s + 1], mi);
+  }
+}
+__global__ void plane_exp_final_kernel(int planes, int *e) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c < planes && e[c] > 0) e[c] -= 1021;
+}
+int plane_exponents(cudaStream_t st, const double *x, long long ldx, long long n, int nsys, int *e) {
+  GFCC_CUDA(cudaMemsetAsync(e, 0, sizeof(int) * 2 * nsys, st));
+  const unsigned chunks = (unsigned)std::max<long long>(1, std::min<long long>((n + 1023) / 1024, 152 * 8 / std::max(1, nsys) + 1));
+  plane_exp_kernel<<<dim3(chunks, (unsigned)nsys), 256, 0, st>>>(x, ldx, n, e);
+  GFCC_LAUNCH_CHECK();
+  plane_exp_final_kernel<<<cdiv(2 * nsys, 128), 128, 0, st>>>(2 * nsys, e);
+  GFCC_LAUNCH_CHECK();
+  return GFCC_OK;
 }
 
 __device__ __forceinline__ double packed_r2(const double *x, long long ldx, int o, int v, int c, int m, int j, int e) {
@@ -352,8 +370,7 @@ int apply_ip_emu(gfcc_ctx *c, const SysBatch &b, double *work, long long work_do
     const double *x = b.x + 2 * (long long)s0 * b.ldx;
     {
     PhaseTimer tu(c, PH_UNPACK);
-    plane_exp_kernel<<<C2, 256, 0, st>>>(x, b.ldx, n, w.ec);
-    GFCC_LAUNCH_CHECK();
+    GFCC_TRY(plane_exponents(st, x, b.ldx, n, (int)(C2 / 2), w.ec));
     digits_ring_kernel<<<grid1d(w.r2b.rows * w.r2b.ld), 256, 0, st>>>(x, b.ldx, C2, (int)o, (int)v, w.ec, S, w.r2b.ld,
                                                                        w.r2b.dig, w.r2b.exp2);
     GFCC_LAUNCH_CHECK();
@@ -430,8 +447,7 @@ int apply_ea_emu(gfcc_ctx *c, const SysBatch &b, double *work, long long work_do
     const double *x = b.x + 2 * (long long)s0 * b.ldx;
     {
       PhaseTimer tu(c, PH_UNPACK);
-      plane_exp_kernel<<<C2, 256, 0, st>>>(x, b.ldx, n, w.ec);
-      GFCC_LAUNCH_CHECK();
+      GFCC_TRY(plane_exponents(st, x, b.ldx, n, (int)(C2 / 2), w.ec));
       digits_ea_ring_kernel<<<grid1d(w.r2e.rows * w.r2e.ld), 256, 0, st>>>(x, b.ldx, C2, (int)o, (int)v, Pv, w.ec, S,
                                                                             w.r2e.ld, w.r2e.dig, w.r2e.exp2);
       GFCC_LAUNCH_CHECK();

@@ -35,6 +35,11 @@ struct Cz {
   float r, i;
 };
 
+// x times the sign of d (+1 or -1), on the integer units
+__device__ __forceinline__ float with_sign(double d, float x) {
+  return __int_as_float(__float_as_int(x) ^ (__double2hiint(d) & 0x80000000));
+}
+
 __device__ __forceinline__ Cz load_u(const SysBatch &b, int s, long long mu) {
   s = sysv(b, s);
   Cz u;
@@ -45,8 +50,8 @@ __device__ __forceinline__ Cz load_u(const SysBatch &b, int s, long long mu) {
     u = {d2f_trunc(b.x[2 * (s * b.ldx + mu)]), d2f_trunc(b.x[2 * (s * b.ldx + mu) + 1])};
   }
   if (b.diag != nullptr && b.omega != nullptr) {
-    const float dr = d2f_trunc(b.omega[s]) + (float)b.dsign * d2f_trunc(b.diag[mu]);
-    const float di = (float)b.zsign * d2f_trunc(b.eta);
+    const float dr = d2f_trunc(b.omega[s]) + with_sign(b.dsign, d2f_trunc(b.diag[mu]));
+    const float di = with_sign(b.zsign, d2f_trunc(b.eta));
     const float inv = 1.0f / (dr * dr + di * di);
     u = {(u.r * dr + u.i * di) * inv, (u.i * dr - u.r * di) * inv};
   }
@@ -141,61 +146,125 @@ __global__ void unpack_k_tiled_kernel(SysBatch b, int o, int v, long long ldk, _
   }
 }
 
+// A system's vector with the right preconditioner, the uniform parts read once
+struct SysIn {
+  const float2 *xf;
+  const double2 *x;
+  const double *diag;
+  float om, di, di2, sgn;
+  __device__ __forceinline__ SysIn(const SysBatch &b, int s) {
+    const int t = sysv(b, s);
+    xf = b.xf ? reinterpret_cast<const float2 *>(b.xf) + t * b.ldx : nullptr;
+    x = b.xf ? nullptr : reinterpret_cast<const double2 *>(b.x) + t * b.ldx;
+    diag = b.omega != nullptr ? b.diag : nullptr;
+    om = diag != nullptr ? d2f_trunc(b.omega[t]) : 0.f;
+    di = with_sign(b.zsign, d2f_trunc(b.eta));
+    di2 = di * di;
+    sgn = with_sign(b.dsign, 1.f);
+  }
+  __device__ __forceinline__ Cz operator()(long long mu) const {
+    Cz u;
+    if (xf != nullptr) {
+      const float2 t = xf[mu];
+      u = {t.x, t.y};
+    } else {
+      const double2 t = x[mu];
+      u = {d2f_trunc(t.x), d2f_trunc(t.y)};
+    }
+    if (diag != nullptr) {
+      const float dr = om + sgn * d2f_trunc(diag[mu]);
+      const float inv = 1.0f / (dr * dr + di2);
+      u = {(u.r * dr + u.i * di) * inv, (u.i * dr - u.r * di) * inv};
+    }
+    return u;
+  }
+};
+
+// BF16 pairs of a run of `len` (re, im) values, packed in 32 bits, to the rows re and re + ld (im): stores of
+// two values wherever the address is a multiple of four bytes.  pack(i) is value i of the run, odd the parity of re's
+// address in values; slot q holds values 2 q - odd and the next, q = 0 .. len / 2.
+template <typename Pack>
+__device__ __forceinline__ void put_pair(__nv_bfloat16 *re, long long ld, int odd, int len, int q, Pack pack) {
+  const int i0 = 2 * q - odd, i1 = i0 + 1;
+  const bool in0 = i0 >= 0 && i0 < len, in1 = i1 < len;
+  const unsigned u0 = in0 ? pack(i0) : 0u, u1 = in1 ? pack(i1) : 0u;
+  const unsigned r = __byte_perm(u0, u1, 0x5410), i = __byte_perm(u0, u1, 0x7632);
+  __nv_bfloat16 *p = re + i0;
+  if (in0 && in1) {
+    *reinterpret_cast<unsigned *>(p) = r;
+    *reinterpret_cast<unsigned *>(p + ld) = i;
+  } else if (in0) {
+    *reinterpret_cast<unsigned short *>(p) = (unsigned short)r;
+    *reinterpret_cast<unsigned short *>(p + ld) = (unsigned short)i;
+  } else if (in1) {
+    *reinterpret_cast<unsigned short *>(p + 1) = (unsigned short)(r >> 16);
+    *reinterpret_cast<unsigned short *>(p + ld + 1) = (unsigned short)(i >> 16);
+  }
+}
+
+__device__ __forceinline__ unsigned pack_bf16(const Cz &u) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(u.r, u.i);
+  return *reinterpret_cast<const unsigned *>(&h);
+}
+
 // All three 2h1p layouts in one pass.  One block per (e tile, m, system s): the tile r2[m, j, e]
 // of system s for every j (each packed element is read by the blocks of its two occupied indices;
-// the right preconditioner is applied once per read), then
+// the right preconditioner is applied once per read), rounded to BF16 in shared memory, then
 //   ring   r2b[(j, c)][(m, e)]  rows of the tile's e range,
 //   oooo   r2o[(e, c)][(m, j)]  rows of o consecutive columns,
 //   long K rk[c][(m, e, j)]     one contiguous run of (e range) x o columns,
-// for both planes c = 2 s + re/im.  Quotients by o come from a 32.32 fixed-point reciprocal
-// (exact while the dividend stays below 2^32 / o; here below 2 UNPACK_ET o).
+// for both planes c = 2 s + re/im, two columns a store.  Bound by instructions: 90 us for 40 systems of o=40 v=200 (154 MB
+// written); one value a store, an index division for each and conversions on the FP64 pipe took 133 us.
 constexpr int UNPACK_ET = 32;   // e values per block (a power of two)
-constexpr int UNPACK_MAX_O = 180;   // tile o x (UNPACK_ET + 1) float2 within the default 48 KB
+constexpr int UNPACK_MAX_O = 180;   // tile o x (UNPACK_ET + 1) words within the default 48 KB
 
-__device__ __forceinline__ int quo(unsigned q, unsigned long long rcp) {
-  return (int)(((unsigned long long)q * rcp) >> 32);
-}
-
-__global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v, unsigned long long rcp_o,
-                                                        long long ld_ov, long long ld_o2, long long ld_k1,
-                                                        __nv_bfloat16 *r2b, __nv_bfloat16 *r2o, __nv_bfloat16 *rk,
-                                                        long long ld_ot, __nv_bfloat16 *rz) {
-  extern __shared__ float2 tl[];   // [o][UNPACK_ET + 1]
+__global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v, long long ld_ov, long long ld_o2,
+                                                        long long ld_k1, __nv_bfloat16 *r2b, __nv_bfloat16 *r2o,
+                                                        __nv_bfloat16 *rk, long long ld_ot, __nv_bfloat16 *rz) {
+  extern __shared__ unsigned tl[];   // [o][UNPACK_ET + 1] (re, im) in BF16
   constexpr int LD = UNPACK_ET + 1;
   const int e0 = blockIdx.x * UNPACK_ET, m = blockIdx.y, s = blockIdx.z;
   const int et = min(UNPACK_ET, v - e0);
-  const int C2 = 2 * b.nsys;
-  for (int t = threadIdx.x; t < o * UNPACK_ET; t += blockDim.x) {
-    const int j = t / UNPACK_ET, el = t % UNPACK_ET;
-    float2 val = make_float2(0.f, 0.f);
-    if (el < et) {
-      const Cz u = r2_at(b, o, v, s, m, j, e0 + el);
-      val = make_float2(u.r, u.i);
+  const int C2 = 2 * b.nsys, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const SysIn in(b, s);
+#pragma unroll 4
+  for (int j = warp; j < o; j += 8) {
+    unsigned h = 0u;
+    if (lane < et && j != m) {
+      const int lo = min(m, j), hi = max(m, j);
+      h = pack_bf16(in(o + (long long)(lo * o - lo * (lo + 1) / 2 + hi - lo - 1) * v + e0 + lane));
+      if (m > j) h ^= 0x80008000u;
     }
-    tl[j * LD + el] = val;
+    tl[j * LD + lane] = h;
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) put_r1(b, s, m, (long long)o * o * v, ld_k1, rk, ld_ot, rz);
   __syncthreads();
-  // ring: rows (j, 2 s + p), columns m v + e0 .. m v + e0 + et
-  for (int t = threadIdx.x; t < 2 * o * UNPACK_ET; t += blockDim.x) {
-    const int el = t % UNPACK_ET, jp = t / UNPACK_ET, p = jp & 1, j = jp >> 1;
-    if (el >= et) continue;
-    const float2 u = tl[j * LD + el];
-    r2b[((long long)j * C2 + 2 * s + p) * ld_ov + (long long)m * v + e0 + el] = __float2bfloat16(p ? u.y : u.x);
+  // ring: rows (j, 2 s + p), columns m v + e0 .. m v + e0 + et, 16 lanes a row (and one value more of an odd start);
+  // row strides are even
+  {
+    const long long col = (long long)m * v + e0;
+    const int q = lane & 15, odd = (int)(col & 1);
+    __nv_bfloat16 *re = r2b + ((long long)(2 * warp + (lane >> 4)) * C2 + 2 * s) * ld_ov + col;
+    for (int j = 2 * warp + (lane >> 4); j < o; j += 16, re += 16LL * C2 * ld_ov) {
+      const unsigned *row = tl + j * LD;
+      auto pack = [&](int i) { return row[i]; };
+      put_pair(re, ld_ov, odd, et, q, pack);
+      if (odd && q == 0) put_pair(re, ld_ov, odd, et, 16, pack);
+    }
   }
-  // oooo: rows (e, 2 s + p), columns m o + j
-  for (int t = threadIdx.x; t < 2 * et * o; t += blockDim.x) {
-    const int ep = quo((unsigned)t, rcp_o), j = t - ep * o, p = ep & 1, el = ep >> 1;
-    const float2 u = tl[j * LD + el];
-    r2o[((long long)(e0 + el) * C2 + 2 * s + p) * ld_o2 + (long long)m * o + j] = __float2bfloat16(p ? u.y : u.x);
-  }
-  // long K: row 2 s + p, columns (m v + e) o + j for the tile's e range
-  for (int p = 0; p < 2; p++) {
-    __nv_bfloat16 *dst = rk + (long long)(2 * s + p) * ld_k1 + ((long long)m * v + e0) * o;
-    for (int t = threadIdx.x; t < et * o; t += blockDim.x) {
-      const int el = quo((unsigned)t, rcp_o), j = t - el * o;
-      const float2 u = tl[j * LD + el];
-      dst[t] = __float2bfloat16(p ? u.y : u.x);
+  // oooo: rows (e, 2 s + p), columns m o + j; long K: row 2 s + p, columns (m v + e) o + j.  16 or 32 lanes a row
+  const int half = o / 2 + 1 <= 16 ? 1 : 0, q0 = half ? lane & 15 : lane, step = half ? 16 : 32;
+  const int el0 = half ? 2 * warp + (lane >> 4) : warp, stride = half ? 16 : 8;
+  __nv_bfloat16 *re_k = rk + (long long)(2 * s) * ld_k1 + ((long long)m * v + e0 + el0) * o;
+  __nv_bfloat16 *re_o = r2o + ((long long)(e0 + el0) * C2 + 2 * s) * ld_o2 + (long long)m * o;
+  const int odd_o = (m * o) & 1;
+  int odd_k = (int)((((long long)m * v + e0 + el0) * o) & 1);   // stays: the stride of el is even
+  for (int el = el0; el < et; el += stride, re_k += stride * o, re_o += (long long)stride * C2 * ld_o2) {
+    const unsigned *col = tl + el;
+    auto pack = [&](int j) { return col[j * LD]; };
+    for (int q = q0; q <= o / 2; q += step) {
+      put_pair(re_o, ld_o2, odd_o, o, q, pack);
+      put_pair(re_k, ld_k1, odd_k, o, q, pack);
     }
   }
 }
@@ -256,39 +325,41 @@ __device__ __forceinline__ Cz y2_at(const SysBatch &b, int v, long long Pv, int 
 // both along e.  grid (cdiv(v, 32), cdiv(v, 32), o * nsys), block (32, 8).
 __global__ void unpack_ea_tile_kernel(SysBatch b, int o, int v, long long Pv, long long ld_ov, long long ldk,
                                       __nv_bfloat16 *r2e, __nv_bfloat16 *rk, long long ld_ot, __nv_bfloat16 *rz) {
-  __shared__ float2 tile[32][33];
+  __shared__ unsigned tile[32][33];   // (re, im) in BF16
   const int e0 = blockIdx.x * 32, a0 = blockIdx.y * 32;
   const int m = (int)(blockIdx.z % (unsigned)o), s = (int)(blockIdx.z / (unsigned)o);
-  const int C2 = 2 * b.nsys;
+  const int C2 = 2 * b.nsys, lane = threadIdx.x;
   // the 1p block, by the blocks of one (a tile, m)
   if (a0 == 0 && m == 0 && threadIdx.y == 0 && e0 + (int)threadIdx.x < v)
     put_r1(b, s, e0 + threadIdx.x, (long long)o * v * v, ldk, rk, ld_ot, rz);
   const bool below = e0 + 31 < a0;   // every a > e: packed pairs (e, a) run along a
+  const SysIn in(b, s);
+#pragma unroll
   for (int r = threadIdx.y; r < 32; r += 8) {
-    const int a = below ? a0 + threadIdx.x : a0 + r, e = below ? e0 + r : e0 + threadIdx.x;
-    float2 val = make_float2(0.f, 0.f);
-    if (a < v && e < v) {
-      const Cz u = y2_at(b, v, Pv, s, m, a, e);
-      val = make_float2(u.r, u.i);
+    const int a = below ? a0 + lane : a0 + r, e = below ? e0 + r : e0 + lane;
+    unsigned h = 0u;
+    if (a < v && e < v && a != e) {
+      h = pack_bf16(in(v + (long long)m * Pv + pair_index(min(a, e), max(a, e), v)));
+      if (a > e) h ^= 0x80008000u;
     }
     if (below)
-      tile[threadIdx.x][r] = val;
+      tile[lane][r] = h;
     else
-      tile[r][threadIdx.x] = val;
+      tile[r][lane] = h;
   }
   __syncthreads();
-  const int e = e0 + threadIdx.x;
-  if (e >= v) return;
-  for (int r = threadIdx.y; r < 32; r += 8) {
-    const int a = a0 + r;
-    if (a >= v) break;
-    const float2 u = tile[r][threadIdx.x];
-    const long long ring = ((long long)a * C2 + 2 * s) * ld_ov + (long long)m * v + e;
-    r2e[ring] = __float2bfloat16(u.x);
-    r2e[ring + ld_ov] = __float2bfloat16(u.y);
-    const long long kk = (long long)(2 * s) * ldk + ((long long)m * v + a) * v + e;
-    rk[kk] = __float2bfloat16(-u.x);
-    rk[kk + ldk] = __float2bfloat16(-u.y);
+  // both along e, two columns a store: 16 lanes a row (and one value more of an odd start)
+  const int et = min(32, v - e0), q = lane & 15;
+  for (int r = 2 * threadIdx.y + (lane >> 4); r < 32 && a0 + r < v; r += 16) {
+    const long long c1 = (long long)m * v + e0, c2 = ((long long)m * v + a0 + r) * v + e0;
+    __nv_bfloat16 *re = r2e + ((long long)(a0 + r) * C2 + 2 * s) * ld_ov + c1, *re_k = rk + (long long)(2 * s) * ldk + c2;
+    const int odd1 = (int)(c1 & 1), odd2 = (int)(c2 & 1);
+    auto plus = [&](int i) { return tile[r][i]; };
+    auto minus = [&](int i) { return tile[r][i] ^ 0x80008000u; };
+    put_pair(re, ld_ov, odd1, et, q, plus);
+    put_pair(re_k, ldk, odd2, et, q, minus);
+    if (q == 0 && odd1) put_pair(re, ld_ov, odd1, et, 16, plus);
+    if (q == 0 && odd2) put_pair(re_k, ldk, odd2, et, 16, minus);
   }
 }
 
@@ -383,10 +454,9 @@ int apply_ip_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
   {
   PhaseTimer tu(c, PH_UNPACK);
   if (v > 0 && o <= UNPACK_MAX_O) {
-    const unsigned long long rcp_o = ((1ULL << 32) + (unsigned long long)o - 1) / (unsigned long long)o;
-    const size_t sm = (size_t)o * (UNPACK_ET + 1) * sizeof(float2);
+    const size_t sm = (size_t)o * (UNPACK_ET + 1) * sizeof(unsigned);
     unpack_ip_kernel<<<dim3(cdiv(v, UNPACK_ET), (unsigned)o, (unsigned)b.nsys), 256, sm, st>>>(
-        b, (int)o, (int)v, rcp_o, c->ld_ov, c->ld_o2, c->ld_k1, w.r2b, w.r2o, w.rk, c->ld_ot, w.rz);
+        b, (int)o, (int)v, c->ld_ov, c->ld_o2, c->ld_k1, w.r2b, w.r2o, w.rk, c->ld_ot, w.rz);
     GFCC_LAUNCH_CHECK();
   } else {
     unpack_ring_kernel<<<grid1d(o * C2 * ov), 256, 0, st>>>(b, (int)o, (int)v, c->ld_ov, w.r2b);
