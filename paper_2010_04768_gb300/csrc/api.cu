@@ -1582,6 +1582,7 @@ void gfcc_destroy(gfcc_ctx *c) {
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
   for (void *p : c->allocs) dfree(p);
   if (c->scratch) dfree(c->scratch);
+  if (c->step_flags) cudaFreeHost(c->step_flags);
   for (auto &lc : c->left_cache)
     if (lc.C) dfree(lc.C);
   if (c->kept.X) dfree(c->kept.X);

@@ -158,6 +158,10 @@ struct gfcc_ctx {
   long long prof_n[PH_COUNT] = {0};
   double prof_flops[PH_COUNT] = {0};
 
+  // where an Arnoldi step reports the state of each system to the host (mapped pinned memory, grown on demand; of the
+  // one solver that runs on the context)
+  int *step_flags = nullptr, *step_flags_dev = nullptr;
+  int step_flags_cap = 0;
   // scratch reused across solves (grown on demand)
   void *scratch = nullptr;
   size_t scratch_bytes = 0;

@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <chrono>
 #include <vector>
 
 #include "ctx.cuh"
@@ -162,7 +163,19 @@ __global__ void vupdate_kernel(const T *V, long long vs_stride, long long vi_str
     CT<T> acc = mkc<T>(0.0, 0.0);
     const double2 *cf = reinterpret_cast<const double2 *>(coef) + (long long)s * NV;
     const int nvv = nvs != nullptr ? nvs[s] : nv;
-    for (int i = 0; i < nvv; i++) {
+    int i = 0;
+    for (; i + 8 <= nvv; i += 8) {   // eight loads in flight
+      CT<T> a[8];
+#pragma unroll
+      for (int u = 0; u < 8; u++) a[u] = ldc(V + 2 * (s * vs_stride + (i + u) * vi_stride), mu);
+#pragma unroll
+      for (int u = 0; u < 8; u++) {
+        const T cx = (T)cf[i + u].x, cy = (T)cf[i + u].y;
+        acc.x += cx * a[u].x - cy * a[u].y;
+        acc.y += cx * a[u].y + cy * a[u].x;
+      }
+    }
+    for (; i < nvv; i++) {
       const CT<T> a = ldc(V + 2 * (s * vs_stride + i * vi_stride), mu);
       const T cx = (T)cf[i].x, cy = (T)cf[i].y;
       acc.x += cx * a.x - cy * a.y;
@@ -220,6 +233,7 @@ struct Lsq {
   double tol;
   int *state, *kcyc, *iters;
   double *est;
+  volatile int *flags;   // mapped host memory (or nullptr): iterations of the system << 3 | its state
 };
 constexpr int LSQ_MAX = 66;   // m + 2 <= 66
 
@@ -290,10 +304,12 @@ __device__ void givens_update(const Lsq &q, int s, int k, const double *h, int N
     const double res = sqrt(g1.x * g1.x + g1.y * g1.y);
     q.est[s] = bn > 0.0 ? res / bn : 0.0;
     const bool breakdown = !(hk1 > 1e-14 * den);
-    if (res <= q.tol * bn || breakdown || k + 1 == m || den == 0.0) {
+    const bool done = res <= q.tol * bn || breakdown || k + 1 == m || den == 0.0;
+    if (done) {
       q.state[s] = ST_CYCLE_DONE;
       q.kcyc[s] = k + 1;
     }
+    if (q.flags != nullptr) q.flags[s] = (it + 1) << 3 | (done ? ST_CYCLE_DONE : ST_IN_CYCLE);
   }
   __syncthreads();
   if (t < k) {
@@ -728,6 +744,16 @@ __global__ void precondition_kernel(T *U, long long n, int nsys, const double *o
   }
 }
 
+// V_0 of every system = 0
+template <typename T>
+__global__ void zero_first_kernel(T *V, long long vs, long long n, int nsys) {
+  const long long tot = n * nsys;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
+    const long long s = t / n;
+    stc(V + 2 * s * vs, t - s * n, mkc<T>(0.0, 0.0));
+  }
+}
+
 __global__ void norm_from_partial_kernel(int nsys, const double *nrm2, int NV, double *out) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s < nsys) out[s] = sqrt(fmax(nrm2[2 * (long long)s * NV], 0.0));
@@ -784,6 +810,19 @@ int Gmres::init(gfcc_ctx *ctx, int sec, long long dim, int ns, int mm, double *w
   f32 = mixed && c->inner_fp64 == 0;
   sector = sec;
   n = dim;
+  if (c->step_flags_cap < ns) {
+    if (c->step_flags) cudaFreeHost(c->step_flags);   // no solver of this context is running
+    c->step_flags = c->step_flags_dev = nullptr;
+    c->step_flags_cap = 0;
+    if (cudaHostAlloc(reinterpret_cast<void **>(&c->step_flags), sizeof(int) * ns, cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer(reinterpret_cast<void **>(&c->step_flags_dev), c->step_flags, 0) != cudaSuccess) {
+      cudaGetLastError();   // none: the steps wait for the stream
+      if (c->step_flags) cudaFreeHost(c->step_flags);
+      c->step_flags = c->step_flags_dev = nullptr;
+    } else {
+      c->step_flags_cap = ns;
+    }
+  }
   nsys = ns;
   m = mm;
   NV = m + 2;
@@ -942,7 +981,7 @@ int Gmres::arnoldi_t(const T *Vb, long long vs, int k, T *w, int active, double 
   // corrected by the FP64-accurate outer residual, only where the first pass cancelled more than 90% of w
   // (orthogonality loss <= 10 x about 1e-6 per vector).
   const double theta = sizeof(T) == sizeof(float) ? REORTH_THETA_F32 : 0.5;
-  const Lsq q{m, H, cs, sn, g, bnorm, tol, state, kcyc, iters, est};
+  const Lsq q{m, H, cs, sn, g, bnorm, tol, state, kcyc, iters, est, c->step_flags_dev};
   cgs_dots_kernel<T><<<dgrid, 32 * DOT_WARPS, 0, st>>>(Vb, vs, n, nv, w, n, dlen, state, nullptr, partial, NV, h, blk_cnt);
   GFCC_LAUNCH_CHECK();
   cgs_update_kernel<T, false><<<ugrid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, ulen, rflag, h, nullptr, theta, partial,
@@ -975,6 +1014,44 @@ int Gmres::solve(double tol, int max_iters, int *h_state, int max_cycles, bool u
              : solve_t<double>(tol, max_iters, h_state, max_cycles, use_x0);
 }
 
+// The Givens update of a system writes its iteration count and state to mapped host memory; the host reads them there
+// while the step's last kernel is still running, instead of a copy and a wait for the stream (some 10 us of idle GPU
+// a step).  Every 100 us without an answer the stream is asked: a failed one is an error, a finished one gives the
+// states by copy.
+int Gmres::wait_step(int *h_state, std::vector<int> &h_it) {
+  cudaStream_t st = c->stream;
+  bool copy = c->step_flags == nullptr;
+  auto last = std::chrono::steady_clock::now();
+  for (int s = 0; s < nsys && !copy; s++) {
+    if (h_state[s] != ST_IN_CYCLE) continue;
+    const int want = h_it[s] + 1;
+    int v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
+    for (unsigned spin = 1; (v >> 3) != want; spin++) {
+      if ((spin & 0xff) == 0 && std::chrono::steady_clock::now() - last > std::chrono::microseconds(100)) {
+        const cudaError_t e = cudaStreamQuery(st);
+        if (e != cudaErrorNotReady) {
+          GFCC_CUDA(e);
+          v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
+          copy = (v >> 3) != want;
+          break;
+        }
+        cudaGetLastError();
+        last = std::chrono::steady_clock::now();
+      }
+      v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
+    }
+    if (copy) break;
+    h_state[s] = v & 7;
+    h_it[s] = want;
+  }
+  if (copy) {
+    GFCC_CUDA(cudaMemcpyAsync(h_state, state, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
+    GFCC_CUDA(cudaMemcpyAsync(h_it.data(), iters, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
+    GFCC_CUDA(cudaStreamSynchronize(st));
+  }
+  return GFCC_OK;
+}
+
 template <typename T>
 int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool use_x0) {
   cudaStream_t st = c->stream;
@@ -1005,7 +1082,10 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
     precondition_kernel<T><<<grid1d(n * nsys), TH, 0, st>>>(Ut, n, nsys, omega, eta, zsg, dg, dsg);
     GFCC_LAUNCH_CHECK();
   }
-  GFCC_CUDA(cudaMemsetAsync(Vt, 0, sizeof(T) * 2 * nsys * (m + 1) * n, st));
+  // V_0 of systems that never enter a cycle is read by the operator (a column of its own): zero.  The other basis
+  // vectors are written before they are read (clearing all of them took 0.45 ms at o=40 v=200).
+  zero_first_kernel<T><<<grid1d(n * nsys), TH, 0, st>>>(Vt, vs, n, nsys);
+  GFCC_LAUNCH_CHECK();
   GFCC_CUDA(cudaMemsetAsync(iters, 0, sizeof(int) * nsys, st));
   GFCC_CUDA(cudaMemsetAsync(state, 0, sizeof(int) * nsys, st));   // ST_PENDING
   GFCC_CUDA(cudaMemsetAsync(blk_cnt, 0, sizeof(unsigned) * nsys, st));
@@ -1014,6 +1094,8 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
   norm_from_partial_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, nrm, NV, bnorm);
   GFCC_LAUNCH_CHECK();
   bool first = !use_x0;
+  std::vector<int> h_it(nsys, 0);
+  for (int s = 0; s < nsys && c->step_flags != nullptr; s++) c->step_flags[s] = 0;   // no step is in flight
   for (int cycle = 0;; cycle++) {
     if (max_cycles > 0 && cycle >= max_cycles) {
       // cycle budget spent: the systems still pending keep their iterate (state 4)
@@ -1113,8 +1195,7 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
         }
       }
       if (!done_step) GFCC_TRY(step());
-      GFCC_CUDA(cudaMemcpyAsync(h_state, state, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
-      GFCC_CUDA(cudaStreamSynchronize(st));
+      GFCC_TRY(wait_step(h_state, h_it));
       active = 0;
       for (int s = 0; s < nsys; s++) active += h_state[s] == ST_IN_CYCLE;
       if (active == 0) break;

@@ -38,6 +38,8 @@ struct Gmres {
   int *state = nullptr, *kcyc = nullptr, *iters = nullptr, *rflag = nullptr;
   unsigned *blk_cnt = nullptr;      // per system: blocks of the running kernel that have finished
   long long partial_chunks = 0;     // chunks of partial sums over all systems that `partial` holds
+  // host side of an Arnoldi step: the state of the systems in cycle, as soon as their Givens update has run
+  int wait_step(int *h_state, std::vector<int> &h_it);
   int *act = nullptr;   // the systems the operator runs on in an Arnoldi step (see solve_t)
   double *relres0 = nullptr;   // relative residual of the initial iterate (first true residual)
   double *sigma_work = nullptr;
