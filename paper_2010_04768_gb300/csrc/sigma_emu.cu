@@ -136,6 +136,93 @@ __global__ void digits_k2_kernel(const double *x, long long ldx, int C2, int o, 
   }
 }
 
+// The digits of a value for the kernel below: Y = round(y 2^(6S)) plus 32 in every base-64 place, so that digit k is a
+// plain field minus 32 (the first may reach 64 - 32); the value of each digit is exact in BF16.
+__device__ __forceinline__ unsigned long long biased_digits(double val, int ex, int S) {
+  const unsigned long long bias = 32ULL * (((S < 10 ? 1ULL << (6 * S) : 0ULL) - 1ULL) / 63ULL);
+  return (unsigned long long)fixed_point(val, ex, 6 * S) + bias;
+}
+// digit k (of S) as the FP32 bits of its value
+__device__ __forceinline__ unsigned digit_bits(unsigned long long Y, int k, int S) {
+  const unsigned u = (unsigned)(Y >> (6 * (S - 1 - k))) & (k == 0 ? 127u : 63u);
+  return __float_as_uint(__uint_as_float(0x4b000000u | u) - 8388640.0f);   // 2^23 + u - (2^23 + 32)
+}
+// the digits of values 2 q - odd and the next of a run of len (get(i): the biased digits of value i) to the S planes of
+// the row at p (odd: the parity of p in values), two values a store where the address allows it
+template <typename Get>
+__device__ __forceinline__ void put_digit_pair(__nv_bfloat16 *p, long long plane, int S, int odd, int len, int q, Get get) {
+  const int i0 = 2 * q - odd, i1 = i0 + 1;
+  const bool in0 = i0 >= 0 && i0 < len, in1 = i1 < len;
+  if (!in0 && !in1) return;
+  const unsigned long long y0 = in0 ? get(i0) : 0ULL, y1 = in1 ? get(i1) : 0ULL;
+  p += i0;
+#pragma unroll 4
+  for (int k = 0; k < S; k++, p += plane) {
+    const unsigned h = __byte_perm(digit_bits(y0, k, S), digit_bits(y1, k, S), 0x7632);
+    if (in0 && in1)
+      *reinterpret_cast<unsigned *>(p) = h;
+    else if (in0)
+      *reinterpret_cast<unsigned short *>(p) = (unsigned short)h;
+    else
+      *reinterpret_cast<unsigned short *>(p + 1) = (unsigned short)(h >> 16);
+  }
+}
+
+// digit planes of the three 2h1p layouts (ring r2b, oooo r2o, long K rk; see the three kernels above) in one pass: one
+// block per (32 e, m, plane c), the fixed-point values of r2[m, j, e] in shared memory.  Bound by instructions and by the
+// 1.2 GB written for 40 systems of o=40 v=200: 432 us (with a kernel for each layout and a digit a store 1040 us).
+constexpr int DIG_ET = 32;
+constexpr int DIG_MAX_O = 180;   // o x (DIG_ET + 1) values within the default 48 KB
+__global__ __launch_bounds__(256) void digits_ip_kernel(const double *x, long long ldx, int C2, int o, int v,
+                                                        const int *ec, int S, long long ld_b, __nv_bfloat16 *r2b,
+                                                        int *exp_b, long long ld_o, __nv_bfloat16 *r2o, int *exp_o,
+                                                        long long ldk, __nv_bfloat16 *rk) {
+  extern __shared__ unsigned long long td[];   // [o][DIG_ET + 1]
+  constexpr int LD = DIG_ET + 1;
+  const int e0 = blockIdx.x * DIG_ET, m = blockIdx.y, c = blockIdx.z;
+  const int et = min(DIG_ET, v - e0), lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ex = ec[c];
+  const double *xs = x + 2 * ((long long)(c >> 1) * ldx + o + e0 + lane) + (c & 1);
+#pragma unroll 4
+  for (int j = warp; j < o; j += 8) {
+    double val = 0.0;
+    if (lane < et && j != m) {
+      const int lo = min(m, j), hi = max(m, j);
+      val = xs[2 * (long long)((lo * o - lo * (lo + 1) / 2 + hi - lo - 1) * v)];
+      if (m > j) val = __hiloint2double(__double2hiint(val) ^ 0x80000000, __double2loint(val));
+    }
+    td[j * LD + lane] = biased_digits(val, ex, S);
+  }
+  if (m == 0) {
+    if (blockIdx.x == 0)
+      for (int j = threadIdx.x; j < o; j += 256) exp_b[(long long)j * C2 + c] = ex;
+    if (threadIdx.x < et) exp_o[(long long)(e0 + threadIdx.x) * C2 + c] = ex;
+  }
+  __syncthreads();
+  const long long plane_b = (long long)o * C2 * ld_b, plane_o = (long long)v * C2 * ld_o, plane_k = (long long)C2 * ldk;
+  {
+    const long long col = (long long)m * v + e0;
+    const int q = lane & 15, odd = (int)(col & 1);
+    for (int j = 2 * warp + (lane >> 4); j < o; j += 16) {
+      const unsigned long long *row = td + j * LD;
+      __nv_bfloat16 *p = r2b + ((long long)j * C2 + c) * ld_b + col;
+      auto get = [&](int i) { return row[i]; };
+      put_digit_pair(p, plane_b, S, odd, et, q, get);
+      if (odd && q == 0) put_digit_pair(p, plane_b, S, odd, et, 16, get);
+    }
+  }
+  const int half = o / 2 + 1 <= 16 ? 1 : 0, q0 = half ? lane & 15 : lane, step = half ? 16 : 32;
+  for (int el = half ? 2 * warp + (lane >> 4) : warp; el < et; el += half ? 16 : 8) {
+    const unsigned long long *col = td + el;
+    auto get = [&](int j) { return col[j * LD]; };
+    __nv_bfloat16 *po = r2o + ((long long)(e0 + el) * C2 + c) * ld_o + (long long)m * o;
+    const long long at = ((long long)m * v + e0 + el) * o;
+    for (int q = q0; q <= o / 2; q += step) {
+      put_digit_pair(po, plane_o, S, (m * o) & 1, o, q, get);
+      put_digit_pair(rk + (long long)c * ldk + at, plane_k, S, (int)(at & 1), o, q, get);
+    }
+  }
+}
+
 // digit planes of the r1 part: rk[c][o2v + m] (and the zero padding of rk up to ldk) and, when ld1 > 0,
 // r1b[c][m] (zero up to ld1); exponents of the operands written
 __global__ void digits_k1_kernel(const double *x, long long ldx, int C2, int o, int v, const int *ec, int S,
@@ -371,15 +458,23 @@ int apply_ip_emu(gfcc_ctx *c, const SysBatch &b, double *work, long long work_do
     {
     PhaseTimer tu(c, PH_UNPACK);
     GFCC_TRY(plane_exponents(st, x, b.ldx, n, (int)(C2 / 2), w.ec));
-    digits_ring_kernel<<<grid1d(w.r2b.rows * w.r2b.ld), 256, 0, st>>>(x, b.ldx, C2, (int)o, (int)v, w.ec, S, w.r2b.ld,
-                                                                       w.r2b.dig, w.r2b.exp2);
-    GFCC_LAUNCH_CHECK();
-    digits_oooo_kernel<<<dim3(cdiv(w.r2o.ld, 32), cdiv(v, 32), C2), dim3(32, 8), 0, st>>>(
-        x, b.ldx, C2, (int)o, (int)v, w.ec, S, w.r2o.ld, w.r2o.dig, w.r2o.exp2);
-    GFCC_LAUNCH_CHECK();
-    digits_k2_kernel<<<dim3(cdiv(o, 32), cdiv(v, 32), o * C2), dim3(32, 8), 0, st>>>(x, b.ldx, C2, (int)o, (int)v,
-                                                                                    w.ec, S, w.rk.ld, w.rk.dig);
-    GFCC_LAUNCH_CHECK();
+    if (v > 0 && o <= DIG_MAX_O) {
+      const size_t sm = (size_t)o * (DIG_ET + 1) * sizeof(unsigned long long);
+      digits_ip_kernel<<<dim3(cdiv(v, DIG_ET), (unsigned)o, (unsigned)C2), 256, sm, st>>>(
+          x, b.ldx, (int)C2, (int)o, (int)v, w.ec, S, w.r2b.ld, w.r2b.dig, w.r2b.exp2, w.r2o.ld, w.r2o.dig, w.r2o.exp2,
+          w.rk.ld, w.rk.dig);
+      GFCC_LAUNCH_CHECK();
+    } else {   // a kernel for each layout, whatever o
+      digits_ring_kernel<<<grid1d(w.r2b.rows * w.r2b.ld), 256, 0, st>>>(x, b.ldx, C2, (int)o, (int)v, w.ec, S, w.r2b.ld,
+                                                                         w.r2b.dig, w.r2b.exp2);
+      GFCC_LAUNCH_CHECK();
+      digits_oooo_kernel<<<dim3(cdiv(w.r2o.ld, 32), cdiv(v, 32), C2), dim3(32, 8), 0, st>>>(
+          x, b.ldx, C2, (int)o, (int)v, w.ec, S, w.r2o.ld, w.r2o.dig, w.r2o.exp2);
+      GFCC_LAUNCH_CHECK();
+      digits_k2_kernel<<<dim3(cdiv(o, 32), cdiv(v, 32), o * C2), dim3(32, 8), 0, st>>>(x, b.ldx, C2, (int)o, (int)v,
+                                                                                      w.ec, S, w.rk.ld, w.rk.dig);
+      GFCC_LAUNCH_CHECK();
+    }
     // (the 1h block also enters [r1 | Z] of the concatenated ovoo / three-body product, sliced there)
     digits_k1_kernel<<<grid1d((long long)C2 * (w.rk.ld - o2v)), 256, 0, st>>>(
         x, b.ldx, C2, (int)o, (int)v, w.ec, S, w.rk.ld, w.rk.dig, w.rk.exp2, 0, nullptr, nullptr);

@@ -162,7 +162,13 @@ struct SysIn {
     di2 = di * di;
     sgn = with_sign(b.dsign, 1.f);
   }
-  __device__ __forceinline__ Cz operator()(long long mu) const {
+  // counting from element off
+  __device__ __forceinline__ void shift(long long off) {
+    if (xf != nullptr) xf += off;
+    if (x != nullptr) x += off;
+    if (diag != nullptr) diag += off;
+  }
+  __device__ __forceinline__ Cz operator()(int mu) const {
     Cz u;
     if (xf != nullptr) {
       const float2 t = xf[mu];
@@ -226,13 +232,14 @@ __global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v
   const int e0 = blockIdx.x * UNPACK_ET, m = blockIdx.y, s = blockIdx.z;
   const int et = min(UNPACK_ET, v - e0);
   const int C2 = 2 * b.nsys, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const SysIn in(b, s);
+  SysIn in(b, s);
+  in.shift(o + e0 + lane);
 #pragma unroll 4
   for (int j = warp; j < o; j += 8) {
     unsigned h = 0u;
     if (lane < et && j != m) {
       const int lo = min(m, j), hi = max(m, j);
-      h = pack_bf16(in(o + (long long)(lo * o - lo * (lo + 1) / 2 + hi - lo - 1) * v + e0 + lane));
+      h = pack_bf16(in((lo * o - lo * (lo + 1) / 2 + hi - lo - 1) * v));
       if (m > j) h ^= 0x80008000u;
     }
     tl[j * LD + lane] = h;
@@ -333,13 +340,15 @@ __global__ void unpack_ea_tile_kernel(SysBatch b, int o, int v, long long Pv, lo
   if (a0 == 0 && m == 0 && threadIdx.y == 0 && e0 + (int)threadIdx.x < v)
     put_r1(b, s, e0 + threadIdx.x, (long long)o * v * v, ldk, rk, ld_ot, rz);
   const bool below = e0 + 31 < a0;   // every a > e: packed pairs (e, a) run along a
-  const SysIn in(b, s);
+  SysIn in(b, s);
+  in.shift(v + (long long)m * Pv);
 #pragma unroll
   for (int r = threadIdx.y; r < 32; r += 8) {
     const int a = below ? a0 + lane : a0 + r, e = below ? e0 + r : e0 + lane;
     unsigned h = 0u;
     if (a < v && e < v && a != e) {
-      h = pack_bf16(in(v + (long long)m * Pv + pair_index(min(a, e), max(a, e), v)));
+      const int lo = min(a, e), hi = max(a, e);
+      h = pack_bf16(in((int)((unsigned)lo * (unsigned)(2 * v - lo - 1) / 2) + hi - lo - 1));   // pair_index in 32 bits
       if (a > e) h ^= 0x80008000u;
     }
     if (below)
@@ -364,15 +373,18 @@ __global__ void unpack_ea_tile_kernel(SysBatch b, int o, int v, long long Pv, lo
 }
 
 // r2p[(i, c)][ef] = y2[i, e < f] (row i of the packed 2p1h block), both planes; grid
-// (cdiv(Pv, 256), o * nsys)
-__global__ void unpack_ea_pairs_kernel(SysBatch b, int o, int v, long long Pv, long long ld, __nv_bfloat16 *out) {
+// (cdiv(Pv, 512), o * nsys)
+__global__ __launch_bounds__(256) void unpack_ea_pairs_kernel(SysBatch b, int o, int v, long long Pv, long long ld,
+                                                              __nv_bfloat16 *out) {
   const int i = (int)(blockIdx.y % (unsigned)o), s = (int)(blockIdx.y / (unsigned)o);
-  const long long ef = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int ef = 2 * (int)(blockIdx.x * 256 + threadIdx.x);   // two values a thread; rows have room for an even count
   if (ef >= Pv) return;
-  const Cz u = load_u(b, s, v + (long long)i * Pv + ef);
-  const long long row = (long long)i * 2 * b.nsys + 2 * s;
-  out[row * ld + ef] = __float2bfloat16(u.r);
-  out[(row + 1) * ld + ef] = __float2bfloat16(u.i);
+  SysIn in(b, s);
+  in.shift(v + (long long)i * Pv);
+  const unsigned u0 = pack_bf16(in(ef)), u1 = ef + 1 < Pv ? pack_bf16(in(ef + 1)) : 0u;
+  __nv_bfloat16 *re = out + ((long long)i * 2 * b.nsys + 2 * s) * ld + ef;
+  *reinterpret_cast<unsigned *>(re) = __byte_perm(u0, u1, 0x5410);
+  *reinterpret_cast<unsigned *>(re + ld) = __byte_perm(u0, u1, 0x7632);
 }
 
 constexpr int KSPLIT = 76;   // split of the long-K contraction (Z and the one-index row): two row tiles fill 152 SMs
@@ -515,7 +527,7 @@ int apply_ea_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
         b, (int)o, (int)v, Pv, c->ld_ov, c->ld_k1e, w.r2e, w.rk, c->ld_ot, w.rz);
     GFCC_LAUNCH_CHECK();
     if (Pv > 0) {
-      unpack_ea_pairs_kernel<<<dim3(cdiv(Pv, 256), (unsigned)(o * b.nsys)), 256, 0, st>>>(b, (int)o, (int)v, Pv,
+      unpack_ea_pairs_kernel<<<dim3(cdiv(Pv, 512), (unsigned)(o * b.nsys)), 256, 0, st>>>(b, (int)o, (int)v, Pv,
                                                                                         c->ld_pv, w.r2p);
       GFCC_LAUNCH_CHECK();
     }
