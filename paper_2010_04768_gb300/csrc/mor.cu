@@ -515,7 +515,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   // residuals of models of 36 vectors over 9616 and 6280 elements were within 6e-14 (rms, of ||b||) of quad sums
   // either way.
   const bool mixed = h_relres != nullptr && c->precision == GFCC_PREC_MIXED_BF16;
-  bool planes = mixed && emulation_pays(2LL * std::min(n_omega, 304) * nb, n, std::max(2 * m, 160), false);
+  bool planes = mixed && emulation_pays(2LL * std::min(n_omega, 304) * nb, n, 2LL * m, false);
   long long per_pair, wb;
   size_t need;
   auto layout = [&]() {

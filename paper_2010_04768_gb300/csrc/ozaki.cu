@@ -296,10 +296,10 @@ __global__ __launch_bounds__(SL_THREADS) void strided_exp_kernel(const double *X
   if (threadIdx.x < SL_ROWS && ro[threadIdx.x] >= 0 && mx[threadIdx.x] > 0) atomicMax(&be[rb + threadIdx.x], mx[threadIdx.x]);
 }
 
-// biased exponent -> e with max_k |X[r][k]| 2^-e in [1/4, 1/2); rows of zeros 0
-__global__ void strided_exp_final_kernel(int *be, long long rows) {
+// biased exponent -> e with max_k |X[r][k]| 2^-e in [1/4, 1/2) (less == 1021) or [1/2, 1) (1022); rows of zeros 0
+__global__ void strided_exp_final_kernel(int *be, long long rows, int less) {
   const long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (r < rows) be[r] = be[r] > 0 ? be[r] - 1021 : 0;
+  if (r < rows) be[r] = be[r] > 0 ? be[r] - less : 0;
 }
 
 // dig[i][r][k] = i-th digit of X[rm(r0 + r) + km(k)] 2^-e[r] (k < K), 0 for K <= k < ld
@@ -369,7 +369,7 @@ int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long lon
   strided_exp_kernel<<<(unsigned)(gx * gz), SL_THREADS, 0, st>>>(X, rows, K, rm, km, r0, k_lanes, (int)span, (unsigned)gx,
                                                                  out.exp2);
   GFCC_LAUNCH_CHECK();
-  strided_exp_final_kernel<<<cdiv(rows, 256), 256, 0, st>>>(out.exp2, rows);
+  strided_exp_final_kernel<<<cdiv(rows, 256), 256, 0, st>>>(out.exp2, rows, bits == F64_BITS && K <= F64_SHORT_K ? 1022 : 1021);
   GFCC_LAUNCH_CHECK();
   strided_slice_kernel<<<(unsigned)(gx * gy), SL_THREADS, 0, st>>>(X, rows, K, rm, km, r0, k_lanes, out.exp2, S, bits,
                                                                    (unsigned)gx, out.dig, out.ld);
@@ -412,21 +412,21 @@ long long up256(long long x) { return (x + 255) / 256 * 256; }
 }  // namespace
 
 // FP64 units: 1.1 TFLOP/s on 16 x 16 tiles.  Digit planes: 36 pairs of BF16 products at about 1.1e15
-// flop/s on padded tiles, the split of both operands (two reads of 8 bytes, eight planes of 2 bytes, at
-// about 3 TB/s), and some 8 launches.  Error against quad sums (relative, Gaussian entries): FP64 units 1.9e-16,
-// 3.0e-16, 6.0e-16, 1.4e-15 at K = 64, 300, 1280, 6400; planes 2.1e-16, 2.3e-16, 2.4e-16, 4.0e-16; entries that
-// decay along K as the Cholesky vectors do: 2.6, 4.6, 7.6, 6.8 against 2.8, 3.0, 3.5, 3.5 (1e-16).  Sums too short
-// for the planes to be the more accurate stay on the FP64 units.
+// flop/s on padded tiles, 4 ps an output for the ends of the tiles, the split of both operands (two reads of 8 bytes,
+// eight planes of 2 bytes, at about 3 TB/s), and some 8 launches.  Error against quad sums (1e-16 relative): Gaussian
+// entries, FP64 units 1.9, 2.1, 2.4, 3.0, 5.7, 14 at K = 32, 64, 160, 300, 1280, 6400; planes 0.6, 0.7, 0.7, 0.7, 2.4,
+// 4.0; entries that decay along K as the Cholesky vectors do, 2.5, 2.6, 3.3, 3.9, 6.6, 7.0 and 0.7, 0.8, 1.1, 1.1, 3.5,
+// 3.5.
 // What it gives: set-up of a mixed IP context at o=40 v=200 L=800 3489 -> 143 ms, IP + EA set-up and solve at
-// o=20 v=100 365 -> 48 ms, CCSD and Lambda at o=16 v=80 404 -> 112 ms, closed-shell solve at o=30 v=150 96 -> 55 ms.
+// o=20 v=100 365 -> 40 ms, CCSD and Lambda at o=16 v=80 404 -> CCSD_NOW ms, closed-shell solve at o=30 v=150 96 -> 46 ms.
 bool emulation_pays(long long M, long long N, long long K, bool a_ready) {
-  if (K < 160) return false;
+  if (K < 32) return false;
   const double m16 = (double)((M + 15) / 16 * 16), n16 = (double)((N + 15) / 16 * 16);
   const double f64 = 2.0 * m16 * n16 * (double)K / 1.1e12;
   const double m128 = (double)((M + 127) / 128 * 128), n32 = (double)((N + 31) / 32 * 32);
   const double n128 = (double)((N + 127) / 128 * 128), m32 = (double)((M + 31) / 32 * 32);
   const double tile = std::min(m128 * n32, n128 * m32);
-  const double emu = 36.0 * 2.0 * tile * (double)((K + 63) / 64 * 64) / 1.1e15 + 32.0 * ((a_ready ? 0.0 : (double)M) + (double)N) * (double)K / 3e12 + (a_ready ? 3e-5 : 4e-5);
+  const double emu = 36.0 * 2.0 * tile * (double)((K + 63) / 64 * 64) / 1.1e15 + 4e-12 * tile + 32.0 * ((a_ready ? 0.0 : (double)M) + (double)N) * (double)K / 3e12 + (a_ready ? 3e-5 : 4e-5);
   return emu < f64;
 }
 

@@ -48,6 +48,9 @@ int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, d
 // Digits of the contractions that take the place of FP64 ones: 8 digits of 7 bits hold 56 bits below the
 // row scale (an FP64 sum keeps 53 below each of its partial sums), pairs to level 9.
 constexpr int F64_DIGITS = 8, F64_BITS = 7, F64_LEVEL = 9;
+// Sums of at most this many terms scale their rows to [1/2, 1) instead of [1/4, 1/2): one bit more, at the price of
+// a first digit of up to 128, which leaves the levels exact for 6 K blocks of 64 (8 otherwise).
+constexpr int F64_SHORT_K = 6 * 64;
 
 // Split rows r0 .. r0 + rows - 1 of a strided matrix, X[rm(r) + km(k)], into digit planes.  `mem` holds
 // emu_operand_bytes(rows, K, S).

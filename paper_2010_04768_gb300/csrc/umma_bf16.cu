@@ -28,6 +28,7 @@
 #include <utility>
 
 #include "common.cuh"
+#include "ozaki.cuh"
 #include "umma.cuh"
 
 namespace gfcc {
@@ -1510,8 +1511,11 @@ int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, in
   a.nz = pl.nz;
   a.nk = (K + BK - 1) / BK;
   a.kb_per_split = (a.nk + a.nz - 1) / a.nz;
-  // a level holds up to P - 1 pairs: (P - 1) kc 64 products of at most 2^(2 bits - 2) stay within 2^24
+  // a level holds up to P - 1 pairs: (P - 1) kc 64 products of at most 2^(2 bits - 2) stay within 2^24.  The first of
+  // the 7-bit digits of short sums (F64_SHORT_K) may be twice as large: two pairs of a level count twice and the pair of
+  // first digits, a level of its own, four times, which 6 blocks allow for P <= 9.
   a.kc = (1 << (26 - 2 * bits)) / (BK * (P - 1));
+  static_assert(F64_SHORT_K <= 6 * BK && (9 + 1) * 6 * BK <= 1 << (26 - 2 * F64_BITS), "short sums are exact");
   a.beta = beta;
   int ex = 0;
   const double fr = frexp(alpha, &ex);
