@@ -51,6 +51,31 @@ long long thread_launch_count();   // the calling thread's share (concurrent sol
     GFCC_CUDA(cudaGetLastError()); \
   } while (0)
 
+// Chained launches: the kernels of an Arnoldi step follow one another with some microseconds of work each, so the
+// gap between two of them counts.  A kernel launched by launch_chained may be scheduled while the kernel before it in
+// the stream still runs (its blocks then hold no more than their slots) and starts with chain_start: it lets its own
+// successor be scheduled, then waits until the kernels before it have completed and their writes are visible.  Every
+// thread does so before it touches memory or TMEM, so the order of the stream's accesses is that of plain launches.
+__device__ __forceinline__ void chain_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                         Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 // Index map of a flattened GEMM index x onto a tensor offset:
 //   d0 <= 0 : x * s0
 //   d0  > 0 : (x % d0) * s0 + (x / d0) * s1      (two tensor indices fused into one GEMM index)

@@ -146,6 +146,7 @@ template <typename TIn, int MODE>
 __global__ __launch_bounds__(THREADS) void ip2_kernel(SysBatch b, int o, int v, long long C2, int s0, int ns, int Po,
                                                        const TIn *T, const TIn *Q, const TIn *U, const TIn *S1,
                                                        const double *diag) {
+  chain_start();
   using P2 = typename Pair<TIn>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   P2 *tile = reinterpret_cast<P2 *>(smem);
@@ -201,6 +202,7 @@ template <typename TIn, int MODE>
 __global__ __launch_bounds__(THREADS) void ea2_kernel(SysBatch b, int o, int v, long long Pv, long long C2, int s0,
                                                        int ns, const TIn *T, const TIn *Qp, const TIn *U, const TIn *S1,
                                                        const double *diag) {
+  chain_start();
   using P2 = typename Pair<TIn>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   P2 *tile = reinterpret_cast<P2 *>(smem);
@@ -267,8 +269,8 @@ int launch_ip(cudaStream_t st, const SysBatch &b, int o, int v, const TIn *S1, c
   for (int s0 = 0; s0 < b.nsys; s0 += max_systems<TIn>()) {
     const int ns = b.nsys - s0 < max_systems<TIn>() ? b.nsys - s0 : max_systems<TIn>();
     const size_t sm = (size_t)A * (ns + 1) * 2 * sizeof(TIn);
-    ip2_kernel<TIn, MODE><<<dim3((unsigned)Po + one_index_blocks(o, ns), std::max(1u, cdiv(v, A))), THREADS, sm, st>>>(
-        b, o, v, C2, s0, ns, (int)Po, T, Q, U, S1, diag);
+    GFCC_CUDA(launch_chained(ip2_kernel<TIn, MODE>, dim3((unsigned)Po + one_index_blocks(o, ns), std::max(1u, cdiv(v, A))), THREADS, sm, st, 
+        b, o, v, C2, s0, ns, (int)Po, T, Q, U, S1, diag));
     GFCC_LAUNCH_CHECK();
   }
   return GFCC_OK;
@@ -282,8 +284,8 @@ int launch_ea(cudaStream_t st, const SysBatch &b, int o, int v, long long Pv, co
   for (int s0 = 0; s0 < b.nsys; s0 += max_systems<TIn>()) {
     const int ns = b.nsys - s0 < max_systems<TIn>() ? b.nsys - s0 : max_systems<TIn>();
     const size_t sm = (size_t)A * (ns + 1) * 2 * sizeof(TIn);
-    ea2_kernel<TIn, MODE><<<dim3((unsigned)o + one_index_blocks(v, ns), std::max(1u, cdiv(Pv, A))), THREADS, sm, st>>>(
-        b, o, v, Pv, C2, s0, ns, T, Qp, U, S1, diag);
+    GFCC_CUDA(launch_chained(ea2_kernel<TIn, MODE>, dim3((unsigned)o + one_index_blocks(v, ns), std::max(1u, cdiv(Pv, A))), THREADS, sm, st, 
+        b, o, v, Pv, C2, s0, ns, T, Qp, U, S1, diag));
     GFCC_LAUNCH_CHECK();
   }
   return GFCC_OK;

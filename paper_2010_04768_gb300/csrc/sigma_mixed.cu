@@ -227,6 +227,7 @@ constexpr int UNPACK_MAX_O = 180;   // tile o x (UNPACK_ET + 1) words within the
 __global__ __launch_bounds__(256) void unpack_ip_kernel(SysBatch b, int o, int v, long long ld_ov, long long ld_o2,
                                                         long long ld_k1, __nv_bfloat16 *r2b, __nv_bfloat16 *r2o,
                                                         __nv_bfloat16 *rk, long long ld_ot, __nv_bfloat16 *rz) {
+  chain_start();
   extern __shared__ unsigned tl[];   // [o][UNPACK_ET + 1] (re, im) in BF16
   constexpr int LD = UNPACK_ET + 1;
   const int e0 = blockIdx.x * UNPACK_ET, m = blockIdx.y, s = blockIdx.z;
@@ -288,6 +289,7 @@ __global__ void unpack_r1_kernel(SysBatch b, int o, int v, long long ldk, __nv_b
 // each: with one thread for an output, which walks all splits, it took 14.7 us whatever the size.
 __global__ __launch_bounds__(256) void reduce_splits_kernel(const float *part, int nsplit, int rows, int cols,
                                                             int nz_rows, __nv_bfloat16 *zT, long long ldT, float *S1) {
+  chain_start();
   __shared__ float sh[8][33];
   const long long tot = (long long)rows * cols;
   const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
@@ -332,6 +334,7 @@ __device__ __forceinline__ Cz y2_at(const SysBatch &b, int v, long long Pv, int 
 // both along e.  grid (cdiv(v, 32), cdiv(v, 32), o * nsys), block (32, 8).
 __global__ void unpack_ea_tile_kernel(SysBatch b, int o, int v, long long Pv, long long ld_ov, long long ldk,
                                       __nv_bfloat16 *r2e, __nv_bfloat16 *rk, long long ld_ot, __nv_bfloat16 *rz) {
+  chain_start();
   __shared__ unsigned tile[32][33];   // (re, im) in BF16
   const int e0 = blockIdx.x * 32, a0 = blockIdx.y * 32;
   const int m = (int)(blockIdx.z % (unsigned)o), s = (int)(blockIdx.z / (unsigned)o);
@@ -376,6 +379,7 @@ __global__ void unpack_ea_tile_kernel(SysBatch b, int o, int v, long long Pv, lo
 // (cdiv(Pv, 512), o * nsys)
 __global__ __launch_bounds__(256) void unpack_ea_pairs_kernel(SysBatch b, int o, int v, long long Pv, long long ld,
                                                               __nv_bfloat16 *out) {
+  chain_start();
   const int i = (int)(blockIdx.y % (unsigned)o), s = (int)(blockIdx.y / (unsigned)o);
   const int ef = 2 * (int)(blockIdx.x * 256 + threadIdx.x);   // two values a thread; rows have room for an even count
   if (ef >= Pv) return;
@@ -467,8 +471,8 @@ int apply_ip_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
   PhaseTimer tu(c, PH_UNPACK);
   if (v > 0 && o <= UNPACK_MAX_O) {
     const size_t sm = (size_t)o * (UNPACK_ET + 1) * sizeof(unsigned);
-    unpack_ip_kernel<<<dim3(cdiv(v, UNPACK_ET), (unsigned)o, (unsigned)b.nsys), 256, sm, st>>>(
-        b, (int)o, (int)v, c->ld_ov, c->ld_o2, c->ld_k1, w.r2b, w.r2o, w.rk, c->ld_ot, w.rz);
+    GFCC_CUDA(launch_chained(unpack_ip_kernel, dim3(cdiv(v, UNPACK_ET), (unsigned)o, (unsigned)b.nsys), 256, sm, st, 
+        b, (int)o, (int)v, c->ld_ov, c->ld_o2, c->ld_k1, w.r2b, w.r2o, w.rk, c->ld_ot, w.rz));
     GFCC_LAUNCH_CHECK();
   } else {
     unpack_ring_kernel<<<grid1d(o * C2 * ov), 256, 0, st>>>(b, (int)o, (int)v, c->ld_ov, w.r2b);
@@ -498,8 +502,8 @@ int apply_ip_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
     const int zs = umma_splits((int)(o2v + o), KSPLIT);
     GFCC_TRY(gemm_bf16_tn(st, c->VU_bf, c->ld_k1, w.rk, c->ld_k1, w.Zp, C2, (int)(v + o), (int)C2, (int)(o2v + o), 1.0f,
                           0.0f, zs, (v + o) * C2));
-    reduce_splits_kernel<<<cdiv((v + o) * C2, 32), 256, 0, st>>>(w.Zp, zs, (int)(v + o), (int)C2, (int)v, w.rz + o,
-                                                                 c->ld_ot, w.S1);
+    GFCC_CUDA(launch_chained(reduce_splits_kernel, cdiv((v + o) * C2, 32), 256, 0, st, w.Zp, zs, (int)(v + o), (int)C2, (int)v, w.rz + o,
+                                                                 c->ld_ot, w.S1));
     GFCC_LAUNCH_CHECK();
     GFCC_TRY(gemm_bf16_tn(st, c->WT_bf, c->ld_ot, w.rz, c->ld_ot, w.U, C2, (int)o2v, (int)C2, (int)(o + v), 1.0f,
                           0.0f));
@@ -523,12 +527,12 @@ int apply_ea_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
   PhaseTimer tsig(c, PH_SIGMA, b.nsys * sigma_flops(c, GFCC_SECTOR_EA));
   {
     PhaseTimer tu(c, PH_UNPACK);
-    unpack_ea_tile_kernel<<<dim3(cdiv(v, 32), cdiv(v, 32), (unsigned)(o * b.nsys)), dim3(32, 8), 0, st>>>(
-        b, (int)o, (int)v, Pv, c->ld_ov, c->ld_k1e, w.r2e, w.rk, c->ld_ot, w.rz);
+    GFCC_CUDA(launch_chained(unpack_ea_tile_kernel, dim3(cdiv(v, 32), cdiv(v, 32), (unsigned)(o * b.nsys)), dim3(32, 8), 0, st, 
+        b, (int)o, (int)v, Pv, c->ld_ov, c->ld_k1e, w.r2e, w.rk, c->ld_ot, w.rz));
     GFCC_LAUNCH_CHECK();
     if (Pv > 0) {
-      unpack_ea_pairs_kernel<<<dim3(cdiv(Pv, 512), (unsigned)(o * b.nsys)), 256, 0, st>>>(b, (int)o, (int)v, Pv,
-                                                                                        c->ld_pv, w.r2p);
+      GFCC_CUDA(launch_chained(unpack_ea_pairs_kernel, dim3(cdiv(Pv, 512), (unsigned)(o * b.nsys)), 256, 0, st, b, (int)o, (int)v, Pv,
+                                                                                        c->ld_pv, w.r2p));
       GFCC_LAUNCH_CHECK();
     }
   }
@@ -551,8 +555,8 @@ int apply_ea_mixed(gfcc_ctx *c, const SysBatch &b, double *work) {
     const int zs = umma_splits((int)(ov2 + v), KSPLIT);
     GFCC_TRY(gemm_bf16_tn(st, c->VUe_bf, c->ld_k1e, w.rk, c->ld_k1e, w.Zp, C2, (int)(o + v), (int)C2, (int)(ov2 + v),
                           1.0f, 0.0f, zs, (o + v) * C2));
-    reduce_splits_kernel<<<cdiv((o + v) * C2, 32), 256, 0, st>>>(w.Zp, zs, (int)(o + v), (int)C2, (int)o, w.rz + v,
-                                                                 c->ld_ot, w.S1);
+    GFCC_CUDA(launch_chained(reduce_splits_kernel, cdiv((o + v) * C2, 32), 256, 0, st, w.Zp, zs, (int)(o + v), (int)C2, (int)o, w.rz + v,
+                                                                 c->ld_ot, w.S1));
     GFCC_LAUNCH_CHECK();
     GFCC_TRY(gemm_bf16_tn(st, c->WTe_bf, c->ld_ot, w.rz, c->ld_ot, w.U, C2, (int)ov2, (int)C2, (int)(v + o), 1.0f,
                           0.0f));

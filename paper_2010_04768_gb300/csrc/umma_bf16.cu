@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     umma_bf16_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float *D,
                           long long ldd, int M, int N, int K, float alpha, float beta, int kb_per_split,
                           long long split_stride, UmmaCtl ctl) {
+  chain_start();
   constexpr int STAGES = Tile<BN, ST>::STAGES, A_BYTES = Tile<BN, ST>::A_BYTES,
                 STAGE_BYTES = Tile<BN, ST>::STAGE_BYTES;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -367,6 +368,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
     umma_persist_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                              float *D, long long ldd, int M, int N, int K, float alpha, float beta, int kb_per_split,
                              long long split_stride, int nM, int nN, int nsplit, UmmaCtl ctl) {
+  chain_start();
   constexpr int STAGES = PTile<BN>::STAGES, A_BYTES = PTile<BN>::A_BYTES, STAGE_BYTES = PTile<BN>::STAGE_BYTES;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -595,6 +597,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     umma_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float *D,
                           long long ldd, int M, int N, int K, float alpha, float beta, int kb_per_split,
                           long long split_stride, UmmaCtl ctl) {
+  chain_start();
   constexpr int STAGES = PairTile<PBN>::STAGES, A_BYTES = PairTile<PBN>::A_BYTES,
                 STAGE_BYTES = PairTile<PBN>::STAGE_BYTES, TMEM_COLS = PairTile<PBN>::TMEM_COLS;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -1199,8 +1202,8 @@ int launch_umma_st(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const
     return GFCC_ERR_ARG;
   }
   dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN, nsplit);
-  umma_bf16_gemm_kernel<BN, ST><<<grid, THREADS, Tile<BN, ST>::SMEM_BYTES, st>>>(ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
-                                                                         split_stride, umma_ctl());
+  GFCC_CUDA(launch_chained(umma_bf16_gemm_kernel<BN, ST>, grid, THREADS, Tile<BN, ST>::SMEM_BYTES, st, ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
+                                                                         split_stride, umma_ctl()));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1233,8 +1236,8 @@ int launch_umma_persist(cudaStream_t st, const __nv_bfloat16 *A, long long lda, 
     return GFCC_ERR_ARG;
   }
   const unsigned grid = (unsigned)std::min<long long>(tiles, sms);
-  umma_persist_gemm_kernel<BN><<<grid, PERSIST_THREADS, PTile<BN>::SMEM_BYTES, st>>>(
-      ma, mb, D, ldd, M, N, K, alpha, beta, kbs, split_stride, (int)nM, (int)nN, nsplit, umma_ctl());
+  GFCC_CUDA(launch_chained(umma_persist_gemm_kernel<BN>, grid, PERSIST_THREADS, PTile<BN>::SMEM_BYTES, st, 
+      ma, mb, D, ldd, M, N, K, alpha, beta, kbs, split_stride, (int)nM, (int)nN, nsplit, umma_ctl()));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1260,8 +1263,8 @@ int launch_umma_pair(cudaStream_t st, const __nv_bfloat16 *A, long long lda, con
     return GFCC_ERR_ARG;
   }
   dim3 grid((unsigned)(2 * mp), (N + PBN - 1) / PBN, nsplit);
-  umma_pair_gemm_kernel<PBN><<<grid, THREADS, PairTile<PBN>::SMEM_BYTES, st>>>(ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
-                                                                              split_stride, umma_ctl());
+  GFCC_CUDA(launch_chained(umma_pair_gemm_kernel<PBN>, grid, THREADS, PairTile<PBN>::SMEM_BYTES, st, ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
+                                                                              split_stride, umma_ctl()));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
