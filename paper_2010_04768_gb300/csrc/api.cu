@@ -70,6 +70,12 @@ int check_extent_bytes(const void *p, long long bytes, const char *what) {
 
 cudaError_t dmalloc(void **p, size_t bytes) {
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && g_emu_arena != nullptr && g_emu_arena->cap > 0) {
+    // no room beside the calling thread's workspace of emulated contractions, which its next one allocates again
+    cudaGetLastError();
+    g_emu_arena->release();
+    e = cudaMalloc(p, bytes);
+  }
   if (e == cudaSuccess) reg_alloc(*p, bytes);
   return e;
 }
