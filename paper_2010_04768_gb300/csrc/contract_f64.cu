@@ -83,6 +83,7 @@ struct KWalk {
 // the K range of a tile; its partial sums meet through distributed shared memory in rank order.
 template <int TM, int RM, int RN>
 __global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kcluster) {
+  chain_start();
   constexpr int TN = NT / TM, BM = TM * RM, BN = TN * RN;
   constexpr int LA = (BM * BK + NT - 1) / NT, LB = (BN * BK + NT - 1) / NT;
   __shared__ double As[2][BK][BM + 1];
@@ -240,19 +241,21 @@ template <int TM, int RM, int RN>
 int launch_contract(const Contract &c, int kcluster, long long mt, long long nt, cudaStream_t st) {
   dim3 grid((unsigned)mt, (unsigned)nt, (unsigned)(c.batch * c.nsplit));
   if (kcluster <= 1) {
-    contract_f64_kernel<TM, RM, RN><<<grid, NT, 0, st>>>(c, 1);
+    GFCC_CUDA(launch_chained(contract_f64_kernel<TM, RM, RN>, grid, dim3(NT), 0, st, c, 1));
   } else {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(NT);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // as launch_chained
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = (unsigned)kcluster;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     GFCC_CUDA(cudaLaunchKernelEx(&cfg, contract_f64_kernel<TM, RM, RN>, c, kcluster));
   }
   GFCC_LAUNCH_CHECK();

@@ -328,6 +328,7 @@ constexpr int VSCALE_UNROLL = 8, VSCALE_PER_BLOCK = 256 * VSCALE_UNROLL;
 template <typename T, bool GIVENS>
 __global__ __launch_bounds__(256) void vscale_kernel(T *w, long long ws_stride, long long n, const double *nrm2, int NV,
                                                      int idx, const int *state, int want, Lsq q) {
+  chain_start();
   __shared__ T factor;
   const int s = blockIdx.y;
   if (state != nullptr && state[s] != want) return;
@@ -474,6 +475,7 @@ template <typename T>
 __global__ __launch_bounds__(32 * DOT_WARPS, CgsShape<T>::DOT_PER_SM) void cgs_dots_kernel(
     const T *V, long long vs, long long vi, int nv, const T *w, long long n, int clen, const int *state, const int *flag,
     double *partial, int NV, double *out, unsigned *cnt) {
+  chain_start();
   constexpr int U = CgsShape<T>::DOT_UNROLL;
   __shared__ double2 parts[DOT_WARPS];
   const int s = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
@@ -580,6 +582,7 @@ __global__ __launch_bounds__(CGS_THREADS, CgsShape<T>::UPD_PER_SM) void cgs_upda
                                                                  long long n, int clen, int *flag, double *h,
                                                                  const double *h2, double theta, double *partial,
                                                                  int NV, unsigned *cnt, const int *state) {
+  chain_start();
   __shared__ CT<T> hh[72];
   __shared__ double sh[CGS_THREADS / 32];
   const int s = blockIdx.y, chunk = blockIdx.x, nch = gridDim.x;
@@ -984,17 +987,17 @@ int Gmres::arnoldi_t(const T *Vb, long long vs, int k, T *w, int active, double 
   const Lsq q{m, H, cs, sn, g, bnorm, tol, state, kcyc, iters, est, c->step_flags_dev};
   cgs_dots_kernel<T><<<dgrid, 32 * DOT_WARPS, 0, st>>>(Vb, vs, n, nv, w, n, dlen, state, nullptr, partial, NV, h, blk_cnt);
   GFCC_LAUNCH_CHECK();
-  cgs_update_kernel<T, false><<<ugrid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, ulen, rflag, h, nullptr, theta, partial,
-                                                             NV, blk_cnt, state);
+  GFCC_CUDA(launch_chained(cgs_update_kernel<T, false>, ugrid, CGS_THREADS, 0, st, Vb, vs, n, nv, w, n, ulen, rflag, h, nullptr, theta, partial,
+                                                             NV, blk_cnt, state));
   GFCC_LAUNCH_CHECK();
-  cgs_dots_kernel<T><<<dgrid, 32 * DOT_WARPS, 0, st>>>(Vb, vs, n, nv, w, n, dlen, state, rflag, partial, NV, h2, blk_cnt);
+  GFCC_CUDA(launch_chained(cgs_dots_kernel<T>, dgrid, 32 * DOT_WARPS, 0, st, Vb, vs, n, nv, w, n, dlen, state, rflag, partial, NV, h2, blk_cnt));
   GFCC_LAUNCH_CHECK();
-  cgs_update_kernel<T, true><<<ugrid, CGS_THREADS, 0, st>>>(Vb, vs, n, nv, w, n, ulen, rflag, h, h2, theta, partial, NV,
-                                                            blk_cnt, state);
+  GFCC_CUDA(launch_chained(cgs_update_kernel<T, true>, ugrid, CGS_THREADS, 0, st, Vb, vs, n, nv, w, n, ulen, rflag, h, h2, theta, partial, NV,
+                                                            blk_cnt, state));
   GFCC_LAUNCH_CHECK();
   dim3 vgrid = vscale_grid(n, nsys);
   vgrid.x += 1;
-  vscale_kernel<T, true><<<vgrid, 256, 0, st>>>(w, vs, n, h, NV, nv, state, ST_IN_CYCLE, q);
+  GFCC_CUDA(launch_chained(vscale_kernel<T, true>, vgrid, 256, 0, st, w, vs, n, h, NV, nv, state, ST_IN_CYCLE, q));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
