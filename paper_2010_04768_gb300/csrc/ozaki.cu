@@ -258,39 +258,57 @@ __device__ __forceinline__ void for_tile(bool k_lanes, F f) {
 }
 
 // be[r] = largest biased exponent among the entries of row r0 + r (be zeroed by the caller); a block
-// covers SL_ROWS rows and `span` K values
+// covers SL_ROWS rows and `span` K values, a tile with eight loads of every thread in flight at a time (41 million
+// entries 66 us; 168 us with a 64-bit division and one load in flight per entry)
 __global__ __launch_bounds__(SL_THREADS) void strided_exp_kernel(const double *X, long long rows, long long K, IMap rm,
                                                                  IMap km, long long r0, bool k_lanes, int span,
                                                                  unsigned gx, int *be) {
+  constexpr int PER = SL_ROWS * SL_K / SL_THREADS;
   __shared__ int mx[SL_ROWS];
-  __shared__ long long ro[SL_ROWS];
+  __shared__ long long ro[SL_ROWS], ko[2][SL_K];   // the K offsets of a tile are formed while the one before is read
   const unsigned bx = blockIdx.x % gx, by = blockIdx.x / gx;
   const long long rb = (long long)bx * SL_ROWS;
   if (threadIdx.x < SL_ROWS) {
     mx[threadIdx.x] = 0;
     ro[threadIdx.x] = rb + threadIdx.x < rows ? imap_apply(rm, r0 + rb + threadIdx.x) : -1;
   }
-  __syncthreads();
   const long long kbeg = (long long)by * span, kend = min(K, kbeg + span);
+  auto offsets = [&](long long k0, long long *dst) {
+    if (threadIdx.x >= 64 && threadIdx.x < 64 + SL_K) {
+      const int k = threadIdx.x - 64;
+      dst[k] = k0 + k < kend ? imap_apply(km, k0 + k) : -1;
+    }
+  };
+  int m[PER];
+#pragma unroll
+  for (int u = 0; u < PER; u++) m[u] = 0;
+  offsets(kbeg, ko[0]);
+  __syncthreads();
+  int cur = 0;
+  for (long long k0 = kbeg; k0 < kend; k0 += SL_K, cur ^= 1) {
+    double v[PER];
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+      const int e = threadIdx.x + u * SL_THREADS;
+      const int r = k_lanes ? e / SL_K : e % SL_ROWS, k = k_lanes ? e % SL_K : e / SL_ROWS;
+      v[u] = ro[r] >= 0 && ko[cur][k] >= 0 ? X[ro[r] + ko[cur][k]] : 0.0;
+    }
+    if (k0 + SL_K < kend) offsets(k0 + SL_K, ko[cur ^ 1]);
+#pragma unroll
+    for (int u = 0; u < PER; u++) m[u] = max(m[u], (__double2hiint(v[u]) >> 20) & 0x7ff);
+    __syncthreads();
+  }
   if (k_lanes) {
-    // a warp per row: lanes along K
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int r = warp; r < SL_ROWS; r += SL_THREADS / 32) {
-      if (ro[r] < 0) continue;
-      int m = 0;
-      for (long long k = kbeg + lane; k < kend; k += 32)
-        m = max(m, (int)((__double_as_longlong(X[ro[r] + imap_apply(km, k)]) >> 52) & 0x7ff));
-      m = __reduce_max_sync(0xffffffffu, m);
-      if (lane == 0) mx[r] = m;
+    // the lanes of a warp share the row of each element
+#pragma unroll
+    for (int u = 0; u < PER; u++) {
+      const int w = __reduce_max_sync(0xffffffffu, m[u]);
+      if ((threadIdx.x & 31) == 0) atomicMax(&mx[(threadIdx.x + u * SL_THREADS) / SL_K], w);
     }
   } else {
-    // lanes along the rows, warps along K
-    const int r = threadIdx.x & 31;
-    int m = 0;
-    if (ro[r] >= 0)
-      for (long long k = kbeg + (threadIdx.x >> 5); k < kend; k += SL_THREADS / 32)
-        m = max(m, (int)((__double_as_longlong(X[ro[r] + imap_apply(km, k)]) >> 52) & 0x7ff));
-    atomicMax(&mx[r], m);
+#pragma unroll
+    for (int u = 1; u < PER; u++) m[0] = max(m[0], m[u]);
+    atomicMax(&mx[threadIdx.x % SL_ROWS], m[0]);
   }
   __syncthreads();
   if (threadIdx.x < SL_ROWS && ro[threadIdx.x] >= 0 && mx[threadIdx.x] > 0) atomicMax(&be[rb + threadIdx.x], mx[threadIdx.x]);
@@ -326,15 +344,21 @@ __global__ __launch_bounds__(SL_THREADS) void strided_slice_kernel(const double 
   for (int t = threadIdx.x; t < SL_ROWS * SL_K / 2; t += SL_THREADS) {
     const int r = t / (SL_K / 2), k = 2 * (t % (SL_K / 2));
     if (ro[r] < 0 || k0 + k >= ld) continue;
-    long long Y0 = fixed_point(tile[r][k], ex[r], bits * S), Y1 = fixed_point(tile[r][k + 1], ex[r], bits * S);
-    __nv_bfloat162 *dst = reinterpret_cast<__nv_bfloat162 *>(dig + (rb + r) * ld + k0 + k);
-    for (int i = 0; i < S; i++) {
-      const int sh = bits * (S - 1 - i);
-      const long long d0 = sh > 0 ? (Y0 + (1LL << (sh - 1))) >> sh : Y0;
-      const long long d1 = sh > 0 ? (Y1 + (1LL << (sh - 1))) >> sh : Y1;
-      Y0 -= d0 << sh;
-      Y1 -= d1 << sh;
-      dst[i * (plane / 2)] = __floats2bfloat162_rn((float)(int)d0, (float)(int)d1);
+    // Half a place added to every digit (and a whole one more to the first, which then is not negative) makes the
+    // digits plain bit fields; each is exact in BF16
+    const unsigned long long bias = ((1ULL << (bits * S)) - 1) / ((1ULL << bits) - 1) << (bits - 1);
+    const unsigned long long lift = 1ULL << (bits * S);   // 2^bits in the first place
+    const unsigned long long Y0 = (unsigned long long)fixed_point(tile[r][k], ex[r], bits * S) + bias + lift,
+                             Y1 = (unsigned long long)fixed_point(tile[r][k + 1], ex[r], bits * S) + bias + lift;
+    unsigned *dst = reinterpret_cast<unsigned *>(dig + (rb + r) * ld + k0 + k);
+    const unsigned mask = (1u << bits) - 1;
+    const float half = 8388608.0f + (float)(1 << (bits - 1));
+    for (int i = 0, sh = bits * (S - 1); i < S; i++, sh -= bits, dst += plane / 2) {
+      const unsigned mi = i == 0 ? 1023u : mask;
+      const float off = i == 0 ? half + (float)(1 << bits) : half;
+      const unsigned f0 = __float_as_uint(__uint_as_float(0x4b000000u | ((unsigned)(Y0 >> sh) & mi)) - off);
+      const unsigned f1 = __float_as_uint(__uint_as_float(0x4b000000u | ((unsigned)(Y1 >> sh) & mi)) - off);
+      *dst = __byte_perm(f0, f1, 0x7632);
     }
   }
 }
@@ -357,8 +381,8 @@ int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long lon
   GFCC_TRY(check_extent_bytes(mem, emu_operand_bytes(rows, K, S), "digit split output"));
   const bool k_lanes = km.s0 == 1 || rm.s0 != 1;
   const long long gx = (rows + SL_ROWS - 1) / SL_ROWS, gy = (out.ld + SL_K - 1) / SL_K;
-  // K values per block of the exponent pass: enough blocks for the chip, at least four tiles each
-  long long span = SL_K * 4;
+  // K values per block of the exponent pass: enough blocks for the chip, one tile at least
+  long long span = SL_K;
   while (gx * ((K + span - 1) / span) > 152 * 16 && span < (1 << 20)) span *= 2;
   const long long gz = (K + span - 1) / span;
   if (gx * gy > 0x7fffffffLL || gx * gz > 0x7fffffffLL) {
@@ -418,7 +442,7 @@ long long up256(long long x) { return (x + 255) / 256 * 256; }
 // 4.0; entries that decay along K as the Cholesky vectors do, 2.5, 2.6, 3.3, 3.9, 6.6, 7.0 and 0.7, 0.8, 1.1, 1.1, 3.5,
 // 3.5.
 // What it gives: set-up of a mixed IP context at o=40 v=200 L=800 3489 -> 143 ms, IP + EA set-up and solve at
-// o=20 v=100 365 -> 40 ms, CCSD and Lambda at o=16 v=80 404 -> CCSD_NOW ms, closed-shell solve at o=30 v=150 96 -> 46 ms.
+// o=20 v=100 365 -> 40 ms, CCSD and Lambda at o=16 v=80 404 -> 99 ms, closed-shell solve at o=30 v=150 96 -> 43 ms.
 bool emulation_pays(long long M, long long N, long long K, bool a_ready) {
   if (K < 32) return false;
   const double m16 = (double)((M + 15) / 16 * 16), n16 = (double)((N + 15) / 16 * 16);

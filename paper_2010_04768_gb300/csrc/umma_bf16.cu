@@ -1394,7 +1394,7 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
 
 namespace {
 constexpr int EMU_SMS = 152;
-constexpr int EMU_MAX_SPLIT_TILES = 4 * EMU_SMS;   // tiles x K splits of a split product: bounds its partial sums
+constexpr int EMU_MAX_SPLIT_TILES = 8 * EMU_SMS;   // tiles x K splits of a split product: bounds its partial sums
 
 // Tiling of a fused digit product: tile width, whether A and B change places, K splits.  The model (in
 // clocks of an SM) weighs the MMAs of 36 digit pairs, the loads of 16 planes at about 55 bytes a clock,
