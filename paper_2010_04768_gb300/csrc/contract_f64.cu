@@ -30,7 +30,7 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int BK = 16, NT = 256;
+constexpr int BK = 16, KSTEP = 4, NT = 256;
 constexpr int NUM_SM = 152;
 
 // x / d by 32-bit division where both fit (the 64-bit one costs several times as many instructions)
@@ -161,17 +161,23 @@ __global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kclust
   for (long long k0 = kbeg; k0 < kend; k0 += BK, buf ^= 1) {
     const bool more = k0 + BK < kend;
     if (more) fetch(k0 + BK);
+    // the last step multiplies no more than its K values, to a multiple of four
+    const int left = (int)min((long long)BK, kend - k0);
 #pragma unroll
-    for (int kk = 0; kk < BK; kk++) {
-      double a[RM], bb[RN];
+    for (int k4 = 0; k4 < BK; k4 += KSTEP) {
+      if (k4 >= left) break;
 #pragma unroll
-      for (int i = 0; i < RM; i++) a[i] = As[buf][kk][ty + TM * i];
+      for (int kk = k4; kk < k4 + KSTEP; kk++) {
+        double a[RM], bb[RN];
 #pragma unroll
-      for (int j = 0; j < RN; j++) bb[j] = Bs[buf][kk][tx + TN * j];
+        for (int i = 0; i < RM; i++) a[i] = As[buf][kk][ty + TM * i];
 #pragma unroll
-      for (int i = 0; i < RM; i++)
+        for (int j = 0; j < RN; j++) bb[j] = Bs[buf][kk][tx + TN * j];
 #pragma unroll
-        for (int j = 0; j < RN; j++) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+        for (int i = 0; i < RM; i++)
+#pragma unroll
+          for (int j = 0; j < RN; j++) acc[i][j] = fma(a[i], bb[j], acc[i][j]);
+      }
     }
     if (more) stage(buf ^ 1);
     __syncthreads();
@@ -225,8 +231,8 @@ Tiling choose_tiling(long long M, long long N, long long K, long long batch, boo
     if ((N + s[1] - 1) / s[1] > 65535) continue;
     for (int S = 1; S <= (cluster ? 8 : 1); S *= 2) {
       if (S > 1 && K < 2 * BK * S) break;
-      const double steps = std::ceil(std::ceil((double)K / S) / BK);
-      const double t = std::ceil(tiles * S / NUM_SM) * (steps * s[0] * s[1] * BK / 2.0 * (s[0] == 32 && s[1] == 32 ? 1.0 : 1.04) +
+      const double ks = S == 1 ? std::ceil((double)K / KSTEP) * KSTEP : std::ceil(std::ceil((double)K / S) / BK) * BK;
+      const double t = std::ceil(tiles * S / NUM_SM) * (ks * s[0] * s[1] / 2.0 * (s[0] == 32 && s[1] == 32 ? 1.0 : 1.04) +
                                                         1000.0 + (S > 1 ? 1500.0 : 0.0));
       if (cost == 0.0 || t < cost) {
         cost = t;

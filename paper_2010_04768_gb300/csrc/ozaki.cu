@@ -32,41 +32,6 @@ namespace {
 
 constexpr int KCHUNK_BLOCKS = (1 << 14) / 64;   // K blocks (of 64) per exact partial sum
 
-// e[r] such that max_k |A[r][k]| * 2^-e[r] lies in [1/4, 1/2); rows of zeros get 0
-__global__ void rowexp_kernel(const double *A, long long rows, long long K, long long lda, int *e) {
-  __shared__ double sh[32];
-  const long long r = blockIdx.x;
-  if (r >= rows) return;
-  double mx = 0.0;
-  for (long long k = threadIdx.x; k < K; k += blockDim.x) mx = fmax(mx, fabs(A[r * lda + k]));
-  for (int off = 16; off > 0; off >>= 1) mx = fmax(mx, __shfl_down_sync(0xffffffffu, mx, off));
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++) mx = fmax(mx, sh[w]);
-    int E = 0;
-    if (mx > 0.0) frexp(mx, &E);   // mx = f 2^E, f in [1/2, 1)
-    e[r] = mx > 0.0 ? E + 1 : 0;
-  }
-}
-
-// dig[i][r][k] = i-th digit of A[r][k] 2^-e[r] (k < K), 0 for K <= k < ld
-__global__ void slice_kernel(const double *A, long long rows, long long K, long long lda, const int *e, int S,
-                             int bits, __nv_bfloat16 *dig, long long ld) {
-  const long long tot = rows * ld;
-  const long long plane = rows * ld;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
-    const long long r = t / ld, k = t - r * ld;
-    long long Y = k < K ? fixed_point(A[r * lda + k], e[r], bits * S) : 0;
-    for (int i = 0; i < S; i++) {
-      const int sh = bits * (S - 1 - i);
-      const long long d = sh > 0 ? (Y + (1LL << (sh - 1))) >> sh : Y;
-      Y -= d << sh;
-      dig[i * plane + t] = __float2bfloat16((float)(int)d);
-    }
-  }
-}
-
 // Exact integer accumulation of digit-pair products: the FP32 partial sums are integers of
 // magnitude <= 2^24, so they convert to int32 exactly; a pair of level L adds (sum_z part) shifted
 // by 6 (Lhi - L) into the high accumulator (levels <= Lsplit) or by 6 (P - L) into the low one.
@@ -111,27 +76,7 @@ long long emu_operand_bytes(long long rows, long long K, int S) {
 
 int emu_slice(cudaStream_t st, const double *A, long long rows, long long K, long long lda, int S, void *mem,
               EmuOperand &out, int bits) {
-  out.bits = bits;
-  out.rows = rows;
-  out.K = K;
-  out.ld = emu_ld(K);
-  out.S = S;
-  unsigned char *p = static_cast<unsigned char *>(mem);
-  out.dig = reinterpret_cast<__nv_bfloat16 *>(p);
-  p += ((long long)S * rows * out.ld * 2 + 255) / 256 * 256;
-  out.exp2 = reinterpret_cast<int *>(p);
-  if (rows <= 0 || K <= 0) return GFCC_OK;
-  GFCC_TRY(check_extent(A, 0, (rows - 1) * lda + K - 1, "digit split input"));
-  GFCC_TRY(check_extent_bytes(mem, emu_operand_bytes(rows, K, S), "digit split output"));
-  if (rows > 0x7fffffffLL) {
-    set_error("emu_slice: too many rows (%lld)", rows);
-    return GFCC_ERR_ARG;
-  }
-  rowexp_kernel<<<(unsigned)rows, 256, 0, st>>>(A, rows, K, lda, out.exp2);
-  GFCC_LAUNCH_CHECK();
-  slice_kernel<<<grid1d(rows * out.ld), 256, 0, st>>>(A, rows, K, lda, out.exp2, S, bits, out.dig, out.ld);
-  GFCC_LAUNCH_CHECK();
-  return GFCC_OK;
+  return emu_slice_strided(st, A, rows, K, imap1(lda), imap1(1), 0, S, bits, mem, out);
 }
 
 // The digit pairs of one level L = i + j share a weight, so several of them can accumulate in the
@@ -344,6 +289,19 @@ __global__ __launch_bounds__(SL_THREADS) void strided_slice_kernel(const double 
   for (int t = threadIdx.x; t < SL_ROWS * SL_K / 2; t += SL_THREADS) {
     const int r = t / (SL_K / 2), k = 2 * (t % (SL_K / 2));
     if (ro[r] < 0 || k0 + k >= ld) continue;
+    if (bits != F64_BITS) {   // digits rounded one after the other (the levels these products drop keep their sums)
+      long long Y0 = fixed_point(tile[r][k], ex[r], bits * S), Y1 = fixed_point(tile[r][k + 1], ex[r], bits * S);
+      __nv_bfloat162 *dst = reinterpret_cast<__nv_bfloat162 *>(dig + (rb + r) * ld + k0 + k);
+      for (int i = 0; i < S; i++) {
+        const int sh = bits * (S - 1 - i);
+        const long long d0 = sh > 0 ? (Y0 + (1LL << (sh - 1))) >> sh : Y0;
+        const long long d1 = sh > 0 ? (Y1 + (1LL << (sh - 1))) >> sh : Y1;
+        Y0 -= d0 << sh;
+        Y1 -= d1 << sh;
+        dst[i * (plane / 2)] = __floats2bfloat162_rn((float)(int)d0, (float)(int)d1);
+      }
+      continue;
+    }
     // Half a place added to every digit (and a whole one more to the first, which then is not negative) makes the
     // digits plain bit fields; each is exact in BF16
     const unsigned long long bias = ((1ULL << (bits * S)) - 1) / ((1ULL << bits) - 1) << (bits - 1);
