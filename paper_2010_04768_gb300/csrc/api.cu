@@ -277,6 +277,7 @@ __global__ void left_ip_1h_kernel(double *C, long long n, int nq, const int *qor
     const int m = q;
     const long long ovv = (long long)o * v * v;
     double acc = 0.0;
+#pragma unroll 8
     for (long long x = threadIdx.x; x < ovv; x += blockDim.x)   // x = (l, c, d)
       acc += t2[(long long)m * ovv + x] * l2[(long long)k * ovv + x];
     double acc1 = 0.0;

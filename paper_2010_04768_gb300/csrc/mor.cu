@@ -145,8 +145,8 @@ __global__ void mor_real_kernel(const double *z, long long n, int rows, double *
 // G[w][a][b] (IP: a over rhs, b over left; EA: a over left, b over rhs) = sum_k ch[k][left] X[k][rhs].
 // Gaussian elimination with partial pivoting by rows; threads split the trailing updates, the back
 // substitution runs by columns.  Bound by the FP64 pipe (m^3 / 3 complex FMAs) once the pivot search is a warp's and
-// the matrix is in shared memory: 256 frequencies at m = 72, nb = 12 took 4 ms with a serial search over the block
-// and one thread per right-hand side in the back substitution.
+// the matrix is in shared memory: 304 frequencies at m = 72, nb = 12 take 0.63 ms (256 took 4 ms with a serial search
+// over the block and one thread per right-hand side in the back substitution).
 __global__ __launch_bounds__(MT) void mor_model_solve_kernel(const double *Hh, int m, const double *omegas, double eta,
                                                              double zsign, double hsign, const double *bh, int nb,
                                                              const double *ch, int nl, int is_ip, double2 *Aw,
@@ -208,15 +208,16 @@ __global__ __launch_bounds__(MT) void mor_model_solve_kernel(const double *Hh, i
       lm[i] = make_double2(a.x * inv.x - a.y * inv.y, a.x * inv.y + a.y * inv.x);
     }
     __syncthreads();
+    // 16 lanes a row (rows are some 50 entries long on average)
     const double2 *rk = A + (long long)k * ld;
-    for (int i = k + 1 + warp; i < m; i += MT / 32) {
+    for (int i = k + 1 + (t0 >> 4); i < m; i += MT / 16) {
       const double2 l = lm[i];
       double2 *ri = A + (long long)i * ld;
-      for (int j = k + 1 + lane; j < ld; j += 32) {
+      for (int j = k + 1 + (t0 & 15); j < ld; j += 16) {
         double2 v = ri[j];
         const double2 src = rk[j];
-        v.x -= l.x * src.x - l.y * src.y;
-        v.y -= l.x * src.y + l.y * src.x;
+        v.x = fma(l.y, src.y, fma(-l.x, src.x, v.x));
+        v.y = fma(-l.y, src.x, fma(-l.x, src.y, v.y));
         ri[j] = v;
       }
     }
@@ -237,8 +238,8 @@ __global__ __launch_bounds__(MT) void mor_model_solve_kernel(const double *Hh, i
       const int row = t / nb, r = t - row * nb;
       const double2 a = A[(long long)row * ld + i], x = xi[r];
       double2 *v = A + (long long)row * ld + m + r;
-      v->x -= a.x * x.x - a.y * x.y;
-      v->y -= a.x * x.y + a.y * x.x;
+      v->x = fma(a.y, x.y, fma(-a.x, x.x, v->x));
+      v->y = fma(-a.y, x.x, fma(-a.x, x.y, v->y));
     }
     __syncthreads();
   }
@@ -280,17 +281,20 @@ __global__ void mor_coef_kernel(const double2 *Xw, int m, int nb, long long pair
   }
 }
 
-// out[2 pr] = ||b_r - (A x)_pr||^2 and out[2 pr + 1] = ||b_r||^2 from Ax [2 pr + re/im][n], one block per pair
+// out[2 pr] = ||b_r - (A x)_pr||^2 from Ax [2 pr + re/im][n] and, of the first frequency's pairs (pr = r), out[2 r + 1] =
+// ||b_r||^2; one block per pair
 __global__ __launch_bounds__(MT) void mor_resnorm_kernel(const double *Ax, const double *B, long long n, int nb,
                                                          double *out) {
   __shared__ double sh[2][MT / 32];
   const long long pr = blockIdx.x;
   const double *ar = Ax + 2 * pr * n, *ai = ar + n, *b = B + (pr % nb) * n;
+  const bool first = pr < nb;
   double rr = 0.0, bb = 0.0;
+#pragma unroll 4
   for (long long e = threadIdx.x; e < n; e += MT) {
     const double x = b[e], d = x - ar[e], i = ai[e];
-    rr += d * d + i * i;
-    bb += x * x;
+    rr = fma(d, d, fma(i, i, rr));
+    if (first) bb = fma(x, x, bb);
   }
   for (int off = 16; off > 0; off >>= 1) {
     rr += __shfl_xor_sync(0xffffffffu, rr, off);
@@ -308,7 +312,7 @@ __global__ __launch_bounds__(MT) void mor_resnorm_kernel(const double *Ax, const
       c += sh[1][t];
     }
     out[2 * pr] = a;
-    out[2 * pr + 1] = c;
+    if (first) out[2 * pr + 1] = c;
   }
 }
 
@@ -510,7 +514,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   int *d_lists = nullptr;
   double *buf = nullptr;
   // The residuals of mixed-precision contexts are products [S | W] x on digit planes (the FP64 units take
-  // 8 n m operations per frequency and right-hand side: 26 ms for 500 x 12 at n = 9616, m = 72, against 4 ms); other
+  // 8 n m operations per frequency and right-hand side: 26 ms for 500 x 12 at n = 9616, m = 72, against 2.4 ms); other
   // contexts and models too small to gain keep the FP64 kernel.  Short sums are as accurate as that kernel here: the
   // residuals of models of 36 vectors over 9616 and 6280 elements were within 6e-14 (rms, of ||b||) of quad sums
   // either way.
@@ -636,8 +640,10 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
       }
       GFCC_CUDA(cudaMemcpyAsync(hres.data(), res, sizeof(double) * 2 * nw * nb, cudaMemcpyDeviceToHost, st));
       GFCC_CUDA(cudaStreamSynchronize(st));
-      for (int t = 0; t < nw * nb; t++)
-        h_relres[(long long)w0 * nb + t] = hres[2 * t + 1] > 0.0 ? std::sqrt(hres[2 * t] / hres[2 * t + 1]) : 0.0;
+      for (int t = 0; t < nw * nb; t++) {
+        const double bb = hres[2 * (done_planes ? t % nb : t) + 1];
+        h_relres[(long long)w0 * nb + t] = bb > 0.0 ? std::sqrt(hres[2 * t] / bb) : 0.0;
+      }
     }
   }
   if (planes) {
