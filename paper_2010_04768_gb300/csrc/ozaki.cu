@@ -10,9 +10,10 @@
 // <= 2^10, so a sum of up to 2^14 of them is an integer of magnitude <= 2^24 and the FP32
 // accumulation of the tensor cores is exact.  The product of two operands is then
 //     sum_k A[m][k] B[n][k] = 2^(e_m + f_n) sum_{i,j} 64^-(i+j) sum_k dA_i[m][k] dB_j[n][k]
-// and the digit-pair products with i + j <= P are evaluated as BF16 GEMMs (K split into
-// chunks of 2^14 with separate FP32 partial sums) and combined in FP64.  The truncation
-// error per term is bounded by about 2^-(6P-4) of 2^(e_m + f_n); P = S + 1.
+// and the digit-pair products with i + j <= P are evaluated on the tensor cores, all of a tile in one kernel
+// (umma_bf16.cu) or as one BF16 GEMM each (K split into chunks of 2^14 with separate FP32 partial sums), and
+// combined with one rounding.  The truncation error per term is bounded by about 2^-(6P-4) of 2^(e_m + f_n);
+// P = S + 1.  Contractions that take the place of FP64 sums use 8 digits of 7 bits instead.
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -7,13 +7,13 @@
 // vectors are rounded to BF16 when they are unpacked, products accumulate in FP32
 // in tensor memory (TMEM).
 //
-// Structure (one 128 x 256 output tile per CTA, 4 warps):
+// Structure (one 128 x 64, 128 x 128 or 128 x 256 output tile per CTA, 4 warps; here the last):
 //   * warp 0, one lane: TMA producer.  A tile 128 x 64 and B tile 256 x 64 (BF16,
 //     128-byte swizzle) per stage into a 4-stage shared-memory ring, completion
 //     tracked by mbarrier transaction counts.
-//   * warp 1, one lane: MMA issuer.  Four tcgen05.mma (M=128, N=256, K=16) per stage,
-//     accumulating in 256 TMEM columns; tcgen05.commit releases the stage.
-//   * all 4 warps: epilogue.  tcgen05.ld of the warp's 32 TMEM lanes, scale, store.
+//   * warp 1: MMA issuer (the whole warp, one elected lane, so that descriptors stay in uniform registers).  Four
+//     tcgen05.mma (M=128, N=256, K=16) per stage, accumulating in 256 TMEM columns; tcgen05.commit releases the stage.
+//   * all 4 warps: epilogue.  tcgen05.ld of the warp's 32 TMEM lanes, scale, store along rows through shared memory.
 // Every wait is bounded (about one second of %globaltimer); on time-out the CTA sets
 // the error flag, stops issuing work, drains what it issued and frees its TMEM.
 #include <cuda.h>
@@ -1356,34 +1356,36 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
       if (it != g_tune.end()) best = it->second;
     }
     if (best == 0) {
-      // first call of this shape: time every tile width (the last two of three launches each, CUDA events on
+      // first call of this shape: time every tile width that may win (the faster of two launches each, CUDA events on
       // the stream; beta == 0, so the repeated launches leave the same D) and keep the fastest
-      cudaEvent_t e0, e1;
-      GFCC_CUDA(cudaEventCreate(&e0));
-      GFCC_CUDA(cudaEventCreate(&e1));
+      cudaEvent_t ev[3];
+      for (cudaEvent_t &e : ev) GFCC_CUDA(cudaEventCreate(&e));
       float best_ms = 0.0f;
+      // 64 columns read the A rows four times as often as 256: not for wide products with a long K loop
+      const bool wide = N >= 512 && K >= 512;
       for (int cand : {64, 128, 256, TILE_PAIR + 128, TILE_PAIR + 192, TILE_PAIR + 256, TILE_PERSIST + 64,
                        TILE_PERSIST + 128, TILE_PERSIST + 256}) {
         const int w = cand > TILE_PERSIST ? cand - TILE_PERSIST : cand > TILE_PAIR ? cand - TILE_PAIR : cand;
         if (cand > TILE_PAIR && cand < TILE_PERSIST
                 ? !pair_ok || pair_cost(w) > 1.15 * pair_cost(pair_best)
-                : ((cand > TILE_PERSIST && !persist_ok) || (w > 64 && w / 2 >= N)))
+                : ((cand > TILE_PERSIST) != persist_ok || (w > 64 && w / 2 >= N) || (w == 64 && wide)))
           continue;   // never better
+        GFCC_CUDA(cudaEventRecord(ev[0], st));
         GFCC_TRY(run(cand));
-        GFCC_CUDA(cudaEventRecord(e0, st));
+        GFCC_CUDA(cudaEventRecord(ev[1], st));
         GFCC_TRY(run(cand));
-        GFCC_TRY(run(cand));
-        GFCC_CUDA(cudaEventRecord(e1, st));
-        GFCC_CUDA(cudaEventSynchronize(e1));
-        float ms = 0.0f;
-        GFCC_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        GFCC_CUDA(cudaEventRecord(ev[2], st));
+        GFCC_CUDA(cudaEventSynchronize(ev[2]));
+        float ms = 0.0f, ms2 = 0.0f;
+        GFCC_CUDA(cudaEventElapsedTime(&ms, ev[0], ev[1]));
+        GFCC_CUDA(cudaEventElapsedTime(&ms2, ev[1], ev[2]));
+        ms = std::min(ms, ms2);
         if (best == 0 || ms < best_ms) {
           best = cand;
           best_ms = ms;
         }
       }
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
+      for (cudaEvent_t e : ev) cudaEventDestroy(e);
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tune[key] = best;
     }
