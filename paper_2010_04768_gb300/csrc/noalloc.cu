@@ -81,7 +81,12 @@ extern "C" int gfcc_sigma_noalloc(gfcc_ctx *c, int sector, int n_vec, const doub
   b.ldx = sector == GFCC_SECTOR_IP ? c->dim_ip : c->dim_ea;
   b.y = y_dev;
   b.ldy = b.ldx;
-  GFCC_TRY(sector == GFCC_SECTOR_IP ? apply_ip(c, b, w) : apply_ea(c, b, w));
+  // the digit planes of a closed-shell context's products would need a workspace: the FP64 units here
+  const int emulate = c->rhf_emulate;
+  c->rhf_emulate = 0;
+  const int s = sector == GFCC_SECTOR_IP ? apply_ip(c, b, w) : apply_ea(c, b, w);
+  c->rhf_emulate = emulate;
+  GFCC_TRY(s);
   GFCC_CUDA(cudaStreamSynchronize(c->stream));
   return GFCC_OK;
 }
