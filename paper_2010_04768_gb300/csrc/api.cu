@@ -468,6 +468,13 @@ int create_impl(int o, int v, int L, const double *fock, const double *chol, con
     return fail(GFCC_ERR_CUDA);
   }
   c->stream = c->own_stream;
+  {
+    double *flag;
+    if ((s = dev_alloc(c, &flag, 1)) < 0) return fail(s);
+    c->umma_flag = reinterpret_cast<unsigned *>(flag);
+  }
+  UmmaScope umma(c->umma_flag);
+  if ((s = umma_error_reset(c->stream)) < 0) return fail(s);
   const long long n = c->n, nn = n * n, ov = (long long)o * v, oovv = ov * ov;
   double *d_fock = nullptr, *d_chol = nullptr;
   if ((s = dev_alloc_tmp(&d_fock, nn)) < 0) return fail(s);
@@ -599,6 +606,8 @@ int grow_scratch(gfcc_ctx *c, size_t bytes) {
 int solve_impl(gfcc_ctx *c, int n_omega, const double *d_om, double eta, const OrbLists &ol, double tol,
                double *d_G) {
   cudaStream_t st = c->stream;
+  UmmaScope umma(c->umma_flag);
+  if (c->precision == GFCC_PREC_MIXED_BF16 || c->rhf) GFCC_TRY(umma_error_reset(st));
   int rc;
   {
     PhaseTimer tm(c, PH_SOLVE);
@@ -803,7 +812,6 @@ int solve_impl_inner(gfcc_ctx *c, int n_omega, const double *d_om, double eta, c
       };
       for (int s = 0; s < nsys; s++) task[s] = next < ntasks ? next++ : -1;
       GFCC_TRY(load_slots(true));
-      GFCC_TRY(umma_error_reset(st));
       bool first = true;
       for (int step = 0;; step++) {
         if (first) {
@@ -972,7 +980,6 @@ int solve_impl_inner(gfcc_ctx *c, int n_omega, const double *d_om, double eta, c
         use_x0 = true;
       }
       if (mixed) {
-        GFCC_TRY(umma_error_reset(st));
         GFCC_TRY(gm.solve_refined(tol, c->inner_tol, c->max_iters, h_state.data(), h_it.data(), use_x0,
                                   h_outer.data()));
         GFCC_TRY(umma_error_check(st));
@@ -1557,8 +1564,9 @@ int gfcc_sigma_ex(gfcc_ctx *c, int sector, int precision, int n_vec, const doubl
   b.nsys = n_vec;
   b.x = dx; b.ldx = n;
   b.y = dy; b.ldy = n;
+  UmmaScope umma(c->umma_flag);
+  if (mixed || emu || c->rhf) GFCC_TRY(umma_error_reset(c->stream));
   if (mixed || emu) {
-    GFCC_TRY(umma_error_reset(c->stream));
     if (ip)
       GFCC_TRY(mixed ? apply_ip_mixed(c, b, w) : apply_ip_emu(c, b, w, ew));
     else
@@ -1636,14 +1644,15 @@ int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double
     set_error("gfcc_selftest_gemm_f64emu: bad arguments");
     return GFCC_ERR_ARG;
   }
-  void *da = nullptr, *db = nullptr, *dc = nullptr, *sa = nullptr, *sb = nullptr, *w = nullptr;
+  void *da = nullptr, *db = nullptr, *dc = nullptr, *sa = nullptr, *sb = nullptr, *w = nullptr, *flag = nullptr;
   cudaStream_t st = nullptr;
   int s = GFCC_OK;
   if (dmalloc(&da, sizeof(double) * M * K) != cudaSuccess || dmalloc(&db, sizeof(double) * N * K) != cudaSuccess ||
       dmalloc(&dc, sizeof(double) * M * N) != cudaSuccess ||
       dmalloc(&sa, emu_operand_bytes(M, K, S)) != cudaSuccess ||
       dmalloc(&sb, emu_operand_bytes(N, K, S)) != cudaSuccess ||
-      dmalloc(&w, emu_gemm_work_bytes(M, N, K)) != cudaSuccess || cudaStreamCreate(&st) != cudaSuccess) {
+      dmalloc(&w, emu_gemm_work_bytes(M, N, K)) != cudaSuccess || dmalloc(&flag, sizeof(unsigned)) != cudaSuccess ||
+      cudaStreamCreate(&st) != cudaSuccess) {
     cudaGetLastError();
     set_error("gfcc_selftest_gemm_f64emu: allocation failed");
     s = GFCC_ERR_OOM;
@@ -1654,6 +1663,7 @@ int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double
     s = GFCC_ERR_CUDA;
   }
   EmuOperand ea, eb;
+  UmmaScope umma(static_cast<unsigned *>(flag));
   if (s == GFCC_OK) s = umma_error_reset(st);
   if (s == GFCC_OK) s = emu_slice(st, static_cast<double *>(da), M, K, K, S, sa, ea);
   if (s == GFCC_OK) s = emu_slice(st, static_cast<double *>(db), N, K, K, S, sb, eb);
@@ -1663,7 +1673,7 @@ int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double
     set_error("gfcc_selftest_gemm_f64emu: copy back failed");
     s = GFCC_ERR_CUDA;
   }
-  for (void *p : {da, db, dc, sa, sb, w}) dfree(p);
+  for (void *p : {da, db, dc, sa, sb, w, flag}) dfree(p);
   if (st) cudaStreamDestroy(st);
   return s;
 }
@@ -1686,11 +1696,12 @@ int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B,
     for (long long k = 0; k < K; k++) ha[i * ld + k] = to_bf16(A[i * K + k]);
   for (long long i = 0; i < N; i++)
     for (long long k = 0; k < K; k++) hb[i * ld + k] = to_bf16(B[i * K + k]);
-  void *da = nullptr, *db = nullptr, *dd = nullptr;
+  void *da = nullptr, *db = nullptr, *dd = nullptr, *flag = nullptr;
   cudaStream_t st = nullptr;
   int s = GFCC_OK;
   if (dmalloc(&da, ha.size() * 2) != cudaSuccess || dmalloc(&db, hb.size() * 2) != cudaSuccess ||
-      dmalloc(&dd, (size_t)M * N * 4) != cudaSuccess || cudaStreamCreate(&st) != cudaSuccess) {
+      dmalloc(&dd, (size_t)M * N * 4) != cudaSuccess || dmalloc(&flag, sizeof(unsigned)) != cudaSuccess ||
+      cudaStreamCreate(&st) != cudaSuccess) {
     cudaGetLastError();
     set_error("gfcc_selftest_gemm_bf16: allocation failed");
     s = GFCC_ERR_OOM;
@@ -1700,6 +1711,7 @@ int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B,
     set_error("gfcc_selftest_gemm_bf16: copy failed");
     s = GFCC_ERR_CUDA;
   }
+  UmmaScope umma(static_cast<unsigned *>(flag));
   if (s == GFCC_OK) s = umma_error_reset(st);
   if (s == GFCC_OK)
     s = gemm_bf16_tn(st, static_cast<const __nv_bfloat16 *>(da), ld, static_cast<const __nv_bfloat16 *>(db), ld,
@@ -1712,6 +1724,7 @@ int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B,
   dfree(da);
   dfree(db);
   dfree(dd);
+  dfree(flag);
   if (st) cudaStreamDestroy(st);
   return s;
 }

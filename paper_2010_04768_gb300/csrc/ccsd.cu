@@ -39,6 +39,7 @@
 #include "ctx.cuh"
 #include "kernels.cuh"
 #include "ozaki.cuh"
+#include "umma.cuh"
 
 namespace gfcc {
 
@@ -619,6 +620,14 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
     set_error("gfcc_ccsd: cannot create a CUDA stream (no usable GPU?)");
     return GFCC_ERR_CUDA;
   }
+  void *flag = nullptr;   // error flag of the call's tensor-core kernels
+  if (dmalloc(&flag, sizeof(unsigned)) != cudaSuccess) {
+    cudaGetLastError();
+    set_error("gfcc_ccsd: allocation failed");
+    cudaStreamDestroy(st);
+    return GFCC_ERR_OOM;
+  }
+  UmmaScope umma(static_cast<unsigned *>(flag));
   const bool prev_emulate = g_emulate_big;
   const double prev_min = g_emulate_min_flops_local;
   EmuArena arena;   // the digit planes' workspace of the whole call
@@ -629,6 +638,7 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
   // Cholesky sums of the singles) are 1e11-1e12 flops each at medium sizes: below the setup threshold
   if (g_emulate_big) g_emulate_min_flops_local = std::min(g_emulate_min_flops, CCSD_EMULATE_MIN_FLOPS);
   auto run = [&](Ccsd &C) -> int {
+    GFCC_TRY(umma_error_reset(st));
     GFCC_TRY(C.init(o, v, L, fock, chol));
     const long long ov = C.ov, N = C.N;
     double it_info[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -690,6 +700,7 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
   g_emu_arena = prev_arena;
   g_emulate_big = prev_emulate;
   g_emulate_min_flops_local = prev_min;
+  dfree(flag);
   cudaGetLastError();
   cudaStreamDestroy(st);
   return s;

@@ -133,6 +133,8 @@ struct gfcc_ctx {
   // digit planes of the FP64 EA operands (full Fock folding) for the FP64-accurate residual
   gfcc::EmuOperand eWre, eWp, eWTe, eV3e, eU1e;   // eWTe: [W3 | T3e] over K = v + o
 
+  unsigned *umma_flag = nullptr;   // error flag of the context's tensor-core kernels (UmmaScope)
+
   std::vector<void *> allocs;
 
   // initial guesses (Algorithm 1: "compute initial guess")

@@ -23,6 +23,7 @@
 #include "gmres.cuh"
 #include "kernels.cuh"
 #include "sigma.cuh"
+#include "umma.cuh"
 
 namespace gfcc {
 
@@ -1260,14 +1261,15 @@ __global__ void absmax_kernel(const double *v, long long n, unsigned long long *
   for (int off = 16; off > 0; off >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, off));
   if ((threadIdx.x & 31) == 0) atomicMax(&amax[s], (unsigned long long)__double_as_longlong(m));
 }
-// per system: relres = ||r|| / ||b0||; done systems get r = 0 so that the inner solve leaves them alone
+// per system: relres = ||r|| / ||b0||; done systems get r = 0 so that the inner solve leaves them alone.  done = -1: a
+// wait of a product so far has run out (*error), and no system's residual means anything.
 __global__ void refine_check_kernel(int nsys, const double *nrm2, int NV, const double *b0norm, double tol, int *done,
-                                    double *relres) {
+                                    double *relres, const unsigned *error) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= nsys) return;
   const double r = sqrt(fmax(nrm2[2 * (long long)s * NV], 0.0));
   relres[s] = b0norm[s] > 0.0 ? r / b0norm[s] : 0.0;
-  done[s] = (b0norm[s] == 0.0 || r <= tol * b0norm[s]) ? 1 : 0;
+  done[s] = *error != 0 ? -1 : (b0norm[s] == 0.0 || r <= tol * b0norm[s]) ? 1 : 0;
 }
 __global__ void zero_done_kernel(double *R, long long n, int nsys, const int *done) {
   const long long tot = n * nsys;
@@ -1390,12 +1392,13 @@ int Gmres::residual_update() {
 int Gmres::refine_residual_free(int *h_done, double *h_relres) {
   cudaStream_t st = c->stream;
   GFCC_TRY(mdot(R, n, 0, 1, R, n, nrm, -1, 0));
-  refine_check_kernel<<<cdiv(nsys, 256), 256, 0, st>>>(nsys, nrm, NV, b0norm, tol_outer, kcyc, relres);
+  refine_check_kernel<<<cdiv(nsys, 256), 256, 0, st>>>(nsys, nrm, NV, b0norm, tol_outer, kcyc, relres,
+                                                         umma_error_flag());
   GFCC_LAUNCH_CHECK();
   GFCC_CUDA(cudaMemcpyAsync(h_done, kcyc, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
   GFCC_CUDA(cudaMemcpyAsync(h_relres, relres, sizeof(double) * nsys, cudaMemcpyDeviceToHost, st));
   GFCC_CUDA(cudaStreamSynchronize(st));
-  return GFCC_OK;
+  return h_done[0] < 0 ? umma_timed_out() : GFCC_OK;
 }
 
 int Gmres::refine_correct(const int *h_done, int *h_state, int *h_iters) {
@@ -1451,11 +1454,13 @@ int Gmres::solve_refined(double tol, double inner_tol, int max_iters, int *h_sta
       GFCC_TRY(residual_update());
     }
     GFCC_TRY(mdot(R, n, 0, 1, R, n, nrm, -1, 0));
-    refine_check_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, nrm, NV, b0norm, tol, done, relres);
+    refine_check_kernel<<<cdiv(nsys, TH), TH, 0, st>>>(nsys, nrm, NV, b0norm, tol, done, relres,
+                                                       umma_error_flag());
     GFCC_LAUNCH_CHECK();
     if (outer == 0) GFCC_CUDA(cudaMemcpyAsync(relres0, relres, sizeof(double) * nsys, cudaMemcpyDeviceToDevice, st));
     GFCC_CUDA(cudaMemcpyAsync(h_done.data(), done, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaStreamSynchronize(st));
+    if (h_done[0] < 0) return umma_timed_out();
     all_done = true;
     bool any_active = false;
     for (int s = 0; s < nsys; s++) {

@@ -500,6 +500,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   const long long n = M->n;
   const int m = M->m;
   const bool ip = M->sector == GFCC_SECTOR_IP;
+  UmmaScope umma(c->umma_flag);
   if (m < 1) {
     set_error("gfcc_mor_green: the subspace is empty (gfcc_mor_expand first)");
     return GFCC_ERR_STATE;
@@ -705,7 +706,17 @@ int mor_expand_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, in
   dfree(sink);
   if (s < 0) return s;
   for (int w = 0; w < n_omega; w++) M->sampled.push_back(h_om[w]);
-  if (M->m > m0) GFCC_TRY(project_new(M, m0));
+  if (M->m > m0) {
+    UmmaScope umma(c->umma_flag);
+    s = umma_error_reset(st);
+    if (s >= 0) s = project_new(M, m0);
+    if (s >= 0) s = umma_error_check(st);
+    if (s < 0) {   // the model stays what it was
+      M->m = m0;
+      M->sampled.resize(M->sampled.size() - n_omega);
+      return s;
+    }
+  }
   GFCC_CUDA(cudaStreamSynchronize(st));
   return rc;
 }

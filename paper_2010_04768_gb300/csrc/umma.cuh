@@ -39,7 +39,19 @@ int umma_tuned_tile(int M, int N, int K, int nsplit);   // 0 if the shape was no
 // test-only switch under which their producers issue no loads (the wait then runs out with nothing
 // in flight and the kernel returns the GFCC_ERR_TIMEOUT status).
 void umma_set_wait(unsigned long long wait_ns, bool skip_loads);
+// The error flag (one device word) of the calling thread's tensor-core kernels for the lifetime of the scope: a bounded
+// wait that gives up sets it.  Each context has its own, and so has each call without one, so that neither a time-out nor
+// a reset reaches another call.
+struct UmmaScope {
+  explicit UmmaScope(unsigned *flag);
+  ~UmmaScope();
+  UmmaScope(const UmmaScope &) = delete;
+  UmmaScope &operator=(const UmmaScope &) = delete;
+  unsigned *prev;
+};
+unsigned *umma_error_flag();             // the flag of the innermost scope
 int umma_error_reset(cudaStream_t st);
 int umma_error_check(cudaStream_t st);   // GFCC_ERR_TIMEOUT if a bounded wait gave up
+int umma_timed_out();                    // records the message and returns GFCC_ERR_TIMEOUT
 
 }  // namespace gfcc

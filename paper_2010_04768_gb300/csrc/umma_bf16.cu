@@ -56,12 +56,22 @@ constexpr unsigned long long DRAIN_NS = 1000000000ULL;
 struct UmmaCtl {
   unsigned long long wait_ns;
   int skip_loads;
+  unsigned *error;   // set by a wait that ran out (the flag of the call that launched the kernel)
 };
 unsigned long long g_wait_ns = 1000000000ULL;
 bool g_skip_loads = false;
-UmmaCtl umma_ctl() { return UmmaCtl{g_wait_ns, g_skip_loads ? 1 : 0}; }
+thread_local unsigned *t_error_flag = nullptr;
 
-__device__ unsigned int g_umma_error = 0;
+// The control block of a launch by the calling thread; a launch outside every UmmaScope is refused (its time-outs
+// would go unreported).
+int umma_ctl(UmmaCtl *ctl) {
+  if (t_error_flag == nullptr) {
+    set_error("internal: tensor-core product outside a call's error scope");
+    return GFCC_ERR_STATE;
+  }
+  *ctl = UmmaCtl{g_wait_ns, g_skip_loads ? 1 : 0, t_error_flag};
+  return GFCC_OK;
+}
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
   return static_cast<unsigned>(__cvta_generic_to_shared(p));
@@ -94,20 +104,37 @@ __device__ __forceinline__ bool mbar_try_wait(unsigned addr, unsigned parity) {
 }
 
 // Bounded wait (limit_ns of %globaltimer) for the phase of the given parity; false on time-out or
-// abort.
+// abort.  Once a kernel of the call has timed out, the waits of the others give up after GIVE_UP_NS, so that a call
+// whose waits run out ends after about one limit and not after one per product.
+constexpr long long GIVE_UP_NS = 50000;
 __device__ __forceinline__ bool mbar_wait(unsigned addr, unsigned parity, volatile int *abort_flag,
-                                          unsigned long long limit_ns) {
+                                          unsigned long long limit_ns, unsigned *error) {
   if (mbar_try_wait(addr, parity)) return true;
   const unsigned long long t0 = globaltimer();
   while (true) {
     if (mbar_try_wait(addr, parity)) return true;
     if (*abort_flag) return false;
-    if (globaltimer() - t0 > limit_ns) {
+    const long long dt = (long long)(globaltimer() - t0);
+    if (dt > (long long)limit_ns) {
       *abort_flag = 1;
-      atomicOr(&g_umma_error, 1u);
+      atomicOr(error, 1u);
+      return false;
+    }
+    if (dt > GIVE_UP_NS && *reinterpret_cast<volatile unsigned *>(error) != 0) {
+      *abort_flag = 1;
       return false;
     }
   }
+}
+
+// The waits of the abort path: for work this CTA has issued, always up to DRAIN_NS.
+__device__ __forceinline__ void drain_wait(unsigned addr, unsigned parity, unsigned *error) {
+  const unsigned long long t0 = globaltimer();
+  while (!mbar_try_wait(addr, parity))
+    if ((long long)(globaltimer() - t0) > (long long)DRAIN_NS) {
+      atomicOr(error, 1u);
+      return;
+    }
 }
 
 __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap *map, unsigned mbar, int x, int y) {
@@ -281,7 +308,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int kb = 0; kb < nk && !ctl.skip_loads; kb++) {
       const int s = kb % STAGES;
       const unsigned ph = (kb / STAGES) & 1;
-      if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns)) break;
+      if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns, ctl.error)) break;
       unsigned char *sa = smem + s * STAGE_BYTES;
       unsigned char *sb = sa + A_BYTES;
       mbar_expect_tx(smem_u32(&full[s]), STAGE_BYTES);
@@ -296,7 +323,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int kb = 0; kb < nk; kb++) {
       const int s = kb % STAGES;
       const unsigned ph = (kb / STAGES) & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns, ctl.error))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned long long da = d0 + s * (STAGE_BYTES >> 4), db = da + (A_BYTES >> 4);
       if (elect_one()) {
@@ -315,7 +342,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   __syncwarp();
 
   // ---------------- epilogue: all 4 warps
-  const bool ready = mbar_wait(smem_u32(done), 0, abort_flag, ctl.wait_ns);
+  const bool ready = mbar_wait(smem_u32(done), 0, abort_flag, ctl.wait_ns, ctl.error);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   // tcgen05.ld is warp-collective: take the decision per warp
   if (__all_sync(0xffffffffu, ready && !*abort_flag)) {
@@ -337,10 +364,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     // freed), then let the TMA copies this CTA issued land before its shared memory goes away.
     // These waits keep the fixed DRAIN_NS limit; if one of them runs out as well, the CTA exits with
     // that work in flight (the error flag is already set).
-    volatile int never = 0;
-    mbar_wait(smem_u32(done), 0, &never, DRAIN_NS);
+    drain_wait(smem_u32(done), 0, ctl.error);
     for (int kb = *consumed; kb < *issued; kb++)
-      mbar_wait(smem_u32(&full[kb % STAGES]), (kb / STAGES) & 1, &never, DRAIN_NS);
+      drain_wait(smem_u32(&full[kb % STAGES]), (kb / STAGES) & 1, ctl.error);
   }
   __syncthreads();
   if (warp == 0) {
@@ -433,7 +459,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
         for (int kb = 0; kb < nk; kb++, it++) {
           const int s = it % STAGES;
           const unsigned ph = (it / STAGES) & 1;
-          if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns)) {
+          if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns, ctl.error)) {
             ok = false;
             break;
           }
@@ -456,13 +482,13 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
       long long zoff;
       tile_of(t, m0, n0, kb0, nk, zoff);
       const int buf = lt & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acce[buf]), ((lt >> 1) & 1) ^ 1, abort_flag, ctl.wait_ns))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acce[buf]), ((lt >> 1) & 1) ^ 1, abort_flag, ctl.wait_ns, ctl.error))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned acc = tmem + (unsigned)(buf * BN);
       for (int kb = 0; kb < nk; kb++, it++) {
         const int s = it % STAGES;
         const unsigned ph = (it / STAGES) & 1;
-        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns, ctl.error))) {
           ok = false;
           break;
         }
@@ -490,7 +516,7 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
       long long zoff;
       tile_of(t, m0, n0, kb0, nk, zoff);
       const int buf = lt & 1;
-      const bool ready = mbar_wait(smem_u32(&accf[buf]), (lt >> 1) & 1, abort_flag, ctl.wait_ns);
+      const bool ready = mbar_wait(smem_u32(&accf[buf]), (lt >> 1) & 1, abort_flag, ctl.wait_ns, ctl.error);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (!__all_sync(0xffffffffu, ready && !*abort_flag)) break;
       const int row0 = m0 + q * 32;
@@ -511,11 +537,10 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
   if (threadIdx.x == 0) {
     // every MMA the issuer committed has completed (the drain barrier); after a time-out also the TMA
     // copies issued but not consumed land before the shared memory goes away (fixed DRAIN_NS limits)
-    volatile int never = 0;
-    mbar_wait(smem_u32(drain), 0, &never, DRAIN_NS);
+    drain_wait(smem_u32(drain), 0, ctl.error);
     if (*abort_flag)
       for (int it = *consumed; it < *issued; it++)
-        mbar_wait(smem_u32(&full[it % STAGES]), (it / STAGES) & 1, &never, DRAIN_NS);
+        drain_wait(smem_u32(&full[it % STAGES]), (it / STAGES) & 1, ctl.error);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -658,7 +683,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     for (int kb = 0; kb < nk && !ctl.skip_loads; kb++) {
       const int s = kb % STAGES;
       const unsigned ph = (kb / STAGES) & 1;
-      if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns)) break;
+      if (!mbar_wait(smem_u32(&empty[s]), ph ^ 1, abort_flag, ctl.wait_ns, ctl.error)) break;
       unsigned char *sa = smem + s * STAGE_BYTES;
       unsigned char *sb = sa + A_BYTES;
       if (leader) mbar_expect_tx(smem_u32(&full[s]), 2 * STAGE_BYTES);
@@ -674,7 +699,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     for (int kb = 0; kb < nk; kb++) {
       const int s = kb % STAGES;
       const unsigned ph = (kb / STAGES) & 1;
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&full[s]), ph, abort_flag, ctl.wait_ns, ctl.error))) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const unsigned long long da = d0 + s * (STAGE_BYTES >> 4), db = da + (A_BYTES >> 4);
       if (elect_one()) {
@@ -691,10 +716,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   __syncwarp();
 
   // ---------------- epilogue: all 4 warps of each CTA, its own 128 rows (skipped once any CTA of the
-  // launch has given up, so that a pair whose leader aborted writes nothing)
-  const bool ready = mbar_wait(smem_u32(done), 0, abort_flag, ctl.wait_ns);
+  // call has given up, so that a pair whose leader aborted writes nothing)
+  const bool ready = mbar_wait(smem_u32(done), 0, abort_flag, ctl.wait_ns, ctl.error);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const bool failed = *reinterpret_cast<volatile unsigned *>(&g_umma_error) != 0;
+  const bool failed = *reinterpret_cast<volatile unsigned *>(ctl.error) != 0;
   if (__all_sync(0xffffffffu, ready && !*abort_flag && !failed) && nk > 0) {
     // the pair's MMAs have completed and all loads landed: the stages hold the blocks on their way out
     float *buf = reinterpret_cast<float *>(smem + warp * STORE_BYTES);
@@ -711,10 +736,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   if (threadIdx.x == 0 && leader && *abort_flag) {
     // leader after a time-out: the committed MMAs (done), then the loads it waited for of both CTAs
     // (the pair's copies complete on the leader's barriers), each with the fixed DRAIN_NS limit
-    volatile int never = 0;
-    mbar_wait(smem_u32(done), 0, &never, DRAIN_NS);
+    drain_wait(smem_u32(done), 0, ctl.error);
     for (int kb = *consumed; kb < *issued; kb++)
-      mbar_wait(smem_u32(&full[kb % STAGES]), (kb / STAGES) & 1, &never, DRAIN_NS);
+      drain_wait(smem_u32(&full[kb % STAGES]), (kb / STAGES) & 1, ctl.error);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync_all();   // neither CTA frees its TMEM or shared memory while the pair's work is in flight
@@ -807,13 +831,13 @@ template <int BN, int P>
 __device__ __forceinline__ bool emu_issue_kblock(unsigned tmem, unsigned sa0, unsigned sb, unsigned long long *afull,
                                                  unsigned long long *aempty, int &ita, bool start,
                                                  volatile int *consumed_a, volatile int *abort_flag,
-                                                 unsigned long long wait_ns) {
+                                                 unsigned long long wait_ns, unsigned *error) {
   using T = EmuTile<BN>;
   const unsigned long long db = smem_desc(sb);
 #pragma unroll
   for (int i = 1; i < P; i++, ita++) {
     const int s = ita % EMU_A_SLOTS;
-    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&afull[s]), (ita / EMU_A_SLOTS) & 1, abort_flag, wait_ns)))
+    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&afull[s]), (ita / EMU_A_SLOTS) & 1, abort_flag, wait_ns, error)))
       return false;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const unsigned long long da = smem_desc(sa0 + s * EMU_A_BYTES);
@@ -858,6 +882,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
   const int SAe = min(a.SA, a.P - 1);   // A planes with at least one partner
   const int SBe = min(a.SB, a.P - 1);
   const unsigned long long wait_ns = a.ctl.wait_ns;
+  unsigned *error = a.ctl.error;
   // tile t: split z, then groups of RASTER_GM row tiles sweep the column tiles
   auto tile_of = [&](int t, int &m0, int &n0, int &z, int &kb0, int &nk) {
     z = t / (a.nM * a.nN);
@@ -907,7 +932,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
         tile_of(t, m0, n0, z, kb0, nk);
         for (int kb = kb0; kb < kb0 + nk && ok; kb++) {
           const int sb = itb & 1;
-          if (!mbar_wait(smem_u32(&bempty[sb]), ((itb >> 1) & 1) ^ 1, abort_flag, wait_ns)) {
+          if (!mbar_wait(smem_u32(&bempty[sb]), ((itb >> 1) & 1) ^ 1, abort_flag, wait_ns, error)) {
             ok = false;
             break;
           }
@@ -916,7 +941,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
           *issued_b = ++itb;
           for (int i = 0; i < SAe; i++) {
             const int s = ita % EMU_A_SLOTS;
-            if (!mbar_wait(smem_u32(&aempty[s]), ((ita / EMU_A_SLOTS) & 1) ^ 1, abort_flag, wait_ns)) {
+            if (!mbar_wait(smem_u32(&aempty[s]), ((ita / EMU_A_SLOTS) & 1) ^ 1, abort_flag, wait_ns, error)) {
               ok = false;
               break;
             }
@@ -936,7 +961,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
       int m0, n0, z, kb0, nk;
       tile_of(t, m0, n0, z, kb0, nk);
       for (int c0 = 0; c0 < nk && ok; c0 += a.kc, ch++) {
-        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(acce), (ch & 1) ^ 1, abort_flag, wait_ns))) {
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(acce), (ch & 1) ^ 1, abort_flag, wait_ns, error))) {
           ok = false;
           break;
         }
@@ -944,7 +969,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
         const int c1 = min(nk, c0 + a.kc);
         for (int kb = c0; kb < c1 && ok; kb++, itb++) {
           const int sbuf = itb & 1;
-          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bfull[sbuf]), (itb >> 1) & 1, abort_flag, wait_ns))) {
+          if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bfull[sbuf]), (itb >> 1) & 1, abort_flag, wait_ns, error))) {
             ok = false;
             break;
           }
@@ -954,7 +979,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
           switch (a.P) {
 #define GFCC_EMU_LEVEL(P)                                                                                       \
   case P:                                                                                                       \
-    ok = emu_issue_kblock<BN, P>(tmem, sa0, sb, afull, aempty, ita, start, consumed_a, abort_flag, wait_ns); \
+    ok = emu_issue_kblock<BN, P>(tmem, sa0, sb, afull, aempty, ita, start, consumed_a, abort_flag, wait_ns, error); \
     break;
             GFCC_EMU_LEVEL(2)
             GFCC_EMU_LEVEL(3)
@@ -994,7 +1019,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
         // one lane polls and decides for the group; the other warps block on a named barrier (polling by
         // all of them takes shared-memory cycles from the loads)
         if (warp == 2 && lane == 0) {
-          const bool ready = mbar_wait(smem_u32(accf), ch & 1, abort_flag, wait_ns);
+          const bool ready = mbar_wait(smem_u32(accf), ch & 1, abort_flag, wait_ns, error);
           go[ch & 1] = ready && !*abort_flag ? 1 : 0;
         }
         __syncwarp();
@@ -1076,13 +1101,12 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
   if (threadIdx.x == 0) {
     // every MMA has completed (the drain barrier); after a time-out also the copies that were issued but
     // not consumed land before the shared memory goes away (fixed DRAIN_NS limits)
-    volatile int never = 0;
-    mbar_wait(smem_u32(drain), 0, &never, DRAIN_NS);
+    drain_wait(smem_u32(drain), 0, error);
     if (*abort_flag) {
       for (int it = *consumed_a; it < *issued_a; it++)
-        mbar_wait(smem_u32(&afull[it % EMU_A_SLOTS]), (it / EMU_A_SLOTS) & 1, &never, DRAIN_NS);
+        drain_wait(smem_u32(&afull[it % EMU_A_SLOTS]), (it / EMU_A_SLOTS) & 1, error);
       for (int it = *consumed_b; it < *issued_b; it++)
-        mbar_wait(smem_u32(&bfull[it & 1]), (it >> 1) & 1, &never, DRAIN_NS);
+        drain_wait(smem_u32(&bfull[it & 1]), (it >> 1) & 1, error);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1153,21 +1177,25 @@ int umma_splits(int K, int nsplit) {
   return (nk + kbs - 1) / kbs;
 }
 
+UmmaScope::UmmaScope(unsigned *flag) : prev(t_error_flag) { t_error_flag = flag; }
+UmmaScope::~UmmaScope() { t_error_flag = prev; }
+unsigned *umma_error_flag() { return t_error_flag; }
+
 int umma_error_reset(cudaStream_t st) {
-  const unsigned zero = 0;
-  GFCC_CUDA(cudaMemcpyToSymbolAsync(g_umma_error, &zero, sizeof(zero), 0, cudaMemcpyHostToDevice, st));
+  GFCC_CUDA(cudaMemsetAsync(t_error_flag, 0, sizeof(unsigned), st));
   return GFCC_OK;
 }
 
 int umma_error_check(cudaStream_t st) {
   unsigned h = 0;
-  GFCC_CUDA(cudaMemcpyFromSymbolAsync(&h, g_umma_error, sizeof(h), 0, cudaMemcpyDeviceToHost, st));
+  GFCC_CUDA(cudaMemcpyAsync(&h, t_error_flag, sizeof(h), cudaMemcpyDeviceToHost, st));
   GFCC_CUDA(cudaStreamSynchronize(st));
-  if (h != 0) {
-    set_error("a tensor-core GEMM wait timed out on the device");
-    return GFCC_ERR_TIMEOUT;
-  }
-  return GFCC_OK;
+  return h != 0 ? umma_timed_out() : GFCC_OK;
+}
+
+int umma_timed_out() {
+  set_error("a tensor-core GEMM wait timed out on the device");
+  return GFCC_ERR_TIMEOUT;
 }
 
 namespace {
@@ -1186,6 +1214,8 @@ template <int BN, int ST>
 int launch_umma_st(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const __nv_bfloat16 *B, long long ldb,
                    float *D, long long ldd, int M, int N, int K, float alpha, float beta, int nsplit, int kbs,
                    long long split_stride) {
+  UmmaCtl ctl;
+  GFCC_TRY(umma_ctl(&ctl));
   CUtensorMap ma, mb;
   GFCC_TRY(make_map(&ma, A, M, K, lda, BM));
   GFCC_TRY(make_map(&mb, B, N, K, ldb, BN));
@@ -1203,7 +1233,7 @@ int launch_umma_st(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const
   }
   dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN, nsplit);
   GFCC_CUDA(launch_chained(umma_bf16_gemm_kernel<BN, ST>, grid, THREADS, Tile<BN, ST>::SMEM_BYTES, st, ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
-                                                                         split_stride, umma_ctl()));
+                                                                         split_stride, ctl));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1212,6 +1242,8 @@ template <int BN>
 int launch_umma_persist(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const __nv_bfloat16 *B, long long ldb,
                         float *D, long long ldd, int M, int N, int K, float alpha, float beta, int nsplit, int kbs,
                         long long split_stride) {
+  UmmaCtl ctl;
+  GFCC_TRY(umma_ctl(&ctl));
   CUtensorMap ma, mb;
   GFCC_TRY(make_map(&ma, A, M, K, lda, BM));
   GFCC_TRY(make_map(&mb, B, N, K, ldb, BN));
@@ -1237,7 +1269,7 @@ int launch_umma_persist(cudaStream_t st, const __nv_bfloat16 *A, long long lda, 
   }
   const unsigned grid = (unsigned)std::min<long long>(tiles, sms);
   GFCC_CUDA(launch_chained(umma_persist_gemm_kernel<BN>, grid, PERSIST_THREADS, PTile<BN>::SMEM_BYTES, st, 
-      ma, mb, D, ldd, M, N, K, alpha, beta, kbs, split_stride, (int)nM, (int)nN, nsplit, umma_ctl()));
+      ma, mb, D, ldd, M, N, K, alpha, beta, kbs, split_stride, (int)nM, (int)nN, nsplit, ctl));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1246,6 +1278,8 @@ template <int PBN>
 int launch_umma_pair(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const __nv_bfloat16 *B, long long ldb,
                      float *D, long long ldd, int M, int N, int K, float alpha, float beta, int nsplit, int kbs,
                      long long split_stride) {
+  UmmaCtl ctl;
+  GFCC_TRY(umma_ctl(&ctl));
   CUtensorMap ma, mb;
   GFCC_TRY(make_map(&ma, A, M, K, lda, BM));
   GFCC_TRY(make_map(&mb, B, N, K, ldb, PairTile<PBN>::HALF));
@@ -1264,7 +1298,7 @@ int launch_umma_pair(cudaStream_t st, const __nv_bfloat16 *A, long long lda, con
   }
   dim3 grid((unsigned)(2 * mp), (N + PBN - 1) / PBN, nsplit);
   GFCC_CUDA(launch_chained(umma_pair_gemm_kernel<PBN>, grid, THREADS, PairTile<PBN>::SMEM_BYTES, st, ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
-                                                                              split_stride, umma_ctl()));
+                                                                              split_stride, ctl));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1527,7 +1561,7 @@ int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, in
   const bool pow2 = fr == 0.5;
   a.alpha_exp = pow2 ? ex - 1 : 0;
   a.alpha_mul = pow2 ? 1.0 : alpha;
-  a.ctl = umma_ctl();
+  GFCC_TRY(umma_ctl(&a.ctl));
   a.part = a.nz > 1 ? work : nullptr;
   if ((long long)a.nM * a.nN * a.nz > 0x7fffffffLL || a.kc < 1) {
     set_error("emu_gemm_fused: too many tiles (M=%d, N=%d)", M, N);

@@ -1,0 +1,64 @@
+"""Calls whose tensor-core products cannot finish report GFCC_ERR_TIMEOUT, and soon.
+
+As in test_gpu_failure.py the bounded waits are made to run out on the host's order: their producers issue no loads
+(GFCC_OPT_TEST_NO_LOADS) and the limit (GFCC_OPT_WAIT_NS) is short.  Afterwards the same calls give what they gave before.
+"""
+import time
+from contextlib import contextmanager
+
+import numpy as np
+import pytest
+
+from paper_2010_04768_gb300 import gfcc
+from paper_2010_04768_gb300.synthetic import make_problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2010_04768_gb300 import build
+    build.build()
+    gfcc.load()
+
+
+@contextmanager
+def no_loads(wait_ns):
+    gfcc.set_process_option(gfcc.OPT_AUTOTUNE, 0.0)   # no tile is chosen from launches that do nothing
+    gfcc.set_process_option(gfcc.OPT_WAIT_NS, wait_ns)
+    gfcc.set_process_option(gfcc.OPT_TEST_NO_LOADS, 1.0)
+    try:
+        yield
+    finally:
+        gfcc.set_process_option(gfcc.OPT_TEST_NO_LOADS, 0.0)
+        gfcc.set_process_option(gfcc.OPT_WAIT_NS, 1e9)
+        gfcc.set_process_option(gfcc.OPT_AUTOTUNE, 1.0)
+
+
+def timed_out(call, wait_ns=2000.0, within=None):
+    t = time.perf_counter()
+    with no_loads(wait_ns):
+        with pytest.raises(gfcc.GFCCError) as e:
+            call()
+    assert e.value.code == gfcc.ERR_TIMEOUT
+    if within is not None:
+        assert time.perf_counter() - t < within
+
+
+@pytest.mark.parametrize("guess", [False, True])
+def test_mixed_solve_ends_after_about_one_limit(guess):
+    # 20 ms a wait: the products of one Arnoldi step alone would take 0.1 s one after the other, a refinement of 60
+    # steps 6 s
+    om, orbs = [-0.7, -0.6], [0, 3, 5]
+    g = gfcc.GFCC(make_problem(6, 30, 60, seed=4), sectors="IP", precision="mixed")
+    if guess:
+        g.set_option(gfcc.OPT_GUESS, gfcc.GUESS_MINRES)
+    other = gfcc.GFCC(make_problem(5, 24, 50, seed=5), sectors="IP", precision="mixed")
+    ref, ref_other = g.solve(om, 0.01, orbs, 1e-9)[0], other.solve(om, 0.01, [1, 2], 1e-9)[0]
+    timed_out(lambda: g.solve(om, 0.01, orbs, 1e-9), wait_ns=2e7, within=1.5)
+    # neither another context nor this one's next call sees it
+    for k, (a, b) in ((other, ([1, 2], ref_other)), (g, (orbs, ref))):
+        G, code = k.solve(om, 0.01, a, 1e-9)
+        assert code == gfcc.OK and np.abs(G - b).max() <= 1e-7 * np.abs(b).max()
+    g.close()
+    other.close()
