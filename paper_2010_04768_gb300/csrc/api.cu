@@ -537,6 +537,8 @@ int create_impl(int o, int v, int L, const double *fock, const double *chol, con
       g_emu_arena = nullptr;
       g_emulate_big = false;
     }
+    // a wait of a digit-plane product that ran out left elements unwritten
+    if (s >= 0 && precision == GFCC_PREC_MIXED_BF16) s = umma_error_check(c->stream);
     if (timed) {
       cudaEventRecord(e1, c->stream);
       cudaEventSynchronize(e1);
@@ -613,6 +615,7 @@ int solve_impl(gfcc_ctx *c, int n_omega, const double *d_om, double eta, const O
     PhaseTimer tm(c, PH_SOLVE);
     rc = solve_impl_inner(c, n_omega, d_om, eta, ol, tol, d_G);
   }
+  if (rc >= 0 && c->rhf) GFCC_TRY(umma_error_check(st));   // the operator's digit-plane products
   if (c->prof) {
     GFCC_CUDA(cudaStreamSynchronize(st));
     prof_resolve(c);
@@ -1574,6 +1577,7 @@ int gfcc_sigma_ex(gfcc_ctx *c, int sector, int precision, int n_vec, const doubl
     GFCC_TRY(umma_error_check(c->stream));
   } else {
     GFCC_TRY(sector == GFCC_SECTOR_IP ? apply_ip(c, b, w) : apply_ea(c, b, w));
+    if (c->rhf) GFCC_TRY(umma_error_check(c->stream));
   }
   GFCC_CUDA(cudaMemcpyAsync(y, dy, sizeof(double) * 2 * n_vec * n, cudaMemcpyDeviceToHost, c->stream));
   GFCC_CUDA(cudaStreamSynchronize(c->stream));

@@ -662,6 +662,7 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
     it_info[2] = rmax;
     it_info[7] = fl;
     GFCC_TRY(C.energy(C.x, &it_info[0]));
+    GFCC_TRY(umma_error_check(st));   // a wait of a digit-plane product that ran out left a result unwritten
     GFCC_CUDA(cudaMemcpyAsync(t1, C.x, sizeof(double) * ov, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaMemcpyAsync(t2, C.x + ov, sizeof(double) * ov * ov, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaStreamSynchronize(st));
@@ -679,7 +680,7 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
       double lr = 0.0;
       const int st_l = C.iterate(true, tol, max_iter, &lit, &lr, nullptr);
       GFCC_TRY(st_l);
-      GFCC_CUDA(cudaStreamSynchronize(st));
+      GFCC_TRY(umma_error_check(st));
       it_info[6] = seconds_since(t0);
       it_info[3] = lit;
       it_info[4] = lr;

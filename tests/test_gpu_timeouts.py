@@ -10,7 +10,7 @@ import numpy as np
 import pytest
 
 from paper_2010_04768_gb300 import gfcc
-from paper_2010_04768_gb300.synthetic import make_problem
+from paper_2010_04768_gb300.synthetic import make_closed_shell_problem, make_problem, random_vector
 
 pytestmark = pytest.mark.gpu
 
@@ -62,3 +62,35 @@ def test_mixed_solve_ends_after_about_one_limit(guess):
         assert code == gfcc.OK and np.abs(G - b).max() <= 1e-7 * np.abs(b).max()
     g.close()
     other.close()
+
+
+def test_mixed_context_creation():
+    pr = make_problem(6, 40, 80, seed=3)
+    timed_out(lambda: gfcc.GFCC(pr, sectors="IP+EA", precision="mixed"))
+    g = gfcc.GFCC(pr, sectors="IP", precision="mixed")
+    assert g.solve([-0.5], 0.01, [0, 1, 2], 1e-9)[1] == gfcc.OK
+    g.close()
+
+
+def test_emulated_ccsd():
+    pr = make_problem(6, 40, 60, seed=3)
+
+    def call():
+        return gfcc.ccsd(pr.fock, pr.chol, pr.o, tol=1e-8, want_lambda=True, emulate=True)
+
+    ref = call()
+    timed_out(call)
+    got = call()
+    assert got[-1] == ref[-1] and all(np.array_equal(a, b) for a, b in zip(got[:4], ref[:4]))
+
+
+def test_closed_shell_operator():
+    g = gfcc.GFCC(make_closed_shell_problem(10, 60, 100, seed=2), sectors="IP", closed_shell=True)
+    x = np.stack([random_vector(k, g.dims()[0]) + 1j * random_vector(20 + k, g.dims()[0]) for k in range(8)])
+    orbs = np.arange(2, 10)
+    ref, G0 = g.sigma("IP", x), g.solve([-0.6], 0.01, orbs, 1e-8)[0]
+    timed_out(lambda: g.sigma("IP", x))
+    timed_out(lambda: g.solve([-0.6], 0.01, orbs, 1e-8))
+    assert np.array_equal(g.sigma("IP", x), ref)
+    assert np.array_equal(g.solve([-0.6], 0.01, orbs, 1e-8)[0], G0)
+    g.close()
