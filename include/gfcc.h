@@ -105,7 +105,8 @@ extern "C" {
                                      the value is above the default                                    */
 #define GFCC_OPT_WAIT_NS    20    /* limit of the bounded waits of the tensor-core kernels in
                                      nanoseconds (1 .. 1e11); default 1e9.  A wait that runs out makes
-                                     the call return GFCC_ERR_TIMEOUT                                   */
+                                     the call return GFCC_ERR_TIMEOUT; so does a solver step that takes
+                                     the GPU more than 60 times this value (and 2 s)                    */
 #define GFCC_OPT_TEST_NO_LOADS 21 /* test only: 1 makes the tensor-core kernels issue no loads, so that
                                      their first wait runs out (with nothing in flight) and the call
                                      returns GFCC_ERR_TIMEOUT; default 0                               */
@@ -335,6 +336,13 @@ int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B,
  * A (M x K), B (N x K), C (M x N): row-major FP64 HOST arrays.
  */
 int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double *B, int S, int P, double *C);
+
+/*
+ * gfcc_selftest_host_wait - the bounded host wait of the solvers on a stream that stays busy for busy_ns
+ * (at most 5e9) nanoseconds: GFCC_ERR_TIMEOUT beyond 60 times GFCC_OPT_WAIT_NS (2 s at least), else GFCC_OK.
+ * The stream is idle again on return.
+ */
+int gfcc_selftest_host_wait(double busy_ns);
 
 /*
  * gfcc_guess_stats - initial-guess statistics of the last gfcc_solve, in the entry order of

@@ -4,6 +4,7 @@
 // right-hand sides, left vectors and overlaps of eqs. gfxn2/gfxn3.
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstdarg>
 #include <cstring>
@@ -84,6 +85,26 @@ void dfree(void *p) {
   if (p == nullptr) return;
   unreg_alloc(p);
   cudaFree(p);
+}
+
+int wait_stream(cudaStream_t st) {
+  const auto begin = std::chrono::steady_clock::now(), limit = begin + std::chrono::nanoseconds(host_wait_limit());
+  for (;;) {
+    const cudaError_t e = cudaStreamQuery(st);
+    if (e == cudaSuccess) return GFCC_OK;
+    if (e != cudaErrorNotReady) GFCC_CUDA(e);
+    cudaGetLastError();
+    const auto now = std::chrono::steady_clock::now();
+    if (now > limit) {
+      set_error("a stream's work has not ended after %.1f s", 1e-9 * (double)host_wait_limit());
+      return GFCC_ERR_TIMEOUT;
+    }
+    // a question takes about a microsecond and a lock that launching threads need
+    if (now - begin > std::chrono::microseconds(20)) {
+      const auto next = now + std::chrono::microseconds(5);
+      while (std::chrono::steady_clock::now() < next) std::this_thread::yield();
+    }
+  }
 }
 
 static std::atomic<long long> g_launches{0};
@@ -609,6 +630,8 @@ int solve_impl(gfcc_ctx *c, int n_omega, const double *d_om, double eta, const O
                double *d_G) {
   cudaStream_t st = c->stream;
   UmmaScope umma(c->umma_flag);
+  // what a caller's stream still holds does not count towards the limits of the solver's host waits
+  if (st != c->own_stream) GFCC_CUDA(cudaStreamSynchronize(st));
   if (c->precision == GFCC_PREC_MIXED_BF16 || c->rhf) GFCC_TRY(umma_error_reset(st));
   int rc;
   {
@@ -1118,6 +1141,11 @@ int solve_host(gfcc_ctx *c, int n_omega, const double *omegas, double eta, int n
       s = GFCC_ERR_CUDA;
     }
   }
+  if (c->stuck && cudaStreamQuery(c->stream) == cudaErrorNotReady) {   // left to the running work
+    cudaGetLastError();
+    return s;
+  }
+  c->stuck = false;
   dfree(d_om);
   dfree(d_P);
   dfree(d_Q);
@@ -1195,6 +1223,18 @@ int solve_for_sink(gfcc_ctx *c, int sector, int n_omega, const double *h_om, dou
   c->sectors = saved;
   return rc;
 }
+
+namespace {
+// holds one thread of the GPU for ns
+__global__ void busy_kernel(unsigned long long ns) {
+  unsigned long long t0, t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t0));
+  do {
+    __nanosleep(1000);
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  } while ((long long)(t - t0) < (long long)ns);
+}
+}  // namespace
 
 }  // namespace gfcc
 
@@ -1596,6 +1636,7 @@ int gfcc_dims(gfcc_ctx *c, long long *dim_ip, long long *dim_ea) {
 
 void gfcc_destroy(gfcc_ctx *c) {
   if (c == nullptr) return;
+  if (c->stuck && wait_stream(c->stream) == GFCC_ERR_TIMEOUT) return;   // its memory is left to the running work
   if (c->stream) cudaStreamSynchronize(c->stream);
   prof_resolve(c);
   for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
@@ -1639,6 +1680,20 @@ int gfcc_profile_read(gfcc_ctx *c, int phase, double *ms, long long *count, doub
   if (count) *count = c->prof_n[phase];
   if (flops) *flops = c->prof_flops[phase];
   return GFCC_OK;
+}
+
+int gfcc_selftest_host_wait(double busy_ns) {
+  if (!(busy_ns >= 0.0 && busy_ns <= 5e9)) {
+    set_error("gfcc_selftest_host_wait: 0 to 5e9 nanoseconds (got %g)", busy_ns);
+    return GFCC_ERR_ARG;
+  }
+  cudaStream_t st = nullptr;
+  GFCC_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+  busy_kernel<<<1, 1, 0, st>>>((unsigned long long)busy_ns);
+  int s = cudaGetLastError() == cudaSuccess ? wait_stream(st) : GFCC_ERR_CUDA;
+  cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return s;
 }
 
 long long gfcc_launch_count(void) { return gfcc::g_launches.load(); }

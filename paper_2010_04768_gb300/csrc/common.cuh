@@ -23,6 +23,13 @@ int check_extent_bytes(const void *p, long long bytes, const char *what);
 cudaError_t dmalloc(void **p, size_t bytes);   // cudaMalloc + reg_alloc
 void dfree(void *p);                           // unreg_alloc + cudaFree
 
+// Waits on the host for the work of a stream, with a limit (host_wait_limit): GFCC_OK, GFCC_ERR_CUDA, or
+// GFCC_ERR_TIMEOUT when the work has not ended by then.
+int wait_stream(cudaStream_t st);
+// Nanoseconds after which the host gives up a step of a solver: far above what a step takes, and above the limits of the
+// device waits that a step may run into one after the other.
+unsigned long long host_wait_limit();
+
 // Evaluate a CUDA runtime call; on failure record the message and return GFCC_ERR_CUDA.
 #define GFCC_CUDA(call)                                                                 \
   do {                                                                                  \

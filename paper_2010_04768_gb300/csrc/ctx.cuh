@@ -164,6 +164,7 @@ struct gfcc_ctx {
   // one solver that runs on the context)
   int *step_flags = nullptr, *step_flags_dev = nullptr;
   int step_flags_cap = 0;
+  bool stuck = false;   // a host wait has given up: the stream may still run, and frees would wait for it without end
   // scratch reused across solves (grown on demand)
   void *scratch = nullptr;
   size_t scratch_bytes = 0;

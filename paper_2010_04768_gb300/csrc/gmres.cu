@@ -17,6 +17,8 @@
 #include <cmath>
 #include <cstring>
 #include <chrono>
+#include <cstdio>
+#include <thread>
 #include <vector>
 
 #include "ctx.cuh"
@@ -1018,29 +1020,52 @@ int Gmres::solve(double tol, int max_iters, int *h_state, int max_cycles, bool u
              : solve_t<double>(tol, max_iters, h_state, max_cycles, use_x0);
 }
 
+int Gmres::gave_up(const char *what, int step, const int *h_state) {
+  char which[96] = "";
+  int len = 0;
+  for (int s = 0; s < nsys && h_state != nullptr && len < 80; s++)
+    if (h_state[s] == ST_IN_CYCLE) len += std::snprintf(which + len, sizeof(which) - len, " %d", s);
+  c->stuck = true;
+  set_error("the GPU has not finished %s of the %s sector after %.1f s (step %d of %d, %d systems, in cycle:%s)", what,
+            sector == GFCC_SECTOR_IP ? "IP" : "EA", 1e-9 * (double)host_wait_limit(), step, m, nsys, which);
+  return GFCC_ERR_TIMEOUT;
+}
+
+int Gmres::wait(const char *what, int step, const int *h_state) {
+  const int s = wait_stream(c->stream);
+  return s == GFCC_ERR_TIMEOUT ? gave_up(what, step, h_state) : s;
+}
+
 // The Givens update of a system writes its iteration count and state to mapped host memory; the host reads them there
 // while the step's last kernel is still running, instead of a copy and a wait for the stream (some 10 us of idle GPU
 // a step).  Every 100 us without an answer the stream is asked: a failed one is an error, a finished one gives the
-// states by copy.
-int Gmres::wait_step(int *h_state, std::vector<int> &h_it) {
+// states by copy, and one that runs on beyond the limit of the host's waits ends the solve.
+int Gmres::wait_step(int step, int *h_state, std::vector<int> &h_it) {
   cudaStream_t st = c->stream;
   bool copy = c->step_flags == nullptr;
-  auto last = std::chrono::steady_clock::now();
+  if (copy) GFCC_TRY(wait("an Arnoldi step", step, h_state));
+  const auto begin = std::chrono::steady_clock::now(), limit = begin + std::chrono::nanoseconds(host_wait_limit());
+  auto last = begin;
   for (int s = 0; s < nsys && !copy; s++) {
     if (h_state[s] != ST_IN_CYCLE) continue;
     const int want = h_it[s] + 1;
     int v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
     for (unsigned spin = 1; (v >> 3) != want; spin++) {
-      if ((spin & 0xff) == 0 && std::chrono::steady_clock::now() - last > std::chrono::microseconds(100)) {
-        const cudaError_t e = cudaStreamQuery(st);
-        if (e != cudaErrorNotReady) {
-          GFCC_CUDA(e);
-          v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
-          copy = (v >> 3) != want;
-          break;
+      if ((spin & 0xff) == 0) {
+        const auto now = std::chrono::steady_clock::now();
+        if (now - last > std::chrono::microseconds(100)) {
+          const cudaError_t e = cudaStreamQuery(st);
+          if (e != cudaErrorNotReady) {
+            GFCC_CUDA(e);
+            v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
+            copy = (v >> 3) != want;
+            break;
+          }
+          cudaGetLastError();
+          if (now > limit) return gave_up("an Arnoldi step", step, h_state);
+          std::this_thread::yield();
+          last = now;
         }
-        cudaGetLastError();
-        last = std::chrono::steady_clock::now();
       }
       v = __atomic_load_n(&c->step_flags[s], __ATOMIC_ACQUIRE);
     }
@@ -1123,6 +1148,7 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
     GFCC_LAUNCH_CHECK();
     if (cycle == 0) GFCC_CUDA(cudaMemcpyAsync(relres0, relres, sizeof(double) * nsys, cudaMemcpyDeviceToDevice, st));
     first = false;
+    GFCC_TRY(wait("the residual of a cycle"));
     GFCC_CUDA(cudaMemcpyAsync(h_state, state, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaStreamSynchronize(st));
     bool any = false;
@@ -1199,7 +1225,7 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
         }
       }
       if (!done_step) GFCC_TRY(step());
-      GFCC_TRY(wait_step(h_state, h_it));
+      GFCC_TRY(wait_step(k, h_state, h_it));
       active = 0;
       for (int s = 0; s < nsys; s++) active += h_state[s] == ST_IN_CYCLE;
       if (active == 0) break;
@@ -1355,6 +1381,7 @@ int Gmres::residual_update() {
     absmax_kernel<<<gr, 256, 0, st>>>(D, n, am + nsys);
     GFCC_LAUNCH_CHECK();
     std::vector<unsigned long long> h(2 * (size_t)nsys);
+    GFCC_TRY(wait("a residual"));
     GFCC_CUDA(cudaMemcpyAsync(h.data(), am, sizeof(unsigned long long) * 2 * nsys, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaStreamSynchronize(st));
     int drop = 1 << 20;
@@ -1395,6 +1422,7 @@ int Gmres::refine_residual_free(int *h_done, double *h_relres) {
   refine_check_kernel<<<cdiv(nsys, 256), 256, 0, st>>>(nsys, nrm, NV, b0norm, tol_outer, kcyc, relres,
                                                          umma_error_flag());
   GFCC_LAUNCH_CHECK();
+  GFCC_TRY(wait("a refinement"));
   GFCC_CUDA(cudaMemcpyAsync(h_done, kcyc, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
   GFCC_CUDA(cudaMemcpyAsync(h_relres, relres, sizeof(double) * nsys, cudaMemcpyDeviceToHost, st));
   GFCC_CUDA(cudaStreamSynchronize(st));
@@ -1415,6 +1443,7 @@ int Gmres::refine_correct(const int *h_done, int *h_state, int *h_iters) {
     GFCC_CUDA(cudaMemcpyAsync(B, R, sizeof(double) * tot, cudaMemcpyDeviceToDevice, st));
   }
   GFCC_TRY(solve(c->inner_tol, c->max_iters, h_state, c->inner_cycles));
+  GFCC_TRY(wait("an inner solve"));
   std::vector<int> it(nsys);
   GFCC_CUDA(cudaMemcpyAsync(it.data(), iters, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
   if (f32)
@@ -1458,6 +1487,7 @@ int Gmres::solve_refined(double tol, double inner_tol, int max_iters, int *h_sta
                                                        umma_error_flag());
     GFCC_LAUNCH_CHECK();
     if (outer == 0) GFCC_CUDA(cudaMemcpyAsync(relres0, relres, sizeof(double) * nsys, cudaMemcpyDeviceToDevice, st));
+    GFCC_TRY(wait("a refinement"));
     GFCC_CUDA(cudaMemcpyAsync(h_done.data(), done, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaStreamSynchronize(st));
     if (h_done[0] < 0) return umma_timed_out();
@@ -1482,6 +1512,7 @@ int Gmres::solve_refined(double tol, double inner_tol, int max_iters, int *h_sta
       GFCC_CUDA(cudaMemcpyAsync(B, R, sizeof(double) * tot, cudaMemcpyDeviceToDevice, st));
     }
     GFCC_TRY(solve(inner_tol, max_iters, h_state, c->inner_cycles));
+    GFCC_TRY(wait("an inner solve"));
     GFCC_CUDA(cudaMemcpyAsync(it.data(), iters, sizeof(int) * nsys, cudaMemcpyDeviceToHost, st));
     GFCC_CUDA(cudaStreamSynchronize(st));
     for (int s = 0; s < nsys; s++) h_iters[s] += it[s];

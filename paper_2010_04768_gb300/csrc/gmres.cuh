@@ -39,7 +39,9 @@ struct Gmres {
   unsigned *blk_cnt = nullptr;      // per system: blocks of the running kernel that have finished
   long long partial_chunks = 0;     // chunks of partial sums over all systems that `partial` holds
   // host side of an Arnoldi step: the state of the systems in cycle, as soon as their Givens update has run
-  int wait_step(int *h_state, std::vector<int> &h_it);
+  int wait_step(int step, int *h_state, std::vector<int> &h_it);
+  int wait(const char *what, int step = -1, const int *h_state = nullptr);   // for the stream, with a limit
+  int gave_up(const char *what, int step, const int *h_state);
   int *act = nullptr;   // the systems the operator runs on in an Arnoldi step (see solve_t)
   double *relres0 = nullptr;   // relative residual of the initial iterate (first true residual)
   double *sigma_work = nullptr;

@@ -1586,6 +1586,8 @@ void umma_set_autotune(bool on) { g_autotune = on; }
 void umma_set_pair_mode(int mode) { g_pair_mode = mode; }
 void umma_set_persist_mode(int mode) { g_persist_mode = mode; }
 
+unsigned long long host_wait_limit() { return std::max(2000000000ULL, 60 * g_wait_ns); }
+
 void umma_set_wait(unsigned long long wait_ns, bool skip_loads) {
   g_wait_ns = wait_ns;
   g_skip_loads = skip_loads;

@@ -85,6 +85,8 @@ def load():
     fp = ctypes.POINTER(ctypes.c_float)
     lib.gfcc_selftest_gemm_bf16.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, fp, fp, fp]
     lib.gfcc_selftest_gemm_bf16.restype = ctypes.c_int
+    lib.gfcc_selftest_host_wait.argtypes = [ctypes.c_double]
+    lib.gfcc_selftest_host_wait.restype = ctypes.c_int
     lib.gfcc_selftest_gemm_f64emu.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, dp, dp, ctypes.c_int,
                                               ctypes.c_int, dp]
     lib.gfcc_selftest_gemm_f64emu.restype = ctypes.c_int
@@ -177,6 +179,11 @@ def selftest_gemm_f64emu(A: np.ndarray, B: np.ndarray, S: int = 8, P: int = 9) -
     C = np.zeros((M, N), dtype=np.float64)
     _check(load().gfcc_selftest_gemm_f64emu(M, N, K, _dp(A), _dp(B), S, P, _dp(C)))
     return C
+
+
+def selftest_host_wait(busy_s: float):
+    """The solvers' bounded host wait on a stream that stays busy for busy_s seconds."""
+    _check(load().gfcc_selftest_host_wait(1e9 * busy_s))
 
 
 def _dp(a: np.ndarray):

@@ -94,3 +94,16 @@ def test_closed_shell_operator():
     assert np.array_equal(g.sigma("IP", x), ref)
     assert np.array_equal(g.solve([-0.6], 0.01, orbs, 1e-8)[0], G0)
     g.close()
+
+
+def test_host_wait_gives_up():
+    gfcc.selftest_host_wait(0.0)
+    gfcc.selftest_host_wait(0.3)
+    gfcc.set_process_option(gfcc.OPT_WAIT_NS, 2000.0)   # the host's limit: 2 s
+    try:
+        with pytest.raises(gfcc.GFCCError) as e:
+            gfcc.selftest_host_wait(2.5)
+    finally:
+        gfcc.set_process_option(gfcc.OPT_WAIT_NS, 1e9)
+    assert e.value.code == gfcc.ERR_TIMEOUT
+    gfcc.selftest_host_wait(2.5)
