@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <thread>
 #include <vector>
@@ -86,6 +87,18 @@ void dfree(void *p) {
   unreg_alloc(p);
   cudaFree(p);
 }
+
+namespace {
+std::atomic<int> g_calls{0};
+thread_local int t_calls = 0;   // nested calls of a thread count once
+}  // namespace
+CallScope::CallScope() {
+  if (t_calls++ == 0) g_calls.fetch_add(1);
+}
+CallScope::~CallScope() {
+  if (--t_calls == 0) g_calls.fetch_sub(1);
+}
+bool concurrent_calls() { return g_calls.load(std::memory_order_relaxed) > 1; }
 
 int wait_stream(cudaStream_t st) {
   const auto begin = std::chrono::steady_clock::now(), limit = begin + std::chrono::nanoseconds(host_wait_limit());
@@ -494,6 +507,7 @@ int create_impl(int o, int v, int L, const double *fock, const double *chol, con
     if ((s = dev_alloc(c, &flag, 1)) < 0) return fail(s);
     c->umma_flag = reinterpret_cast<unsigned *>(flag);
   }
+  CallScope call;
   UmmaScope umma(c->umma_flag);
   if ((s = umma_error_reset(c->stream)) < 0) return fail(s);
   const long long n = c->n, nn = n * n, ov = (long long)o * v, oovv = ov * ov;
@@ -629,6 +643,7 @@ int grow_scratch(gfcc_ctx *c, size_t bytes) {
 int solve_impl(gfcc_ctx *c, int n_omega, const double *d_om, double eta, const OrbLists &ol, double tol,
                double *d_G) {
   cudaStream_t st = c->stream;
+  CallScope call;
   UmmaScope umma(c->umma_flag);
   // what a caller's stream still holds does not count towards the limits of the solver's host waits
   if (st != c->own_stream) GFCC_CUDA(cudaStreamSynchronize(st));
@@ -1499,6 +1514,8 @@ int gfcc_solve_batch(gfcc_ctx *const *ctxs, int n_ctx, const gfcc_request *reqs,
     share[i] = ctxs[i]->mem_share;
     ctxs[i]->mem_share = share[i] / nthreads;   // concurrent solves split the free memory
   }
+  // counts beside the threads' calls, so that they take the shared GPU into account from the first
+  const std::unique_ptr<CallScope> batch(nthreads > 1 ? new CallScope : nullptr);
   std::atomic<int> next{0};
   auto worker = [&]() {
     if (cudaSetDevice(dev) != cudaSuccess) {
@@ -1607,6 +1624,7 @@ int gfcc_sigma_ex(gfcc_ctx *c, int sector, int precision, int n_vec, const doubl
   b.nsys = n_vec;
   b.x = dx; b.ldx = n;
   b.y = dy; b.ldy = n;
+  CallScope call;
   UmmaScope umma(c->umma_flag);
   if (mixed || emu || c->rhf) GFCC_TRY(umma_error_reset(c->stream));
   if (mixed || emu) {
@@ -1722,6 +1740,7 @@ int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double
     s = GFCC_ERR_CUDA;
   }
   EmuOperand ea, eb;
+  CallScope call;
   UmmaScope umma(static_cast<unsigned *>(flag));
   if (s == GFCC_OK) s = umma_error_reset(st);
   if (s == GFCC_OK) s = emu_slice(st, static_cast<double *>(da), M, K, K, S, sa, ea);
@@ -1770,6 +1789,7 @@ int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B,
     set_error("gfcc_selftest_gemm_bf16: copy failed");
     s = GFCC_ERR_CUDA;
   }
+  CallScope call;
   UmmaScope umma(static_cast<unsigned *>(flag));
   if (s == GFCC_OK) s = umma_error_reset(st);
   if (s == GFCC_OK)

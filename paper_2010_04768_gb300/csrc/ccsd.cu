@@ -627,6 +627,7 @@ int ccsd_impl(int o, int v, int L, const double *fock, const double *chol, doubl
     cudaStreamDestroy(st);
     return GFCC_ERR_OOM;
   }
+  CallScope call;
   UmmaScope umma(static_cast<unsigned *>(flag));
   const bool prev_emulate = g_emulate_big;
   const double prev_min = g_emulate_min_flops_local;

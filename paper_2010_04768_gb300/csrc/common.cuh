@@ -58,6 +58,19 @@ long long thread_launch_count();   // the calling thread's share (concurrent sol
     GFCC_CUDA(cudaGetLastError()); \
   } while (0)
 
+// Calls that use the GPU, counted over all threads from entry to return.
+struct CallScope {
+  CallScope();
+  ~CallScope();
+  CallScope(const CallScope &) = delete;
+  CallScope &operator=(const CallScope &) = delete;
+};
+// Whether another thread's call shares the GPU (or will: gfcc_solve_batch counts as one beside its threads' calls).
+// Then launches are plain ones, no tile is chosen from timings, and products stay on one-CTA tiles: batches of
+// mixed-precision solves on four streams stalled now and then with chained launches, CTA-pair tiles and timings taken
+// beside other streams, and which of these did it is not known.
+bool concurrent_calls();
+
 // Chained launches: the kernels of an Arnoldi step follow one another with some microseconds of work each, so the
 // gap between two of them counts.  A kernel launched by launch_chained may be scheduled while the kernel before it in
 // the stream still runs (its blocks then hold no more than their slots) and starts with chain_start: it lets its own
@@ -82,7 +95,7 @@ static inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, di
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = concurrent_calls() ? 0 : 1;   // without its predecessor's overlap chain_start does nothing
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

@@ -500,6 +500,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   const long long n = M->n;
   const int m = M->m;
   const bool ip = M->sector == GFCC_SECTOR_IP;
+  CallScope call;
   UmmaScope umma(c->umma_flag);
   if (m < 1) {
     set_error("gfcc_mor_green: the subspace is empty (gfcc_mor_expand first)");
@@ -668,6 +669,7 @@ int mor_expand_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, in
   cudaStream_t st = c->stream;
   const long long n = M->n;
   const long long ntasks = (long long)n_omega * n_orb;
+  CallScope call;
   // solutions of the full systems (the hot path), then Gram-Schmidt of their real and imaginary parts
   double *sink = nullptr;
   if (dmalloc(reinterpret_cast<void **>(&sink), sizeof(double) * 2 * (size_t)ntasks * n) != cudaSuccess) {

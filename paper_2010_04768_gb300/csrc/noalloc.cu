@@ -73,6 +73,7 @@ extern "C" int gfcc_sigma_noalloc(gfcc_ctx *c, int sector, int n_vec, const doub
               n_vec, need, NOALLOC_SCRATCH_DOUBLES, longk);
     return GFCC_ERR_ARG;
   }
+  CallScope call;
   double *w = nullptr;
   GFCC_TRY(scratch_address(&w));
   SysBatch b;

@@ -1359,7 +1359,8 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
   // the pair kernel needs two row tiles and pays off on wide products with a long K loop; its widths by the waves of
   // 76 pairs (clocks of a tile: a K block's loads at 55 bytes a clock, some 16 a column and 6000 for its ends).
   // 3591 x 1620 x 3591: 192 columns 38 us, 256 columns 50 us; 8000 x 3200 x 8000: 256 columns 257 us, 128 348 us.
-  const bool pair_ok = g_pair_mode != 2 && M > BM && N > 128 && kbs >= 8;
+  const bool alone = !concurrent_calls();
+  const bool pair_ok = g_pair_mode != 2 && M > BM && N > 128 && kbs >= 8 && alone;
   auto pair_cost = [&](int w) {
     const long long tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + w - 1LL) / w) * nsplit;
     return (double)((tiles + 75) / 76) * (kbs * (298.0 + 1.16 * w) + 16.0 * w + 6000.0);
@@ -1375,7 +1376,17 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
   const bool persist_ok = g_persist_mode != 2 && tiles_narrow > 2 * 152;
   // default: the narrowest tile that covers N (wide N keeps the 256-column tile)
   int bn = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
-  if (g_autotune && beta != 0.0f) {
+  if (!alone) {
+    // beside other calls no launch is timed: the one-CTA tile whose busiest SM has the least to do, by the clocks of
+    // pair_cost (without the halved B tile)
+    auto cost = [&](int w) {
+      const long long tiles = ((M + BM - 1LL) / BM) * ((N + w - 1LL) / w) * nsplit;
+      return (double)((tiles + 151) / 152) * (kbs * (298.0 + 2.33 * w) + 16.0 * w + 6000.0);
+    };
+    bn = 64;
+    for (int w : {128, 256})
+      if (w / 2 < N && cost(w) < cost(bn)) bn = w;
+  } else if (g_autotune && beta != 0.0f) {
     // accumulating calls are not timed (they would change D); they reuse a tuned choice if any
     const int t = umma_tuned_tile(M, N, K, nsplit);
     if (t) bn = t;
