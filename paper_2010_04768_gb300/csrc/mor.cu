@@ -492,6 +492,8 @@ int project_new(gfcc_mor *M, int k0) {
 
 }  // namespace
 
+constexpr int MODEL_SMEM = 220 * 1024;   // shared memory of a model solve at most
+
 // Model Green's function on a frequency grid (the sector of the object): rows / columns as gfcc_solve_block.
 int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int nP, const int *h_P, int nQ,
                    const int *h_Q, double *h_G, double *h_relres) {
@@ -561,48 +563,55 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   double *Ax = res + 2LL * wb * nb;                    // [2 wb nb][n]
   double *Cx = Ax + (planes ? 2LL * wb * nb * n : 0);  // [2 wb nb][2 m]
   int s = GFCC_OK;
-  auto done = [&](int code) {
-    dfree(d_lists);
-    return code;
-  };
+  double *Hm = nullptr;
+  struct Free {   // on every way out
+    int *&lists;
+    double *&H;
+    ~Free() {
+      dfree(lists);
+      dfree(H);
+    }
+  } free_both{d_lists, Hm};
   if (cudaMemcpyAsync(d_lists, h_b, sizeof(int) * nb, cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(d_lists + nb, h_l, sizeof(int) * nl, cudaMemcpyHostToDevice, st) != cudaSuccess ||
       cudaMemcpyAsync(om, h_om, sizeof(double) * n_omega, cudaMemcpyHostToDevice, st) != cudaSuccess) {
     set_error("gfcc_mor_green: host-to-device copy failed");
-    return done(GFCC_ERR_CUDA);
+    return GFCC_ERR_CUDA;
   }
-  if ((s = build_rhs(c, M->sector, nb, d_lists, Bc, st)) < 0) return done(s);
+  if ((s = build_rhs(c, M->sector, nb, d_lists, Bc, st)) < 0) return s;
   mor_real_kernel<<<grid1d((long long)nb * n), MT, 0, st>>>(Bc, n, nb, Br);
   GFCC_LAUNCH_CHECK();
-  if ((s = build_left_vectors(c, M->sector, nl, d_lists + nb, Cl, st)) < 0) return done(s);
+  if ((s = build_left_vectors(c, M->sector, nl, d_lists + nb, Cl, st)) < 0) return s;
   // bh[k][r] = S_k . b_r, ch[k][q] = S_k . c_q
   if ((s = gemm_f64(st, m, nb, n, 1.0, M->S, imap1(n), imap1(1), Br, imap1(1), imap1(n), 0.0, bh, imap1(nb),
                     imap1(1))) < 0)
-    return done(s);
+    return s;
   if ((s = gemm_f64(st, m, nl, n, 1.0, M->S, imap1(n), imap1(1), Cl, imap1(1), imap1(n), 0.0, ch, imap1(nl),
                     imap1(1))) < 0)
-    return done(s);
+    return s;
   // Hhat packed with row stride m for the model kernel
-  double *Hm = nullptr;
   if (dmalloc(reinterpret_cast<void **>(&Hm), sizeof(double) * (size_t)m * m) != cudaSuccess) {
     cudaGetLastError();
     set_error("gfcc_mor_green: allocation failed");
-    return done(GFCC_ERR_OOM);
+    return GFCC_ERR_OOM;
   }
   if (cudaMemcpy2DAsync(Hm, sizeof(double) * m, M->H, sizeof(double) * M->cap, sizeof(double) * m, m,
                         cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
-    dfree(Hm);
     set_error("gfcc_mor_green: copy failed");
-    return done(GFCC_ERR_CUDA);
+    return GFCC_ERR_CUDA;
   }
   const double zsign = ip ? -1.0 : 1.0, hsign = ip ? 1.0 : -1.0;
   std::vector<double> hres(2 * wb * nb);
   // the model matrix in shared memory where it fits (multipliers + m x (m + nb))
   const size_t smem_lm = sizeof(double2) * (size_t)m, smem_all = smem_lm + sizeof(double2) * (size_t)m * (m + nb);
-  const bool in_smem = smem_all <= 220 * 1024;
+  const bool in_smem = smem_all <= MODEL_SMEM;
   const size_t smem = in_smem ? smem_all : smem_lm;
-  if (smem > 48 * 1024)
-    GFCC_CUDA(cudaFuncSetAttribute(mor_model_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // the limit belongs to the function, not to this call: every call sets the same
+  if (cudaFuncSetAttribute(mor_model_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MODEL_SMEM) !=
+      cudaSuccess) {
+    set_error("gfcc_mor_green: %s", cudaGetErrorString(cudaGetLastError()));
+    return GFCC_ERR_CUDA;
+  }
   EmuArena arena;   // digit planes of the residual products
   EmuArena *prev_arena = g_emu_arena;
   for (int w0 = 0; w0 < n_omega; w0 += (int)wb) {
@@ -629,8 +638,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
           GFCC_LAUNCH_CHECK();
           done_planes = true;
         } else if (s != GFCC_ERR_OOM) {
-          dfree(Hm);
-          return done(s);
+          return s;
         }
         s = GFCC_OK;   // no room for the planes: the FP64 units
       }
@@ -651,16 +659,14 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   if (planes) {
     const int e = umma_error_check(st);
     if (e < 0) {
-      dfree(Hm);
-      return done(e);
+      return e;
     }
   }
-  dfree(Hm);
   if (h_G) {
     GFCC_CUDA(cudaMemcpyAsync(h_G, Gd, sizeof(double) * 2 * n_omega * nb * nl, cudaMemcpyDeviceToHost, st));
   }
   GFCC_CUDA(cudaStreamSynchronize(st));
-  return done(GFCC_OK);
+  return GFCC_OK;
 }
 
 int mor_expand_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int n_orb, const int *h_orb, double tol,
