@@ -492,6 +492,12 @@ int project_new(gfcc_mor *M, int k0) {
 
 }  // namespace
 
+// Doubles before the model matrices in the workspace of a call (right-hand sides, left vectors and their projections); the
+// matrices are read and written as pairs, so an odd count of doubles before them is rounded up
+long long model_offset(long long n, long long m, long long nb, long long nl) {
+  return (3 * nb * n + nl * n + m * (nb + nl) + 1) & ~1LL;
+}
+
 constexpr int MODEL_SMEM = 220 * 1024;   // shared memory of a model solve at most
 
 // Model Green's function on a frequency grid (the sector of the object): rows / columns as gfcc_solve_block.
@@ -531,9 +537,8 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
     // frequencies per model launch: their dense model matrices, solutions and residuals within about 4 GB
     const long long per_w = 16LL * m * (m + nb) + per_pair * nb;
     wb = std::max<long long>(1, std::min<long long>({(long long)n_omega, 304LL, (4LL << 30) / per_w}));
-    need = sizeof(double) * (size_t)(2LL * nb * n + (long long)nb * n + (long long)nl * n + (long long)m * (nb + nl) +
-                                     2LL * wb * m * (m + nb) + 2LL * wb * m * nb + 2LL * n_omega * nb * nl + n_omega +
-                                     2LL * wb * nb + 64) +
+    need = sizeof(double) * (size_t)(model_offset(n, m, nb, nl) + 2LL * wb * m * (m + nb) + 2LL * wb * m * nb +
+                                     2LL * n_omega * nb * nl + n_omega + 2LL * wb * nb + 64) +
            (size_t)(per_pair * wb * nb);
   };
   layout();
@@ -555,7 +560,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   double *Cl = Br + (long long)nb * n;       // [nl][n]
   double *bh = Cl + (long long)nl * n;       // [m][nb]
   double *ch = bh + (long long)m * nb;       // [m][nl]
-  double2 *Aw = reinterpret_cast<double2 *>(ch + (long long)m * nl);
+  double2 *Aw = reinterpret_cast<double2 *>(buf + model_offset(n, m, nb, nl));
   double2 *Xw = Aw + wb * m * (m + nb);
   double *Gd = reinterpret_cast<double *>(Xw + wb * m * nb);
   double *om = Gd + 2LL * n_omega * nb * nl;
