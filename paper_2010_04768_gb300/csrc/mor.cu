@@ -140,8 +140,8 @@ __global__ void mor_real_kernel(const double *z, long long n, int rows, double *
     out[t] = z[2 * t];
 }
 
-// Model solves: one CTA per frequency w.  [A | X] = [z_w I + s Hhat | bh] (complex, m x (m + nb), row-major, in
-// shared memory when it fits, else in work [w][m][m + nb]); solution X [w][m][nb] complex; then
+// Model solves: one CTA per frequency w.  [A | X] = [z_w I + s Hhat | bh] (complex, m x (m + nb), row-major) behind the
+// multipliers of a step [m], in shared memory when both fit, else in work [w][m + m (m + nb)]; solution X [w][m][nb] complex; then
 // G[w][a][b] (IP: a over rhs, b over left; EA: a over left, b over rhs) = sum_k ch[k][left] X[k][rhs].
 // Gaussian elimination with partial pivoting by rows; threads split the trailing updates, the back
 // substitution runs by columns.  Bound by the FP64 pipe (m^3 / 3 complex FMAs) once the pivot search is a warp's and
@@ -155,8 +155,8 @@ __global__ __launch_bounds__(MT) void mor_model_solve_kernel(const double *Hh, i
   __shared__ int piv;
   __shared__ double2 inv_s;
   const int w = blockIdx.x, ld = m + nb, t0 = threadIdx.x, lane = t0 & 31, warp = t0 >> 5;
-  double2 *lm = sm;                                                       // multipliers of a step [m]
-  double2 *A = Aw != nullptr ? Aw + (long long)w * m * ld : sm + m;       // [m][ld]
+  double2 *lm = Aw != nullptr ? Aw + w * (m + (long long)m * ld) : sm;
+  double2 *A = lm + m;   // [m][ld]
   const double om = omegas[w];
   for (int t = t0; t < m * ld; t += MT) {
     const int i = t / ld, j = t - i * ld;
@@ -535,9 +535,9 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   auto layout = [&]() {
     per_pair = planes ? 16LL * n + 32LL * m : 0;   // A x and the coefficient rows
     // frequencies per model launch: their dense model matrices, solutions and residuals within about 4 GB
-    const long long per_w = 16LL * m * (m + nb) + per_pair * nb;
+    const long long per_w = 16LL * m * (m + nb + 1) + per_pair * nb;
     wb = std::max<long long>(1, std::min<long long>({(long long)n_omega, 304LL, (4LL << 30) / per_w}));
-    need = sizeof(double) * (size_t)(model_offset(n, m, nb, nl) + 2LL * wb * m * (m + nb) + 2LL * wb * m * nb +
+    need = sizeof(double) * (size_t)(model_offset(n, m, nb, nl) + 2LL * wb * m * (m + nb + 1) + 2LL * wb * m * nb +
                                      2LL * n_omega * nb * nl + n_omega + 2LL * wb * nb + 64) +
            (size_t)(per_pair * wb * nb);
   };
@@ -561,7 +561,7 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   double *bh = Cl + (long long)nl * n;       // [m][nb]
   double *ch = bh + (long long)m * nb;       // [m][nl]
   double2 *Aw = reinterpret_cast<double2 *>(buf + model_offset(n, m, nb, nl));
-  double2 *Xw = Aw + wb * m * (m + nb);
+  double2 *Xw = Aw + wb * m * (m + nb + 1);
   double *Gd = reinterpret_cast<double *>(Xw + wb * m * nb);
   double *om = Gd + 2LL * n_omega * nb * nl;
   double *res = om + n_omega;
@@ -608,9 +608,9 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   const double zsign = ip ? -1.0 : 1.0, hsign = ip ? 1.0 : -1.0;
   std::vector<double> hres(2 * wb * nb);
   // the model matrix in shared memory where it fits (multipliers + m x (m + nb))
-  const size_t smem_lm = sizeof(double2) * (size_t)m, smem_all = smem_lm + sizeof(double2) * (size_t)m * (m + nb);
+  const size_t smem_all = sizeof(double2) * (size_t)m * (m + nb + 1);
   const bool in_smem = smem_all <= MODEL_SMEM;
-  const size_t smem = in_smem ? smem_all : smem_lm;
+  const size_t smem = in_smem ? smem_all : 0;
   // the limit belongs to the function, not to this call: every call sets the same
   if (cudaFuncSetAttribute(mor_model_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MODEL_SMEM) !=
       cudaSuccess) {

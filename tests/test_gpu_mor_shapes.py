@@ -31,3 +31,16 @@ def test_rows_and_columns_of_different_count(o, v):
         assert np.abs(r - rr[:, rows]).max() <= 1e-12
     mor.close()
     g.close()
+
+
+def test_model_beyond_shared_memory():
+    # m of about 240: matrix and multipliers in the call's workspace; the model interpolates its samples
+    om, orbs, eta = np.linspace(-1.0, -0.2, 20), np.arange(6), 0.05
+    g = gfcc.GFCC(make_problem(6, 60, 60, seed=3), sectors="IP")
+    mor = gfcc.MOR(g, "IP")
+    ref, code = mor.expand(om, eta, orbs, 1e-11)
+    assert code == gfcc.OK and mor.dim() > 200
+    G = mor.green(om, eta, orbs)
+    assert np.abs(G - ref).max() <= 1e-8 * np.abs(ref).max()
+    mor.close()
+    g.close()
