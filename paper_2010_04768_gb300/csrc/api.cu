@@ -644,6 +644,7 @@ int solve_impl(gfcc_ctx *c, int n_omega, const double *d_om, double eta, const O
                double *d_G) {
   cudaStream_t st = c->stream;
   CallScope call;
+  ArenaScope arena(c);
   UmmaScope umma(c->umma_flag);
   // what a caller's stream still holds does not count towards the limits of the solver's host waits
   if (st != c->own_stream) GFCC_CUDA(cudaStreamSynchronize(st));
@@ -1625,6 +1626,7 @@ int gfcc_sigma_ex(gfcc_ctx *c, int sector, int precision, int n_vec, const doubl
   b.x = dx; b.ldx = n;
   b.y = dy; b.ldy = n;
   CallScope call;
+  ArenaScope arena(c);
   UmmaScope umma(c->umma_flag);
   if (mixed || emu || c->rhf) GFCC_TRY(umma_error_reset(c->stream));
   if (mixed || emu) {

@@ -93,7 +93,7 @@ struct gfcc_ctx {
   double *rU1 = nullptr;    // [i][m | (m,n,e)]: the 1h row (o x (o + o^2 v))
   // digit planes of the ring matrices, [-t | -W], oooo, Vz and the 1h row (those that fit)
   gfcc::EmuOperand rM1e, rM2e, rM3e, rWTe, rWqe, rVze, rU1e;
-  gfcc::EmuArena emu_arena;   // workspace of the emulated contractions of the operator
+  gfcc::EmuArena emu_arena;   // workspace of the emulated contractions of the operator, held during a call (ArenaScope)
 
   // mixed-precision IP operands: BF16, K-major, row strides padded to multiples of 8.  The exact
   // Fock-like diagonal d (diag_ip) is left out of them and applied in FP64 by the epilogue.
@@ -183,6 +183,14 @@ struct gfcc_ctx {
 };
 
 namespace gfcc {
+// Gives the closed-shell operator's workspace back at the end of a call: between calls the device memory is the caller's.
+struct ArenaScope {
+  gfcc_ctx *c;
+  explicit ArenaScope(gfcc_ctx *ctx) : c(ctx) {}
+  ~ArenaScope() {
+    if (!c->stuck) c->emu_arena.release();
+  }
+};
 // Times the enclosed region on the context's stream when profiling is on.
 struct PhaseTimer {
   gfcc_ctx *c;

@@ -681,6 +681,7 @@ int mor_expand_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, in
   const long long n = M->n;
   const long long ntasks = (long long)n_omega * n_orb;
   CallScope call;
+  ArenaScope arena(c);
   // solutions of the full systems (the hot path), then Gram-Schmidt of their real and imaginary parts
   double *sink = nullptr;
   if (dmalloc(reinterpret_cast<void **>(&sink), sizeof(double) * 2 * (size_t)ntasks * n) != cudaSuccess) {
