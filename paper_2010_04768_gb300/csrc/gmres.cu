@@ -430,6 +430,7 @@ __global__ __launch_bounds__(32) void backsolve_kernel(int m, const double *H, c
 // from L1 between the basis loads took 107 and 78 us.
 constexpr int CGS_THREADS = 256, CGS_MIN_CHUNK = 256, CGS_BATCH = 8;
 constexpr int DOT_WARPS = 4, DOT_RUN = 4096;   // FP32 sums of at most DOT_RUN / 32 terms, then FP64
+constexpr int NORM_RUN = 32;                   // of the update's norm (even: a thread takes two elements at a time)
 template <typename T>
 struct CgsShape {   // blocks per SM (by registers), elements a round of the dots
   static constexpr bool F32 = sizeof(T) == sizeof(float);
@@ -602,6 +603,7 @@ __global__ __launch_bounds__(CGS_THREADS, CgsShape<T>::UPD_PER_SM) void cgs_upda
   T *ws = w + 2 * s * vs;
   const T *Vs = V + 2 * s * vs;
   T nn = T(0);
+  double t = 0.0;   // ||w'||^2: FP32 sums of at most NORM_RUN elements, then FP64
   if (clen <= CGS_THREADS) {   // one element per thread
     const long long e = e0 + threadIdx.x;
     if (e < e1) {
@@ -630,7 +632,8 @@ __global__ __launch_bounds__(CGS_THREADS, CgsShape<T>::UPD_PER_SM) void cgs_upda
       nn = x.x * x.x + x.y * x.y;
     }
   } else
-  for (long long e = e0 + threadIdx.x; e < e1; e += 2 * CGS_THREADS) {
+  for (long long r0 = e0; r0 < e1; r0 += NORM_RUN * CGS_THREADS, t += (double)nn, nn = T(0))
+  for (long long e = r0 + threadIdx.x; e < min(r0 + NORM_RUN * CGS_THREADS, e1); e += 2 * CGS_THREADS) {
     const long long f = e + CGS_THREADS;
     const bool inf = f < e1;
     CT<T> acc0 = mkc<T>(0.0, 0.0), acc1 = mkc<T>(0.0, 0.0);
@@ -676,7 +679,7 @@ __global__ __launch_bounds__(CGS_THREADS, CgsShape<T>::UPD_PER_SM) void cgs_upda
       nn += x1.x * x1.x + x1.y * x1.y;
     }
   }
-  double t = (double)nn;
+  t += (double)nn;
   for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = t;
   __syncthreads();
