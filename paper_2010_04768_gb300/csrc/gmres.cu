@@ -326,21 +326,25 @@ __device__ void givens_update(const Lsq &q, int s, int k, const double *h, int N
 // FP64 per thread held this kernel to a quarter of the memory rate: 54 us for 100 MB); each thread scales
 // VSCALE_UNROLL elements with independent loads.
 constexpr int VSCALE_UNROLL = 8, VSCALE_PER_BLOCK = 256 * VSCALE_UNROLL;
-// GIVENS: one more block per system makes the Givens update of column idx - 1 meanwhile (a system that it takes
-// out of its cycle may or may not be scaled; the vector is not used again).
+// GIVENS: one more block per system makes the Givens update of column idx - 1 meanwhile, which may take the system out of
+// its cycle; the vector is not used again then.  So that a block scales all of its part or none of it, one thread reads the
+// state for the block.
 template <typename T, bool GIVENS>
 __global__ __launch_bounds__(256) void vscale_kernel(T *w, long long ws_stride, long long n, const double *nrm2, int NV,
                                                      int idx, const int *state, int want, Lsq q) {
   chain_start();
   __shared__ T factor;
+  __shared__ bool scale;
   const int s = blockIdx.y;
-  if (state != nullptr && state[s] != want) return;
   if (GIVENS && blockIdx.x == gridDim.x - 1) {
-    givens_update(q, s, idx - 1, nrm2, NV);
+    if (state[s] == want) givens_update(q, s, idx - 1, nrm2, NV);   // writes the state behind a barrier
     return;
   }
-  const double nn = nrm2[2 * ((long long)s * NV + idx)];
-  if (!(nn > 0.0)) return;
+  if (threadIdx.x == 0) {
+    const double nn = nrm2[2 * ((long long)s * NV + idx)];
+    scale = *const_cast<const volatile int *>(state + s) == want && nn > 0.0;
+    factor = (T)(1.0 / sqrt(nn));
+  }
   T *ws = w + 2 * s * ws_stride;
   const long long t0 = (long long)blockIdx.x * VSCALE_PER_BLOCK + threadIdx.x;
   CT<T> x[VSCALE_UNROLL];
@@ -349,8 +353,8 @@ __global__ __launch_bounds__(256) void vscale_kernel(T *w, long long ws_stride, 
     const long long t = t0 + (long long)u * 256;
     x[u] = t < n ? ldc(ws, t) : mkc<T>(0.0, 0.0);
   }
-  if (threadIdx.x == 0) factor = (T)(1.0 / sqrt(nn));
   __syncthreads();
+  if (!scale) return;
   const T inv = factor;
 #pragma unroll
   for (int u = 0; u < VSCALE_UNROLL; u++) {
