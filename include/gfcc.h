@@ -338,6 +338,13 @@ int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B,
 int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double *B, int S, int P, double *C);
 
 /*
+ * gfcc_selftest_gemm_planes - C[M][N] = sum_k A[m][k] B[n][k] + beta C by the digit planes (8 of 7 bits) that
+ * take the place of FP64 contractions.  mode 0: planes alone; 1: outputs whose sum of magnitudes is small
+ * beside the largest entries of their row and column are summed in FP64; 2: the same with A split beforehand.
+ */
+int gfcc_selftest_gemm_planes(int M, int N, int K, const double *A, const double *B, double beta, int mode, double *C);
+
+/*
  * gfcc_selftest_host_wait - the bounded host wait of the solvers on a stream that stays busy for busy_ns
  * (at most 5e9) nanoseconds: GFCC_ERR_TIMEOUT beyond 60 times GFCC_OPT_WAIT_NS (2 s at least), else GFCC_OK.
  * The stream is idle again on return.

@@ -1758,6 +1758,52 @@ int gfcc_selftest_gemm_f64emu(int M, int N, int K, const double *A, const double
   return s;
 }
 
+int gfcc_selftest_gemm_planes(int M, int N, int K, const double *A, const double *B, double beta, int mode, double *C) {
+  if (M <= 0 || N <= 0 || K <= 0 || mode < 0 || mode > 2 || A == nullptr || B == nullptr || C == nullptr) {
+    set_error("gfcc_selftest_gemm_planes: bad arguments");
+    return GFCC_ERR_ARG;
+  }
+  void *da = nullptr, *db = nullptr, *dc = nullptr, *sa = nullptr, *flag = nullptr;
+  cudaStream_t st = nullptr;
+  int s = GFCC_OK;
+  if (dmalloc(&da, sizeof(double) * M * K) != cudaSuccess || dmalloc(&db, sizeof(double) * N * K) != cudaSuccess ||
+      dmalloc(&dc, sizeof(double) * M * N) != cudaSuccess ||
+      dmalloc(&sa, emu_operand_bytes(M, K, F64_DIGITS + 1)) != cudaSuccess ||
+      dmalloc(&flag, sizeof(unsigned)) != cudaSuccess || cudaStreamCreate(&st) != cudaSuccess) {
+    cudaGetLastError();
+    set_error("gfcc_selftest_gemm_planes: allocation failed");
+    s = GFCC_ERR_OOM;
+  }
+  if (s == GFCC_OK && (cudaMemcpy(da, A, sizeof(double) * M * K, cudaMemcpyHostToDevice) != cudaSuccess ||
+                       cudaMemcpy(db, B, sizeof(double) * N * K, cudaMemcpyHostToDevice) != cudaSuccess ||
+                       cudaMemcpy(dc, C, sizeof(double) * M * N, cudaMemcpyHostToDevice) != cudaSuccess)) {
+    set_error("gfcc_selftest_gemm_planes: copy failed");
+    s = GFCC_ERR_CUDA;
+  }
+  CallScope call;
+  UmmaScope umma(static_cast<unsigned *>(flag));
+  if (s == GFCC_OK) s = umma_error_reset(st);
+  const double *a = static_cast<const double *>(da), *b = static_cast<const double *>(db);
+  double *c = static_cast<double *>(dc);
+  if (s == GFCC_OK && mode == 2) {
+    EmuOperand ea;
+    s = emu_slice_strided(st, a, M, K, imap1(K), imap1(1), 0, F64_DIGITS, F64_BITS, sa, ea, true);
+    if (s == GFCC_OK)
+      s = gemm_f64_emulated_pre(st, ea, a, imap1(K), imap1(1), N, b, imap1(1), imap1(K), 1.0, beta, c, imap1(N), imap1(1), true);
+  } else if (s == GFCC_OK) {
+    s = gemm_f64_emulated(st, M, N, K, 1.0, a, imap1(K), imap1(1), b, imap1(1), imap1(K), beta, c, imap1(N), imap1(1),
+                          mode == 1);
+  }
+  if (s == GFCC_OK) s = umma_error_check(st);
+  if (s == GFCC_OK && cudaMemcpy(C, dc, sizeof(double) * M * N, cudaMemcpyDeviceToHost) != cudaSuccess) {
+    set_error("gfcc_selftest_gemm_planes: copy back failed");
+    s = GFCC_ERR_CUDA;
+  }
+  for (void *p : {da, db, dc, sa, flag}) dfree(p);
+  if (st) cudaStreamDestroy(st);
+  return s;
+}
+
 int gfcc_selftest_gemm_bf16(int M, int N, int K, const float *A, const float *B, float *D) {
   if (M <= 0 || N <= 0 || K <= 0 || A == nullptr || B == nullptr || D == nullptr) {
     set_error("gfcc_selftest_gemm_bf16: bad arguments");

@@ -82,8 +82,7 @@ struct KWalk {
 // memory while this one is multiplied.  A cluster of gridDim.z / batch blocks (along z) may share
 // the K range of a tile; its partial sums meet through distributed shared memory in rank order.
 template <int TM, int RM, int RN>
-__global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kcluster) {
-  chain_start();
+__device__ __forceinline__ void contract_tile(const Contract &c, int kcluster, long long m0, long long n0) {
   constexpr int TN = NT / TM, BM = TM * RM, BN = TN * RN;
   constexpr int LA = (BM * BK + NT - 1) / NT, LB = (BN * BK + NT - 1) / NT;
   __shared__ double As[2][BK][BM + 1];
@@ -97,8 +96,6 @@ __global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kclust
   double *C = c.C + b * c.scb + (kcluster > 1 ? 0 : z * c.scz);
   const long long kbeg = z * c.kchunk;
   const long long kend = min(c.K, kbeg + c.kchunk);
-  const long long m0 = (long long)blockIdx.x * BM;
-  const long long n0 = (long long)blockIdx.y * BN;
 
   // this thread's elements of the A and B tiles: lanes run along K where K is the contiguous index
   // of the operand, else along M (N)
@@ -214,6 +211,28 @@ __global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kclust
     for (int j = 0; j < RN; j++) store(ty + TM * i, tx + TN * j, acc[i][j]);
 }
 
+template <int TM, int RM, int RN>
+__global__ __launch_bounds__(NT) void contract_f64_kernel(Contract c, int kcluster) {
+  chain_start();
+  contract_tile<TM, RM, RN>(c, kcluster, (long long)blockIdx.x * TM * RM, (long long)blockIdx.y * (NT / TM) * RN);
+}
+
+// One launch for both ends of a guarded digit-plane product: blocks of one wave store the listed values, or walk the
+// 32 x 32 tiles if the list has overflowed (a block for each of 40 000 tiles took 30 us to find that it has not).
+constexpr int LISTED_BLOCKS = NUM_SM * 4;
+__global__ __launch_bounds__(NT) void contract_listed_kernel(Contract c, GuardList list, long long mt, long long tiles) {
+  const unsigned count = *list.count;
+  if (count <= list.cap) {
+    for (unsigned i = blockIdx.x * NT + threadIdx.x; i < count; i += gridDim.x * NT)
+      c.C[map_offset(c.cm, list.at[i].x) + map_offset(c.cn, list.at[i].y)] = list.value[i];
+    return;
+  }
+  for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
+    contract_tile<16, 2, 2>(c, 1, t % mt * 32, t / mt * 32);
+    __syncthreads();
+  }
+}
+
 struct Tiling {
   int bm, bn, kcluster;
 };
@@ -313,6 +332,20 @@ int contract_f64(const Contract &c, cudaStream_t st) {
   return launch_contract<16, 1, 1>(cc, t.kcluster, mt, nt, st);
 }
 
+int contract_listed(const Contract &c, const GuardList &list, cudaStream_t st) {
+  Contract cc = c;
+  cc.nsplit = 1;
+  cc.kchunk = cc.K;
+  const long long mt = (c.M + 31) / 32, tiles = mt * ((c.N + 31) / 32);
+  const long long ka = imap_max(c.am, c.M) + imap_max(c.ak, c.K), kb = imap_max(c.bk, c.K) + imap_max(c.bn, c.N);
+  GFCC_TRY(check_extent(c.A, 0, ka, "contraction operand A"));
+  GFCC_TRY(check_extent(c.B, 0, kb, "contraction operand B"));
+  GFCC_TRY(check_extent(c.C, 0, imap_max(c.cm, c.M) + imap_max(c.cn, c.N), "contraction output C"));
+  contract_listed_kernel<<<(unsigned)std::min<long long>(tiles, LISTED_BLOCKS), NT, 0, st>>>(cc, list, mt, tiles);
+  GFCC_LAUNCH_CHECK();
+  return GFCC_OK;
+}
+
 namespace {
 // C = alpha * sum_z part[z] + beta * C
 __global__ void splitk_reduce_kernel(const double *part, int nsplit, long long M, long long N, double alpha, double beta,
@@ -352,14 +385,14 @@ int gemm_f64(cudaStream_t st, long long M, long long N, long long K, double alph
   c.batch = batch; c.sab = sab; c.sbb = sbb; c.scb = scb;
   c.alpha = alpha; c.beta = beta;
   // Contractions whose owner allows it (mixed-precision set-up, emulated CCSD, closed-shell operator) run on
-  // the tensor cores from digit planes that hold more bits than FP64 sums keep: all of at least emu_min
-  // flops, and the smaller ones where the planes are faster (unless the threshold was raised above its default).
-  // Without room for the planes the FP64 units do it.
+  // the tensor cores from digit planes: all of at least emu_min flops, and the smaller ones where the planes are faster
+  // (unless the threshold was raised above its default), these with the outputs that 56 bits below the largest entries
+  // do not serve summed in FP64.  Without room for the planes the FP64 units do it.
   const double emu_min = g_emulate_min_flops_local >= 0.0 ? g_emulate_min_flops_local : g_emulate_min_flops;
+  const bool large = 2.0 * (double)M * (double)N * (double)K >= emu_min;
   if (batch == 1 && K > 0 && g_emulate_big &&
-      (2.0 * (double)M * (double)N * (double)K >= emu_min ||
-       (g_emulate_min_flops <= EMULATE_MIN_FLOPS_DEFAULT && emulation_pays(M, N, K, false)))) {
-    const int s = gemm_f64_emulated(st, M, N, K, alpha, A, am, ak, B, bk, bn, beta, C, cm, cn);
+      (large || (g_emulate_min_flops <= EMULATE_MIN_FLOPS_DEFAULT && emulation_pays(M, N, K, false)))) {
+    const int s = gemm_f64_emulated(st, M, N, K, alpha, A, am, ak, B, bk, bn, beta, C, cm, cn, !large);
     if (s != GFCC_ERR_OOM) return s;
   }
   // A few 16 x 16 output tiles and a long K: the K ranges of a cluster (8 at most) would not fill the

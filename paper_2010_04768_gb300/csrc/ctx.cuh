@@ -91,8 +91,8 @@ struct gfcc_ctx {
   double *rWT = nullptr;    // [(i,j,a)][e | m]: -t_ij^ea | -W_maij  (o^2 v x (v + o))
   double *rVz = nullptr;    // [e][(m,n,f)]: 2 u_mnef - u_mnfe  (v x o^2 v)
   double *rU1 = nullptr;    // [i][m | (m,n,e)]: the 1h row (o x (o + o^2 v))
-  // digit planes of the ring matrices, [-t | -W], oooo, Vz and the 1h row (those that fit)
-  gfcc::EmuOperand rM1e, rM2e, rM3e, rWTe, rWqe, rVze, rU1e;
+  // digit planes of the ring matrices, -t, oooo, Vz and the 2h1p part of the 1h row (those that fit)
+  gfcc::EmuOperand rM1e, rM2e, rM3e, rTe, rWqe, rVze, rU1e;
   gfcc::EmuArena emu_arena;   // workspace of the emulated contractions of the operator, held during a call (ArenaScope)
 
   // mixed-precision IP operands: BF16, K-major, row strides padded to multiples of 8.  The exact

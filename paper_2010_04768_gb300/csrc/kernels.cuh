@@ -1,6 +1,7 @@
 // Declarations of the device-side building blocks of libgfcc.
 #pragma once
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace gfcc {
 
@@ -17,6 +18,8 @@ struct Contract {
   long long nsplit = 1, kchunk = 0, scz = 0;
 };
 int contract_f64(const Contract &c, cudaStream_t st);
+// The contraction (batch and nsplit 1) if the list has overflowed, else the list's values stored to C
+int contract_listed(const Contract &c, const GuardList &list, cudaStream_t st);
 // gemm_f64 sends contractions of at least g_emulate_min_flops to the FP64-accurate digit-plane
 // path when g_emulate_big is set (mixed-precision contexts set it during their setup)
 extern thread_local bool g_emulate_big;

@@ -282,14 +282,16 @@ __global__ void mor_coef_kernel(const double2 *Xw, int m, int nb, long long pair
 }
 
 // out[2 pr] = ||b_r - (A x)_pr||^2 from Ax [2 pr + re/im][n] and, of the first frequency's pairs (pr = r), out[2 r + 1] =
-// ||b_r||^2; one block per pair
+// ||b_r||^2; one block per pair.  Infinities and NaN of the pair's coefficient rows (nc numbers), which digit planes do
+// not hold, make it NaN.
 __global__ __launch_bounds__(MT) void mor_resnorm_kernel(const double *Ax, const double *B, long long n, int nb,
-                                                         double *out) {
+                                                         const double *coef, long long nc, double *out) {
   __shared__ double sh[2][MT / 32];
   const long long pr = blockIdx.x;
   const double *ar = Ax + 2 * pr * n, *ai = ar + n, *b = B + (pr % nb) * n;
   const bool first = pr < nb;
   double rr = 0.0, bb = 0.0;
+  for (long long k = threadIdx.x; k < nc; k += MT) rr += 0.0 * coef[pr * nc + k];
 #pragma unroll 4
   for (long long e = threadIdx.x; e < n; e += MT) {
     const double x = b[e], d = x - ar[e], i = ai[e];
@@ -525,9 +527,11 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
   double *buf = nullptr;
   // The residuals of mixed-precision contexts are products [S | W] x on digit planes (the FP64 units take
   // 8 n m operations per frequency and right-hand side: 26 ms for 500 x 12 at n = 9616, m = 72, against 2.4 ms); other
-  // contexts and models too small to gain keep the FP64 kernel.  Short sums are as accurate as that kernel here: the
-  // residuals of models of 36 vectors over 9616 and 6280 elements were within 6e-14 (rms, of ||b||) of quad sums
-  // either way.
+  // contexts and models too small to gain keep the FP64 kernel.  What is returned is the norm of A x - b, and whatever the
+  // spread of the entries the planes' error of A x is within the norm of FP64's: an element's is below
+  // 2^-54 2m max|x| max_k|S_k|, and FP64's bound 2m 2^-53 |x| |S| of the same element is no smaller in the norms of x and
+  // of the elements.  The residuals of models of 36 vectors over 9616 and 6280 elements were within 6e-14 (rms, of ||b||)
+  // of quad sums either way.
   const bool mixed = h_relres != nullptr && c->precision == GFCC_PREC_MIXED_BF16;
   bool planes = mixed && emulation_pays(2LL * std::min(n_omega, 304) * nb, n, 2LL * m, false);
   long long per_pair, wb;
@@ -636,10 +640,10 @@ int mor_green_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, int
         if (w0 == 0) s = umma_error_reset(st);
         if (s == GFCC_OK)
           s = gemm_f64_emulated(st, 2 * pairs, n, 2LL * m, 1.0, Cx, imap1(2LL * m), imap1(1), M->S,
-                                imap2(m, n, (long long)M->cap * n), imap1(1), 0.0, Ax, imap1(n), imap1(1));
+                                imap2(m, n, (long long)M->cap * n), imap1(1), 0.0, Ax, imap1(n), imap1(1), false);
         g_emu_arena = prev_arena;
         if (s == GFCC_OK) {
-          mor_resnorm_kernel<<<(unsigned)pairs, MT, 0, st>>>(Ax, Br, n, nb, res);
+          mor_resnorm_kernel<<<(unsigned)pairs, MT, 0, st>>>(Ax, Br, n, nb, Cx, 4LL * m, res);
           GFCC_LAUNCH_CHECK();
           done_planes = true;
         } else if (s != GFCC_ERR_OOM) {

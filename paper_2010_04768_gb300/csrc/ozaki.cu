@@ -122,7 +122,7 @@ int emu_max_exponent(cudaStream_t st, const EmuOperand &e, int *out) {
 }
 
 int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, double alpha, double beta, double *C,
-             IMap cm, IMap cn, void *work, long long n0, long long m0) {
+             IMap cm, IMap cn, void *work, long long n0, long long m0, const GuardList *gate) {
   P = std::max(2, P - A.drop);
   const long long M = A.rows, N = B.rows, K = A.K;
   if (M <= 0 || N <= 0) return GFCC_OK;
@@ -132,8 +132,8 @@ int emu_gemm(cudaStream_t st, const EmuOperand &A, const EmuOperand &B, int P, d
   }
   if ((N <= g_fused_max_n || A.bits != 6) && emu_fused_takes(A.S, B.S, P) && M <= (1LL << 31) - 256 && N <= (1LL << 31) - 256)
     return emu_gemm_fused(st, A.dig, A.rows * A.ld, A.S, A.exp2, B.dig, B.rows * B.ld, B.S, B.exp2, A.ld, (int)M,
-                          (int)N, (int)K, P, A.bits, alpha, beta, C, cm, cn, n0, static_cast<double *>(work), m0);
-  if (A.bits != 6 || m0 != 0) {
+                          (int)N, (int)K, P, A.bits, alpha, beta, C, cm, cn, n0, static_cast<double *>(work), m0, gate);
+  if (A.bits != 6 || m0 != 0 || gate != nullptr) {
     set_error("emu_gemm: %d-bit digits to level %d are beyond the digit-pair products", A.bits, P);
     return GFCC_ERR_ARG;
   }
@@ -266,11 +266,22 @@ __global__ void strided_exp_final_kernel(int *be, long long rows, int less) {
   if (r < rows) be[r] = be[r] > 0 ? be[r] - less : 0;
 }
 
-// dig[i][r][k] = i-th digit of X[rm(r0 + r) + km(k)] 2^-e[r] (k < K), 0 for K <= k < ld
+// |x| 2^-e in BF16, rounded down (infinities and NaN kept); what is not zero counts as 2^-60 at least, so that a sum of
+// products of magnitudes is zero only where every product is
+__device__ __forceinline__ unsigned magnitude_bf16(double x, int e) {
+  const int hi = __double2hiint(x) & 0x7fffffff, E = hi >> 20;
+  if (hi == 0 && __double2loint(x) == 0) return 0u;
+  if (E == 0x7ff) return (hi & 0xfffff) != 0 || __double2loint(x) != 0 ? 0x7fc0u : 0x7f80u;
+  const int f = E - 1023 - e + 127;
+  return E == 0 || f < 127 - 60 ? (unsigned)(127 - 60) << 7 : (unsigned)f << 7 | ((hi >> 13) & 0x7f);
+}
+
+// dig[i][r][k] = i-th digit of X[rm(r0 + r) + km(k)] 2^-e[r] (k < K), 0 for K <= k < ld; mag: plane S of dig holds the
+// magnitudes
 __global__ __launch_bounds__(SL_THREADS) void strided_slice_kernel(const double *X, long long rows, long long K, IMap rm,
                                                                    IMap km, long long r0, bool k_lanes, const int *e,
                                                                    int S, int bits, unsigned gx, __nv_bfloat16 *dig,
-                                                                   long long ld) {
+                                                                   long long ld, bool mag) {
   __shared__ double tile[SL_ROWS][SL_K + 1];
   __shared__ long long ro[SL_ROWS], ko[SL_K];
   __shared__ int ex[SL_ROWS];
@@ -319,13 +330,14 @@ __global__ __launch_bounds__(SL_THREADS) void strided_slice_kernel(const double 
       const unsigned f1 = __float_as_uint(__uint_as_float(0x4b000000u | ((unsigned)(Y1 >> sh) & mi)) - off);
       *dst = __byte_perm(f0, f1, 0x7632);
     }
+    if (mag) *dst = magnitude_bf16(tile[r][k], ex[r]) | magnitude_bf16(tile[r][k + 1], ex[r]) << 16;
   }
 }
 
 }  // namespace
 
 int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long long K, IMap rm, IMap km, long long r0,
-                      int S, int bits, void *mem, EmuOperand &out) {
+                      int S, int bits, void *mem, EmuOperand &out, bool mag) {
   out.rows = rows;
   out.K = K;
   out.ld = emu_ld(K);
@@ -333,11 +345,16 @@ int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long lon
   out.bits = bits;
   unsigned char *p = static_cast<unsigned char *>(mem);
   out.dig = reinterpret_cast<__nv_bfloat16 *>(p);
-  p += ((long long)S * rows * out.ld * 2 + 255) / 256 * 256;
+  out.mag = mag ? out.dig + S * rows * out.ld : nullptr;
+  p += ((long long)(S + (mag ? 1 : 0)) * rows * out.ld * 2 + 255) / 256 * 256;
   out.exp2 = reinterpret_cast<int *>(p);
   if (rows <= 0 || K <= 0) return GFCC_OK;
+  if (mag && bits != F64_BITS) {
+    set_error("emu_slice_strided: magnitudes go with %d-bit digits", F64_BITS);
+    return GFCC_ERR_ARG;
+  }
   GFCC_TRY(check_extent(X, 0, imap_max(rm, r0 + rows) + imap_max(km, K), "digit split input"));
-  GFCC_TRY(check_extent_bytes(mem, emu_operand_bytes(rows, K, S), "digit split output"));
+  GFCC_TRY(check_extent_bytes(mem, emu_operand_bytes(rows, K, S + (mag ? 1 : 0)), "digit split output"));
   const bool k_lanes = km.s0 == 1 || rm.s0 != 1;
   const long long gx = (rows + SL_ROWS - 1) / SL_ROWS, gy = (out.ld + SL_K - 1) / SL_K;
   // K values per block of the exponent pass: enough blocks for the chip, one tile at least
@@ -355,7 +372,7 @@ int emu_slice_strided(cudaStream_t st, const double *X, long long rows, long lon
   strided_exp_final_kernel<<<cdiv(rows, 256), 256, 0, st>>>(out.exp2, rows, bits == F64_BITS && K <= F64_SHORT_K ? 1022 : 1021);
   GFCC_LAUNCH_CHECK();
   strided_slice_kernel<<<(unsigned)(gx * gy), SL_THREADS, 0, st>>>(X, rows, K, rm, km, r0, k_lanes, out.exp2, S, bits,
-                                                                   (unsigned)gx, out.dig, out.ld);
+                                                                   (unsigned)gx, out.dig, out.ld, mag);
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -385,23 +402,91 @@ void EmuArena::release() {
 namespace {
 constexpr long long EMU_BLOCK_BYTES = 4LL << 30;
 
-// rows (or columns) of a block whose digit planes stay within EMU_BLOCK_BYTES
+// rows (or columns) of a block whose planes (magnitudes among them) stay within EMU_BLOCK_BYTES
 long long block_rows(long long rows, long long K) {
-  const long long per = emu_ld(K) * 2 * F64_DIGITS + 8;
+  const long long per = emu_ld(K) * 2 * (F64_DIGITS + 1) + 8;
   return std::min(rows, std::max<long long>(256, EMU_BLOCK_BYTES / per / 128 * 128));
 }
 
 long long up256(long long x) { return (x + 255) / 256 * 256; }
+
+// The error of a digit-plane output in units of its row and column scales is, with remainders of both signs, about
+// sqrt(K) 2^-58 (seven digit pairs of level 10 and above dropped from each product, each below 2^-58; both entries
+// rounded to 2^-57), and the FP64 sum's bound K 2^-53 times the sum of magnitudes: 2^-5 / sqrt(K) is where one standard
+// deviation meets it, GUARD_THETA / sqrt(K) asks for six.
+constexpr float GUARD_THETA = 0.2f;
+float guard_theta(long long K) { return GUARD_THETA / std::sqrt((float)K); }
+// Listed outputs are summed at about 0.4 of the rate of the contraction: beyond an eighth of them it takes over
+unsigned guard_cap(long long M, long long N) {
+  return (unsigned)std::min<long long>(1LL << 26, std::max<long long>(1024, M * N / 8));
+}
+long long guard_bytes(unsigned cap) { return 256 + up256(8LL * cap) + 8LL * cap; }
+GuardList guard_list(void *mem, unsigned cap) {
+  GuardList g;
+  unsigned char *p = static_cast<unsigned char *>(mem);
+  g.count = reinterpret_cast<unsigned *>(p);
+  g.at = reinterpret_cast<int2 *>(p + 256);
+  g.value = reinterpret_cast<double *>(p + 256 + up256(8LL * cap));
+  g.cap = cap;
+  return g;
+}
+
+// value[i] = alpha sum_k A(m, k) B(k, n) + beta C(m, n) of the listed outputs, WARPS warps each
+template <int WARPS>
+__global__ __launch_bounds__(256) void guard_values_kernel(Contract c, GuardList g) {
+  constexpr int PER = 8 / WARPS;   // outputs a block
+  __shared__ double part[8];
+  const unsigned count = *g.count;
+  if (count > g.cap) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, first = threadIdx.x % (32 * WARPS);
+  for (unsigned i0 = blockIdx.x * PER; i0 < count; i0 += gridDim.x * PER) {
+    const unsigned i = i0 + warp / WARPS;
+    double s = 0.0;
+    int2 at = make_int2(0, 0);
+    if (i < count) {
+      at = g.at[i];
+      const double *a = c.A + imap_apply(c.am, at.x), *b = c.B + imap_apply(c.bn, at.y);
+#pragma unroll 4
+      for (long long k = first; k < c.K; k += 32 * WARPS) s = fma(a[imap_apply(c.ak, k)], b[imap_apply(c.bk, k)], s);
+    }
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (WARPS > 1) {
+      if (lane == 0) part[warp] = s;
+      __syncthreads();
+      s = 0.0;
+      for (int w = 0; w < WARPS; w++) s += part[warp / WARPS * WARPS + w];
+      __syncthreads();
+    }
+    if (first == 0 && i < count) {
+      s *= c.alpha;
+      if (c.beta != 0.0) s += c.beta * c.C[imap_apply(c.cm, at.x) + imap_apply(c.cn, at.y)];
+      g.value[i] = s;
+    }
+  }
+}
+// A guarded product in the order its kernels need: the list of all blocks, the listed values (from C as it was), the
+// planes' product or the FP64 contraction, the listed values stored.
+template <typename List, typename Product>
+int guarded_product(cudaStream_t st, const Contract &p, const GuardList &g, List list, Product product) {
+  GFCC_CUDA(cudaMemsetAsync(g.count, 0, sizeof(unsigned), st));
+  GFCC_TRY(list());
+  if (p.K >= 4096)
+    guard_values_kernel<8><<<152 * 8, 256, 0, st>>>(p, g);
+  else
+    guard_values_kernel<1><<<152 * 8, 256, 0, st>>>(p, g);
+  GFCC_LAUNCH_CHECK();
+  GFCC_TRY(product());
+  return contract_listed(p, g, st);
+}
 }  // namespace
 
-// FP64 units: 1.1 TFLOP/s on 16 x 16 tiles.  Digit planes: 36 pairs of BF16 products at about 1.1e15
+// FP64 units: 1.1 TFLOP/s on 16 x 16 tiles.  Digit planes: 36 pairs of BF16 products and one of magnitudes at about 1.1e15
 // flop/s on padded tiles, 4 ps an output for the ends of the tiles, the split of both operands (two reads of 8 bytes,
-// eight planes of 2 bytes, at about 3 TB/s), and some 8 launches.  Error against quad sums (1e-16 relative): Gaussian
+// nine planes of 2 bytes, at about 3 TB/s), and some 12 launches.  Error against quad sums (1e-16 relative): Gaussian
 // entries, FP64 units 1.9, 2.1, 2.4, 3.0, 5.7, 14 at K = 32, 64, 160, 300, 1280, 6400; planes 0.6, 0.7, 0.7, 0.7, 2.4,
 // 4.0; entries that decay along K as the Cholesky vectors do, 2.5, 2.6, 3.3, 3.9, 6.6, 7.0 and 0.7, 0.8, 1.1, 1.1, 3.5,
-// 3.5.
-// What it gives: set-up of a mixed IP context at o=40 v=200 L=800 3489 -> 143 ms, IP + EA set-up and solve at
-// o=20 v=100 365 -> 40 ms, CCSD and Lambda at o=16 v=80 404 -> 99 ms, closed-shell solve at o=30 v=150 96 -> 43 ms.
+// 3.5.  What the guard costs: CCSD and Lambda at o=16 v=80 103 -> 114 ms, closed-shell solve at o=30 v=150 63 -> 69 ms,
+// IP + EA set-up and solve at o=20 v=100 39 -> 41 ms.
 bool emulation_pays(long long M, long long N, long long K, bool a_ready) {
   if (K < 32) return false;
   const double m16 = (double)((M + 15) / 16 * 16), n16 = (double)((N + 15) / 16 * 16);
@@ -409,58 +494,121 @@ bool emulation_pays(long long M, long long N, long long K, bool a_ready) {
   const double m128 = (double)((M + 127) / 128 * 128), n32 = (double)((N + 31) / 32 * 32);
   const double n128 = (double)((N + 127) / 128 * 128), m32 = (double)((M + 31) / 32 * 32);
   const double tile = std::min(m128 * n32, n128 * m32);
-  const double emu = 36.0 * 2.0 * tile * (double)((K + 63) / 64 * 64) / 1.1e15 + 4e-12 * tile + 32.0 * ((a_ready ? 0.0 : (double)M) + (double)N) * (double)K / 3e12 + (a_ready ? 3e-5 : 4e-5);
+  const double emu = 37.0 * 2.0 * tile * (double)((K + 63) / 64 * 64) / 1.1e15 + 4e-12 * tile +
+                     34.0 * ((a_ready ? 0.0 : (double)M) + (double)N) * (double)K / 3e12 + (a_ready ? 4e-5 : 5e-5);
   return emu < f64;
 }
 
-int gemm_f64_emulated_pre(cudaStream_t st, const EmuOperand &A, long long N, const double *B, IMap bk, IMap bn,
-                          double alpha, double beta, double *C, IMap cm, IMap cn) {
-  const long long M = A.rows, K = A.K;
+int gemm_f64_emulated_pre(cudaStream_t st, const EmuOperand &Ae, const double *A, IMap am, IMap ak, long long N,
+                          const double *B, IMap bk, IMap bn, double alpha, double beta, double *C, IMap cm, IMap cn,
+                          bool guarded) {
+  const long long M = Ae.rows, K = Ae.K;
   if (M <= 0 || N <= 0) return GFCC_OK;
   GFCC_TRY(check_extent(B, 0, imap_max(bk, K) + imap_max(bn, N), "emulated contraction operand B"));
   GFCC_TRY(check_extent(C, 0, imap_max(cm, M) + imap_max(cn, N), "emulated contraction output C"));
+  if (guarded && Ae.mag == nullptr) {
+    set_error("emulated contraction: the sliced operand has no magnitudes");
+    return GFCC_ERR_ARG;
+  }
   const long long nb = block_rows(N, K);
-  const long long bbytes = up256(emu_operand_bytes(nb, K, F64_DIGITS)), wbytes = emu_fused_work_bytes(M, nb, K);
+  const unsigned cap = guarded ? guard_cap(M, N) : 0;
+  const long long bbytes = up256(emu_operand_bytes(nb, K, F64_DIGITS + 1)), gbytes = guarded ? up256(guard_bytes(cap)) : 0;
+  const long long wbytes = std::max(emu_fused_work_bytes(M, nb, K), guarded ? emu_guard_work_bytes(M, nb, K) : 0);
   EmuArena local;
   EmuArena *ar = g_emu_arena ? g_emu_arena : &local;
   void *mem = nullptr;
-  if (ar->get((size_t)(bbytes + wbytes), &mem) < 0) {
+  if (ar->get((size_t)(bbytes + gbytes + wbytes), &mem) < 0) {
     set_error("emulated contraction: cannot allocate its temporaries (M=%lld N-block=%lld K=%lld)", M, nb, K);
     return GFCC_ERR_OOM;
   }
-  void *gw = static_cast<unsigned char *>(mem) + bbytes;
+  void *gm = static_cast<unsigned char *>(mem) + bbytes, *gw = static_cast<unsigned char *>(gm) + gbytes;
   EmuOperand eb;
-  for (long long n0 = 0; n0 < N; n0 += nb) {
-    GFCC_TRY(emu_slice_strided(st, B, std::min(nb, N - n0), K, bn, bk, n0, F64_DIGITS, F64_BITS, mem, eb));
-    GFCC_TRY(emu_gemm(st, A, eb, F64_LEVEL, alpha, beta, C, cm, cn, gw, n0));
-  }
-  return GFCC_OK;
+  long long sliced = -1;   // the first column of the block that eb holds
+  auto slice = [&](long long n0) -> int {
+    if (sliced == n0) return GFCC_OK;
+    sliced = n0;
+    return emu_slice_strided(st, B, std::min(nb, N - n0), K, bn, bk, n0, F64_DIGITS, F64_BITS, mem, eb, guarded);
+  };
+  const GuardList g = guarded ? guard_list(gm, cap) : GuardList();
+  auto list = [&]() -> int {
+    for (long long n0 = 0; n0 < N; n0 += nb) {
+      GFCC_TRY(slice(n0));
+      GFCC_TRY(emu_guard(st, Ae.mag, eb.mag, Ae.ld, (int)M, (int)eb.rows, (int)K, guard_theta(K), g, 0, n0,
+                         static_cast<float *>(gw)));
+    }
+    return GFCC_OK;
+  };
+  auto product = [&]() -> int {
+    for (long long n0 = 0; n0 < N; n0 += nb) {
+      GFCC_TRY(slice(n0));
+      GFCC_TRY(emu_gemm(st, Ae, eb, F64_LEVEL, alpha, beta, C, cm, cn, gw, n0, 0, guarded ? &g : nullptr));
+    }
+    return GFCC_OK;
+  };
+  if (!guarded) return product();
+  Contract c;
+  c.A = A; c.B = B; c.C = C;
+  c.M = M; c.N = N; c.K = K;
+  c.am = am; c.ak = ak; c.bk = bk; c.bn = bn; c.cm = cm; c.cn = cn;
+  c.alpha = alpha; c.beta = beta;
+  return guarded_product(st, c, g, list, product);
 }
 
 int gemm_f64_emulated(cudaStream_t st, long long M, long long N, long long K, double alpha, const double *A, IMap am,
-                      IMap ak, const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn) {
+                      IMap ak, const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn,
+                      bool guarded) {
   if (M <= 0 || N <= 0) return GFCC_OK;
   GFCC_TRY(check_extent(A, 0, imap_max(am, M) + imap_max(ak, K), "emulated contraction operand A"));
   GFCC_TRY(check_extent(B, 0, imap_max(bk, K) + imap_max(bn, N), "emulated contraction operand B"));
   GFCC_TRY(check_extent(C, 0, imap_max(cm, M) + imap_max(cn, N), "emulated contraction output C"));
   const long long mb = block_rows(M, K), nb = block_rows(N, K);
-  const long long abytes = up256(emu_operand_bytes(mb, K, F64_DIGITS)), bbytes = up256(emu_operand_bytes(nb, K, F64_DIGITS));
+  const int planes = F64_DIGITS + (guarded ? 1 : 0);
+  const unsigned cap = guarded ? guard_cap(M, N) : 0;
+  const long long abytes = up256(emu_operand_bytes(mb, K, planes)), bbytes = up256(emu_operand_bytes(nb, K, planes));
+  const long long gbytes = guarded ? up256(guard_bytes(cap)) : 0;
+  const long long wbytes = std::max(emu_fused_work_bytes(mb, nb, K), guarded ? emu_guard_work_bytes(mb, nb, K) : 0);
   EmuArena local;
   EmuArena *ar = g_emu_arena ? g_emu_arena : &local;
   void *mem = nullptr;
-  GFCC_TRY(ar->get((size_t)(abytes + bbytes + emu_fused_work_bytes(mb, nb, K)), &mem));
-  void *bm = static_cast<unsigned char *>(mem) + abytes, *gw = static_cast<unsigned char *>(bm) + bbytes;
+  GFCC_TRY(ar->get((size_t)(abytes + bbytes + gbytes + wbytes), &mem));
+  unsigned char *bm = static_cast<unsigned char *>(mem) + abytes, *gm = bm + bbytes;
+  void *gw = gm + gbytes;
   EmuOperand ea, eb;
-  for (long long m0 = 0; m0 < M; m0 += mb) {
-    const long long rows = std::min(mb, M - m0);
-    GFCC_TRY(emu_slice_strided(st, A, rows, K, am, ak, m0, F64_DIGITS, F64_BITS, mem, ea));
-    for (long long n0 = 0; n0 < N; n0 += nb) {
-      const long long cols = std::min(nb, N - n0);
-      if (m0 == 0 || nb < N) GFCC_TRY(emu_slice_strided(st, B, cols, K, bn, bk, n0, F64_DIGITS, F64_BITS, bm, eb));
-      GFCC_TRY(emu_gemm(st, ea, eb, F64_LEVEL, alpha, beta, C, cm, cn, gw, n0, m0));
-    }
-  }
-  return GFCC_OK;
+  long long am0 = -1, bn0 = -1;   // first row and column of the blocks that ea and eb hold
+  auto slice = [&](long long m0, long long n0) -> int {
+    if (am0 != m0)
+      GFCC_TRY(emu_slice_strided(st, A, std::min(mb, M - m0), K, am, ak, m0, F64_DIGITS, F64_BITS, mem, ea, guarded));
+    am0 = m0;
+    if (bn0 != n0)
+      GFCC_TRY(emu_slice_strided(st, B, std::min(nb, N - n0), K, bn, bk, n0, F64_DIGITS, F64_BITS, bm, eb, guarded));
+    bn0 = n0;
+    return GFCC_OK;
+  };
+  const GuardList g = guarded ? guard_list(gm, cap) : GuardList();
+  auto list = [&]() -> int {
+    for (long long m0 = 0; m0 < M; m0 += mb)
+      for (long long n0 = 0; n0 < N; n0 += nb) {
+        GFCC_TRY(slice(m0, n0));
+        GFCC_TRY(emu_guard(st, ea.mag, eb.mag, ea.ld, (int)ea.rows, (int)eb.rows, (int)K, guard_theta(K), g, m0, n0,
+                           static_cast<float *>(gw)));
+      }
+    return GFCC_OK;
+  };
+  auto product = [&]() -> int {
+    for (long long m0 = 0; m0 < M; m0 += mb)
+      for (long long n0 = 0; n0 < N; n0 += nb) {
+        GFCC_TRY(slice(m0, n0));
+        GFCC_TRY(emu_gemm(st, ea, eb, F64_LEVEL, alpha, beta, C, cm, cn, gw, n0, m0, guarded ? &g : nullptr));
+      }
+    return GFCC_OK;
+  };
+  if (!guarded) return product();
+  Contract c;
+  c.A = A; c.B = B; c.C = C;
+  c.M = M; c.N = N; c.K = K;
+  c.am = am; c.ak = ak; c.bk = bk; c.bn = bn; c.cm = cm; c.cn = cn;
+  c.alpha = alpha; c.beta = beta;
+  return guarded_product(st, c, g, list, product);
 }
 
 }  // namespace gfcc

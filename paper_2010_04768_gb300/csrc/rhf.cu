@@ -30,8 +30,9 @@
 namespace gfcc {
 
 // With the context's emulation option on, the operator's contractions run from digit planes (F64_DIGITS of
-// F64_BITS, more bits than FP64 sums keep): those of at least this many flops, and the smaller ones where the
-// planes are faster.  The planes of the constant operands are cut once at setup.
+// F64_BITS): those of at least this many flops, and the smaller ones where the planes are faster, these with the outputs
+// that 56 bits below the largest entries do not serve summed in FP64.  The planes of the constant operands are cut once
+// at setup.
 constexpr double RHF_EMULATE_MIN_FLOPS = 1e9;
 
 namespace {
@@ -392,20 +393,20 @@ int build_hbar_rhf(gfcc_ctx *c, const double *d_fock, const double *d_chol) {
     }
     double left = 0.25 * (double)fr;
     auto planes = [&](const double *X, long long rows, long long K, IMap rm, IMap km, EmuOperand &e) -> int {
-      const long long bytes = emu_operand_bytes(rows, K, F64_DIGITS);
+      const long long bytes = emu_operand_bytes(rows, K, F64_DIGITS + 1);
       if ((double)bytes > left) return GFCC_OK;
       left -= (double)bytes;
       double *mem;
       GFCC_TRY(dev_alloc(c, &mem, bytes / 8 + 1));
-      return emu_slice_strided(st, X, rows, K, rm, km, 0, F64_DIGITS, F64_BITS, mem, e);
+      return emu_slice_strided(st, X, rows, K, rm, km, 0, F64_DIGITS, F64_BITS, mem, e, true);
     };
     GFCC_TRY(planes(c->rM1, ov, ov, imap1(ov), imap1(1), c->rM1e));
     GFCC_TRY(planes(c->rM2, ov, ov, imap1(ov), imap1(1), c->rM2e));
     GFCC_TRY(planes(c->rM3, ov, ov, imap1(ov), imap1(1), c->rM3e));
     GFCC_TRY(planes(c->Woooo, oo, oo, imap1(1), imap1(oo), c->rWqe));
-    GFCC_TRY(planes(c->rWT, o2v, v + o, imap1(v + o), imap1(1), c->rWTe));
+    GFCC_TRY(planes(c->rWT, o2v, v, imap1(v + o), imap1(1), c->rTe));
     GFCC_TRY(planes(c->rVz, v, o2v, imap1(o2v), imap1(1), c->rVze));
-    GFCC_TRY(planes(c->rU1, o, o + o2v, imap1(o + o2v), imap1(1), c->rU1e));
+    GFCC_TRY(planes(c->rU1 + o, o, o2v, imap1(o + o2v), imap1(1), c->rU1e));
   }
   GFCC_TRY(dev_alloc(c, &c->diag_ip, c->dim_ip));
   rhf_diag_kernel<<<grid1d(c->dim_ip), 256, 0, st>>>(c->Foo, c->Fvv, o, v, c->diag_ip);
@@ -448,9 +449,9 @@ int apply_ip_rhf(gfcc_ctx *c, const SysBatch &b, double *work) {
   // C (+)= X B with X's digit planes where the operator runs on them, else through gemm_f64
   auto product = [&](const double *X, IMap xm, IMap xk, const EmuOperand &Xe, long long M, long long N, long long K,
                      const double *B, IMap bk, IMap bn, double beta, double *C, IMap cm, IMap cn) -> int {
-    if (c->rhf_emulate && Xe.dig != nullptr &&
-        (2.0 * (double)M * (double)N * (double)K >= RHF_EMULATE_MIN_FLOPS || emulation_pays(M, N, K, true))) {
-      const int s = gemm_f64_emulated_pre(st, Xe, N, B, bk, bn, 1.0, beta, C, cm, cn);
+    const bool large = 2.0 * (double)M * (double)N * (double)K >= RHF_EMULATE_MIN_FLOPS;
+    if (c->rhf_emulate && Xe.dig != nullptr && (large || emulation_pays(M, N, K, true))) {
+      const int s = gemm_f64_emulated_pre(st, Xe, X, xm, xk, N, B, bk, bn, 1.0, beta, C, cm, cn, !large);
       if (s != GFCC_ERR_OOM) return s;
     }
     return gemm_f64(st, M, N, K, 1.0, X, xm, xk, B, bk, bn, beta, C, cm, cn);
@@ -458,8 +459,12 @@ int apply_ip_rhf(gfcc_ctx *c, const SysBatch &b, double *work) {
   // z[e][c] = Vz[e][(m,n,f)] r2u[(m,n,f)][c];  S2 = [-t | -W_maij] [z; r1u]
   GFCC_TRY(product(c->rVz, imap1(o2v), imap1(1), c->rVze, v, C2, o2v, r2u, imap1(C2), imap1(1), 0.0, P, imap1(C2),
                    imap1(1)));
-  GFCC_TRY(product(c->rWT, imap1(v + o), imap1(1), c->rWTe, o2v, C2, v + o, P, imap1(C2), imap1(1), 0.0, S2, imap1(C2),
+  // (as two products: t and W, z and r1 each have a magnitude of their own, and the outputs that planes scaled to the
+  // larger ones did not serve made the product of both 1.3 ms for 10 vectors of o=30 v=150)
+  GFCC_TRY(product(c->rWT, imap1(v + o), imap1(1), c->rTe, o2v, C2, v, P, imap1(C2), imap1(1), 0.0, S2, imap1(C2),
                    imap1(1)));
+  GFCC_TRY(gemm_f64(st, o2v, C2, o, 1.0, c->rWT + v, imap1(v + o), imap1(1), r1u, imap1(C2), imap1(1), 1.0, S2, imap1(C2),
+                    imap1(1)));
   // + W_mnij r_mn^a
   GFCC_TRY(product(c->Woooo, imap1(1), imap1(oo), c->rWqe, oo, v * C2, oo, r2u, imap1(v * C2), imap1(1), 1.0, S2,
                    imap1(v * C2), imap1(1)));
@@ -475,9 +480,11 @@ int apply_ip_rhf(gfcc_ctx *c, const SysBatch &b, double *work) {
     GFCC_TRY(ring(c->rM2, c->rM2e, imap1(C2), imap2(C2, 1, ov * C2), imap1(C2), imap2(C2, 1, ov * C2)));
     GFCC_TRY(ring(c->rM3, c->rM3e, imap2(v, C2, ov * C2), imap2(C2, 1, v * C2), imap1(C2), imap2(C2, 1, ov * C2)));
   }
-  // S1 = U1 [r1u; r2u]
-  GFCC_TRY(product(c->rU1, imap1(o + o2v), imap1(1), c->rU1e, o, C2, o + o2v, r1u, imap1(C2), imap1(1), 0.0, S1,
+  // S1 = U1 [r1u; r2u] (two products likewise: the Fock diagonal is far above the rest of its row)
+  GFCC_TRY(product(c->rU1 + o, imap1(o + o2v), imap1(1), c->rU1e, o, C2, o2v, r2u, imap1(C2), imap1(1), 0.0, S1,
                    imap1(C2), imap1(1)));
+  GFCC_TRY(gemm_f64(st, o, C2, o, 1.0, c->rU1, imap1(o + o2v), imap1(1), r1u, imap1(C2), imap1(1), 1.0, S1, imap1(C2),
+                    imap1(1)));
   rhf_epilogue_kernel<<<grid1d(dim * b.nsys), 256, 0, st>>>(b, dim, C2, r1u, S1);
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;

@@ -6,6 +6,15 @@
 
 namespace gfcc {
 
+// Entries of a digit-plane product that are to be summed in FP64 instead: (row, column) of the first min(count, cap).
+// With more than cap of them the whole product is (kernels of the other way then return at once).
+struct GuardList {
+  unsigned *count = nullptr;
+  int2 *at = nullptr;
+  double *value = nullptr;
+  unsigned cap = 0;
+};
+
 // D[m][n] = alpha * sum_k A[m][k] B[n][k] + beta * D[m][n]; A: M x K, B: N x K (BF16, K-major,
 // row strides lda / ldb multiples of 8 elements, 16-byte aligned), D: FP32 row-major.
 // nsplit > 1 splits K: partial sum z goes to D + z * split_stride (with beta != 0 each partial
@@ -22,7 +31,12 @@ int umma_splits(int K, int nsplit);
 int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, int SA, const int *eA,
                    const __nv_bfloat16 *Bdig, long long plB, int SB, const int *eB, long long ld, int M, int N, int K,
                    int P, int bits, double alpha, double beta, double *C, IMap cm, IMap cn, long long n0,
-                   double *work, long long m0 = 0);
+                   double *work, long long m0 = 0, const GuardList *gate = nullptr);
+// Appends to the list the entries (m0 + m, n0 + n) whose sum over k of A[m][k] B[n][k] (planes of magnitudes, row stride ld)
+// is neither zero nor from theta up to a finite value.  `work` holds emu_guard_work_bytes.
+int emu_guard(cudaStream_t st, const __nv_bfloat16 *A, const __nv_bfloat16 *B, long long ld, int M, int N, int K,
+              float theta, const GuardList &list, long long m0, long long n0, float *work);
+long long emu_guard_work_bytes(long long M, long long N, long long K);
 long long emu_fused_work_bytes(long long M, long long N, long long K);
 bool emu_fused_takes(int SA, int SB, int P);   // digit counts and level that emu_gemm_fused evaluates
 // Tile autotuning (on by default): the first call of each GEMM shape with beta == 0 times the

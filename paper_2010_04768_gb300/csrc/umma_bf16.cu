@@ -244,11 +244,29 @@ __device__ __forceinline__ void store_block(float *buf, const float (&v)[32], fl
   __syncwarp();
 }
 
-template <int BN, int ST>
+// GUARD: the outputs are not stored; those beside [theta, infinity) and not zero are listed (emu_guard)
+struct GuardArgs {
+  GuardList list;
+  float theta = 0.0f;
+  int m0 = 0, n0 = 0;
+};
+
+// mask: which of the 32 entries (row, col ..) go on the list
+__device__ __forceinline__ void guard_append(const GuardArgs &g, unsigned mask, int row, int col) {
+  const unsigned n = __popc(mask);
+  if (n == 0 || *reinterpret_cast<volatile unsigned *>(g.list.count) > g.list.cap) return;
+  unsigned i = atomicAdd(g.list.count, n);
+  for (; mask != 0; mask &= mask - 1, i++)
+    if (i < g.list.cap) g.list.at[i] = make_int2(g.m0 + row, g.n0 + col + __ffs(mask) - 1);
+}
+
+__device__ __forceinline__ bool guard_hit(float v, float theta) { return v != 0.0f && !(v >= theta && v < 1e30f); }
+
+template <int BN, int ST, bool GUARD = false>
 __global__ void __launch_bounds__(THREADS, 1)
     umma_bf16_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, float *D,
                           long long ldd, int M, int N, int K, float alpha, float beta, int kb_per_split,
-                          long long split_stride, UmmaCtl ctl) {
+                          long long split_stride, UmmaCtl ctl, GuardArgs guard) {
   chain_start();
   constexpr int STAGES = Tile<BN, ST>::STAGES, A_BYTES = Tile<BN, ST>::A_BYTES,
                 STAGE_BYTES = Tile<BN, ST>::STAGE_BYTES;
@@ -353,7 +371,16 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int c0 = 0; c0 < BN && n0 + c0 < N && row0 < M; c0 += 32) {
       float v[32];
       tmem_ld_32(tmem + ((unsigned)(warp * 32) << 16) + c0, v);
-      store_block(buf, v, alpha, beta, D, ldd, row0, M, n0 + c0, N);
+      if constexpr (GUARD) {
+        unsigned mask = 0;
+#pragma unroll
+        for (int i = 0; i < 32; i++)
+          if (row0 + lane < M && n0 + c0 + i < N && guard_hit(v[i], guard.theta)) mask |= 1u << i;
+        guard_append(guard, mask, row0 + lane, n0 + c0);
+        __syncwarp();
+      } else {
+        store_block(buf, v, alpha, beta, D, ldd, row0, M, n0 + c0, N);
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -784,6 +811,8 @@ struct EmuArgs {
   double *C, *part;
   IMap rm, cm;                  // row / column maps of C
   long long r0g, c0g;           // first row / column index
+  const unsigned *gate;         // nothing is done when *gate > gate_cap (nullptr: always)
+  unsigned gate_cap;
   UmmaCtl ctl;
 };
 
@@ -865,6 +894,7 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
     umma_emu_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ EmuArgs a) {
   using T = EmuTile<BN>;
+  if (a.gate != nullptr && *a.gate > a.gate_cap) return;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char *smA = smem, *smB = smem + EMU_A_SLOTS * EMU_A_BYTES;
@@ -1120,7 +1150,8 @@ __global__ void __launch_bounds__(EmuTile<BN>::THREADS, 1)
 // C = alpha 2^(eA + eB) sum_z part[z] + beta C (the K splits of umma_emu_kernel)
 __global__ void emu_split_reduce_kernel(const double *part, int nz, int M, int N, const int *eA, const int *eB,
                                         double alpha, double beta, double *C, IMap cm, IMap cn, long long m0g,
-                                        long long n0g) {
+                                        long long n0g, const unsigned *gate, unsigned gate_cap) {
+  if (gate != nullptr && *gate > gate_cap) return;
   const long long tot = (long long)M * N;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
     const int m = (int)(t / N), n = (int)(t - (long long)m * N);
@@ -1210,10 +1241,10 @@ int g_persist_mode = 0;
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int, int, int>, int> g_tune;
 
-template <int BN, int ST>
+template <int BN, int ST, bool GUARD = false>
 int launch_umma_st(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const __nv_bfloat16 *B, long long ldb,
                    float *D, long long ldd, int M, int N, int K, float alpha, float beta, int nsplit, int kbs,
-                   long long split_stride) {
+                   long long split_stride, const GuardArgs &guard = GuardArgs()) {
   UmmaCtl ctl;
   GFCC_TRY(umma_ctl(&ctl));
   CUtensorMap ma, mb;
@@ -1223,7 +1254,7 @@ int launch_umma_st(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const
   int dev = 0;
   GFCC_CUDA(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64 || !attr[dev]) {
-    GFCC_CUDA(cudaFuncSetAttribute(umma_bf16_gemm_kernel<BN, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    GFCC_CUDA(cudaFuncSetAttribute(umma_bf16_gemm_kernel<BN, ST, GUARD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    Tile<BN, ST>::SMEM_BYTES));
     if (dev >= 0 && dev < 64) attr[dev] = true;
   }
@@ -1232,8 +1263,8 @@ int launch_umma_st(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const
     return GFCC_ERR_ARG;
   }
   dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN, nsplit);
-  GFCC_CUDA(launch_chained(umma_bf16_gemm_kernel<BN, ST>, grid, THREADS, Tile<BN, ST>::SMEM_BYTES, st, ma, mb, D, ldd, M, N, K, alpha, beta, kbs,
-                                                                         split_stride, ctl));
+  GFCC_CUDA(launch_chained(umma_bf16_gemm_kernel<BN, ST, GUARD>, grid, THREADS, Tile<BN, ST>::SMEM_BYTES, st, ma, mb, D,
+                           ldd, M, N, K, alpha, beta, kbs, split_stride, ctl, guard));
   GFCC_LAUNCH_CHECK();
   return GFCC_OK;
 }
@@ -1531,7 +1562,7 @@ bool emu_fused_takes(int SA, int SB, int P) {
 int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, int SA, const int *eA,
                    const __nv_bfloat16 *Bdig, long long plB, int SB, const int *eB, long long ld, int M, int N, int K,
                    int P, int bits, double alpha, double beta, double *C, IMap cm, IMap cn, long long n0,
-                   double *work, long long m0) {
+                   double *work, long long m0, const GuardList *gate) {
   if (M <= 0 || N <= 0) return GFCC_OK;
   if (!emu_fused_takes(SA, SB, P) || bits < 1 || bits > 7 || K <= 0 || (ld % 8) ||
       (reinterpret_cast<uintptr_t>(Adig) & 15) || (reinterpret_cast<uintptr_t>(Bdig) & 15) || (plA % 8) ||
@@ -1574,6 +1605,8 @@ int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, in
   a.alpha_mul = pow2 ? 1.0 : alpha;
   GFCC_TRY(umma_ctl(&a.ctl));
   a.part = a.nz > 1 ? work : nullptr;
+  a.gate = gate != nullptr ? gate->count : nullptr;
+  a.gate_cap = gate != nullptr ? gate->cap : 0;
   if ((long long)a.nM * a.nN * a.nz > 0x7fffffffLL || a.kc < 1) {
     set_error("emu_gemm_fused: too many tiles (M=%d, N=%d)", M, N);
     return GFCC_ERR_ARG;
@@ -1586,7 +1619,65 @@ int emu_gemm_fused(cudaStream_t st, const __nv_bfloat16 *Adig, long long plA, in
   GFCC_TRY(pl.bn == 64 ? launch_emu<64>(st, ma, mb, a) : launch_emu<32>(st, ma, mb, a));
   if (a.nz > 1) {
     emu_split_reduce_kernel<<<grid1d((long long)M * N), 256, 0, st>>>(work, a.nz, a.M, a.N, a.eA, a.eB, alpha, beta, C,
-                                                                       a.rm, a.cm, a.r0g, a.c0g);
+                                                                       a.rm, a.cm, a.r0g, a.c0g, a.gate, a.gate_cap);
+    GFCC_LAUNCH_CHECK();
+  }
+  return GFCC_OK;
+}
+
+namespace {
+// K splits of the sum of magnitudes: few tiles and a long K would leave SMs idle
+int guard_splits(long long M, long long N, long long K) {
+  const long long bn = N <= 64 ? 64 : (N <= 128 ? 128 : 256), nk = (K + BK - 1) / BK;
+  const long long tiles = ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
+  return umma_splits((int)K, (int)std::max<long long>(1, std::min<long long>(nk / 4, 2 * EMU_SMS / tiles)));
+}
+
+__global__ void guard_sum_kernel(const float *part, int nsplit, int M, int N, GuardArgs g) {
+  const long long tot = (long long)M * N;
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < tot; t += (long long)gridDim.x * blockDim.x) {
+    float v = 0.0f;
+    for (int z = 0; z < nsplit; z++) v += part[z * tot + t];
+    if (guard_hit(v, g.theta)) guard_append(g, 1u, (int)(t / N), (int)(t % N));
+  }
+}
+
+template <int BN>
+int launch_guard(cudaStream_t st, const __nv_bfloat16 *A, const __nv_bfloat16 *B, long long ld, int M, int N, int K,
+                 int nsplit, int kbs, float *work, const GuardArgs &g) {
+  if (nsplit > 1) return launch_umma<BN>(st, A, ld, B, ld, work, N, M, N, K, 1.0f, 0.0f, nsplit, kbs, (long long)M * N);
+  if (kbs <= 2) return launch_umma_st<BN, 2, true>(st, A, ld, B, ld, nullptr, 0, M, N, K, 1.0f, 0.0f, 1, kbs, 0, g);
+  return launch_umma_st<BN, 0, true>(st, A, ld, B, ld, nullptr, 0, M, N, K, 1.0f, 0.0f, 1, kbs, 0, g);
+}
+}  // namespace
+
+long long emu_guard_work_bytes(long long M, long long N, long long K) {
+  const int nsplit = guard_splits(M, N, K);
+  return nsplit > 1 ? 4LL * nsplit * M * N : 0;
+}
+
+int emu_guard(cudaStream_t st, const __nv_bfloat16 *A, const __nv_bfloat16 *B, long long ld, int M, int N, int K,
+              float theta, const GuardList &list, long long m0, long long n0, float *work) {
+  if (M <= 0 || N <= 0) return GFCC_OK;
+  if (K <= 0 || (ld % 8) || (reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(B) & 15) ||
+      m0 + M > (1LL << 31) - 1 || n0 + N > (1LL << 31) - 1) {
+    set_error("emu_guard: unsupported shape or alignment (M=%d N=%d K=%d)", M, N, K);
+    return GFCC_ERR_ARG;
+  }
+  GFCC_TRY(check_extent_bytes(A, (long long)(M - 1) * ld * 2 + (long long)K * 2, "magnitudes A"));
+  GFCC_TRY(check_extent_bytes(B, (long long)(N - 1) * ld * 2 + (long long)K * 2, "magnitudes B"));
+  const int nsplit = guard_splits(M, N, K), nk = (K + BK - 1) / BK, kbs = (nk + nsplit - 1) / nsplit;
+  if (nsplit > 1) GFCC_TRY(check_extent_bytes(work, emu_guard_work_bytes(M, N, K), "partial sums of magnitudes"));
+  GuardArgs g;
+  g.list = list;
+  g.theta = theta;
+  g.m0 = (int)m0;
+  g.n0 = (int)n0;
+  GFCC_TRY(N <= 64    ? launch_guard<64>(st, A, B, ld, M, N, K, nsplit, kbs, work, g)
+           : N <= 128 ? launch_guard<128>(st, A, B, ld, M, N, K, nsplit, kbs, work, g)
+                      : launch_guard<256>(st, A, B, ld, M, N, K, nsplit, kbs, work, g));
+  if (nsplit > 1) {
+    guard_sum_kernel<<<grid1d((long long)M * N), 256, 0, st>>>(work, nsplit, M, N, g);
     GFCC_LAUNCH_CHECK();
   }
   return GFCC_OK;

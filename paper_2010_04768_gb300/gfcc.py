@@ -85,6 +85,9 @@ def load():
     fp = ctypes.POINTER(ctypes.c_float)
     lib.gfcc_selftest_gemm_bf16.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, fp, fp, fp]
     lib.gfcc_selftest_gemm_bf16.restype = ctypes.c_int
+    lib.gfcc_selftest_gemm_planes.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, dp, dp, ctypes.c_double,
+                                              ctypes.c_int, dp]
+    lib.gfcc_selftest_gemm_planes.restype = ctypes.c_int
     lib.gfcc_selftest_host_wait.argtypes = [ctypes.c_double]
     lib.gfcc_selftest_host_wait.restype = ctypes.c_int
     lib.gfcc_selftest_gemm_f64emu.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, dp, dp, ctypes.c_int,
@@ -179,6 +182,16 @@ def selftest_gemm_f64emu(A: np.ndarray, B: np.ndarray, S: int = 8, P: int = 9) -
     C = np.zeros((M, N), dtype=np.float64)
     _check(load().gfcc_selftest_gemm_f64emu(M, N, K, _dp(A), _dp(B), S, P, _dp(C)))
     return C
+
+
+def selftest_gemm_planes(A: np.ndarray, B: np.ndarray, mode: int = 1, C: np.ndarray | None = None) -> np.ndarray:
+    """A @ B.T (+ C) from the digit planes of FP64 contractions (mode 0: alone, 1: guarded, 2: guarded, A split first)."""
+    A, B = _f64(A), _f64(B)
+    M, K = A.shape
+    N = B.shape[0]
+    out = np.zeros((M, N)) if C is None else np.array(C, dtype=np.float64)
+    _check(load().gfcc_selftest_gemm_planes(M, N, K, _dp(A), _dp(B), 0.0 if C is None else 1.0, mode, _dp(out)))
+    return out
 
 
 def selftest_host_wait(busy_s: float):
