@@ -695,6 +695,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
     *consumed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  // The allocation reaches into the peer's SM, so both CTAs of the pair have to be running before either asks for it: a
+  // CTA that asked while its peer's SM was still held by another stream's kernel waited without end, about once in 150
+  // solves of four streams.
+  cluster_sync_all();
   if (warp == 0) {   // TMEM of both CTAs: 256 FP32 columns x 128 lanes each (one warp per CTA)
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS));
@@ -773,6 +777,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   if (warp == 0) {
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS));
   }
+  // and stay until both have given it back
+  cluster_sync_all();
 }
 
 // ---------------------------------------------------------------------------------------------
