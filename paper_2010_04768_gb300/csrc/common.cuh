@@ -65,10 +65,8 @@ struct CallScope {
   CallScope(const CallScope &) = delete;
   CallScope &operator=(const CallScope &) = delete;
 };
-// Whether another thread's call shares the GPU (or will: gfcc_solve_batch counts as one beside its threads' calls).
-// Then launches are plain ones, no tile is chosen from timings, and products stay on one-CTA tiles: batches of
-// mixed-precision solves on four streams stalled now and then with chained launches, CTA-pair tiles and timings taken
-// beside other streams, and which of these did it is not known.
+// Whether another thread's call shares the GPU (or will: gfcc_solve_batch counts as one beside its threads' calls).  Then
+// no tile is chosen from timings, which the other calls' kernels would be part of.
 bool concurrent_calls();
 
 // Chained launches: the kernels of an Arnoldi step follow one another with some microseconds of work each, so the
@@ -95,7 +93,7 @@ static inline cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, di
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = concurrent_calls() ? 0 : 1;   // without its predecessor's overlap chain_start does nothing
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 

@@ -280,7 +280,7 @@ int launch_contract(const Contract &c, int kcluster, long long mt, long long nt,
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = (unsigned)kcluster;
     cfg.attrs = at;
-    cfg.numAttrs = concurrent_calls() ? 1 : 2;
+    cfg.numAttrs = 2;
     GFCC_CUDA(cudaLaunchKernelEx(&cfg, contract_f64_kernel<TM, RM, RN>, c, kcluster));
   }
   GFCC_LAUNCH_CHECK();

@@ -1103,9 +1103,8 @@ int Gmres::solve_t(double tol, int max_iters, int *h_state, int max_cycles, bool
   const bool use_graphs =
       sizeof(T) == sizeof(float) && mixed && c->use_graphs && graphs_ok && !c->prof && st != nullptr;
   if (use_graphs) {
-    if (gnsys != nsys || gchained == concurrent_calls()) {
+    if (gnsys != nsys) {
       drop_graphs();
-      gchained = !concurrent_calls();
       gexec.assign(m, nullptr);
       glaunch.assign(m, 0);
       gnsys = nsys;

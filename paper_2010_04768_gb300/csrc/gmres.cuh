@@ -91,7 +91,7 @@ struct Gmres {
   std::vector<cudaGraphExec_t> gexec;
   std::vector<long long> glaunch;
   int gnsys = -1, gseen = 0;
-  bool gbroken = false, gchained = false;   // gchained: the captured launches are chained (not replayed beside other calls)
+  bool gbroken = false;
   void drop_graphs();
   // y = A x for the batch (nact < 0) or for the nact systems listed in the device array idx (SysBatch::idx)
   template <typename T>

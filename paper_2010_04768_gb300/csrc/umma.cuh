@@ -39,11 +39,12 @@ int emu_guard(cudaStream_t st, const __nv_bfloat16 *A, const __nv_bfloat16 *B, l
 long long emu_guard_work_bytes(long long M, long long N, long long K);
 long long emu_fused_work_bytes(long long M, long long N, long long K);
 bool emu_fused_takes(int SA, int SB, int P);   // digit counts and level that emu_gemm_fused evaluates
-// Tile autotuning (on by default): the first call of each GEMM shape with beta == 0 times the
-// 64 / 128 / 256-column tiles and every later call of the shape uses the fastest.
+// Tile autotuning (on by default): the first call of each GEMM shape with beta == 0 times the tiles that may win (one
+// CTA, CTA pair, persistent, each in three widths), unless other calls share the GPU, and every later call of the shape
+// uses the fastest.
 void umma_set_autotune(bool on);
-// CTA-pair tile (cta_group::2, 256 rows x 128, 192 or 256 columns per pair): 0 timed by the autotuner beside the one-CTA tiles
-// (default), 1 used whenever it applies, 2 never
+// CTA-pair tiles (cta_group::2, 256 rows x 128, 192 or 256 columns per pair): 0 timed by the autotuner beside the one-CTA
+// tiles (default), 1 used whenever they apply, 2 never
 void umma_set_pair_mode(int mode);
 // persistent tile loop (one CTA per SM, two TMEM accumulators): 0 timed by the autotuner (default),
 // 1 always, 2 never

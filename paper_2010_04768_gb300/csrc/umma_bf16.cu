@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     *consumed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {   // TMEM: 256 FP32 columns x 128 lanes for the accumulator
+  if (warp == 0) {   // TMEM: BN FP32 columns x 128 lanes for the accumulator
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(BN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -579,8 +579,8 @@ __global__ void __launch_bounds__(PERSIST_THREADS, 1)
 
 // ---------------------------------------------------------------------------------------------
 // The same product on CTA pairs (tcgen05 cta_group::2): a cluster of two CTAs on two SMs computes a
-// 256 x 256 output tile with M = 256 MMAs.  Each CTA stages its own 128 rows of A and one half (128
-// columns) of the B tile, so per SM the shared memory holds and the tensor core reads half of the B
+// 256 x 256 (192, 128) output tile with M = 256 MMAs.  Each CTA stages its own 128 rows of A and one half of
+// the columns of the B tile, so per SM the shared memory holds and the tensor core reads half of the B
 // tile of the one-CTA kernel: with a 128 x 256 tile per SM the operand traffic through shared
 // memory (TMA writes plus MMA reads, about 1.5x the shared-memory bandwidth at the full MMA rate in
 // the one-CTA kernel) drops to about the bandwidth.  The leader CTA (cluster rank 0) issues the MMAs
@@ -699,7 +699,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
   // CTA that asked while its peer's SM was still held by another stream's kernel waited without end, about once in 150
   // solves of four streams.
   cluster_sync_all();
-  if (warp == 0) {   // TMEM of both CTAs: 256 FP32 columns x 128 lanes each (one warp per CTA)
+  if (warp == 0) {   // TMEM of both CTAs: TMEM_COLS FP32 columns x 128 lanes each (one warp per CTA)
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(TMEM_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
@@ -724,7 +724,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
       *issued = kb + 1;
     }
   } else if (warp == 1 && leader) {
-    // ---------------- MMA issuer (leader only): M = 256 over the pair, N = 256
+    // ---------------- MMA issuer (leader only): M = 256 over the pair, N = PBN
     const unsigned idesc = idesc_bf16(2 * BM, PBN);
     const unsigned long long d0 = smem_desc(smem_u32(smem));
     for (int kb = 0; kb < nk; kb++) {
@@ -1396,8 +1396,7 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
   // the pair kernel needs two row tiles and pays off on wide products with a long K loop; its widths by the waves of
   // 76 pairs (clocks of a tile: a K block's loads at 55 bytes a clock, some 16 a column and 6000 for its ends).
   // 3591 x 1620 x 3591: 192 columns 38 us, 256 columns 50 us; 8000 x 3200 x 8000: 256 columns 257 us, 128 348 us.
-  const bool alone = !concurrent_calls();
-  const bool pair_ok = g_pair_mode != 2 && M > BM && N > 128 && kbs >= 8 && alone;
+  const bool pair_ok = g_pair_mode != 2 && M > BM && N > 128 && kbs >= 8;
   auto pair_cost = [&](int w) {
     const long long tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + w - 1LL) / w) * nsplit;
     return (double)((tiles + 75) / 76) * (kbs * (298.0 + 1.16 * w) + 16.0 * w + 6000.0);
@@ -1413,9 +1412,9 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
   const bool persist_ok = g_persist_mode != 2 && tiles_narrow > 2 * 152;
   // default: the narrowest tile that covers N (wide N keeps the 256-column tile)
   int bn = N <= 64 ? 64 : (N <= 128 ? 128 : 256);
-  if (!alone) {
-    // beside other calls no launch is timed: the one-CTA tile whose busiest SM has the least to do, by the clocks of
-    // pair_cost (without the halved B tile)
+  if (concurrent_calls()) {
+    // beside other calls no launch is timed: a choice made alone, or the tile whose busiest SM has the least to do, by the
+    // clocks of pair_cost (one-CTA tiles without the halved B tile)
     auto cost = [&](int w) {
       const long long tiles = ((M + BM - 1LL) / BM) * ((N + w - 1LL) / w) * nsplit;
       return (double)((tiles + 151) / 152) * (kbs * (298.0 + 2.33 * w) + 16.0 * w + 6000.0);
@@ -1423,6 +1422,9 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
     bn = 64;
     for (int w : {128, 256})
       if (w / 2 < N && cost(w) < cost(bn)) bn = w;
+    if (pair_ok && pair_cost(pair_best) < cost(bn)) bn = TILE_PAIR + pair_best;
+    const int t = umma_tuned_tile(M, N, K, nsplit);
+    if (t) bn = t;
   } else if (g_autotune && beta != 0.0f) {
     // accumulating calls are not timed (they would change D); they reuse a tuned choice if any
     const int t = umma_tuned_tile(M, N, K, nsplit);
