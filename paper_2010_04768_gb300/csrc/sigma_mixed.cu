@@ -312,22 +312,8 @@ __global__ __launch_bounds__(256) void reduce_splits_kernel(const float *part, i
 }
 
 // ---------------------------------------------------------------------------------------- EA
-// y2[m, a, e] of system s (antisymmetric in a, e; zero for a == e) from the packed EA vector
-// (1p a, then i-major 2p1h with pairs a < b)
-__device__ __forceinline__ Cz y2_at(const SysBatch &b, int v, long long Pv, int s, int m, int a, int e) {
-  if (a == e) return {0.0f, 0.0f};
-  const long long lo = a < e ? a : e, hi = a < e ? e : a;
-  const long long mu = v + (long long)m * Pv + pair_index(lo, hi, v);
-  Cz u = load_u(b, s, mu);
-  if (a > e) {
-    u.r = -u.r;
-    u.i = -u.i;
-  }
-  return u;
-}
-
 // The ring and long-K layouts of the 2p1h block in one pass: block (e tile, a tile, (m, s)) holds the
-// 32 x 32 tile Y[a][e] = y2[m, a, e] of system s (antisymmetric: packed a < e, read along e above
+// 32 x 32 tile Y[a][e] = y2[m, a, e] of system s (antisymmetric, zero for a == e: packed a < e, read along e above
 // the diagonal and along a below it, so that reads stay coalesced), then writes, for both planes,
 //   ring   r2e[(a, c)][(m, e)] =  Y[a][e]
 //   long K rk[c][(m, a, e)]     = -Y[a][e]  (= y2[m, e, a])
