@@ -977,14 +977,14 @@ def roofline_entries(prof, spec, peaks, closed_shell=False):
         ("ring_bf16", "tensor", "umma_bf16_gemm_kernel (BF16 ring contraction of the inner sigma)"),
         ("bf16_other", "tensor", "umma_bf16_gemm_kernel + reduce_splits_kernel (the other BF16 products of the "
                                  "inner sigma: oooo, three-body, 1h row)"),
-        ("ring_emu", "tensor", "umma_bf16_gemm_kernel / umma_emu_kernel + combine_int_kernel + finalize_kernel "
+        ("ring_emu", "tensor", "umma_emu_kernel "
                                "(FP64-accurate ring contraction of the refinement residual from BF16 digit planes)"),
         ("emu_other", "tensor", "umma_emu_kernel / umma_bf16_gemm_kernel + digit slicing (the other FP64-accurate "
                                 "products of the residual: oooo / vvvv, three-body, 1h / 1p row)"),
         ("unpack", "hbm", "unpack_ip_kernel / unpack_ea_tile_kernel / digit kernels (packed vectors into the "
                           "contraction layouts)"),
         ("epilogue", "hbm", "epi::ip2_kernel / epi::ea2_kernel (sigma epilogues)"),
-        ("arnoldi", "hbm", "cgs_dots_kernel + cgs_update_norm_kernel (+ vscale) of the Arnoldi step"),
+        ("arnoldi", "hbm", "cgs_dots_kernel + cgs_update_kernel (+ vscale) of the Arnoldi step"),
     ]
     rf = {}
     for ph, bound, kernel in cands:

@@ -429,9 +429,9 @@ __global__ __launch_bounds__(32) void backsolve_kernel(int m, const double *H, c
 // once.  The last block of a system adds up its chunks' partial sums in chunk order and takes
 // what follows from them: coefficients, the test for a second pass.  The Givens update runs beside the scaling of the
 // new vector.
-// At 30 systems of o=27 v=133 (n = 46710, FP32) and 51 vectors the dots take 77 us and the update 57 us (3.9 and
-// 5.3 TB/s of basis read from HBM, the rest from L2); blocks of eight warps, 1.13 and 1.46 waves of them, and w read
-// from L1 between the basis loads took 107 and 78 us.
+// At 51 vectors of a batch of 30 systems of o=27 v=133 (n = 46710, FP32; those still in cycle take part) the dots take
+// 77 us and the update 57 us; blocks of eight warps, 1.13 and 1.46 waves of them, and w read from L1 between the basis
+// loads took 107 and 78 us.
 constexpr int CGS_THREADS = 256, CGS_MIN_CHUNK = 256, CGS_BATCH = 8;
 constexpr int DOT_WARPS = 4, DOT_RUN = 4096;   // FP32 sums of at most DOT_RUN / 32 terms, then FP64
 constexpr int NORM_RUN = 32;                   // of the update's norm (even: a thread takes two elements at a time)
