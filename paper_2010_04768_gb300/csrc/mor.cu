@@ -695,7 +695,7 @@ int mor_expand_impl(gfcc_mor *M, int n_omega, const double *h_om, double eta, in
   }
   int rc = solve_for_sink(c, M->sector, n_omega, h_om, eta, n_orb, h_orb, tol, sink, h_G);
   if (rc < 0) {
-    dfree(sink);
+    if (!c->stuck) dfree(sink);   // else left to the work that still runs
     return rc;
   }
   std::vector<int> status(c->st_status);
