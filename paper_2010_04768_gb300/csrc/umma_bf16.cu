@@ -1442,8 +1442,15 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
     if (best == 0) {
       // first call of this shape: time every tile width that may win (the faster of two launches each, CUDA events on
       // the stream; beta == 0, so the repeated launches leave the same D) and keep the fastest
-      cudaEvent_t ev[3];
-      for (cudaEvent_t &e : ev) GFCC_CUDA(cudaEventCreate(&e));
+      struct Events {
+        cudaEvent_t e[3] = {nullptr, nullptr, nullptr};
+        ~Events() {
+          for (cudaEvent_t x : e)
+            if (x) cudaEventDestroy(x);
+        }
+      } events;
+      cudaEvent_t *ev = events.e;
+      for (cudaEvent_t &x : events.e) GFCC_CUDA(cudaEventCreate(&x));
       float best_ms = 0.0f;
       // 64 columns read the A rows four times as often as 256: not for wide products with a long K loop
       const bool wide = N >= 512 && K >= 512;
@@ -1469,7 +1476,7 @@ int gemm_bf16_tn(cudaStream_t st, const __nv_bfloat16 *A, long long lda, const _
           best_ms = ms;
         }
       }
-      for (cudaEvent_t e : ev) cudaEventDestroy(e);
+      GFCC_TRY(umma_error_check(st));   // no choice is kept from launches that gave up
       std::lock_guard<std::mutex> lk(g_tune_mu);
       g_tune[key] = best;
     }

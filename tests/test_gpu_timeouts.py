@@ -96,6 +96,28 @@ def test_closed_shell_operator():
     g.close()
 
 
+def test_tuning_keeps_no_choice_from_launches_that_gave_up():
+    # a shape of its own whose first call times out: the next one times its tiles again, the one after that does not
+    rng = np.random.default_rng(9)
+    A, B = rng.standard_normal((391, 517), dtype=np.float32), rng.standard_normal((263, 517), dtype=np.float32)
+    n = gfcc.launch_count()
+    gfcc.set_process_option(gfcc.OPT_WAIT_NS, 2000.0)
+    gfcc.set_process_option(gfcc.OPT_TEST_NO_LOADS, 1.0)
+    try:
+        with pytest.raises(gfcc.GFCCError) as e:
+            gfcc.selftest_gemm_bf16(A, B)
+    finally:
+        gfcc.set_process_option(gfcc.OPT_TEST_NO_LOADS, 0.0)
+        gfcc.set_process_option(gfcc.OPT_WAIT_NS, 1e9)
+    assert e.value.code == gfcc.ERR_TIMEOUT
+    tried = gfcc.launch_count() - n
+    n = gfcc.launch_count()
+    first = gfcc.selftest_gemm_bf16(A, B)
+    assert gfcc.launch_count() - n >= tried > 2      # timed again: the tiles, then the product
+    n = gfcc.launch_count()
+    assert np.array_equal(gfcc.selftest_gemm_bf16(A, B), first) and gfcc.launch_count() - n == 1
+
+
 def test_host_wait_gives_up():
     gfcc.selftest_host_wait(0.0)
     gfcc.selftest_host_wait(0.3)
